@@ -15,7 +15,8 @@ LIB_PATH = os.path.join(HERE, "libsteps_gpu.so")
 SOURCES = ["steps_host.cpp", "steps_kernels.cu", "steps_batch.cu", "steps_api.cu", "steps_spec.cpp",
            "steps_server.cpp"]
 # device sources embedded into the library for the run-time compiler (NVRTC)
-EMBEDDED = [("kSrcDeviceH", "steps_device.h"), ("kSrcStepCuh", "steps_step.cuh")]
+EMBEDDED = [("kSrcDeviceH", "steps_device.h"), ("kSrcStepCuh", "steps_step.cuh"),
+            ("kSrcWarpCuh", "steps_warp.cuh")]
 EMBED_CPP = "steps_rtc_sources.cpp"
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

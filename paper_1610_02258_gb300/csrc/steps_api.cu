@@ -64,6 +64,24 @@ __global__ void any_negative(const int32_t *src, int64_t n, uint32_t *flag) {
     if (__any_sync(0xFFFFFFFFu, neg) && (threadIdx.x & 31) == 0) atomicOr(flag, 1u);
 }
 
+// The tiles every tile of a flow launch waits for (CSR): itself and every tile
+// holding a face neighbour of one of its tets. Tiles of B tets in device
+// order; `base` is added to every index.
+void flow_neighbours(const std::vector<int32_t> &nbr_dev, int64_t T, int64_t B, int64_t base,
+                     std::vector<int32_t> &off, std::vector<int32_t> &nb) {
+    std::vector<int32_t> tmp;
+    for (int64_t t = 0; t * B < T; ++t) {
+        tmp.assign(1, (int32_t)(base + t));
+        for (int64_t d = 4 * t * B; d < 4 * std::min(T, (t + 1) * B); ++d) {
+            const int32_t j = nbr_dev[(size_t)d];
+            if (j >= 0 && j / B != t) tmp.push_back((int32_t)(base + j / B));
+        }
+        std::sort(tmp.begin(), tmp.end());
+        off.push_back((int32_t)nb.size());
+        nb.insert(nb.end(), tmp.begin(), std::unique(tmp.begin(), tmp.end()));
+    }
+}
+
 // Launch-form choices of tuned simulations, shared by every simulation of
 // the same compiled kernel, tet count and block size (clones of one
 // prototype, the jobs of a stream): the first one's tuning run decides.
@@ -122,9 +140,9 @@ struct steps_sim {
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     // flow launches (a run's full windows in one launch), per block size: [0]
     // the simulation's, [1] 512 (a tuning candidate when the block is smaller).
-    // Each holds its step kernel, every tile's neighbour tiles (tiles of
-    // `block` tets in device order, CSR), the tiles' finished-window words and
-    // the item counter (d_flow[ntiles]).
+    // Each holds its step kernel, the tiles' finished-window words and the item
+    // counter (d_flow[nwords]) and, for a block-tile kernel, every tile's
+    // neighbour tiles (tiles of `block` tets in device order, CSR).
     struct Flow {
         void *spec = nullptr;  // null with `generic`: the generic kernel's flow form (256-thread blocks)
         bool generic = false;
@@ -133,7 +151,8 @@ struct steps_sim {
         int32_t *d_tnb_off = nullptr;
         int32_t *d_tnb = nullptr;
         uint32_t *d_flow = nullptr;
-        int64_t ntiles = 0;
+        int64_t ntiles = 0;  // items per window
+        int64_t nwords = 0;
         size_t bytes = 0;
     } flow[2];
     int flow_pick = -1;  // flow = 0 (tuned): -1 not yet timed, 0 window launches, 1 + k flow launches of flow[k]
@@ -179,30 +198,23 @@ struct steps_sim {
         void *sp = k == 0 ? spec : (spec ? spec_kernel(model, 512, nullptr) : nullptr);
         const bool generic = k == 0 && !spec;
         if (!sp && !(generic && B == 256)) return STEPS_OK;
-        const int64_t nt = (T + B - 1) / B;
-        std::vector<int32_t> off, nb, tmp;
-        try {
-            off.resize((size_t)nt + 1);
-            for (int64_t t = 0; t < nt; ++t) {
-                tmp.assign(1, (int32_t)t);
-                for (int64_t d = t * B; d < std::min(T, (t + 1) * B); ++d)
-                    for (int f = 0; f < 4; ++f) {
-                        const int32_t j = tab.nbr_dev[(size_t)(4 * d + f)];
-                        if (j >= 0 && j / B != t) tmp.push_back((int32_t)(j / B));
-                    }
-                std::sort(tmp.begin(), tmp.end());
-                tmp.erase(std::unique(tmp.begin(), tmp.end()), tmp.end());
-                off[(size_t)t] = (int32_t)nb.size();
-                nb.insert(nb.end(), tmp.begin(), tmp.end());
+        // a warp-tile kernel publishes per 32 tets and finds the tiles it waits
+        // for from its tets' neighbours: it needs no lists
+        const bool warp = sp && spec_warp_tile(model);
+        const int64_t nt = (T + B - 1) / B, nwords = warp ? nt * (B / 32) : nt;
+        std::vector<int32_t> off, nb;
+        if (!warp) {
+            try {
+                flow_neighbours(tab.nbr_dev, T, B, 0, off, nb);
+                off.push_back((int32_t)nb.size());
+            } catch (const std::bad_alloc &) {
+                set_error("flow tables: out of host memory");
+                return STEPS_ERR_OOM;
             }
-            off[(size_t)nt] = (int32_t)nb.size();
-        } catch (const std::bad_alloc &) {
-            set_error("flow tables: out of host memory");
-            return STEPS_ERR_OOM;
         }
-        if (!cuda_ok(cudaMalloc((void **)&fl.d_tnb_off, off.size() * 4), "flow tables") ||
-            !cuda_ok(cudaMalloc((void **)&fl.d_tnb, nb.size() * 4), "flow tables") ||
-            !cuda_ok(cudaMalloc((void **)&fl.d_flow, ((size_t)nt + 1) * 4), "flow tables")) {
+        if ((!warp && (!cuda_ok(cudaMalloc((void **)&fl.d_tnb_off, off.size() * 4), "flow tables") ||
+                       !cuda_ok(cudaMalloc((void **)&fl.d_tnb, nb.size() * 4), "flow tables"))) ||
+            !cuda_ok(cudaMalloc((void **)&fl.d_flow, ((size_t)nwords + 1) * 4), "flow tables")) {
             cudaFree(fl.d_tnb_off);
             cudaFree(fl.d_tnb);
             cudaFree(fl.d_flow);
@@ -210,15 +222,17 @@ struct steps_sim {
             fl.d_flow = nullptr;
             return STEPS_ERR_OOM;
         }
-        if (!cuda_ok(cudaMemcpy(fl.d_tnb_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice), "flow tables") ||
-            !cuda_ok(cudaMemcpy(fl.d_tnb, nb.data(), nb.size() * 4, cudaMemcpyHostToDevice), "flow tables") ||
-            !cuda_ok(cudaMemset(fl.d_flow, 0, ((size_t)nt + 1) * 4), "flow tables"))
+        if ((!warp &&
+             (!cuda_ok(cudaMemcpy(fl.d_tnb_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice), "flow tables") ||
+              !cuda_ok(cudaMemcpy(fl.d_tnb, nb.data(), nb.size() * 4, cudaMemcpyHostToDevice), "flow tables"))) ||
+            !cuda_ok(cudaMemset(fl.d_flow, 0, ((size_t)nwords + 1) * 4), "flow tables"))
             return STEPS_ERR_CUDA;
         fl.spec = sp;
         fl.generic = generic;
         fl.block = (int)B;
         fl.ntiles = nt;
-        fl.bytes = (off.size() + nb.size() + (size_t)nt + 1) * 4;
+        fl.nwords = nwords;
+        fl.bytes = (off.size() + nb.size() + (size_t)nwords + 1) * 4;
         return STEPS_OK;
     }
 
@@ -271,6 +285,10 @@ struct steps_sim {
         a.Tpad = (int32_t)Tpad;
         a.key0 = (uint32_t)seed;
         a.key1 = (uint32_t)(seed >> 32);
+        for (uint32_t k0 = a.key0, k1 = a.key1, r = 0; r < 10; ++r, k0 += 0x9E3779B9u, k1 += 0xBB67AE85u) {
+            (r & 1 ? a.rk[r / 2].z : a.rk[r / 2].x) = k0;  // Philox key schedule: Weyl steps of the key
+            (r & 1 ? a.rk[r / 2].w : a.rk[r / 2].y) = k1;
+        }
         a.window = window;
         a.window_base = base;
         a.tau_k = tau_k;
@@ -455,13 +473,13 @@ struct steps_sim {
         const int64_t cap = std::max<int64_t>(1, (int64_t)0x7FFFFFFF / ntiles);
         for (int64_t done = 0; done < n;) {
             const int64_t nw = std::min(n - done, cap);
-            if (!cuda_ok(cudaMemsetAsync(d_flow + ntiles, 0, 4, stream), "flow counter")) return STEPS_ERR_CUDA;
+            if (!cuda_ok(cudaMemsetAsync(d_flow + fl.nwords, 0, 4, stream), "flow counter")) return STEPS_ERR_CUDA;
             StepArgs a = args(cur, k_total, nullptr, tab.tau, scale_full);
             FlowArgs f;
             f.tnb_off = fl.d_tnb_off;
             f.tnb = fl.d_tnb;
             f.tile_done = d_flow;
-            f.fetch = d_flow + ntiles;
+            f.fetch = d_flow + fl.nwords;
             f.nwin = (uint32_t)nw;
             f.ntiles = (uint32_t)ntiles;
             rc = fl.generic ? launch_flow(model.dev, a, f, fl.block, stream)
@@ -1282,6 +1300,7 @@ struct steps_batch {
         int32_t *d_tnb = nullptr;
         uint32_t *d_flow = nullptr;
         std::vector<std::pair<int64_t, int64_t>> groups;  // (first work entry, entries)
+        int64_t nwords = 0;
     } fl[4];
     uint64_t flow_launches = 0;
 
@@ -1375,9 +1394,10 @@ struct steps_batch {
         if (!cuda_ok(cudaGetDevice(&dev), "steps_batch: device") ||
             !cuda_ok(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev), "steps_batch: L2 size"))
             return STEPS_ERR_CUDA;
-        std::vector<int32_t> off, nb, tmp;
+        std::vector<int32_t> off, nb;
         std::vector<std::pair<int64_t, int64_t>> groups;
         int64_t nwork = 0;
+        const bool warp = spec_warp_tile(members[0]->model);  // (flow runs on specialised kernels only)
         try {
             int64_t gfirst = 0, gbytes = 0;
             for (steps_sim *m : members) {
@@ -1390,18 +1410,7 @@ struct steps_batch {
                     gbytes = 0;
                 }
                 gbytes += bytes;
-                for (int64_t t = 0; t < tiles; ++t) {
-                    tmp.assign(1, (int32_t)(base + t));
-                    for (int64_t d = t * B; d < std::min(T, (t + 1) * B); ++d)
-                        for (int q = 0; q < 4; ++q) {
-                            const int32_t j = m->tab.nbr_dev[(size_t)(4 * d + q)];
-                            if (j >= 0 && j / B != t) tmp.push_back((int32_t)(base + j / B));
-                        }
-                    std::sort(tmp.begin(), tmp.end());
-                    tmp.erase(std::unique(tmp.begin(), tmp.end()), tmp.end());
-                    off.push_back((int32_t)nb.size());
-                    nb.insert(nb.end(), tmp.begin(), tmp.end());
-                }
+                if (!warp) flow_neighbours(m->tab.nbr_dev, T, B, base, off, nb);
                 nwork += tiles;
             }
             off.push_back((int32_t)nb.size());
@@ -1414,9 +1423,11 @@ struct steps_batch {
             set_error("steps_batch: flow tables do not match the work list");
             return STEPS_ERR_STATE;
         }
-        if (!cuda_ok(cudaMalloc((void **)&f.d_tnb_off, off.size() * 4), "steps_batch: flow tables") ||
-            !cuda_ok(cudaMalloc((void **)&f.d_tnb, nb.size() * 4), "steps_batch: flow tables") ||
-            !cuda_ok(cudaMalloc((void **)&f.d_flow, ((size_t)nwork + 1) * 4), "steps_batch: flow tables")) {
+        // (a warp-tile kernel publishes per 32 tets and needs no lists)
+        const int64_t nwords = warp ? nwork * (b / 32) : nwork;
+        if ((!warp && (!cuda_ok(cudaMalloc((void **)&f.d_tnb_off, off.size() * 4), "steps_batch: flow tables") ||
+                       !cuda_ok(cudaMalloc((void **)&f.d_tnb, nb.size() * 4), "steps_batch: flow tables"))) ||
+            !cuda_ok(cudaMalloc((void **)&f.d_flow, ((size_t)nwords + 1) * 4), "steps_batch: flow tables")) {
             cudaFree(f.d_tnb_off);
             cudaFree(f.d_tnb);
             cudaFree(f.d_flow);
@@ -1424,10 +1435,12 @@ struct steps_batch {
             f.d_flow = nullptr;
             return STEPS_ERR_OOM;
         }
-        if (!cuda_ok(cudaMemcpy(f.d_tnb_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice), "steps_batch") ||
-            !cuda_ok(cudaMemcpy(f.d_tnb, nb.data(), nb.size() * 4, cudaMemcpyHostToDevice), "steps_batch") ||
-            !cuda_ok(cudaMemset(f.d_flow, 0, ((size_t)nwork + 1) * 4), "steps_batch"))
+        if ((!warp &&
+             (!cuda_ok(cudaMemcpy(f.d_tnb_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice), "steps_batch") ||
+              !cuda_ok(cudaMemcpy(f.d_tnb, nb.data(), nb.size() * 4, cudaMemcpyHostToDevice), "steps_batch"))) ||
+            !cuda_ok(cudaMemset(f.d_flow, 0, ((size_t)nwords + 1) * 4), "steps_batch"))
             return STEPS_ERR_CUDA;
+        f.nwords = nwords;
         f.groups = std::move(groups);
         return STEPS_OK;
     }
@@ -1443,13 +1456,13 @@ struct steps_batch {
             const int64_t cap = std::max<int64_t>(1, (int64_t)0x7FFFFFFF / g.second);
             for (int64_t done = 0; done < n;) {
                 const int64_t nw = std::min(n - done, cap);
-                if (!cuda_ok(cudaMemsetAsync(f.d_flow + work[slot(b)].n, 0, 4, stream), "steps_batch: flow counter"))
+                if (!cuda_ok(cudaMemsetAsync(f.d_flow + f.nwords, 0, 4, stream), "steps_batch: flow counter"))
                     return STEPS_ERR_CUDA;
                 FlowArgs a;
                 a.tnb_off = f.d_tnb_off;
                 a.tnb = f.d_tnb;
                 a.tile_done = f.d_flow;
-                a.fetch = f.d_flow + work[slot(b)].n;
+                a.fetch = f.d_flow + f.nwords;
                 a.nwin = (uint32_t)nw;
                 a.ntiles = (uint32_t)g.second;
                 rc = launch_spec_batch_flow(spec[slot(b)], work[slot(b)].d, d_reps, a, (uint32_t)g.first, max_S, b,

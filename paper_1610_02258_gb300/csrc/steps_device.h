@@ -77,6 +77,7 @@ struct StepArgs {
     uint32_t *err;                // device error word
     int32_t T, Tpad;
     uint32_t key0, key1;          // Philox key = seed
+    uint4 rk[5];                  // its round keys: (k0, k1) of rounds 2i and 2i + 1
     uint64_t window;              // window index of this launch (RNG counter)
     const uint64_t *window_base;  // if set, window = *window_base + window (graph replay)
     double tau_k, inv_tau_k;
@@ -88,14 +89,41 @@ struct StepArgs {
     uint32_t scale[kMaxSpecies];  // per-species fixed-point scale for this window length
 };
 
+// Shared memory of one warp of the warp-tile step (steps_warp.cuh): 32
+// consecutive tets, one per lane, of a model with up to kWarpMaxSpecies
+// species.
+constexpr int kWarpMaxSpecies = 12;
+constexpr int kWarpMapCap = 160;    // Philox blocks listed at a time
+constexpr int kWarpQueueCap = 160;  // waiting movers: 31 left over + four words of 32 lanes
+
+template <int SM>
+struct WarpTile {
+    int32_t cnt[SM + 1][32];        // counts; row SM ones (a missing reactant)
+    int32_t trial[SM][32];          // trial counts that differ from the count, and those drawn by bit planes
+    uint4 thr[32];
+    int4 nbr[32];
+    uint4 pre[32];                  // words of the species up to and including each, a byte each (x, y, z); w: all words
+    uint32_t tet[32];
+    union {
+        struct {
+            uint16_t map[kWarpMapCap];  // lane | block-in-tet << 5
+            uint2 q[kWarpQueueCap];     // waiting movers: 31-bit uniform, lane | species << 5 (bit-plane groups: the group)
+        } d;
+        struct {                        // species whose occupancy is to be rounded: the integral up to the
+            uint64_t O[64], tS[64];     // last change and its time (doubles), or after a single event
+            uint16_t ls[64];            // (lane | species << 5, bit 15 set) the change and the time as float
+        } r;
+    };
+};
+
 // Full windows of one simulation in one flow launch (flow_tiles; the batched
 // form: a group of members, batch_flow_tile): one block per item (window q,
 // tile t), q-major; the item (q, t) waits until every tile sharing a face
 // with t, t included, has finished window q - 1.
 struct FlowArgs {
-    const int32_t *tnb_off;  // [ntiles + 1] offsets into tnb of each tile's neighbour tiles
+    const int32_t *tnb_off;  // [ntiles + 1] offsets into tnb of each tile's neighbour tiles (not for warp tiles)
     const int32_t *tnb;      // neighbour tiles (each tile lists itself)
-    uint32_t *tile_done;     // [ntiles] low word of (last window the tile finished + 1)
+    uint32_t *tile_done;     // low word of (last window the tile finished + 1): [ntiles], or one per warp tile
     uint32_t *fetch;         // item counter, zero when the launch starts
     uint32_t nwin;           // windows a.window, a.window + 1, ... (nwin * ntiles < 2^31)
     uint32_t ntiles;

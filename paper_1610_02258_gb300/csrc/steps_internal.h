@@ -16,6 +16,12 @@ static_assert(kMaxSpecies == STEPS_MAX_SPECIES && kMaxReac == STEPS_MAX_REACTION
 
 void set_error(const std::string &msg);
 
+// sizeof(WarpTile<S>) for a species count known at run time
+constexpr size_t warp_tile_bytes(int S) {
+    return sizeof(WarpTile<1>) + (size_t)(S - 1) * (sizeof(WarpTile<2>) - sizeof(WarpTile<1>));
+}
+static_assert(warp_tile_bytes(kWarpMaxSpecies) == sizeof(WarpTile<kWarpMaxSpecies>), "warp tile rows");
+
 // ---------------------------------------------------------------- host objects
 struct HostMesh {
     int64_t nv = 0, nt = 0;
@@ -91,6 +97,8 @@ int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEnt
 std::string spec_program_source(const HostModel &hm, int block);
 // whether the specialised kernels keep the trial counts in StepArgs::trial
 bool spec_global_trial(const HostModel &hm);
+// whether they run on warp tiles: flow launches then wait and publish per 32 tets, whatever the block size
+bool spec_warp_tile(const HostModel &hm);
 
 // steps_api.cu: steps_batch_run in two parts (enqueue every window and the
 // error word's copy; then wait and map the word to a return code), so that

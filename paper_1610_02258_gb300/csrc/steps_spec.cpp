@@ -31,6 +31,7 @@ namespace steps {
 
 extern const char *const kSrcDeviceH;  // steps_device.h, embedded at build time
 extern const char *const kSrcStepCuh;  // steps_step.cuh, embedded at build time
+extern const char *const kSrcWarpCuh;  // steps_warp.cuh, embedded at build time
 
 namespace {
 
@@ -81,6 +82,10 @@ Nvrtc &nvrtc() {
 // Models with many species keep the trial counts in a global buffer: their
 // tile's shared memory then fits more resident blocks per SM.
 bool spec_global_trial(const HostModel &hm) { return hm.dev.S >= 16; }
+
+// Models with few species run on warp tiles (steps_warp.cuh): their loops
+// over species are unrolled.
+bool spec_warp_tile(const HostModel &hm) { return hm.dev.S <= kWarpMaxSpecies; }
 
 namespace {
 
@@ -138,10 +143,101 @@ std::string policy_source(const HostModel &hm, int block) {
     return o.str();
 }
 
+// The generated policy of the warp-tile step. The counts of a tet are read and
+// converted once per sweep; every propensity is then two or three products in
+// registers (the forms above, the same operations in the same order), and one
+// with an absent reactant is exactly 0 by itself.
+std::string warp_policy_source(const HostModel &hm) {
+    const ModelDev &m = hm.dev;
+    std::ostringstream o;
+    o << "namespace steps {\nnamespace {\nstruct SpecModel {\n";
+    o << "    static constexpr bool kExpLeave = " << (hm.leave_exp ? "true" : "false") << ";\n";
+    o << "    __device__ static constexpr int S(const ModelDev &) { return " << m.S << "; }\n";
+    o << "    __device__ static constexpr int R(const ModelDev &) { return " << m.R << "; }\n";
+    o << "    __device__ static constexpr uint32_t diffusive(const ModelDev &) { return " << hex_u32(m.diffusive)
+      << "; }\n";
+    o << "    template <int BLOCK>\n    __device__ static void build(const ModelDev &m, RxnTab &tb) {\n";
+    o << "        build_rxn_tab<BLOCK, 32>(m, tb);\n    }\n";
+    o << "    template <class F>\n    __device__ static void for_changes(const RxnTab &tb, int r, F f) {\n";
+    o << "        RtModel<false>::for_changes(tb, r, f);\n    }\n";
+    o << "    template <int RM, bool MASKED>\n    __device__ __forceinline__ static float sums_of(const ModelDev &m, "
+         "const int32_t *cnt, float inv_nav, uint32_t active, float *psum) {\n";
+    uint32_t used = 0;
+    for (int r = 0; r < m.R; ++r) {
+        if (m.reac[r].ia < m.S) used |= 1u << m.reac[r].ia;
+        if (m.reac[r].ib < m.S && m.reac[r].type == kOrder2) used |= 1u << m.reac[r].ib;
+    }
+    for (int s = 0; s < m.S; ++s)
+        if ((used >> s) & 1u) o << "        const float x" << s << " = __int2float_rn(cnt[" << s * 32 << "]);\n";
+    o << "        float a0 = 0.0f, ar;\n";
+    for (int r = 0; r < m.R; ++r) {
+        const ReacDesc &d = m.reac[r];
+        const std::string k = "m.reac[" + std::to_string(r) + "].k", x = "x" + std::to_string(d.ia);
+        o << "        ar = ";
+        switch (d.type) {
+        case kOrder0: o << "__fdiv_rn(" << k << ", inv_nav)"; break;
+        case kOrder1: o << "__fmul_rn(" << k << ", " << x << ")"; break;
+        case kOrder2:
+            o << "__fmul_rn(__fmul_rn(__fmul_rn(" << k << ", inv_nav), " << x << "), x" << d.ib << ")";
+            break;
+        default:
+            o << "__fmul_rn(__fmul_rn(__fmul_rn(" << k << ", inv_nav), " << x << "), __int2float_rn(cnt["
+              << d.ib * 32 << "] - 1))";
+            break;
+        }
+        o << ";\n        if (MASKED && !((active >> " << r << ") & 1u)) ar = 0.0f;\n";
+        o << "        psum[" << r << "] = a0 = __fadd_rn(a0, ar);\n";
+    }
+    o << "        return a0;\n    }\n";
+    o << "    template <int RM>\n    __device__ __forceinline__ static float sums(const RxnTab &, const ModelDev &m, "
+         "const int32_t *cnt, float inv_nav, uint32_t active, bool masked, float *psum) {\n"
+         "        return masked ? sums_of<RM, true>(m, cnt, inv_nav, active, psum)\n"
+         "                      : sums_of<RM, false>(m, cnt, inv_nav, active, psum);\n    }\n";
+    o << "    template <int RM>\n    __device__ __forceinline__ static float first_sums(const RxnTab &tb, const "
+         "ModelDev &m, const int32_t *cnt, float inv_nav, uint32_t active, bool masked, float *psum) {\n"
+         "        const float a0 = sums<RM>(tb, m, cnt, inv_nav, active, masked, psum);\n"
+         "        if (a0 <= 3.0e38f) return a0;\n"
+         "        float ps[RM];\n"
+         "        const float a1 = careful_sums<RM>(tb, m, cnt, inv_nav, active, ps);\n"
+         "        for (int r = 0; r < " << m.R << "; ++r) psum[r] = ps[r];\n"
+         "        return a1;\n    }\n";
+    o << "    template <int RM>\n    __device__ __forceinline__ static int pick(const RxnTab &tb, const ModelDev &m, "
+         "const float *psum, float target, const int32_t *cnt, float inv_nav, uint32_t active) {\n"
+         "        int n = 0;\n"
+         "#pragma unroll\n"
+         "        for (int r = 0; r < " << m.R << "; ++r) n += psum[r] <= target ? 1 : 0;\n"
+         "        return n < " << m.R << " ? n : last_positive_tab(tb, m, cnt, inv_nav, active);\n    }\n";
+    o << "};\n}  // namespace\n}  // namespace steps\n";
+    return o.str();
+}
+
 int reaction_bucket(int R) { return R <= 8 ? 8 : R <= 16 ? 16 : R <= 24 ? 24 : 32; }
 
 std::string program_source(const HostModel &hm, int block) {
     std::ostringstream o;
+    const std::string b = std::to_string(block);
+    if (spec_warp_tile(hm)) {
+        const std::string args = "<" + b + ", " + std::to_string(std::max(1, hm.dev.R)) + ", " +
+                                 std::to_string(hm.dev.S) + ", steps::SpecModel";
+        const std::string head = "extern \"C\" __global__ void __launch_bounds__(" + b + ", " +
+                                 std::to_string(1024 / block) + ")\n";
+        const std::string member = "const steps::BlockWork *__restrict__ work, const steps::RepEntry *__restrict__ reps, ";
+        o << "#include \"steps_warp.cuh\"\n" << warp_policy_source(hm);
+        o << head << "steps_spec_step(const __grid_constant__ steps::ModelDev m, const __grid_constant__ "
+          << "steps::StepArgs a) {\n    steps::warp_step" << args << ">(m, a, (int64_t)blockIdx.x);\n}\n";
+        o << head << "steps_spec_flow(const __grid_constant__ steps::ModelDev m, const __grid_constant__ "
+          << "steps::StepArgs a, const __grid_constant__ steps::FlowArgs f) {\n    steps::warp_step" << args
+          << ", 1>(m, a, 0, &f);\n}\n";
+        o << head << "steps_spec_batch(" << member << "int32_t prefetch) {\n"
+          << "    steps::batch_member<" << b << ">(work, reps, prefetch, [](const steps::ModelDev &m, const "
+          << "steps::StepArgs &a, int64_t tile) { steps::warp_step" << args << ">(m, a, tile); });\n}\n";
+        o << head << "steps_spec_batch_flow(" << member << "const __grid_constant__ steps::FlowArgs f, uint32_t work0, "
+          << "int32_t prefetch) {\n"
+          << "    steps::batch_flow_member<" << b << ">(work, reps, f, work0, prefetch, [&f](const steps::ModelDev &m, "
+          << "const steps::StepArgs &a, int64_t tile, uint32_t q, uint32_t dep) { steps::warp_step" << args
+          << ", 2>(m, a, tile, &f, q, dep); });\n}\n";
+        return o.str();
+    }
     // models with many species keep trial counts in global memory; at 256
     // threads their tiles then fit five resident blocks per SM with a 32-entry
     // block map and 48 registers per thread
@@ -179,7 +275,7 @@ struct Compiled {
     size_t smem_set_flow = 0;           // the flow kernel
     size_t smem_set_batch_flow = 0;     // the batched flow kernel
     size_t smem_set_batch = 0;          // and the batched one
-    bool global_trial = false;          // trial counts in StepArgs::trial, not shared memory
+    size_t smem = 0;                    // dynamic shared memory per block
 };
 
 std::mutex g_mu;
@@ -206,9 +302,9 @@ Compiled *compiled(const HostModel &hm, int block, std::string *why) {
         return it->second.get();
     }
     nvrtc_program prog = nullptr;
-    const char *hdr_src[2] = {kSrcDeviceH, kSrcStepCuh};
-    const char *hdr_name[2] = {"steps_device.h", "steps_step.cuh"};
-    if (nv.create(&prog, src.c_str(), "steps_spec.cu", 2, hdr_src, hdr_name) != 0) {
+    const char *hdr_src[3] = {kSrcDeviceH, kSrcStepCuh, kSrcWarpCuh};
+    const char *hdr_name[3] = {"steps_device.h", "steps_step.cuh", "steps_warp.cuh"};
+    if (nv.create(&prog, src.c_str(), "steps_spec.cu", 3, hdr_src, hdr_name) != 0) {
         if (why) *why = "nvrtcCreateProgram failed";
         g_cache[src] = nullptr;
         return nullptr;
@@ -236,7 +332,9 @@ Compiled *compiled(const HostModel &hm, int block, std::string *why) {
         return nullptr;
     }
     auto c = std::make_shared<Compiled>();
-    c->global_trial = spec_global_trial(hm);
+    const size_t S = (size_t)hm.dev.S;
+    c->smem = spec_warp_tile(hm) ? (size_t)(block / 32) * warp_tile_bytes(hm.dev.S)
+                                 : (S + 1 + (spec_global_trial(hm) ? 0 : S)) * (size_t)block * sizeof(int32_t);
     if (cudaLibraryLoadData(&c->lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0) != cudaSuccess ||
         cudaLibraryGetKernel(&c->kern, c->lib, "steps_spec_step") != cudaSuccess ||
         cudaLibraryGetKernel(&c->kern_batch, c->lib, "steps_spec_batch") != cudaSuccess ||
@@ -274,7 +372,7 @@ int launch_spec(void *spec, const ModelDev &m, const StepArgs &a, int block, voi
     if (a.T <= 0) return STEPS_OK;
     Compiled *c = static_cast<Compiled *>(spec);
     const void *fn = (const void *)c->kern;
-    const size_t smem = ((size_t)m.S + 1 + (c->global_trial ? 0 : (size_t)m.S)) * (size_t)block * sizeof(int32_t);
+    const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set)) return STEPS_ERR_CUDA;
     StepArgs b = a;
     if (b.prefetch) b.prefetch = prefetch_distance(fn, block, smem);
@@ -304,7 +402,7 @@ int launch_spec_flow(void *spec, const ModelDev &m, const StepArgs &a, const Flo
     if (a.T <= 0 || f.nwin == 0) return STEPS_OK;
     Compiled *c = static_cast<Compiled *>(spec);
     const void *fn = (const void *)c->kern_flow;
-    const size_t smem = ((size_t)m.S + 1 + (c->global_trial ? 0 : (size_t)m.S)) * (size_t)block * sizeof(int32_t);
+    const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set_flow)) return STEPS_ERR_CUDA;
     int per_sm = 0, dev = 0, sms = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, smem) != cudaSuccess ||
@@ -334,7 +432,7 @@ int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, co
     if (f.nwin == 0 || f.ntiles == 0) return STEPS_OK;
     Compiled *c = static_cast<Compiled *>(spec);
     const void *fn = (const void *)c->kern_batch_flow;
-    const size_t smem = ((size_t)S + 1 + (c->global_trial ? 0 : (size_t)S)) * (size_t)block * sizeof(int32_t);
+    const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set_batch_flow)) return STEPS_ERR_CUDA;
     int32_t prefetch = prefetch_distance(fn, block, smem);
     FlowArgs ff = f;
@@ -353,7 +451,7 @@ int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEnt
     if (nblocks <= 0) return STEPS_OK;
     Compiled *c = static_cast<Compiled *>(spec);
     const void *fn = (const void *)c->kern_batch;
-    const size_t smem = ((size_t)S + 1 + (c->global_trial ? 0 : (size_t)S)) * (size_t)block * sizeof(int32_t);
+    const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set_batch)) return STEPS_ERR_CUDA;
     int32_t prefetch = prefetch_distance(fn, block, smem);
     void *args[3] = {(void *)&work, (void *)&reps, (void *)&prefetch};

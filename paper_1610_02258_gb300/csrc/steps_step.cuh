@@ -138,14 +138,15 @@ struct RxnTab {
     uint32_t need[kMaxReac];
 };
 
-template <int BLOCK>
+// BLOCK threads fill it; STRIDE: entries of a count row.
+template <int BLOCK, int STRIDE = BLOCK>
 __device__ __forceinline__ void build_rxn_tab(const ModelDev &m, RxnTab &tb) {
     for (int r = threadIdx.x; r < m.R; r += BLOCK) {
         const ReacDesc &d = m.reac[r];
         const uint32_t fl = (uint32_t)d.sub | (d.type == kOrder2 || d.type == kDimer ? 0x100u : 0u) |
                             (d.type == kOrder0 ? 0x200u : 0u);
-        tb.p[r] = make_float4(d.k, __uint_as_float((uint32_t)(d.ia * BLOCK * 4)),
-                              __uint_as_float((uint32_t)(d.ib * BLOCK * 4)), __uint_as_float(fl));
+        tb.p[r] = make_float4(d.k, __uint_as_float((uint32_t)(d.ia * STRIDE * 4)),
+                              __uint_as_float((uint32_t)(d.ib * STRIDE * 4)), __uint_as_float(fl));
         uint32_t w[4] = {0u, 0u, 0u, 0u};
         for (int q = 0; q < d.nchg; ++q) {
             w[q >> 2] |= (uint32_t)(uint8_t)d.chg_s[q] << (8 * (q & 3));
@@ -990,9 +991,9 @@ __device__ __forceinline__ void flow_tiles(const ModelDev &m, const StepArgs &a,
 // its model and window arguments from the device table into shared memory
 // (cur/nxt by the member's buffer parity) and runs the tile body. A member
 // whose windows are done returns at once (block-uniform).
-template <int BLOCK, int RM, class P>
-__device__ __forceinline__ void batch_tile(const BlockWork *__restrict__ work, const RepEntry *__restrict__ reps,
-                                           int32_t prefetch) {
+template <int BLOCK, class F>
+__device__ __forceinline__ void batch_member(const BlockWork *__restrict__ work, const RepEntry *__restrict__ reps,
+                                             int32_t prefetch, F step) {
     __shared__ __align__(16) ModelDev t_model;
     __shared__ __align__(16) StepArgs t_args;
     __shared__ int32_t t_tile;
@@ -1014,7 +1015,15 @@ __device__ __forceinline__ void batch_tile(const BlockWork *__restrict__ work, c
         t_tile = bw.tile;
     }
     __syncthreads();
-    step_tile<BLOCK, RM, P>(t_model, t_args, (int64_t)t_tile);
+    step(t_model, t_args, (int64_t)t_tile);
+}
+
+template <int BLOCK, int RM, class P>
+__device__ __forceinline__ void batch_tile(const BlockWork *__restrict__ work, const RepEntry *__restrict__ reps,
+                                           int32_t prefetch) {
+    batch_member<BLOCK>(work, reps, prefetch, [](const ModelDev &m, const StepArgs &a, int64_t tile) {
+        step_tile<BLOCK, RM, P>(m, a, tile);
+    });
 }
 
 // Full windows of a group of batch members in one launch (the batched form of
@@ -1023,9 +1032,10 @@ __device__ __forceinline__ void batch_tile(const BlockWork *__restrict__ work, c
 // window index and buffers). A member whose windows end earlier skips its
 // later items; nothing depends on them (the dependencies stay within a
 // member). f's tile lists and words are indexed by work entry.
-template <int BLOCK, int RM, class P>
-__device__ __forceinline__ void batch_flow_tile(const BlockWork *__restrict__ work, const RepEntry *__restrict__ reps,
-                                                const FlowArgs &f, uint32_t work0, int32_t prefetch) {
+template <int BLOCK, class F>
+__device__ __forceinline__ void batch_flow_member(const BlockWork *__restrict__ work,
+                                                  const RepEntry *__restrict__ reps, const FlowArgs &f, uint32_t work0,
+                                                  int32_t prefetch, F step) {
     __shared__ __align__(16) ModelDev t_model;
     __shared__ __align__(16) StepArgs t_args;
     __shared__ uint32_t s_q, s_dep;
@@ -1061,7 +1071,16 @@ __device__ __forceinline__ void batch_flow_tile(const BlockWork *__restrict__ wo
         t_args.prefetch = prefetch;  // tiles ahead within the member
     }
     __syncthreads();
-    step_tile<BLOCK, RM, P, 2>(t_model, t_args, (int64_t)s_tile, &f, s_q, s_dep);
+    step(t_model, t_args, (int64_t)s_tile, s_q, s_dep);
+}
+
+template <int BLOCK, int RM, class P>
+__device__ __forceinline__ void batch_flow_tile(const BlockWork *__restrict__ work, const RepEntry *__restrict__ reps,
+                                                const FlowArgs &f, uint32_t work0, int32_t prefetch) {
+    batch_flow_member<BLOCK>(work, reps, f, work0, prefetch,
+                             [&f](const ModelDev &m, const StepArgs &a, int64_t tile, uint32_t q, uint32_t dep) {
+                                 step_tile<BLOCK, RM, P, 2>(m, a, tile, &f, q, dep);
+                             });
 }
 
 }  // namespace
