@@ -16,7 +16,7 @@ SOURCES = ["steps_host.cpp", "steps_kernels.cu", "steps_batch.cu", "steps_api.cu
            "steps_server.cpp"]
 # device sources embedded into the library for the run-time compiler (NVRTC)
 EMBEDDED = [("kSrcDeviceH", "steps_device.h"), ("kSrcStepCuh", "steps_step.cuh"),
-            ("kSrcWarpCuh", "steps_warp.cuh")]
+            ("kSrcWarpCuh", "steps_warp.cuh"), ("kSrcListCuh", "steps_list.cuh")]
 EMBED_CPP = "steps_rtc_sources.cpp"
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

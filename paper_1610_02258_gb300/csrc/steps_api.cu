@@ -36,6 +36,14 @@ struct steps_model {
 namespace {
 
 constexpr int kGraphWindows = 16;  // full windows per captured graph (even: buffer parity is restored)
+// The list form runs a state of at most this many listed tets (or, from set
+// counts, non-zero counts) per tet. us per window, block tiles -> list form:
+// 1.03M-tet dendrite, 0.12: 39.8 -> 14.8; 294,780-tet box with 14, 20 and 30
+// species at 0.2, 0.31, 0.49: 19.2 -> 14.2, 23.3 -> 21.0, 27.6 -> 21.9, at
+// 1.0, 1.6, 2.4: 25 -> 42, 35 -> 46, 45 -> 55; 300k-tet dendrite, 0.35: 17 -> 23.
+constexpr double kListFill = 0.25;
+constexpr uint64_t kListWindows = 128;       // windows after which a list is built afresh
+constexpr int64_t kListCheckWindows = 1024;  // windows after which a run looks at the list's length
 constexpr int64_t kFlowTuneWindows = 72;  // windows the launch-form tuning takes (3 rounds of up to 3 groups)
 
 __global__ void scatter_to_device_order(const int32_t *src, int64_t nt, int32_t S, const int32_t *inv_perm,
@@ -54,14 +62,79 @@ __global__ void gather_to_original_order(const int32_t *src, int64_t nt, int32_t
     for (int s = 0; s < S; ++s) dst[s * (size_t)nt + i] = src[s * Tpad + d];
 }
 
+// Species words (StepArgs::tm_cur, tm_nxt) of a count buffer, for the list form:
+// one coalesced pass over the counts.
+__global__ void build_species_words(const int32_t *cnt, int64_t T, size_t Tpad, int32_t S, uint32_t *cur, uint32_t *nxt) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= T) return;
+    uint32_t nz = 0;
+#pragma unroll 4
+    for (int s = 0; s < S; ++s) nz |= cnt[s * Tpad + i] != 0 ? 1u << s : 0u;
+    cur[i] = nz;
+    nxt[i] = 0u;
+}
+
+// The list of the next window: the tets with a species
+// bit that are not sources, a block's together, in order.
+__global__ void build_list(const uint32_t *tm, int64_t T, const uint32_t *srcbits, int32_t *list, uint32_t *n) {
+    __shared__ uint32_t at[9];
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const bool in = i < T && tm[i] != 0u && !(srcbits && ((srcbits[i >> 5] >> (i & 31)) & 1u));
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
+    if (lane == 0) at[warp] = (uint32_t)__popc(m);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t sum = 0;
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t c = at[k];
+            at[k] = sum;
+            sum += c;
+        }
+        at[8] = sum ? atomicAdd(n, sum) : 0u;
+    }
+    __syncthreads();
+    if (in) list[at[8] + at[warp] + __popc(m & ((1u << lane) - 1u))] = (int32_t)i;
+}
+
+// The tets' records, and those with an active order-0 reaction (rmask null:
+// all are active): a bit each and a list (list null: the model has none).
+__global__ void build_sources(const uint32_t *rmask, uint32_t order0, int64_t T, const uint4 *thr, const int32_t *orig,
+                              const float *inv_nav, uint4 *rec, uint32_t *bits, int32_t *list, uint32_t *n) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t act = i < T && rmask ? rmask[i] : 0xFFFFFFFFu;
+    if (i < T)
+        rec[i] = make_uint4(thr[i].w, orig ? (uint32_t)orig[i] : (uint32_t)i, __float_as_uint(inv_nav[i]), act);
+    if (!list) return;
+    const bool in = i < T && (act & order0) != 0u;
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
+    uint32_t at = 0;
+    if (lane == 0 && i < T) {
+        bits[i >> 5] = m;
+        if (m) at = atomicAdd(n, (uint32_t)__popc(m));
+    }
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    if (in) list[at + __popc(m & ((1u << lane) - 1u))] = (int32_t)i;
+}
+
 __global__ void set_u64_kernel(uint64_t *p, uint64_t v) { *p = v; }
 
-// *flag |= 1 if any of src[0..n) is negative (grid-stride; one atomic per warp at most)
+// flag[0] |= 1 if any of src[0..n) is negative; flag[1] += the non-zero ones, if
+// asked for (grid-stride; one atomic per warp at most)
+template <bool COUNT>
 __global__ void any_negative(const int32_t *src, int64_t n, uint32_t *flag) {
     bool neg = false;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    uint32_t nz = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         neg |= src[i] < 0;
+        if (COUNT) nz += src[i] != 0 ? 1u : 0u;
+    }
     if (__any_sync(0xFFFFFFFFu, neg) && (threadIdx.x & 31) == 0) atomicOr(flag, 1u);
+    if (COUNT) {
+        nz = __reduce_add_sync(0xFFFFFFFFu, nz);
+        if (nz && (threadIdx.x & 31) == 0) atomicAdd(flag + 1, nz);
+    }
 }
 
 // The tiles every tile of a flow launch waits for (CSR): itself and every tile
@@ -121,7 +194,7 @@ struct steps_sim {
     int32_t *d_inv_perm = nullptr;  // original id -> device index (null without reordering)
     uint32_t *d_rmask = nullptr;
     std::vector<uint32_t> h_rmask;  // device order
-    uint32_t *d_err = nullptr;      // [2]: window error word, input check flag
+    uint32_t *d_err = nullptr;      // [3]: window error word, input check flag, non-zero input counts
     uint64_t *d_window_base = nullptr;
     int32_t *d_stage = nullptr;     // [S * nt] original-order staging
     int32_t *d_rec = nullptr;       // recording selection (species, then tets)
@@ -130,6 +203,20 @@ struct steps_sim {
     int32_t *d_trial = nullptr;     // [S][Tpad] trial counts for specialised kernels that keep them in global memory
     uint32_t *d_leave[2] = {nullptr, nullptr};  // EXP leave law: [S][Tpad] tables of the full and the last window
     std::string spec_why;           // why there is none
+    // list form (steps_list.cuh): its kernel, and per-simulation buffers
+    void *spec_list = nullptr;
+    uint32_t *d_tm[2] = {nullptr, nullptr};   // [Tpad] species words of both count buffers
+    int32_t *d_list[2] = {nullptr, nullptr};  // [2 Tpad] the lists (a tet is listed twice at most)
+    uint32_t *d_lcnt = nullptr;     // [4] their lengths (StepArgs::lcnt)
+    uint4 *d_tetrec = nullptr;      // [Tpad] the tets' records (StepArgs::rec)
+    int32_t *d_src = nullptr;       // models with order-0 reactions: the sources, a list
+    uint32_t *d_srcbits = nullptr;  // and a bit each
+    bool tm_valid = false;          // the species words match the counts
+    bool list_valid = false;        // the next window's list matches the species words
+    bool src_valid = false;         // the records and the sources match the reaction masks
+    bool listing = false;           // the present run's windows go through the list form
+    uint64_t list_built = 0;        // the window the list was last built for
+    double fill = 0.0;              // listed tets or non-zero counts per tet, last known
     // time
     double t_base = 0.0;
     int64_t k_grid = 0;
@@ -176,6 +263,7 @@ struct steps_sim {
         cudaFree(d_stage);
         cudaFree(d_rec);
         cudaFree(d_trial);
+        free_list();
         cudaFree(d_leave[0]);
         cudaFree(d_leave[1]);
         for (Flow &f : flow) {
@@ -256,11 +344,95 @@ struct steps_sim {
 
     // the global trial buffer the model-specialised kernels of this model need (if any)
     int ensure_trial() {
-        if (d_trial || !spec_global_trial(model)) return STEPS_OK;
+        if (d_trial || !(spec_global_trial(model) || spec_list)) return STEPS_OK;
         if (!cuda_ok(cudaMalloc((void **)&d_trial, (size_t)S * (size_t)Tpad * 4), "trial buffer"))
             return STEPS_ERR_OOM;
         drop_graphs();  // the captured launches hold the old arguments
         return STEPS_OK;
+    }
+
+    void free_list() {
+        for (void **p : {(void **)&d_tm[0], (void **)&d_tm[1], (void **)&d_list[0], (void **)&d_list[1],
+                         (void **)&d_lcnt, (void **)&d_tetrec, (void **)&d_src, (void **)&d_srcbits}) {
+            cudaFree(*p);
+            *p = nullptr;
+        }
+    }
+
+    // the list form's buffers
+    cudaError_t alloc_list() {
+        const size_t n = (size_t)Tpad * 4;
+        cudaError_t e = cudaSuccess;
+        auto get = [&](void **p, size_t bytes) {
+            if (e == cudaSuccess) e = cudaMalloc(p, bytes);
+        };
+        get((void **)&d_tm[0], n);
+        get((void **)&d_tm[1], n);
+        get((void **)&d_list[0], 2 * n);
+        get((void **)&d_list[1], 2 * n);
+        get((void **)&d_lcnt, 16);
+        get((void **)&d_tetrec, 4 * n);
+        if (model.dev.order0) {
+            get((void **)&d_src, n);
+            get((void **)&d_srcbits, n / 32);
+        }
+        if (e != cudaSuccess) free_list();
+        return e;
+    }
+
+    // Before a run: the form of its windows, by what is known of the state.
+    int choose_form() {
+        const bool want = spec_list && opt.flow != 1 && fill <= kListFill;
+        if (want != listing) drop_graphs();
+        listing = want;
+        if (!listing) tm_valid = list_valid = false;  // the other kernels leave them behind
+        return STEPS_OK;
+    }
+
+    // Before windows in the list form: the species words match the counts, the
+    // records and sources the masks, and the list is window k_total's. Windows
+    // append tets in the order their warps meet them; building the list afresh
+    // now and then keeps neighbours together.
+    int prepare_list() {
+        if (!listing || (tm_valid && src_valid && list_valid && k_total - list_built < kListWindows)) return STEPS_OK;
+        const unsigned grid = (unsigned)((T + 255) / 256);
+        if (!tm_valid)
+            build_species_words<<<grid, 256, 0, stream>>>(d_cnt[cur], T, (size_t)Tpad, S, d_tm[cur], d_tm[1 - cur]);
+        if (!cuda_ok(cudaMemsetAsync(d_lcnt, 0, src_valid ? 12 : 16, stream), "tet lists")) return STEPS_ERR_CUDA;
+        if (!src_valid)
+            build_sources<<<grid, 256, 0, stream>>>(d_rmask, model.dev.order0, T, d_thr, d_orig, d_inv_nav, d_tetrec,
+                                                    d_srcbits, d_src, d_lcnt + 3);
+        build_list<<<grid, 256, 0, stream>>>(d_tm[cur], T, d_srcbits, d_list[k_total & 1], d_lcnt + k_total % 3);
+        if (!cuda_ok(cudaGetLastError(), "tet lists")) return STEPS_ERR_CUDA;
+        tm_valid = src_valid = list_valid = true;
+        list_built = k_total;
+        return STEPS_OK;
+    }
+
+    // n full windows in the list form, as long as the state stays sparse: their
+    // number into *done. The list's length is looked at every kListCheckWindows.
+    int list_windows(int64_t n, int64_t *done) {
+        while (listing && *done < n) {
+            const int64_t m = std::min(n - *done, kListCheckWindows);
+            int rc = window_launches(m);
+            if (rc) return rc;
+            *done += m;
+            if (*done < n) {
+                uint32_t c[4];
+                if (!cuda_ok(cudaMemcpyAsync(c, d_lcnt, 16, cudaMemcpyDeviceToHost, stream), "list length") ||
+                    !cuda_ok(cudaStreamSynchronize(stream), "list length"))
+                    return STEPS_ERR_CUDA;
+                fill_from(c);
+                rc = choose_form();
+                if (rc) return rc;
+            }
+        }
+        return STEPS_OK;
+    }
+
+    // the fill from the list's lengths after the last window enqueued
+    void fill_from(const uint32_t c[4]) {
+        if (list_valid) fill = ((double)c[k_total % 3] + (d_src ? 0.5 * (double)c[3] : 0.0)) / (double)T;
     }
 
     void drop_graphs() {
@@ -298,6 +470,14 @@ struct steps_sim {
         a.occ = opt.occupancy;
         a.prefetch = 1;  // the launch sets the distance: half a resident wave
         a.trial = d_trial;
+        a.tm_cur = d_tm[from];
+        a.tm_nxt = d_tm[1 - from];
+        a.rec = d_tetrec;
+        a.list[0] = d_list[0];
+        a.list[1] = d_list[1];
+        a.lcnt = d_lcnt;
+        a.src = d_src;
+        a.srcbits = d_srcbits;
         a.leave = d_leave[0] ? (tau_k == tab.tau ? d_leave[0] : d_leave[1]) : nullptr;
         std::memcpy(a.scale, scale, sizeof(a.scale));
         return a;
@@ -305,6 +485,7 @@ struct steps_sim {
 
     // one window on the model-specialised kernel if there is one, else the generic one
     int launch(const StepArgs &a, cudaStream_t st) const {
+        if (listing) return launch_spec(spec_list, model.dev, a, opt.block, st);
         return spec ? launch_spec(spec, model.dev, a, opt.block, st) : launch_step(model.dev, a, opt.block, st);
     }
 
@@ -316,7 +497,8 @@ struct steps_sim {
             if (rc) return rc;
         }
         StepArgs a = args(cur, k_total, nullptr, tau_k, scale);
-        int rc = launch(a, stream);
+        int rc = prepare_list();
+        if (!rc) rc = launch(a, stream);
         if (rc) return rc;
         ++launches;
         cur = 1 - cur;
@@ -354,6 +536,10 @@ struct steps_sim {
 
     // n full windows: flow launches or window launches (all give the same bits)
     int full_windows(int64_t n) {
+        int64_t listed = 0;
+        if (int rl = list_windows(n, &listed)) return rl;
+        n -= listed;
+        if (n == 0) return STEPS_OK;
         if (opt.flow == 0 && flow_pick < 0 && flow_possible() && n >= kFlowTuneWindows) {
             int64_t used = 0;
             int rc = tune_flow(&used);
@@ -445,6 +631,8 @@ struct steps_sim {
             if (!cuda_ok(cudaGetLastError(), "set window base")) return STEPS_ERR_CUDA;
             ++launches;
             while (n - done >= kGraphWindows) {
+                int rc = prepare_list();
+                if (rc) return rc;
                 if (!cuda_ok(cudaGraphLaunch(graph[cur], stream), "cudaGraphLaunch")) return STEPS_ERR_CUDA;
                 launches += kGraphWindows + 1;
                 done += kGraphWindows;
@@ -453,7 +641,8 @@ struct steps_sim {
         }
         for (; done < n; ++done) {
             StepArgs a = args(cur, k_total, nullptr, tab.tau, scale_full);
-            int rc = launch(a, stream);
+            int rc = prepare_list();
+            if (!rc) rc = launch(a, stream);
             if (rc) return rc;
             ++launches;
             cur = 1 - cur;
@@ -638,7 +827,7 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
     alloc((void **)&s->d_nbr, Tpad * 16);
     alloc((void **)&s->d_thr, Tpad * 16);
     alloc((void **)&s->d_inv_nav, Tpad * 4);
-    alloc((void **)&s->d_err, 8);
+    alloc((void **)&s->d_err, 12);
     alloc((void **)&s->d_window_base, 8);
     alloc((void **)&s->d_stage, S * T * 4);
     if (reordered) {
@@ -663,7 +852,7 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
                       "upload inv_nav") &&
               cuda_ok(cudaMemset(s->d_cnt[0], 0, S * Tpad * 4), "memset") &&
               cuda_ok(cudaMemset(s->d_cnt[1], 0, S * Tpad * 4), "memset") &&
-              cuda_ok(cudaMemset(s->d_err, 0, 8), "memset") && cuda_ok(cudaMemset(s->d_window_base, 0, 8), "memset");
+              cuda_ok(cudaMemset(s->d_err, 0, 12), "memset") && cuda_ok(cudaMemset(s->d_window_base, 0, 8), "memset");
     if (ok && reordered)
         ok = cuda_ok(cudaMemset(s->d_orig, 0, Tpad * 4), "memset") &&
              cuda_ok(cudaMemcpy(s->d_orig, s->tab.perm.data(), T * 4, cudaMemcpyHostToDevice), "upload perm") &&
@@ -683,6 +872,12 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
             return STEPS_ERR_CUDA;
         }
         if (s->spec) {
+            s->spec_list = spec_list_kernel(s->model);
+            if (s->spec_list && (e = s->alloc_list()) != cudaSuccess) {
+                set_error(std::string("steps_sim_create: device allocation failed: ") + cudaGetErrorString(e));
+                cudaGetLastError();
+                return STEPS_ERR_OOM;
+            }
             int rc = s->ensure_trial();
             if (rc) return rc;
         }
@@ -713,6 +908,7 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
     s->seed = seed;
     s->h_rmask = src->h_rmask;
     s->spec = src->spec;
+    s->spec_list = src->spec_list;
     s->spec_why = src->spec_why;
     std::memcpy(s->scale_full, src->scale_full, sizeof(s->scale_full));
     const size_t Tpad = (size_t)s->Tpad, S = (size_t)s->S, T = (size_t)s->T;
@@ -725,7 +921,7 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
     alloc((void **)&s->d_nbr, Tpad * 16);
     alloc((void **)&s->d_thr, Tpad * 16);
     alloc((void **)&s->d_inv_nav, Tpad * 4);
-    alloc((void **)&s->d_err, 8);
+    alloc((void **)&s->d_err, 12);
     alloc((void **)&s->d_window_base, 8);
     alloc((void **)&s->d_stage, S * T * 4);
     if (src->d_orig) {
@@ -734,6 +930,7 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
     }
     if (src->d_rmask) alloc((void **)&s->d_rmask, Tpad * 4);
     if (src->d_trial) alloc((void **)&s->d_trial, S * Tpad * 4);
+    if (src->d_tm[0] && e == cudaSuccess) e = s->alloc_list();
     if (src->d_leave[0]) {
         alloc((void **)&s->d_leave[0], S * Tpad * 4);
         alloc((void **)&s->d_leave[1], S * Tpad * 4);
@@ -749,7 +946,7 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
               cuda_ok(cudaMemcpyAsync(s->d_inv_nav, src->d_inv_nav, Tpad * 4, cudaMemcpyDeviceToDevice, st), "clone") &&
               cuda_ok(cudaMemsetAsync(s->d_cnt[0], 0, S * Tpad * 4, st), "clone") &&
               cuda_ok(cudaMemsetAsync(s->d_cnt[1], 0, S * Tpad * 4, st), "clone") &&
-              cuda_ok(cudaMemsetAsync(s->d_err, 0, 8, st), "clone") &&
+              cuda_ok(cudaMemsetAsync(s->d_err, 0, 12, st), "clone") &&
               cuda_ok(cudaMemsetAsync(s->d_window_base, 0, 8, st), "clone");
     if (ok && src->d_orig)
         ok = cuda_ok(cudaMemcpyAsync(s->d_orig, src->d_orig, Tpad * 4, cudaMemcpyDeviceToDevice, st), "clone") &&
@@ -769,7 +966,8 @@ int steps_sim_device_bytes(const steps_sim *sim, int64_t *bytes) {
     CHECK_NULL(bytes, "steps_sim_device_bytes");
     const int64_t Tpad = sim->Tpad, S = sim->S, T = sim->T;
     *bytes = 2 * S * Tpad * 4 + Tpad * 16 * 2 + Tpad * 4 + 16 + S * T * 4 + (sim->d_orig ? Tpad * 4 + T * 4 : 0) +
-             (sim->d_trial ? S * Tpad * 4 : 0) + (sim->d_leave[0] ? 2 * S * Tpad * 4 : 0) +
+             (sim->d_trial ? S * Tpad * 4 : 0) + (sim->d_tm[0] ? 10 * Tpad * 4 + 16 : 0) +
+             (sim->d_src ? Tpad * 4 + Tpad / 8 : 0) + (sim->d_leave[0] ? 2 * S * Tpad * 4 : 0) +
              (sim->d_rmask ? Tpad * 4 : 0) + (int64_t)(sim->flow[0].bytes + sim->flow[1].bytes);
     return STEPS_OK;
 }
@@ -787,20 +985,24 @@ static int put_counts(steps_sim *sim, int32_t s0, int32_t ns, const int32_t *cou
                  "steps_set_counts: copy"))
         return STEPS_ERR_CUDA;
     // reject negative counts on the device, before anything of the state changes
-    uint32_t neg = 0;
+    uint32_t seen[2] = {0, 0};  // a negative count; non-zero ones
     const int64_t n = (int64_t)ns * (int64_t)T;
-    if (!cuda_ok(cudaMemsetAsync(sim->d_err + 1, 0, 4, sim->stream), "steps_set_counts: check"))
+    if (!cuda_ok(cudaMemsetAsync(sim->d_err + 1, 0, 8, sim->stream), "steps_set_counts: check"))
         return STEPS_ERR_CUDA;
-    any_negative<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, sim->stream>>>(sim->d_stage, n,
-                                                                                               sim->d_err + 1);
+    const unsigned grid = (unsigned)std::min<int64_t>((n + 255) / 256, 4096);
+    if (sim->spec_list) any_negative<true><<<grid, 256, 0, sim->stream>>>(sim->d_stage, n, sim->d_err + 1);
+    else any_negative<false><<<grid, 256, 0, sim->stream>>>(sim->d_stage, n, sim->d_err + 1);
     if (!cuda_ok(cudaGetLastError(), "steps_set_counts: check") ||
-        !cuda_ok(cudaMemcpyAsync(&neg, sim->d_err + 1, 4, cudaMemcpyDeviceToHost, sim->stream), "steps_set_counts: check") ||
+        !cuda_ok(cudaMemcpyAsync(seen, sim->d_err + 1, 8, cudaMemcpyDeviceToHost, sim->stream), "steps_set_counts: check") ||
         !cuda_ok(cudaStreamSynchronize(sim->stream), "steps_set_counts: check"))
         return STEPS_ERR_CUDA;
-    if (neg) {
+    if (seen[0]) {
         set_error("steps_set_counts: negative count");
         return STEPS_ERR_ARG;
     }
+    sim->tm_valid = sim->list_valid = false;
+    // counts of every species replace the state; of one, they add to what is known of it
+    sim->fill = (ns == sim->S ? 0.0 : sim->fill) + seen[1] / (double)T;
     scatter_to_device_order<<<(unsigned)((T + 255) / 256), 256, 0, sim->stream>>>(
         sim->d_stage, (int64_t)T, ns, sim->d_inv_perm, sim->d_cnt[sim->cur] + (size_t)s0 * Tpad, Tpad);
     if (!cuda_ok(cudaGetLastError(), "steps_set_counts: scatter")) return STEPS_ERR_CUDA;
@@ -877,6 +1079,7 @@ int steps_set_reac_mask(steps_sim *sim, int32_t reac, const uint8_t *active) {
             return STEPS_ERR_OOM;
         sim->drop_graphs();  // kernel arguments change
     }
+    sim->src_valid = sim->list_valid = false;
     if (!cuda_ok(cudaStreamSynchronize(sim->stream), "steps_set_reac_mask") ||
         !cuda_ok(cudaMemcpy(sim->d_rmask, sim->h_rmask.data(), T * 4, cudaMemcpyHostToDevice),
                  "steps_set_reac_mask: copy"))
@@ -900,6 +1103,7 @@ int refuse_failed(const steps_sim *sim, const char *who) {
 // Enqueues the windows of Algorithm 1 from the simulation's time to t_end
 // (full windows of tau, then a shortened last window); no synchronisation.
 int enqueue_run(steps_sim *sim, double t_end) {
+    if (int rf = sim->choose_form()) return rf;
     const double tau = sim->tab.tau;
     const bool finite = std::isfinite(tau);
     const double tol = finite ? 1e-9 * tau : 0.0;
@@ -932,10 +1136,12 @@ int enqueue_run(steps_sim *sim, double t_end) {
 // Waits for the simulation's stream and turns the device error word into a
 // return code (and clears it).
 int finish_run(steps_sim *sim, const char *who) {
-    uint32_t err = 0;
+    uint32_t err = 0, c[4];
     if (!cuda_ok(cudaMemcpyAsync(&err, sim->d_err, 4, cudaMemcpyDeviceToHost, sim->stream), "error word") ||
+        (sim->listing && !cuda_ok(cudaMemcpyAsync(c, sim->d_lcnt, 16, cudaMemcpyDeviceToHost, sim->stream), who)) ||
         !cuda_ok(cudaStreamSynchronize(sim->stream), who))
         return STEPS_ERR_CUDA;
+    if (sim->listing) sim->fill_from(c);
     if (err) {
         cudaMemsetAsync(sim->d_err, 0, 4, sim->stream);
         if (err & 4u) {
@@ -1641,6 +1847,7 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
         nfull[j] = k;
         nmax = std::max(nmax, k);
     }
+    for (steps_sim *m : b->members) m->tm_valid = m->list_valid = false;  // the batched kernels leave them behind
     // table for the full windows
     for (size_t j = 0; j < n; ++j) {
         steps_sim *m = b->members[j];
@@ -1904,7 +2111,7 @@ extern "C" int steps_run_noalloc(steps_sim *sim, int32_t *d_counts, double t_end
     {
         const int64_t n = (int64_t)(S * T);
         uint32_t neg = 0;
-        any_negative<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, st>>>(d_counts, n, sc.err + 1);
+        any_negative<false><<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, st>>>(d_counts, n, sc.err + 1);
         if (!cuda_ok(cudaGetLastError(), "steps_run_noalloc: check") ||
             !cuda_ok(cudaMemcpyAsync(&neg, sc.err + 1, 4, cudaMemcpyDeviceToHost, st), "steps_run_noalloc: check") ||
             !cuda_ok(cudaStreamSynchronize(st), "steps_run_noalloc: check"))
@@ -1918,7 +2125,9 @@ extern "C" int steps_run_noalloc(steps_sim *sim, int32_t *d_counts, double t_end
     scatter_to_device_order<<<grid, 256, 0, st>>>(d_counts, (int64_t)T, (int32_t)S, sim->d_inv_perm, buf[0], Tpad);
     if (!cuda_ok(cudaGetLastError(), "steps_run_noalloc: scatter")) return STEPS_ERR_CUDA;
 
-    // the window loop of steps_run (Algorithm 1), with plain launches on the scratch buffers
+    // the window loop of steps_run (Algorithm 1), with plain launches on the scratch buffers (never the list form)
+    if (sim->listing) sim->drop_graphs();
+    sim->listing = sim->tm_valid = sim->list_valid = false;
     const double tau = sim->tab.tau;
     const bool finite = std::isfinite(tau);
     const double tol = finite ? 1e-9 * tau : 0.0;

@@ -85,6 +85,12 @@ struct StepArgs {
     int32_t occ;                  // STEPS_OCC_*
     int32_t prefetch;             // tiles ahead whose tables a block prefetches into L2 (0 = none)
     int32_t *trial;               // [S][Tpad] trial counts, for kernels that keep them in global memory
+    uint32_t *tm_cur, *tm_nxt;    // list form: [T] species bits of cur and nxt, a clear bit means count 0
+    const uint4 *rec;             // [T] last face threshold, RNG key, 1 / (N_A V_L), active reactions
+    int32_t *list[2];             // the tets with a species bit, by window parity (sources left out),
+    uint32_t *lcnt;               // [4]: their number, by window mod 3; and the number of sources
+    const int32_t *src;           // tets with an active order-0 reaction,
+    const uint32_t *srcbits;      // a bit each (nullptr: the model has no order-0 reaction)
     const uint32_t *leave;        // [S][Tpad] EXP leave law: floor(2^31 (1 - exp(-tau_k D_S G_tet))), or nullptr
     uint32_t scale[kMaxSpecies];  // per-species fixed-point scale for this window length
 };
@@ -115,6 +121,39 @@ struct WarpTile {
         } r;
     };
 };
+
+// Shared memory of one warp of the list form (steps_list.cuh): 32 tets, one per lane.
+constexpr int kListMapCap = 64;
+
+template <int SM>
+struct ListTile {
+    int32_t cnt[SM + 1][32];          // counts; row SM ones
+    uint32_t thr_w[32];               // last face threshold
+    uint32_t tet[32];
+    int32_t idx[32];                  // device index (-1: none)
+    uint16_t words[32];               // word-stream molecules
+    union {
+        struct {
+            uint32_t map[kListMapCap];  // lane | block-in-tet << 5 | species of the four words << 12
+            uint2 q[kWarpQueueCap];     // WarpTile
+        } d;
+        struct {
+            uint64_t O[64], tS[64];
+            uint16_t ls[64];
+        } r;
+    };
+};
+
+// Blocks of a launch in the list form over T tets: a warp for every two lines
+// of 32 tets, but no more than a resident wave; a warp takes several chunks
+// where more tets are listed.
+#if defined(__CUDACC__) || defined(__CUDACC_RTC__)
+__host__ __device__
+#endif
+inline int64_t list_blocks(int64_t T, int block) {
+    const int64_t per = 2 * (int64_t)block, n = (T + per - 1) / per, most = 608 * 256 / block;
+    return n < most ? n : most;
+}
 
 // Full windows of one simulation in one flow launch (flow_tiles; the batched
 // form: a group of members, batch_flow_tile): one block per item (window q,

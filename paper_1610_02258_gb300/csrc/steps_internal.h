@@ -21,6 +21,11 @@ constexpr size_t warp_tile_bytes(int S) {
     return sizeof(WarpTile<1>) + (size_t)(S - 1) * (sizeof(WarpTile<2>) - sizeof(WarpTile<1>));
 }
 static_assert(warp_tile_bytes(kWarpMaxSpecies) == sizeof(WarpTile<kWarpMaxSpecies>), "warp tile rows");
+// and sizeof(ListTile<S>)
+constexpr size_t list_tile_bytes(int S) {
+    return sizeof(ListTile<1>) + (size_t)(S - 1) * (sizeof(ListTile<2>) - sizeof(ListTile<1>));
+}
+static_assert(list_tile_bytes(kMaxSpecies) == sizeof(ListTile<kMaxSpecies>), "list tile rows");
 
 // ---------------------------------------------------------------- host objects
 struct HostMesh {
@@ -95,10 +100,13 @@ int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, co
 int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEntry *reps, int S, int block,
                       void *stream);
 std::string spec_program_source(const HostModel &hm, int block);
-// whether the specialised kernels keep the trial counts in StepArgs::trial
+// whether the specialised block-tile kernels keep the trial counts in StepArgs::trial
 bool spec_global_trial(const HostModel &hm);
-// whether they run on warp tiles: flow launches then wait and publish per 32 tets, whatever the block size
+// whether the specialised kernels run on warp tiles: flow launches then wait and publish per 32 tets, whatever
+// the block size
 bool spec_warp_tile(const HostModel &hm);
+// the list form's step kernel for launch_spec (models of more species than warp tiles take), or nullptr
+void *spec_list_kernel(const HostModel &hm);
 
 // steps_api.cu: steps_batch_run in two parts (enqueue every window and the
 // error word's copy; then wait and map the word to a return code), so that

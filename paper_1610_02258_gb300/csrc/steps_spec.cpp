@@ -32,6 +32,7 @@ namespace steps {
 extern const char *const kSrcDeviceH;  // steps_device.h, embedded at build time
 extern const char *const kSrcStepCuh;  // steps_step.cuh, embedded at build time
 extern const char *const kSrcWarpCuh;  // steps_warp.cuh, embedded at build time
+extern const char *const kSrcListCuh;  // steps_list.cuh, embedded at build time
 
 namespace {
 
@@ -99,8 +100,9 @@ std::string hex_u32(uint32_t v) {
 // structure as constants. Propensity forms (all in float, as RtModel):
 //   order 0: k / inv_nav            order 1: k x
 //   order 2: ((k inv_nav) x) y      dimer:   ((k inv_nav) x) (x - 1)
-// (RtModel's extra factors of 1 are exact and left out.)
-std::string policy_source(const HostModel &hm, int block) {
+// (RtModel's extra factors of 1 are exact and left out.) block: entries of a
+// count row; list: for the list form.
+std::string policy_source(const HostModel &hm, int block, bool list) {
     const ModelDev &m = hm.dev;
     std::ostringstream o;
     o << "namespace steps {\nnamespace {\nstruct SpecModel {\n";
@@ -111,7 +113,7 @@ std::string policy_source(const HostModel &hm, int block) {
     o << "    __device__ static uint32_t diffusive(const ModelDev &) { return " << hex_u32(m.diffusive) << "; }\n";
     o << "    __device__ static uint32_t need(const RxnTab &tb, int r) { return tb.need[r]; }\n";
     o << "    template <int BLOCK>\n    __device__ static void build(const ModelDev &m, RxnTab &tb) {\n";
-    o << "        build_rxn_tab<BLOCK>(m, tb);\n    }\n";
+    o << "        build_rxn_tab<BLOCK, " << block << ">(m, tb);\n    }\n";
     o << "    __device__ static float prop(const RxnTab &, const ModelDev &m, int r, const int32_t *cnt, float inv_nav) {\n";
     o << "        switch (r) {\n";
     for (int r = 0; r < m.R; ++r) {
@@ -138,6 +140,13 @@ std::string policy_source(const HostModel &hm, int block) {
     // SSA loop would inline every reaction's occupancy update there
     o << "    template <class F>\n    __device__ static void for_changes(const RxnTab &tb, int r, F f) {\n";
     o << "        RtModel<false>::for_changes(tb, r, f);\n    }\n";
+    if (list)  // as ssa_lane calls them
+        o << "    template <int RM>\n    __device__ __forceinline__ static float sums(const RxnTab &tb, const ModelDev &m, "
+             "const int32_t *cnt, float inv_nav, uint32_t active, bool, float *psum) {\n"
+             "        return propensity_sums<SpecModel, RM>(tb, m, cnt, inv_nav, active, psum);\n    }\n"
+             "    template <int RM>\n    __device__ __forceinline__ static int pick(const RxnTab &tb, const ModelDev &m, "
+             "const float *psum, float target, const int32_t *cnt, float inv_nav, uint32_t active) {\n"
+             "        return pick_reaction<SpecModel, RM>(tb, m, psum, target, cnt, inv_nav, active);\n    }\n";
     o << "};\n}  // namespace\n}  // namespace steps\n";
 
     return o.str();
@@ -243,7 +252,7 @@ std::string program_source(const HostModel &hm, int block) {
     // block map and 48 registers per thread
     const bool five = spec_global_trial(hm) && block == 256;
     if (five) o << "#define STEPS_MAP_CAP 32\n";
-    o << "#include \"steps_step.cuh\"\n" << policy_source(hm, block);
+    o << "#include \"steps_step.cuh\"\n" << policy_source(hm, block, false);
     o << "extern \"C\" __global__ void __launch_bounds__(" << block << ", " << (five ? 5 : 2048 / block / 2) << ")\n"
       << "steps_spec_step(const __grid_constant__ steps::ModelDev m, const __grid_constant__ steps::StepArgs a) {\n"
       << "    steps::step_tile<" << block << ", " << reaction_bucket(hm.dev.R) << ", steps::SpecModel>(m, a, "
@@ -265,6 +274,20 @@ std::string program_source(const HostModel &hm, int block) {
     return o.str();
 }
 
+// The list form's program: one step kernel (256-thread blocks).
+constexpr int kListBlock = 256;
+
+std::string list_program_source(const HostModel &hm) {
+    std::ostringstream o;
+    const std::string b = std::to_string(kListBlock);
+    o << "#include \"steps_list.cuh\"\n" << policy_source(hm, 32, true);
+    o << "extern \"C\" __global__ void __launch_bounds__(" << b << ", " << 1024 / kListBlock << ")\n"
+      << "steps_spec_list(const __grid_constant__ steps::ModelDev m, const __grid_constant__ steps::StepArgs a) {\n"
+      << "    steps::list_step<" << b << ", " << std::max(1, hm.dev.R) << ", " << hm.dev.S
+      << ", steps::SpecModel>(m, a, blockIdx.x, gridDim.x);\n}\n";
+    return o.str();
+}
+
 struct Compiled {
     cudaLibrary_t lib = nullptr;
     cudaKernel_t kern = nullptr;        // plain step kernel
@@ -275,6 +298,7 @@ struct Compiled {
     size_t smem_set_flow = 0;           // the flow kernel
     size_t smem_set_batch_flow = 0;     // the batched flow kernel
     size_t smem_set_batch = 0;          // and the batched one
+    cudaKernel_t kern_list = nullptr;   // or the list form's step kernel alone
     size_t smem = 0;                    // dynamic shared memory per block
 };
 
@@ -288,13 +312,13 @@ std::string spec_program_source(const HostModel &hm, int block) { return program
 namespace {
 
 // Compiles (once per generated source) and loads the plain and batched kernels.
-Compiled *compiled(const HostModel &hm, int block, std::string *why) {
+Compiled *compiled(const HostModel &hm, int block, bool list, std::string *why) {
     Nvrtc &nv = nvrtc();
     if (!nv.handle) {
         if (why) *why = nv.why;
         return nullptr;
     }
-    const std::string src = program_source(hm, block);
+    const std::string src = list ? list_program_source(hm) : program_source(hm, block);
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_cache.find(src);
     if (it != g_cache.end()) {
@@ -302,9 +326,9 @@ Compiled *compiled(const HostModel &hm, int block, std::string *why) {
         return it->second.get();
     }
     nvrtc_program prog = nullptr;
-    const char *hdr_src[3] = {kSrcDeviceH, kSrcStepCuh, kSrcWarpCuh};
-    const char *hdr_name[3] = {"steps_device.h", "steps_step.cuh", "steps_warp.cuh"};
-    if (nv.create(&prog, src.c_str(), "steps_spec.cu", 3, hdr_src, hdr_name) != 0) {
+    const char *hdr_src[4] = {kSrcDeviceH, kSrcStepCuh, kSrcWarpCuh, kSrcListCuh};
+    const char *hdr_name[4] = {"steps_device.h", "steps_step.cuh", "steps_warp.cuh", "steps_list.cuh"};
+    if (nv.create(&prog, src.c_str(), "steps_spec.cu", 4, hdr_src, hdr_name) != 0) {
         if (why) *why = "nvrtcCreateProgram failed";
         g_cache[src] = nullptr;
         return nullptr;
@@ -333,13 +357,19 @@ Compiled *compiled(const HostModel &hm, int block, std::string *why) {
     }
     auto c = std::make_shared<Compiled>();
     const size_t S = (size_t)hm.dev.S;
-    c->smem = spec_warp_tile(hm) ? (size_t)(block / 32) * warp_tile_bytes(hm.dev.S)
-                                 : (S + 1 + (spec_global_trial(hm) ? 0 : S)) * (size_t)block * sizeof(int32_t);
-    if (cudaLibraryLoadData(&c->lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0) != cudaSuccess ||
-        cudaLibraryGetKernel(&c->kern, c->lib, "steps_spec_step") != cudaSuccess ||
-        cudaLibraryGetKernel(&c->kern_batch, c->lib, "steps_spec_batch") != cudaSuccess ||
-        cudaLibraryGetKernel(&c->kern_flow, c->lib, "steps_spec_flow") != cudaSuccess ||
-        cudaLibraryGetKernel(&c->kern_batch_flow, c->lib, "steps_spec_batch_flow") != cudaSuccess) {
+    c->smem = list                 ? (size_t)(kListBlock / 32) * list_tile_bytes(hm.dev.S)
+              : spec_warp_tile(hm) ? (size_t)(block / 32) * warp_tile_bytes(hm.dev.S)
+                                   : (S + 1 + (spec_global_trial(hm) ? 0 : S)) * (size_t)block * sizeof(int32_t);
+    bool ok = cudaLibraryLoadData(&c->lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0) == cudaSuccess;
+    if (list) {
+        ok = ok && cudaLibraryGetKernel(&c->kern_list, c->lib, "steps_spec_list") == cudaSuccess;
+    } else {
+        ok = ok && cudaLibraryGetKernel(&c->kern, c->lib, "steps_spec_step") == cudaSuccess &&
+             cudaLibraryGetKernel(&c->kern_batch, c->lib, "steps_spec_batch") == cudaSuccess &&
+             cudaLibraryGetKernel(&c->kern_flow, c->lib, "steps_spec_flow") == cudaSuccess &&
+             cudaLibraryGetKernel(&c->kern_batch_flow, c->lib, "steps_spec_batch_flow") == cudaSuccess;
+    }
+    if (!ok) {
         cudaGetLastError();
         if (why) *why = "loading the compiled kernel failed";
         g_cache[src] = nullptr;
@@ -364,21 +394,25 @@ bool opt_in(const void *fn, size_t smem, size_t *done) {
 }  // namespace
 
 void *spec_kernel(const HostModel &hm, int block, std::string *why) {
-    Compiled *c = compiled(hm, block, why);
-    return c ? (void *)c : nullptr;
+    return (void *)compiled(hm, block, false, why);
+}
+
+void *spec_list_kernel(const HostModel &hm) {
+    return hm.dev.S > kWarpMaxSpecies ? (void *)compiled(hm, kListBlock, true, nullptr) : nullptr;
 }
 
 int launch_spec(void *spec, const ModelDev &m, const StepArgs &a, int block, void *stream) {
     if (a.T <= 0) return STEPS_OK;
     Compiled *c = static_cast<Compiled *>(spec);
-    const void *fn = (const void *)c->kern;
+    const void *fn = (const void *)(c->kern_list ? c->kern_list : c->kern);
+    if (c->kern_list) block = kListBlock;
     const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set)) return STEPS_ERR_CUDA;
     StepArgs b = a;
     if (b.prefetch) b.prefetch = prefetch_distance(fn, block, smem);
     ModelDev mm = m;
     void *args[2] = {(void *)&mm, (void *)&b};
-    const unsigned grid = (unsigned)((a.T + block - 1) / block);
+    const unsigned grid = (unsigned)(c->kern_list ? list_blocks(a.T, block) : (a.T + block - 1) / block);
     // programmatic dependent launch, as the generic step kernel
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);

@@ -127,6 +127,7 @@ __device__ __forceinline__ uint32_t ssa_lane(const RxnTab &tb, const ModelDev &m
         tS[s] = dt_acc;
     });
     for (uint32_t j = 1;; ++j) {
+        asm volatile("" ::: "memory");  // keep the reaction table out of registers across iterations
         const uint4 w = philox_rk(a.rk, c0, tet, j, (kPurposeReac << 28) | c3);
         float psum[RM];
         const float a0 = P::template sums<RM>(tb, m, cnt, inv_nav, active, a.rmask != nullptr, psum);
@@ -196,56 +197,64 @@ __device__ __forceinline__ void move_out(const StepArgs &a, WarpTile<SM> &w, int
     }
 }
 
-// Up to 32 queued groups of 32 trial molecules, one per lane (the bit-plane
-// draws of bulk_species, one group).
+// The bit-plane draws of bulk_species for group g of species s: bit j of l[f]
+// says that molecule 32 g + j is below threshold T_f.
+__device__ __forceinline__ void plane_group(const StepArgs &a, const uint4 A, uint32_t R, uint32_t M, uint32_t g,
+                                            uint32_t tet, int s, uint32_t c0, uint32_t c3, uint32_t l[4]) {
+    const uint32_t m = min(32u, M - 32u * g);
+    const uint32_t valid = m == 32u ? 0xFFFFFFFFu : (1u << m) - 1u;
+    uint32_t T0, T1, T2, T3;
+    species_thresholds(A, R, T0, T1, T2, T3);
+    const uint32_t c3b = (kPurposeBulk << 28) | ((uint32_t)s << 23) | (c3 & 0x007FFFFFu);
+    // T_f = 2^31: every x < T_f; T_f = 0: none
+    uint32_t l0 = T0 >= 0x80000000u ? valid : 0u, u0 = (T0 >= 0x80000000u || T0 == 0u) ? 0u : valid;
+    uint32_t l1 = T1 >= 0x80000000u ? valid : 0u, u1 = (T1 >= 0x80000000u || T1 == 0u) ? 0u : valid;
+    uint32_t l2 = T2 >= 0x80000000u ? valid : 0u, u2 = (T2 >= 0x80000000u || T2 == 0u) ? 0u : valid;
+    uint32_t l3 = T3 >= 0x80000000u ? valid : 0u, u3 = (T3 >= 0x80000000u || T3 == 0u) ? 0u : valid;
+    for (uint32_t blk = 0; blk < 8u && (u0 | u1 | u2 | u3); ++blk) {
+        const uint4 r = philox_rk(a.rk, c0, tet, (g << 3) | blk, c3b);
+        const int sh = 30 - 4 * (int)blk;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (q < 3 || blk < 7u) {  // 31 planes
+                const uint32_t Rw = word_of(r, (uint32_t)q);
+                plane_compare(T0, sh - q, Rw, u0, l0);
+                plane_compare(T1, sh - q, Rw, u1, l1);
+                plane_compare(T2, sh - q, Rw, u2, l2);
+                plane_compare(T3, sh - q, Rw, u3, l3);
+            }
+        }
+        // a molecule that stays needs no face
+        const uint32_t may = u3 | l3;
+        u0 &= may;
+        u1 &= may;
+        u2 &= may;
+    }
+    l[0] = l0;
+    l[1] = l1;
+    l[2] = l2;
+    l[3] = l3;
+}
+
+// Up to 32 queued groups of 32 trial molecules, one per lane.
 template <int SM, class P>
 __device__ __forceinline__ void plane_groups(const StepArgs &a, WarpTile<SM> &w, int32_t *nxt, const uint32_t *s_scale,
                                              int64_t i0, int first, int n, uint32_t c0, uint32_t c3) {
     const int lane = threadIdx.x & 31;
     if (lane < n) {
         const uint2 e = w.d.q[first + lane];
-        const uint32_t g = e.x;
         const int t = (int)(e.y & 31u), s = (int)(e.y >> 5);
-        const uint32_t m = min(32u, (uint32_t)w.trial[s][t] - 32u * g);
-        const uint32_t valid = m == 32u ? 0xFFFFFFFFu : (1u << m) - 1u;
-        const uint32_t R = warp_R<P>(a, s_scale, s, i0 + t);
-        uint32_t T0, T1, T2, T3;
-        species_thresholds(w.thr[t], R, T0, T1, T2, T3);
-        const uint32_t c3b = (kPurposeBulk << 28) | ((uint32_t)s << 23) | (c3 & 0x007FFFFFu);
-        const uint32_t tet = w.tet[t];
-        // T_f = 2^31: every x < T_f; T_f = 0: none
-        uint32_t l0 = T0 >= 0x80000000u ? valid : 0u, u0 = (T0 >= 0x80000000u || T0 == 0u) ? 0u : valid;
-        uint32_t l1 = T1 >= 0x80000000u ? valid : 0u, u1 = (T1 >= 0x80000000u || T1 == 0u) ? 0u : valid;
-        uint32_t l2 = T2 >= 0x80000000u ? valid : 0u, u2 = (T2 >= 0x80000000u || T2 == 0u) ? 0u : valid;
-        uint32_t l3 = T3 >= 0x80000000u ? valid : 0u, u3 = (T3 >= 0x80000000u || T3 == 0u) ? 0u : valid;
-        for (uint32_t blk = 0; blk < 8u && (u0 | u1 | u2 | u3); ++blk) {
-            const uint4 r = philox_rk(a.rk, c0, tet, (g << 3) | blk, c3b);
-            const int sh = 30 - 4 * (int)blk;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (q < 3 || blk < 7u) {  // 31 planes
-                    const uint32_t Rw = word_of(r, (uint32_t)q);
-                    plane_compare(T0, sh - q, Rw, u0, l0);
-                    plane_compare(T1, sh - q, Rw, u1, l1);
-                    plane_compare(T2, sh - q, Rw, u2, l2);
-                    plane_compare(T3, sh - q, Rw, u3, l3);
-                }
-            }
-            // a molecule that stays needs no face
-            const uint32_t may = u3 | l3;
-            u0 &= may;
-            u1 &= may;
-            u2 &= may;
-        }
-        // cumulative thresholds: l0 within l1 within l2 within l3
-        const int32_t n0 = __popc(l0), n1 = __popc(l1 & ~l0), n2 = __popc(l2 & ~l1), n3 = __popc(l3 & ~l2);
+        uint32_t l[4];
+        plane_group(a, w.thr[t], warp_R<P>(a, s_scale, s, i0 + t), (uint32_t)w.trial[s][t], e.x, w.tet[t], s, c0, c3, l);
+        // cumulative thresholds: l[0] within l[1] within l[2] within l[3]
+        const int32_t n0 = __popc(l[0]), n1 = __popc(l[1] & ~l[0]), n2 = __popc(l[2] & ~l[1]), n3 = __popc(l[3] & ~l[2]);
         const int4 nb = w.nbr[t];
         int32_t *row = nxt + (uint64_t)(uint32_t)s * (uint32_t)a.Tpad;
         if (n0) atomicAdd(row + nb.x, n0);
         if (n1) atomicAdd(row + nb.y, n1);
         if (n2) atomicAdd(row + nb.z, n2);
         if (n3) atomicAdd(row + nb.w, n3);
-        if (l3) atomicSub(&w.cnt[s][t], n0 + n1 + n2 + n3);
+        if (l[3]) atomicSub(&w.cnt[s][t], n0 + n1 + n2 + n3);
     }
 }
 
