@@ -120,7 +120,8 @@ class Clocks:
 
 
 KERNEL_SOURCES = ["paper_1610_02258_gb300/csrc/steps_step.cuh", "paper_1610_02258_gb300/csrc/steps_warp.cuh",
-                  "paper_1610_02258_gb300/csrc/steps_list.cuh", "paper_1610_02258_gb300/csrc/steps_kernels.cu",
+                  "paper_1610_02258_gb300/csrc/steps_list.cuh", "paper_1610_02258_gb300/csrc/steps_warp.cu",
+                  "paper_1610_02258_gb300/csrc/steps_kernels.cu",
                   "paper_1610_02258_gb300/csrc/steps_batch.cu", "paper_1610_02258_gb300/csrc/steps_internal.h",
                   "paper_1610_02258_gb300/csrc/steps_device.h", "paper_1610_02258_gb300/csrc/steps_spec.cpp"]
 

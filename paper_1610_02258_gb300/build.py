@@ -12,7 +12,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB_PATH = os.path.join(HERE, "libsteps_gpu.so")
-SOURCES = ["steps_host.cpp", "steps_kernels.cu", "steps_batch.cu", "steps_api.cu", "steps_spec.cpp",
+SOURCES = ["steps_host.cpp", "steps_kernels.cu", "steps_warp.cu", "steps_batch.cu", "steps_api.cu", "steps_spec.cpp",
            "steps_server.cpp"]
 # device sources embedded into the library for the run-time compiler (NVRTC)
 EMBEDDED = [("kSrcDeviceH", "steps_device.h"), ("kSrcStepCuh", "steps_step.cuh"),

@@ -288,7 +288,7 @@ struct steps_sim {
         if (!sp && !(generic && B == 256)) return STEPS_OK;
         // a warp-tile kernel publishes per 32 tets and finds the tiles it waits
         // for from its tets' neighbours: it needs no lists
-        const bool warp = sp && spec_warp_tile(model);
+        const bool warp = warp_tiles(model);
         const int64_t nt = (T + B - 1) / B, nwords = warp ? nt * (B / 32) : nt;
         std::vector<int32_t> off, nb;
         if (!warp) {
@@ -1603,7 +1603,7 @@ struct steps_batch {
         std::vector<int32_t> off, nb;
         std::vector<std::pair<int64_t, int64_t>> groups;
         int64_t nwork = 0;
-        const bool warp = spec_warp_tile(members[0]->model);  // (flow runs on specialised kernels only)
+        const bool warp = warp_tiles(members[0]->model);  // (flow runs on specialised kernels only)
         try {
             int64_t gfirst = 0, gbytes = 0;
             for (steps_sim *m : members) {

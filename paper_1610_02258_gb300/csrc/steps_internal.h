@@ -73,6 +73,10 @@ void exp_leave_table(const HostModel &model, const Tables &t, double tau_k, size
 // shared-memory size.
 int prefetch_distance(const void *kernel, int block, size_t smem);
 int launch_step(const ModelDev &m, const StepArgs &a, int block, void *stream);
+// the same for models of up to kWarpMaxSpecies species, on warp tiles (steps_warp.cu)
+int launch_warp(const ModelDev &m, const StepArgs &a, int block, void *stream);
+int launch_warp_flow(const ModelDev &m, const StepArgs &a, const FlowArgs &f, int block, void *stream);
+int launch_warp_batch(const BlockWork *work, int64_t nblocks, const RepEntry *reps, int max_S, int block, void *stream);
 int launch_philox_test(uint64_t seed, const uint32_t *d_ctr, int64_t n, uint32_t *d_out, void *stream);
 int launch_logf_test(const float *d_x, int64_t n, float *d_out, void *stream);
 int launch_wait_test(const void *d_src, int deliver, long long limit, uint32_t *d_status, void *stream);
@@ -102,9 +106,9 @@ int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEnt
 std::string spec_program_source(const HostModel &hm, int block);
 // whether the specialised block-tile kernels keep the trial counts in StepArgs::trial
 bool spec_global_trial(const HostModel &hm);
-// whether the specialised kernels run on warp tiles: flow launches then wait and publish per 32 tets, whatever
+// whether a model's kernels, specialised or not, run on warp tiles: flow launches then wait and publish per 32 tets, whatever
 // the block size
-bool spec_warp_tile(const HostModel &hm);
+bool warp_tiles(const HostModel &hm);
 // the list form's step kernel for launch_spec (models of more species than warp tiles take), or nullptr
 void *spec_list_kernel(const HostModel &hm);
 

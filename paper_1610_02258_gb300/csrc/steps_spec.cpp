@@ -86,7 +86,7 @@ bool spec_global_trial(const HostModel &hm) { return hm.dev.S >= 16; }
 
 // Models with few species run on warp tiles (steps_warp.cuh): their loops
 // over species are unrolled.
-bool spec_warp_tile(const HostModel &hm) { return hm.dev.S <= kWarpMaxSpecies; }
+bool warp_tiles(const HostModel &hm) { return hm.dev.S <= kWarpMaxSpecies; }
 
 namespace {
 
@@ -165,8 +165,8 @@ std::string warp_policy_source(const HostModel &hm) {
     o << "    __device__ static constexpr int R(const ModelDev &) { return " << m.R << "; }\n";
     o << "    __device__ static constexpr uint32_t diffusive(const ModelDev &) { return " << hex_u32(m.diffusive)
       << "; }\n";
-    o << "    template <int BLOCK>\n    __device__ static void build(const ModelDev &m, RxnTab &tb) {\n";
-    o << "        build_rxn_tab<BLOCK, 32>(m, tb);\n    }\n";
+    o << "    template <int THREADS>\n    __device__ static void build(const ModelDev &m, RxnTab &tb) {\n";
+    o << "        if (threadIdx.x < THREADS) build_rxn_tab<THREADS, 32>(m, tb);\n    }\n";
     o << "    template <class F>\n    __device__ static void for_changes(const RxnTab &tb, int r, F f) {\n";
     o << "        RtModel<false>::for_changes(tb, r, f);\n    }\n";
     o << "    template <int RM, bool MASKED>\n    __device__ __forceinline__ static float sums_of(const ModelDev &m, "
@@ -207,7 +207,7 @@ std::string warp_policy_source(const HostModel &hm) {
          "        const float a0 = sums<RM>(tb, m, cnt, inv_nav, active, masked, psum);\n"
          "        if (a0 <= 3.0e38f) return a0;\n"
          "        float ps[RM];\n"
-         "        const float a1 = careful_sums<RM>(tb, m, cnt, inv_nav, active, ps);\n"
+         "        const float a1 = careful_sums(tb, m, cnt, inv_nav, active, ps);\n"
          "        for (int r = 0; r < " << m.R << "; ++r) psum[r] = ps[r];\n"
          "        return a1;\n    }\n";
     o << "    template <int RM>\n    __device__ __forceinline__ static int pick(const RxnTab &tb, const ModelDev &m, "
@@ -225,7 +225,7 @@ int reaction_bucket(int R) { return R <= 8 ? 8 : R <= 16 ? 16 : R <= 24 ? 24 : 3
 std::string program_source(const HostModel &hm, int block) {
     std::ostringstream o;
     const std::string b = std::to_string(block);
-    if (spec_warp_tile(hm)) {
+    if (warp_tiles(hm)) {
         const std::string args = "<" + b + ", " + std::to_string(std::max(1, hm.dev.R)) + ", " +
                                  std::to_string(hm.dev.S) + ", steps::SpecModel";
         const std::string head = "extern \"C\" __global__ void __launch_bounds__(" + b + ", " +
@@ -358,7 +358,7 @@ Compiled *compiled(const HostModel &hm, int block, bool list, std::string *why) 
     auto c = std::make_shared<Compiled>();
     const size_t S = (size_t)hm.dev.S;
     c->smem = list                 ? (size_t)(kListBlock / 32) * list_tile_bytes(hm.dev.S)
-              : spec_warp_tile(hm) ? (size_t)(block / 32) * warp_tile_bytes(hm.dev.S)
+              : warp_tiles(hm) ? (size_t)(block / 32) * warp_tile_bytes(hm.dev.S)
                                    : (S + 1 + (spec_global_trial(hm) ? 0 : S)) * (size_t)block * sizeof(int32_t);
     bool ok = cudaLibraryLoadData(&c->lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0) == cudaSuccess;
     if (list) {

@@ -997,16 +997,17 @@ __device__ __forceinline__ void batch_member(const BlockWork *__restrict__ work,
     __shared__ __align__(16) ModelDev t_model;
     __shared__ __align__(16) StepArgs t_args;
     __shared__ int32_t t_tile;
+    const int threads = BLOCK ? BLOCK : (int)blockDim.x;
     const BlockWork bw = work[blockIdx.x];
     const RepEntry *e = reps + bw.rep;
     if (e->args.window >= e->window_end) return;
     static_assert(sizeof(ModelDev) % 4 == 0 && sizeof(StepArgs) % 4 == 0, "word copy");
     const uint32_t *src_m = reinterpret_cast<const uint32_t *>(&e->model);
     uint32_t *dst_m = reinterpret_cast<uint32_t *>(&t_model);
-    for (int k = threadIdx.x; k < (int)(sizeof(ModelDev) / 4); k += BLOCK) dst_m[k] = src_m[k];
+    for (int k = threadIdx.x; k < (int)(sizeof(ModelDev) / 4); k += threads) dst_m[k] = src_m[k];
     const uint32_t *src_a = reinterpret_cast<const uint32_t *>(&e->args);
     uint32_t *dst_a = reinterpret_cast<uint32_t *>(&t_args);
-    for (int k = threadIdx.x; k < (int)(sizeof(StepArgs) / 4); k += BLOCK) dst_a[k] = src_a[k];
+    for (int k = threadIdx.x; k < (int)(sizeof(StepArgs) / 4); k += threads) dst_a[k] = src_a[k];
     __syncthreads();
     if (threadIdx.x == 0) {
         t_args.cur = e->cnt[e->parity];

@@ -1,0 +1,105 @@
+// The warp-tile step for models given at run time (meshes below the
+// specialisation size, or without the run-time compiler) of up to
+// kWarpMaxSpecies species: plain, flow and batched kernels. The loops over
+// species are unrolled to 4 or 12, the reaction table is walked in loops.
+#include <algorithm>
+#include <string>
+
+#include "steps_warp.cuh"
+
+namespace steps {
+
+namespace {
+
+template <int SM>
+__global__ void __launch_bounds__(512, 2)
+    warp_kernel(const __grid_constant__ ModelDev m, const __grid_constant__ StepArgs a) {
+    warp_step<0, 1, SM, RtWarp>(m, a, (int64_t)blockIdx.x);
+}
+
+template <int SM>
+__global__ void __launch_bounds__(512, 2)
+    warp_flow_kernel(const __grid_constant__ ModelDev m, const __grid_constant__ StepArgs a,
+                     const __grid_constant__ FlowArgs f) {
+    warp_step<0, 1, SM, RtWarp, 1>(m, a, 0, &f);
+}
+
+template <int SM>
+__global__ void __launch_bounds__(512, 2)
+    warp_batch_kernel(const BlockWork *__restrict__ work, const RepEntry *__restrict__ reps) {
+    batch_member<0>(work, reps, 0, [](const ModelDev &m, const StepArgs &a, int64_t tile) {
+        warp_step<0, 1, SM, RtWarp>(m, a, tile);
+    });
+}
+
+bool opt_in(const void *fn, size_t smem) {
+    if (smem <= 44 * 1024) return true;  // with the static arrays below the 48 KB every launch may have
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) return true;
+    set_error(std::string("warp-tile kernel shared memory: ") + cudaGetErrorString(e));
+    return false;
+}
+
+int checked(cudaError_t e, const char *what) {
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) return STEPS_OK;
+    set_error(std::string(what) + ": " + cudaGetErrorString(e));
+    return STEPS_ERR_CUDA;
+}
+
+template <int SM>
+int launch_plain(const ModelDev &m, const StepArgs &a, int block, void *stream) {
+    // a small mesh's tiles go into smaller blocks until the blocks cover the
+    // SMs twice: its windows are bound by the latency of a tile, and warps of
+    // one block share an SM
+    while (block > 32 && ((int64_t)a.T + block - 1) / block < 2 * 152) block /= 2;
+    const size_t smem = (size_t)(block / 32) * sizeof(WarpTile<SM>);
+    if (!opt_in((const void *)warp_kernel<SM>, smem)) return STEPS_ERR_CUDA;
+    // programmatic dependent launch, as the block-tile kernel
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(((int64_t)a.T + block - 1) / block));
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return checked(cudaLaunchKernelEx(&cfg, warp_kernel<SM>, m, a), "warp-tile kernel launch");
+}
+
+template <int SM>
+int launch_flow_sm(const ModelDev &m, const StepArgs &a, const FlowArgs &f, int block, void *stream) {
+    const size_t smem = (size_t)(block / 32) * sizeof(WarpTile<SM>);
+    if (!opt_in((const void *)warp_flow_kernel<SM>, smem)) return STEPS_ERR_CUDA;
+    StepArgs b = a;
+    b.window_base = nullptr;
+    warp_flow_kernel<SM><<<f.nwin * f.ntiles, block, smem, (cudaStream_t)stream>>>(m, b, f);  // one item per block
+    return checked(cudaSuccess, "warp-tile flow kernel launch");
+}
+
+template <int SM>
+int launch_batch_sm(const BlockWork *work, int64_t nblocks, const RepEntry *reps, int block, void *stream) {
+    const size_t smem = (size_t)(block / 32) * sizeof(WarpTile<SM>);
+    if (!opt_in((const void *)warp_batch_kernel<SM>, smem)) return STEPS_ERR_CUDA;
+    warp_batch_kernel<SM><<<(unsigned)nblocks, block, smem, (cudaStream_t)stream>>>(work, reps);
+    return checked(cudaSuccess, "warp-tile batch kernel launch");
+}
+
+}  // namespace
+
+int launch_warp(const ModelDev &m, const StepArgs &a, int block, void *stream) {
+    return m.S <= 4 ? launch_plain<4>(m, a, block, stream) : launch_plain<kWarpMaxSpecies>(m, a, block, stream);
+}
+
+int launch_warp_flow(const ModelDev &m, const StepArgs &a, const FlowArgs &f, int block, void *stream) {
+    return m.S <= 4 ? launch_flow_sm<4>(m, a, f, block, stream) : launch_flow_sm<kWarpMaxSpecies>(m, a, f, block, stream);
+}
+
+int launch_warp_batch(const BlockWork *work, int64_t nblocks, const RepEntry *reps, int max_S, int block, void *stream) {
+    return max_S <= 4 ? launch_batch_sm<4>(work, nblocks, reps, block, stream)
+                      : launch_batch_sm<kWarpMaxSpecies>(work, nblocks, reps, block, stream);
+}
+
+}  // namespace steps

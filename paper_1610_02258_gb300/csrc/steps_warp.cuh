@@ -75,7 +75,6 @@ __device__ __forceinline__ int32_t round_trials32(double nbar, uint32_t w, int32
 
 // First propensity sums of a tet whose plain sums are not finite (rates near
 // the float range): a reaction without all its reactants counts 0.
-template <int RM>
 __device__ __noinline__ float careful_sums(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
                                            uint32_t active, float *psum) {
     float a0 = 0.0f;
@@ -84,7 +83,7 @@ __device__ __noinline__ float careful_sums(const RxnTab &tb, const ModelDev &m, 
         const bool have = *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(cnt) + __float_as_uint(p.y)) &&
                           *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(cnt) + __float_as_uint(p.z));
         a0 = __fadd_rn(a0, ((active >> r) & 1u) && have ? propensity(p, cnt, inv_nav, true) : 0.0f);
-        psum[r] = a0;
+        if (psum) psum[r] = a0;
     }
     return a0;
 }
@@ -98,6 +97,54 @@ __device__ __noinline__ int last_positive_tab(const RxnTab &tb, const ModelDev &
         if (((active >> r) & 1u) && propensity(tb.p[r], cnt, inv_nav, true) > 0.0f) last = r;
     return last;
 }
+
+// Model access for models given at run time: the reaction table, walked in a
+// loop; the running sums are summed again for a pick instead of kept
+// (unrolled by four, or with the sums kept, the loops were slower). 30,720
+// tets at 151 molecules each, us per window: block tiles 79.7, this 63.8
+// (compiled for the model 43); the 1,920-tet cuboid 9.7 -> 7.4.
+struct RtWarp {
+    static constexpr bool kExpLeave = false;
+    __device__ static int S(const ModelDev &m) { return m.S; }
+    __device__ static int R(const ModelDev &m) { return m.R; }
+    __device__ static uint32_t diffusive(const ModelDev &m) { return m.diffusive; }
+    template <int THREADS>
+    __device__ static void build(const ModelDev &m, RxnTab &tb) {
+        if (threadIdx.x < THREADS) build_rxn_tab<THREADS, 32>(m, tb);
+    }
+    template <class F>
+    __device__ static void for_changes(const RxnTab &tb, int r, F f) {
+        RtModel<false>::for_changes(tb, r, f);
+    }
+    template <int RM>
+    __device__ __forceinline__ static float sums(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
+                                                 uint32_t active, bool, float *) {
+        const bool z = m.order0 != 0u;
+        float a0 = 0.0f;
+#pragma unroll 2
+        for (int r = 0; r < m.R; ++r)
+            a0 = __fadd_rn(a0, ((active >> r) & 1u) ? propensity(tb.p[r], cnt, inv_nav, z) : 0.0f);
+        return a0;
+    }
+    template <int RM>
+    __device__ __forceinline__ static float first_sums(const RxnTab &tb, const ModelDev &m, const int32_t *cnt,
+                                                       float inv_nav, uint32_t active, bool masked, float *psum) {
+        const float a0 = sums<RM>(tb, m, cnt, inv_nav, active, masked, psum);
+        if (a0 <= 3.0e38f) return a0;
+        return careful_sums(tb, m, cnt, inv_nav, active, nullptr);
+    }
+    template <int RM>
+    __device__ __forceinline__ static int pick(const RxnTab &tb, const ModelDev &m, const float *, float target,
+                                               const int32_t *cnt, float inv_nav, uint32_t active) {
+        const bool z = m.order0 != 0u;
+        float sum = 0.0f;
+        for (int r = 0; r < m.R; ++r) {
+            sum = __fadd_rn(sum, ((active >> r) & 1u) ? propensity(tb.p[r], cnt, inv_nav, z) : 0.0f);
+            if (!(sum <= target)) return r;
+        }
+        return last_positive_tab(tb, m, cnt, inv_nav, active);
+    }
+};
 
 // The tile's species factor of species s for lane t's tet (species_R).
 template <class P>
@@ -346,17 +393,21 @@ __device__ __forceinline__ bool flow_nbr_wait(const uint32_t *done, uint32_t own
     const uint32_t *p[4] = {nb.x < 0 ? done + own : base + (nb.x >> 5), nb.y < 0 ? done + own : base + (nb.y >> 5),
                             nb.z < 0 ? done + own : base + (nb.z >> 5), nb.w < 0 ? done + own : base + (nb.w >> 5)};
     const long long t0 = clock64();
-    for (;;) {
+    uint32_t open = 31u;  // words not seen done yet: a lane reads only those again
+    for (uint32_t ns = 32;;) {
         uint32_t v[5];
 #pragma unroll
         for (int k = 0; k < 5; ++k)
-            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v[k]) : "l"(k < 4 ? p[k] : done + own) : "memory");
-        bool ok = true;
+            if ((open >> k) & 1u)
+                asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v[k]) : "l"(k < 4 ? p[k] : done + own) : "memory");
 #pragma unroll
-        for (int k = 0; k < 5; ++k) ok &= (int32_t)(v[k] - need) >= 0;
-        if (__all_sync(0xFFFFFFFFu, ok)) break;
+        for (int k = 0; k < 5; ++k)
+            if (((open >> k) & 1u) && (int32_t)(v[k] - need) >= 0) open &= ~(1u << k);
+        if (__all_sync(0xFFFFFFFFu, open == 0u)) break;
         if (__any_sync(0xFFFFFFFFu, clock64() - t0 > limit)) return false;
-        __nanosleep(64);
+        // every waiting warp polls: back off, so that the ones at work are not held up
+        __nanosleep(ns);
+        ns = min(2u * ns, 1024u);
     }
     asm volatile("fence.acq_rel.gpu;" ::: "memory");
     __syncwarp();
@@ -420,7 +471,7 @@ __device__ __forceinline__ void warp_window(const ModelDev &m, const StepArgs &a
         int32_t *row = cur + i;
 #pragma unroll
         for (int s = 0; s < SM; ++s) {
-            w.cnt[s][lane] = n[s];
+            w.cnt[s][lane] = s < P::S(m) ? n[s] : 1;  // (row S holds ones: a missing reactant)
             any |= n[s];
             if (n[s] != 0) *row = 0;
             row += Tpad;
@@ -602,6 +653,7 @@ __device__ __forceinline__ void warp_window(const ModelDev &m, const StepArgs &a
 // the tiles of block tile `tile`. 1 (a launch of several windows): the block
 // takes its item (window, block tile) from f's counter, as in flow_tiles. 2
 // (batched): the caller took the block's item; dep is its work entry.
+// BLOCK 0: as many threads as the launch has.
 template <int BLOCK, int RM, int SM, class P, int FLOW = 0>
 __device__ __forceinline__ void warp_step(const ModelDev &m, const StepArgs &a, int64_t tile,
                                           const FlowArgs *f = nullptr, uint32_t q = 0, uint32_t dep = 0) {
@@ -609,11 +661,11 @@ __device__ __forceinline__ void warp_step(const ModelDev &m, const StepArgs &a, 
     __shared__ RxnTab tb;
     __shared__ uint32_t s_scale[kMaxSpecies];
     static_assert(SM <= kWarpMaxSpecies, "species bound");
-    constexpr int WARPS = BLOCK / 32;
+    const int threads = BLOCK ? BLOCK : (int)blockDim.x, warps = threads / 32;
     const int tid = threadIdx.x, warp = tid >> 5;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    P::template build<BLOCK>(m, tb);
+    P::template build<32>(m, tb);  // (of up to 32 reactions, by the first warp)
     if (tid < kMaxSpecies) s_scale[tid] = a.scale[tid];
     __syncthreads();
     WarpTile<SM> &w = reinterpret_cast<WarpTile<SM> *>(warp_smem)[warp];
@@ -625,11 +677,11 @@ __device__ __forceinline__ void warp_step(const ModelDev &m, const StepArgs &a, 
         const uint32_t item = s_item;
         if (item >= items) return;
         const uint32_t qq = item / f->ntiles, t = item - qq * f->ntiles;
-        const int64_t i0 = (int64_t)t * BLOCK + warp * 32;
-        if (i0 < a.T) warp_window<RM, SM, P, FLOW>(m, a, w, tb, s_scale, i0, f, qq, t * WARPS + (uint32_t)warp);
+        const int64_t i0 = (int64_t)t * threads + warp * 32;
+        if (i0 < a.T) warp_window<RM, SM, P, FLOW>(m, a, w, tb, s_scale, i0, f, qq, t * (uint32_t)warps + (uint32_t)warp);
     } else {
-        const int64_t i0 = tile * BLOCK + warp * 32;
-        if (i0 < a.T) warp_window<RM, SM, P, FLOW>(m, a, w, tb, s_scale, i0, f, q, dep * WARPS + (uint32_t)warp);
+        const int64_t i0 = tile * threads + warp * 32;
+        if (i0 < a.T) warp_window<RM, SM, P, FLOW>(m, a, w, tb, s_scale, i0, f, q, dep * (uint32_t)warps + (uint32_t)warp);
     }
 }
 }  // namespace

@@ -1,5 +1,5 @@
-"""GPU parity of the warp-tile step (models of up to 12 species on the
-model-specialised kernels) against the CPU oracle, bit for bit, where its
+"""GPU parity of the warp-tile step (models of up to 12 species, on the
+model-specialised kernels and on those for models given at run time) against the CPU oracle, bit for bit, where its
 tiles, queues and packed tables have edges: meshes that end inside, at and
 just past a warp's 32 tets and a block's 256; 1 to 13 species (the table of
 words per species holds four to a word; 13 is the first model on the other
@@ -40,19 +40,26 @@ def _model(S):
 
 
 def _check(capi, S, grid, values, occ=OCC, leave=0, flow=False, block=256, mask=True, windows=(3.0, 5.4)):
+    _check_kernel(capi, S, grid, values, occ, leave, flow, block, mask, windows, 1)
+    if leave == 0 and not (flow and block != 256):  # the kernels for models given at run time
+        _check_kernel(capi, S, grid, values, occ, leave, flow, block, mask, windows, -1)
+
+
+def _check_kernel(capi, S, grid, values, occ, leave, flow, block, mask, windows, specialize):
     verts, tets = I.kuhn_box_mesh(*grid, 0.5 * I.UM)
     nt = tets.shape[0]
     m = _model(S)
     rng = np.random.default_rng(S * 1000 + nt)
     counts = rng.choice(np.asarray(values, np.int32), size=(S, nt)).astype(np.int32)
     on = (rng.random(nt) < 0.5).astype(np.uint8)
-    g = capi.Simulation(verts, tets, m, 7, occupancy=occ, leave_law=leave, specialize=1, flow=flow, block=block)
+    g = capi.Simulation(verts, tets, m, 7, occupancy=occ, leave_law=leave, specialize=specialize, flow=flow,
+                        block=block)
     o = oracle.OracleSim(verts, tets, m, seed=7, occ=occ, prec=32, leave=leave)
     for obj in (g, o):
         obj.set_counts(counts)
         if mask:
             obj.set_reac_mask(0, on)
-    assert g.specialized and g.tau == o.tau
+    assert g.specialized == (specialize > 0) and g.tau == o.tau
     for k in windows:
         g.run(k * o.tau)
         o.run(k * o.tau)
