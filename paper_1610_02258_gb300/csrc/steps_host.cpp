@@ -373,6 +373,13 @@ void build_tables(const HostMesh &mesh, const HostModel &model, int reorder, Tab
     }
 }
 
+uint32_t exp_leave_entry(double tauD, double G) {
+    const double x = tauD * G;
+    double fl = std::floor((1.0 - std::exp(-x)) * 2147483648.0);
+    fl = std::min(2147483648.0, std::max(0.0, fl));
+    return (uint32_t)fl;
+}
+
 void exp_leave_table(const HostModel &model, const Tables &t, double tau_k, size_t Tpad, std::vector<uint32_t> &out) {
     const size_t T = t.G_dev.size();
     out.assign((size_t)model.S * Tpad, 0u);
@@ -380,12 +387,7 @@ void exp_leave_table(const HostModel &model, const Tables &t, double tau_k, size
     for (int s = 0; s < model.S; ++s) {
         const double D = model.D[(size_t)s];
         if (!(D > 0.0)) continue;
-        for (size_t d = 0; d < T; ++d) {
-            const double x = (tau_k * D) * t.G_dev[d];
-            double fl = std::floor((1.0 - std::exp(-x)) * 2147483648.0);
-            fl = std::min(2147483648.0, std::max(0.0, fl));
-            out[(size_t)s * Tpad + d] = (uint32_t)fl;
-        }
+        for (size_t d = 0; d < T; ++d) out[(size_t)s * Tpad + d] = exp_leave_entry(tau_k * D, t.G_dev[d]);
     }
 }
 

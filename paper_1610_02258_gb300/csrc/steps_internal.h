@@ -66,6 +66,7 @@ uint32_t species_scale(const HostModel &model, const Tables &t, int s, double ta
 // EXP leave law: out[s * Tpad + d] = floor(2^31 (1 - exp(-(tau_k D_s) G_d))) for every
 // species and device-order tet (0 for immobile species and the padding).
 void exp_leave_table(const HostModel &model, const Tables &t, double tau_k, size_t Tpad, std::vector<uint32_t> &out);
+uint32_t exp_leave_entry(double tauD, double G);  // one entry, tauD = tau_k D_s
 
 // steps_kernels.cu
 // L2 prefetch distance in tiles: half of the blocks of a kernel resident on
