@@ -213,8 +213,11 @@ bool cuda_ok(cudaError_t e, const char *what) {
 }  // namespace
 
 struct steps_sim {
+    // the host tables, built once and shared by a simulation's clones (copied,
+    // about 50 bytes a tet, they were half of what admitting a job cost)
+    std::shared_ptr<Tables> tables;
+    Tables &tab;
     HostModel model;
-    Tables tab;
     steps_options opt{};
     cudaStream_t stream = nullptr;
     int device = -1;                // the device current at creation (owns every buffer below)
@@ -286,34 +289,62 @@ struct steps_sim {
     int flow_pick = -1;  // flow = 0 (tuned): -1 not yet timed, 0 window launches, 1 + k flow launches of flow[k]
     float flow_ms[3] = {0.f, 0.f, 0.f};  // tuning: ms per window of window launches, flow[0], flow[1]
 
+    // a clone's buffers: one allocation (a dozen, and as many frees, were most
+    // of the time of admitting and retiring a served job)
+    char *arena = nullptr;
+    size_t arena_bytes = 0;
+    void drop(void *p) {
+        if (!(arena && static_cast<char *>(p) >= arena && static_cast<char *>(p) < arena + arena_bytes)) cudaFree(p);
+    }
+
+    using Request = std::pair<void **, size_t>;
+    cudaError_t alloc_arena(const std::vector<Request> &want) {
+        size_t n = 0;
+        for (const Request &r : want) n += (r.second + 255) / 256 * 256;
+        void *p = nullptr;
+        const cudaError_t e = cudaMalloc(&p, n);
+        if (e != cudaSuccess) return e;
+        arena = static_cast<char *>(p);
+        arena_bytes = n;
+        size_t at = 0;
+        for (const Request &r : want) {
+            *r.first = arena + at;
+            at += (r.second + 255) / 256 * 256;
+        }
+        return cudaSuccess;
+    }
+
+    explicit steps_sim(std::shared_ptr<Tables> t) : tables(std::move(t)), tab(*tables) {}
+
     double time() const { return k_grid == 0 ? t_base : t_base + (double)k_grid * tab.tau; }
 
     ~steps_sim() {
         for (auto &g : graph)
             if (g) cudaGraphExecDestroy(g);
-        cudaFree(d_cnt[0]);
-        cudaFree(d_cnt[1]);
-        cudaFree(d_nbr);
-        cudaFree(d_thr);
-        cudaFree(d_inv_nav);
-        cudaFree(d_orig);
-        cudaFree(d_inv_perm);
-        cudaFree(d_rmask);
-        cudaFree(d_err);
-        cudaFree(d_window_base);
-        cudaFree(d_stage);
-        cudaFree(d_rec);
-        cudaFree(d_trial);
+        drop(d_cnt[0]);
+        drop(d_cnt[1]);
+        drop(d_nbr);
+        drop(d_thr);
+        drop(d_inv_nav);
+        drop(d_orig);
+        drop(d_inv_perm);
+        drop(d_rmask);
+        drop(d_err);
+        drop(d_window_base);
+        drop(d_stage);
+        drop(d_rec);
+        drop(d_trial);
         free_list();
-        cudaFree(d_leave[0]);
-        cudaFree(d_leave[1]);
-        cudaFree(d_G);
-        cudaFree(d_leave_list);
+        drop(d_leave[0]);
+        drop(d_leave[1]);
+        drop(d_G);
+        drop(d_leave_list);
         for (Flow &f : flow) {
             cudaFree(f.d_tnb_off);
             cudaFree(f.d_tnb);
             cudaFree(f.d_flow);
         }
+        cudaFree(arena);
     }
 
     // flow[k]'s kernel and tables (once): tile t lists itself and every tile
@@ -450,30 +481,21 @@ struct steps_sim {
     void free_list() {
         for (void **p : {(void **)&d_tm[0], (void **)&d_tm[1], (void **)&d_list[0], (void **)&d_list[1],
                          (void **)&d_lcnt, (void **)&d_tetrec, (void **)&d_src, (void **)&d_srcbits}) {
-            cudaFree(*p);
+            drop(*p);
             *p = nullptr;
         }
     }
 
     // the list form's buffers
-    cudaError_t alloc_list() {
+    std::vector<Request> list_requests() {
         const size_t n = (size_t)Tpad * 4;
-        cudaError_t e = cudaSuccess;
-        auto get = [&](void **p, size_t bytes) {
-            if (e == cudaSuccess) e = cudaMalloc(p, bytes);
-        };
-        get((void **)&d_tm[0], n);
-        get((void **)&d_tm[1], n);
-        get((void **)&d_list[0], 2 * n);
-        get((void **)&d_list[1], 2 * n);
-        get((void **)&d_lcnt, 16);
-        get((void **)&d_tetrec, 4 * n);
+        std::vector<Request> r = {{(void **)&d_tm[0], n},       {(void **)&d_tm[1], n}, {(void **)&d_list[0], 2 * n},
+                                  {(void **)&d_list[1], 2 * n}, {(void **)&d_lcnt, 16}, {(void **)&d_tetrec, 4 * n}};
         if (model.dev.order0) {
-            get((void **)&d_src, n);
-            get((void **)&d_srcbits, n / 32);
+            r.emplace_back((void **)&d_src, n);
+            r.emplace_back((void **)&d_srcbits, n / 32);
         }
-        if (e != cudaSuccess) free_list();
-        return e;
+        return r;
     }
 
     // Before a run: the form of its windows, by what is known of the state.
@@ -849,8 +871,10 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
     *out = nullptr;
     CHECK_NULL(mesh, "steps_sim_create");
     CHECK_NULL(model, "steps_sim_create");
-    std::unique_ptr<steps_sim> s(new (std::nothrow) steps_sim);
-    if (!s) {
+    std::unique_ptr<steps_sim> s;
+    try {
+        s.reset(new steps_sim(std::make_shared<Tables>()));
+    } catch (const std::bad_alloc &) {
         set_error("steps_sim_create: out of host memory");
         return STEPS_ERR_OOM;
     }
@@ -970,7 +994,9 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
         }
         if (s->spec) {
             s->spec_list = spec_list_kernel(s->model);
-            if (s->spec_list && (e = s->alloc_list()) != cudaSuccess) {
+            if (s->spec_list)
+                for (const steps_sim::Request &r : s->list_requests()) alloc(r.first, r.second);
+            if (e != cudaSuccess) {
                 set_error(std::string("steps_sim_create: device allocation failed: ") + cudaGetErrorString(e));
                 cudaGetLastError();
                 return STEPS_ERR_OOM;
@@ -989,13 +1015,15 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
     CHECK_NULL(out, "steps_sim_clone");
     *out = nullptr;
     CHECK_NULL(src, "steps_sim_clone");
-    std::unique_ptr<steps_sim> s(new (std::nothrow) steps_sim);
-    if (!s) {
+    std::unique_ptr<steps_sim> s;
+    try {
+        s.reset(new steps_sim(src->tables));
+        s->model = src->model;
+        s->h_rmask = src->h_rmask;
+    } catch (const std::bad_alloc &) {
         set_error("steps_sim_clone: out of host memory");
         return STEPS_ERR_OOM;
     }
-    s->model = src->model;
-    s->tab = src->tab;
     s->opt = src->opt;
     s->stream = (cudaStream_t)cuda_stream;
     s->device = src->device;
@@ -1003,16 +1031,13 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
     s->Tpad = src->Tpad;
     s->S = src->S;
     s->seed = seed;
-    s->h_rmask = src->h_rmask;
     s->spec = src->spec;
     s->spec_list = src->spec_list;
     s->spec_why = src->spec_why;
     std::memcpy(s->scale_full, src->scale_full, sizeof(s->scale_full));
     const size_t Tpad = (size_t)s->Tpad, S = (size_t)s->S, T = (size_t)s->T;
-    cudaError_t e = cudaSuccess;
-    auto alloc = [&](void **p, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMalloc(p, bytes);
-    };
+    std::vector<steps_sim::Request> want;
+    auto alloc = [&](void **p, size_t bytes) { want.emplace_back(p, bytes); };
     alloc((void **)&s->d_cnt[0], S * Tpad * 4);
     alloc((void **)&s->d_cnt[1], S * Tpad * 4);
     alloc((void **)&s->d_nbr, Tpad * 16);
@@ -1027,13 +1052,15 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
     }
     if (src->d_rmask) alloc((void **)&s->d_rmask, Tpad * 4);
     if (src->d_trial) alloc((void **)&s->d_trial, S * Tpad * 4);
-    if (src->d_tm[0] && e == cudaSuccess) e = s->alloc_list();
+    if (src->d_tm[0])
+        for (const steps_sim::Request &r : s->list_requests()) want.push_back(r);
     if (src->d_leave[0]) {
         alloc((void **)&s->d_leave[0], S * Tpad * 4);
         alloc((void **)&s->d_leave[1], S * Tpad * 4);
         alloc((void **)&s->d_G, Tpad * 8);
         alloc((void **)&s->d_leave_list, kLeaveListBytes);
     }
+    const cudaError_t e = s->alloc_arena(want);
     if (e != cudaSuccess) {
         set_error(std::string("steps_sim_clone: device allocation failed: ") + cudaGetErrorString(e));
         cudaGetLastError();
