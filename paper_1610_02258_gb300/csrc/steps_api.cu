@@ -159,20 +159,30 @@ __global__ void patch_leave(const uint2 *list, const uint32_t *value, uint32_t n
 
 __global__ void set_u64_kernel(uint64_t *p, uint64_t v) { *p = v; }
 
-// flag[0] |= 1 if any of src[0..n) is negative; flag[1] += the non-zero ones, if
-// asked for (grid-stride; one atomic per warp at most)
+// What an input holds: word 0 |= 1 if any of src[0..n) is negative; asked for
+// more, word 1 += the non-zero ones and words 2-3 (64 bits) += their sum
+// (grid-stride; one atomic per warp and word at most)
 template <bool COUNT>
 __global__ void any_negative(const int32_t *src, int64_t n, uint32_t *flag) {
     bool neg = false;
     uint32_t nz = 0;
+    unsigned long long sum = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        neg |= src[i] < 0;
-        if (COUNT) nz += src[i] != 0 ? 1u : 0u;
+        const int32_t v = src[i];
+        neg |= v < 0;
+        if (COUNT) {
+            nz += v != 0 ? 1u : 0u;
+            sum += (unsigned long long)max(v, 0);
+        }
     }
     if (__any_sync(0xFFFFFFFFu, neg) && (threadIdx.x & 31) == 0) atomicOr(flag, 1u);
     if (COUNT) {
         nz = __reduce_add_sync(0xFFFFFFFFu, nz);
-        if (nz && (threadIdx.x & 31) == 0) atomicAdd(flag + 1, nz);
+        for (int d = 16; d > 0; d >>= 1) sum += __shfl_down_sync(0xFFFFFFFFu, sum, d);
+        if (nz && (threadIdx.x & 31) == 0) {
+            atomicAdd(flag + 1, nz);
+            atomicAdd(reinterpret_cast<unsigned long long *>(flag + 2), sum);
+        }
     }
 }
 
@@ -195,14 +205,16 @@ void flow_neighbours(const std::vector<int32_t> &nbr_dev, int64_t T, int64_t B, 
 }
 
 // Launch-form choices of tuned simulations, shared by every simulation of
-// the same compiled kernel, tet count and block size (clones of one
-// prototype, the jobs of a stream): the first one's tuning run decides.
+// the same compiled kernel, tet count, block size and molecules per tet (to a
+// power of two; clones of one prototype, the jobs of a stream): the first
+// one's tuning run decides. (A tenth of the benchmark box's molecules runs 14 %
+// faster in another form than the box.)
 struct FlowChoice {
     int pick;
     float ms[3];
 };
 std::mutex g_flow_mu;
-std::map<std::tuple<const void *, int64_t, int>, FlowChoice> g_flow_choice;
+std::map<std::tuple<const void *, int64_t, int, int>, FlowChoice> g_flow_choice;
 
 bool cuda_ok(cudaError_t e, const char *what) {
     if (e == cudaSuccess) return true;
@@ -236,7 +248,7 @@ struct steps_sim {
     int32_t *d_inv_perm = nullptr;  // original id -> device index (null without reordering)
     uint32_t *d_rmask = nullptr;
     std::vector<uint32_t> h_rmask;  // device order
-    uint32_t *d_err = nullptr;      // [3]: window error word, input check flag, non-zero input counts
+    uint32_t *d_err = nullptr;      // [6]: window error word, unused, then any_negative's four
     uint64_t *d_window_base = nullptr;
     int32_t *d_stage = nullptr;     // [S * nt] original-order staging
     int32_t *d_rec = nullptr;       // recording selection (species, then tets)
@@ -260,6 +272,7 @@ struct steps_sim {
     bool src_valid = false;         // the records and the sources match the reaction masks
     bool listing = false;           // the present run's windows go through the list form
     uint64_t list_built = 0;        // the window the list was last built for
+    double density = 0.0;           // molecules per tet when counts were last set
     double fill = 0.0;              // listed tets or non-zero counts per tet, last known
     // time
     double t_base = 0.0;
@@ -677,7 +690,8 @@ struct steps_sim {
     // fastest flow form is kept when it is more than 2 % faster than window
     // launches. The windows taken are ordinary windows of the run.
     int tune_flow(int64_t *used) {
-        const auto key = std::make_tuple((const void *)spec, T, opt.block);
+        // the best form depends on the state: by powers of two of the molecules per tet
+        const auto key = std::make_tuple((const void *)spec, T, opt.block, (int)std::lrint(std::log2(density + 0.01)));
         {
             std::lock_guard<std::mutex> lock(g_flow_mu);
             auto it = g_flow_choice.find(key);
@@ -943,7 +957,7 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
     alloc((void **)&s->d_nbr, Tpad * 16);
     alloc((void **)&s->d_thr, Tpad * 16);
     alloc((void **)&s->d_inv_nav, Tpad * 4);
-    alloc((void **)&s->d_err, 12);
+    alloc((void **)&s->d_err, 24);
     alloc((void **)&s->d_window_base, 8);
     alloc((void **)&s->d_stage, S * T * 4);
     if (reordered) {
@@ -970,7 +984,7 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
                       "upload inv_nav") &&
               cuda_ok(cudaMemset(s->d_cnt[0], 0, S * Tpad * 4), "memset") &&
               cuda_ok(cudaMemset(s->d_cnt[1], 0, S * Tpad * 4), "memset") &&
-              cuda_ok(cudaMemset(s->d_err, 0, 12), "memset") && cuda_ok(cudaMemset(s->d_window_base, 0, 8), "memset");
+              cuda_ok(cudaMemset(s->d_err, 0, 24), "memset") && cuda_ok(cudaMemset(s->d_window_base, 0, 8), "memset");
     if (ok && reordered)
         ok = cuda_ok(cudaMemset(s->d_orig, 0, Tpad * 4), "memset") &&
              cuda_ok(cudaMemcpy(s->d_orig, s->tab.perm.data(), T * 4, cudaMemcpyHostToDevice), "upload perm") &&
@@ -1043,7 +1057,7 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
     alloc((void **)&s->d_nbr, Tpad * 16);
     alloc((void **)&s->d_thr, Tpad * 16);
     alloc((void **)&s->d_inv_nav, Tpad * 4);
-    alloc((void **)&s->d_err, 12);
+    alloc((void **)&s->d_err, 24);
     alloc((void **)&s->d_window_base, 8);
     alloc((void **)&s->d_stage, S * T * 4);
     if (src->d_orig) {
@@ -1072,7 +1086,7 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
               cuda_ok(cudaMemcpyAsync(s->d_inv_nav, src->d_inv_nav, Tpad * 4, cudaMemcpyDeviceToDevice, st), "clone") &&
               cuda_ok(cudaMemsetAsync(s->d_cnt[0], 0, S * Tpad * 4, st), "clone") &&
               cuda_ok(cudaMemsetAsync(s->d_cnt[1], 0, S * Tpad * 4, st), "clone") &&
-              cuda_ok(cudaMemsetAsync(s->d_err, 0, 12, st), "clone") &&
+              cuda_ok(cudaMemsetAsync(s->d_err, 0, 24, st), "clone") &&
               cuda_ok(cudaMemsetAsync(s->d_window_base, 0, 8, st), "clone");
     if (ok && src->d_orig)
         ok = cuda_ok(cudaMemcpyAsync(s->d_orig, src->d_orig, Tpad * 4, cudaMemcpyDeviceToDevice, st), "clone") &&
@@ -1113,15 +1127,14 @@ static int put_counts(steps_sim *sim, int32_t s0, int32_t ns, const int32_t *cou
                  "steps_set_counts: copy"))
         return STEPS_ERR_CUDA;
     // reject negative counts on the device, before anything of the state changes
-    uint32_t seen[2] = {0, 0};  // a negative count; non-zero ones
+    uint32_t seen[4] = {0, 0, 0, 0};  // a negative count; non-zero ones; their sum
     const int64_t n = (int64_t)ns * (int64_t)T;
-    if (!cuda_ok(cudaMemsetAsync(sim->d_err + 1, 0, 8, sim->stream), "steps_set_counts: check"))
+    if (!cuda_ok(cudaMemsetAsync(sim->d_err + 2, 0, 16, sim->stream), "steps_set_counts: check"))
         return STEPS_ERR_CUDA;
-    const unsigned grid = (unsigned)std::min<int64_t>((n + 255) / 256, 4096);
-    if (sim->spec_list) any_negative<true><<<grid, 256, 0, sim->stream>>>(sim->d_stage, n, sim->d_err + 1);
-    else any_negative<false><<<grid, 256, 0, sim->stream>>>(sim->d_stage, n, sim->d_err + 1);
+    any_negative<true><<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, sim->stream>>>(sim->d_stage, n,
+                                                                                                  sim->d_err + 2);
     if (!cuda_ok(cudaGetLastError(), "steps_set_counts: check") ||
-        !cuda_ok(cudaMemcpyAsync(seen, sim->d_err + 1, 8, cudaMemcpyDeviceToHost, sim->stream), "steps_set_counts: check") ||
+        !cuda_ok(cudaMemcpyAsync(seen, sim->d_err + 2, 16, cudaMemcpyDeviceToHost, sim->stream), "steps_set_counts: check") ||
         !cuda_ok(cudaStreamSynchronize(sim->stream), "steps_set_counts: check"))
         return STEPS_ERR_CUDA;
     if (seen[0]) {
@@ -1130,7 +1143,9 @@ static int put_counts(steps_sim *sim, int32_t s0, int32_t ns, const int32_t *cou
     }
     sim->tm_valid = sim->list_valid = false;
     // counts of every species replace the state; of one, they add to what is known of it
+    const double sum = (double)((uint64_t)seen[3] << 32 | seen[2]);
     sim->fill = (ns == sim->S ? 0.0 : sim->fill) + seen[1] / (double)T;
+    sim->density = (ns == sim->S ? 0.0 : sim->density) + sum / (double)T;
     scatter_to_device_order<<<(unsigned)((T + 255) / 256), 256, 0, sim->stream>>>(
         sim->d_stage, (int64_t)T, ns, sim->d_inv_perm, sim->d_cnt[sim->cur] + (size_t)s0 * Tpad, Tpad);
     if (!cuda_ok(cudaGetLastError(), "steps_set_counts: scatter")) return STEPS_ERR_CUDA;

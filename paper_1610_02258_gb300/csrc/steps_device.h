@@ -102,6 +102,13 @@ constexpr int kWarpMaxSpecies = 12;
 constexpr int kWarpMapCap = 160;    // Philox blocks listed at a time
 constexpr int kWarpQueueCap = 160;  // waiting movers: 31 left over + four words of 32 lanes
 
+// Whether a flow launch's blocks (of a compile-time size) stay resident and take
+// item after item, else one item each.
+#if defined(__CUDACC__) || defined(__CUDACC_RTC__)
+__host__ __device__
+#endif
+constexpr bool warp_flow_persists(int block) { return block > 0 && block < 512; }
+
 template <int SM>
 struct WarpTile {
     int32_t cnt[SM + 1][32];        // counts; row SM ones (a missing reactant)

@@ -120,7 +120,7 @@ __device__ __forceinline__ void list_planes(const StepArgs &a, const ListCtx<SM>
         i = x.w.idx[t];
         const int32_t M = a.trial[(uint64_t)(uint32_t)s * (uint32_t)a.Tpad + (uint32_t)i];
         uint32_t l[4];
-        plane_group(a, __ldg(a.thr + i), list_R<P>(a, x.s_scale, s, i), (uint32_t)M, e.x, x.w.tet[t], s, x.c0, x.c3, l);
+        plane_group(n == 32 ? 0xFFFFFFFFu : (1u << n) - 1u, a, __ldg(a.thr + i), list_R<P>(a, x.s_scale, s, i), (uint32_t)M, e.x, x.w.tet[t], s, x.c0, x.c3, l);
         // cumulative thresholds: l[0] within l[1] within l[2] within l[3]
         moved = (uint32_t)__popc(l[0]) | (uint32_t)__popc(l[1] & ~l[0]) << 8 | (uint32_t)__popc(l[2] & ~l[1]) << 16 |
                 (uint32_t)__popc(l[3] & ~l[2]) << 24;

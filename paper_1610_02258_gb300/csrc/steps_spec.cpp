@@ -298,6 +298,7 @@ struct Compiled {
     size_t smem_set_flow = 0;           // the flow kernel
     size_t smem_set_batch_flow = 0;     // the batched flow kernel
     size_t smem_set_batch = 0;          // and the batched one
+    bool warp = false;                  // warp-tile kernels
     cudaKernel_t kern_list = nullptr;   // or the list form's step kernel alone
     size_t smem = 0;                    // dynamic shared memory per block
 };
@@ -357,6 +358,7 @@ Compiled *compiled(const HostModel &hm, int block, bool list, std::string *why) 
     }
     auto c = std::make_shared<Compiled>();
     const size_t S = (size_t)hm.dev.S;
+    c->warp = !list && warp_tiles(hm);
     c->smem = list                 ? (size_t)(kListBlock / 32) * list_tile_bytes(hm.dev.S)
               : warp_tiles(hm) ? (size_t)(block / 32) * warp_tile_bytes(hm.dev.S)
                                    : (S + 1 + (spec_global_trial(hm) ? 0 : S)) * (size_t)block * sizeof(int32_t);
@@ -452,7 +454,9 @@ int launch_spec_flow(void *spec, const ModelDev &m, const StepArgs &a, const Flo
     ModelDev mm = m;
     FlowArgs ff = f;
     void *args[3] = {(void *)&mm, (void *)&b, (void *)&ff};
-    const unsigned grid = f.nwin * f.ntiles;  // one item per block
+    // one item per block, or the blocks resident at once
+    const unsigned items = f.nwin * f.ntiles;
+    const unsigned grid = c->warp && warp_flow_persists(block) ? std::min(items, (unsigned)(per_sm * sms)) : items;
     cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3((unsigned)block), args, smem, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         set_error(std::string("flow step kernel launch: ") + cudaGetErrorString(e));

@@ -245,8 +245,11 @@ __device__ __forceinline__ void move_out(const StepArgs &a, WarpTile<SM> &w, int
 }
 
 // The bit-plane draws of bulk_species for group g of species s: bit j of l[f]
-// says that molecule 32 g + j is below threshold T_f.
-__device__ __forceinline__ void plane_group(const StepArgs &a, const uint4 A, uint32_t R, uint32_t M, uint32_t g,
+// says that molecule 32 g + j is below threshold T_f. Called by the lanes of
+// `lanes`. Planes above every lane's last threshold (slow species leave with a
+// per cent or so) settle the molecules with a bit there, for all thresholds
+// alike: four planes in six operations instead of eighty.
+__device__ __forceinline__ void plane_group(uint32_t lanes, const StepArgs &a, const uint4 A, uint32_t R, uint32_t M, uint32_t g,
                                             uint32_t tet, int s, uint32_t c0, uint32_t c3, uint32_t l[4]) {
     const uint32_t m = min(32u, M - 32u * g);
     const uint32_t valid = m == 32u ? 0xFFFFFFFFu : (1u << m) - 1u;
@@ -258,9 +261,18 @@ __device__ __forceinline__ void plane_group(const StepArgs &a, const uint4 A, ui
     uint32_t l1 = T1 >= 0x80000000u ? valid : 0u, u1 = (T1 >= 0x80000000u || T1 == 0u) ? 0u : valid;
     uint32_t l2 = T2 >= 0x80000000u ? valid : 0u, u2 = (T2 >= 0x80000000u || T2 == 0u) ? 0u : valid;
     uint32_t l3 = T3 >= 0x80000000u ? valid : 0u, u3 = (T3 >= 0x80000000u || T3 == 0u) ? 0u : valid;
+    const uint32_t zeros = __reduce_min_sync(lanes, (uint32_t)max(0, __clz((int)T3) - 1)) / 4u;
     for (uint32_t blk = 0; blk < 8u && (u0 | u1 | u2 | u3); ++blk) {
         const uint4 r = philox_rk(a.rk, c0, tet, (g << 3) | blk, c3b);
         const int sh = 30 - 4 * (int)blk;
+        if (blk < zeros && blk < 7u) {
+            const uint32_t rest = ~(r.x | r.y | r.z | r.w);
+            u0 &= rest;
+            u1 &= rest;
+            u2 &= rest;
+            u3 &= rest;
+            continue;
+        }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             if (q < 3 || blk < 7u) {  // 31 planes
@@ -292,7 +304,7 @@ __device__ __forceinline__ void plane_groups(const StepArgs &a, WarpTile<SM> &w,
         const uint2 e = w.d.q[first + lane];
         const int t = (int)(e.y & 31u), s = (int)(e.y >> 5);
         uint32_t l[4];
-        plane_group(a, w.thr[t], warp_R<P>(a, s_scale, s, i0 + t), (uint32_t)w.trial[s][t], e.x, w.tet[t], s, c0, c3, l);
+        plane_group(n == 32 ? 0xFFFFFFFFu : (1u << n) - 1u, a, w.thr[t], warp_R<P>(a, s_scale, s, i0 + t), (uint32_t)w.trial[s][t], e.x, w.tet[t], s, c0, c3, l);
         // cumulative thresholds: l[0] within l[1] within l[2] within l[3]
         const int32_t n0 = __popc(l[0]), n1 = __popc(l[1] & ~l[0]), n2 = __popc(l[2] & ~l[1]), n3 = __popc(l[3] & ~l[2]);
         const int4 nb = w.nbr[t];
@@ -392,22 +404,29 @@ __device__ __forceinline__ bool flow_nbr_wait(const uint32_t *done, uint32_t own
     const uint32_t *base = done + own - (uint32_t)(i0 >> 5);
     const uint32_t *p[4] = {nb.x < 0 ? done + own : base + (nb.x >> 5), nb.y < 0 ? done + own : base + (nb.y >> 5),
                             nb.z < 0 ? done + own : base + (nb.z >> 5), nb.w < 0 ? done + own : base + (nb.w >> 5)};
-    const long long t0 = clock64();
-    uint32_t open = 31u;  // words not seen done yet: a lane reads only those again
-    for (uint32_t ns = 32;;) {
-        uint32_t v[5];
+    uint32_t v[5];
 #pragma unroll
-        for (int k = 0; k < 5; ++k)
-            if ((open >> k) & 1u)
-                asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v[k]) : "l"(k < 4 ? p[k] : done + own) : "memory");
+    for (int k = 0; k < 5; ++k)
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v[k]) : "l"(k < 4 ? p[k] : done + own) : "memory");
+    uint32_t open = 0u;  // words not seen done yet: a lane reads only those again
 #pragma unroll
-        for (int k = 0; k < 5; ++k)
-            if (((open >> k) & 1u) && (int32_t)(v[k] - need) >= 0) open &= ~(1u << k);
-        if (__all_sync(0xFFFFFFFFu, open == 0u)) break;
-        if (__any_sync(0xFFFFFFFFu, clock64() - t0 > limit)) return false;
-        // every waiting warp polls: back off, so that the ones at work are not held up
-        __nanosleep(ns);
-        ns = min(2u * ns, 1024u);
+    for (int k = 0; k < 5; ++k) open |= (int32_t)(v[k] - need) >= 0 ? 0u : 1u << k;
+    if (!__all_sync(0xFFFFFFFFu, open == 0u)) {
+        const long long t0 = clock64();
+        uint32_t ns = 32;
+        do {
+            if (__any_sync(0xFFFFFFFFu, clock64() - t0 > limit)) return false;
+            // every waiting warp polls: back off, so that the ones at work are not held up
+            __nanosleep(ns);
+            ns = min(2u * ns, 1024u);
+            for (uint32_t left = open; left; left &= left - 1) {
+                const int k = __ffs(left) - 1;
+                const uint32_t *w = k == 0 ? p[0] : k == 1 ? p[1] : k == 2 ? p[2] : k == 3 ? p[3] : done + own;
+                uint32_t x;
+                asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(w) : "memory");
+                if ((int32_t)(x - need) >= 0) open &= ~(1u << k);
+            }
+        } while (!__all_sync(0xFFFFFFFFu, open == 0u));
     }
     asm volatile("fence.acq_rel.gpu;" ::: "memory");
     __syncwarp();
@@ -416,9 +435,10 @@ __device__ __forceinline__ bool flow_nbr_wait(const uint32_t *done, uint32_t own
 
 // One diffusion window for the 32 tets from i0 on, one warp. FLOW as in
 // step_tile, with the finished-window words by warp tile
-// (dep): window a.window + q, buffers swapped when q is odd.
+// (dep): window a.window + q, buffers swapped when q is odd. False when the
+// tiles it waits for did not finish within the wait limit.
 template <int RM, int SM, class P, int FLOW>
-__device__ __forceinline__ void warp_window(const ModelDev &m, const StepArgs &a, WarpTile<SM> &w, const RxnTab &tb,
+__device__ __forceinline__ bool warp_window(const ModelDev &m, const StepArgs &a, WarpTile<SM> &w, const RxnTab &tb,
                                             const uint32_t *s_scale, int64_t i0, const FlowArgs *f, uint32_t q,
                                             uint32_t dep) {
     constexpr int NP = (SM + 3) / 4;
@@ -451,7 +471,7 @@ __device__ __forceinline__ void warp_window(const ModelDev &m, const StepArgs &a
     if constexpr (FLOW != 0) {
         if (q > 0 && !flow_nbr_wait(f->tile_done, dep, i0, nb4, (uint32_t)(a.window + q))) {
             if (lane == 0) atomicOr(a.err, 8u);
-            return;
+            return false;
         }
     } else {
         asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -646,6 +666,7 @@ __device__ __forceinline__ void warp_window(const ModelDev &m, const StepArgs &a
         __syncwarp();
         if (lane == 0) st_release_gpu(f->tile_done + dep, (uint32_t)(a.window + q + 1));
     }
+    return true;
 }
 
 // The warps of a block: they share the reaction table and the species scales;
@@ -662,6 +683,7 @@ __device__ __forceinline__ void warp_step(const ModelDev &m, const StepArgs &a, 
     __shared__ uint32_t s_scale[kMaxSpecies];
     static_assert(SM <= kWarpMaxSpecies, "species bound");
     const int threads = BLOCK ? BLOCK : (int)blockDim.x, warps = threads / 32;
+    constexpr bool PERSIST = warp_flow_persists(BLOCK);
     const int tid = threadIdx.x, warp = tid >> 5;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -672,13 +694,22 @@ __device__ __forceinline__ void warp_step(const ModelDev &m, const StepArgs &a, 
     if constexpr (FLOW == 1) {
         __shared__ uint32_t s_item;
         const uint32_t items = f->nwin * f->ntiles;
-        if (tid == 0) s_item = atomicAdd(f->fetch, 1u);
-        __syncthreads();
-        const uint32_t item = s_item;
-        if (item >= items) return;
-        const uint32_t qq = item / f->ntiles, t = item - qq * f->ntiles;
-        const int64_t i0 = (int64_t)t * threads + warp * 32;
-        if (i0 < a.T) warp_window<RM, SM, P, FLOW>(m, a, w, tb, s_scale, i0, f, qq, t * (uint32_t)warps + (uint32_t)warp);
+        uint32_t next = 0;
+        if (tid == 0) next = atomicAdd(f->fetch, 1u);
+        for (;;) {
+            if (tid == 0) s_item = next;
+            __syncthreads();
+            const uint32_t item = s_item;
+            if (item >= items) return;
+            // the next item, fetched while this one runs
+            if (PERSIST && tid == 0) next = atomicAdd(f->fetch, 1u);
+            const uint32_t qq = item / f->ntiles, t = item - qq * f->ntiles;
+            const int64_t i0 = (int64_t)t * threads + warp * 32;
+            bool done = true;
+            if (i0 < a.T)
+                done = warp_window<RM, SM, P, FLOW>(m, a, w, tb, s_scale, i0, f, qq, t * (uint32_t)warps + (uint32_t)warp);
+            if (!PERSIST || __syncthreads_or(!done)) return;  // (a wait that ran out ends the block)
+        }
     } else {
         const int64_t i0 = tile * threads + warp * 32;
         if (i0 < a.T) warp_window<RM, SM, P, FLOW>(m, a, w, tb, s_scale, i0, f, q, dep * (uint32_t)warps + (uint32_t)warp);
