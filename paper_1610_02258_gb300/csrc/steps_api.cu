@@ -37,11 +37,12 @@ namespace {
 
 constexpr int kGraphWindows = 16;  // full windows per captured graph (even: buffer parity is restored)
 // The list form runs a state of at most this many listed tets (or, from set
-// counts, non-zero counts) per tet. us per window, block tiles -> list form:
-// 1.03M-tet dendrite, 0.12: 39.8 -> 14.8; 294,780-tet box with 14, 20 and 30
-// species at 0.2, 0.31, 0.49: 19.2 -> 14.2, 23.3 -> 21.0, 27.6 -> 21.9, at
-// 1.0, 1.6, 2.4: 25 -> 42, 35 -> 46, 45 -> 55; 300k-tet dendrite, 0.35: 17 -> 23.
-constexpr double kListFill = 0.25;
+// counts, non-zero counts) per tet. us per window, warp tiles -> list form:
+// 1.03M-tet dendrite, 0.12: 61.8 -> 14.6; 294,780-tet box with 14, 20 and 30
+// species at 0.2, 0.31, 0.48: 19.6 -> 15.3, 22.0 -> 16.2, 34.1 -> 16.7; but
+// with 14 at 1.0: 23.3 -> 28.3, and the 300k-tet dendrite, whose molecules
+// crowd at one end, 0.37: 15.8 -> 19.1.
+constexpr double kListFill = 0.33;
 constexpr uint64_t kListWindows = 128;       // windows after which a list is built afresh
 constexpr int64_t kListCheckWindows = 1024;  // windows after which a run looks at the list's length
 constexpr int64_t kFlowTuneWindows = 72;  // windows the launch-form tuning takes (3 rounds of up to 3 groups)
@@ -187,16 +188,15 @@ __global__ void any_negative(const int32_t *src, int64_t n, uint32_t *flag) {
 }
 
 // The tiles every tile of a flow launch waits for (CSR): itself and every tile
-// holding a face neighbour of one of its tets. Tiles of B tets in device
-// order; `base` is added to every index.
-void flow_neighbours(const std::vector<int32_t> &nbr_dev, int64_t T, int64_t B, int64_t base,
-                     std::vector<int32_t> &off, std::vector<int32_t> &nb) {
+// holding a face neighbour of one of its tets. Tiles of B tets in device order.
+void flow_neighbours(const std::vector<int32_t> &nbr_dev, int64_t T, int64_t B, std::vector<int32_t> &off,
+                     std::vector<int32_t> &nb) {
     std::vector<int32_t> tmp;
     for (int64_t t = 0; t * B < T; ++t) {
-        tmp.assign(1, (int32_t)(base + t));
+        tmp.assign(1, (int32_t)t);
         for (int64_t d = 4 * t * B; d < 4 * std::min(T, (t + 1) * B); ++d) {
             const int32_t j = nbr_dev[(size_t)d];
-            if (j >= 0 && j / B != t) tmp.push_back((int32_t)(base + j / B));
+            if (j >= 0 && j / B != t) tmp.push_back((int32_t)(j / B));
         }
         std::sort(tmp.begin(), tmp.end());
         off.push_back((int32_t)nb.size());
@@ -254,7 +254,7 @@ struct steps_sim {
     int32_t *d_rec = nullptr;       // recording selection (species, then tets)
     size_t rec_bytes = 0;
     void *spec = nullptr;           // step kernel compiled for this model (cached process-wide), or null
-    int32_t *d_trial = nullptr;     // [S][Tpad] trial counts for specialised kernels that keep them in global memory
+    int32_t *d_trial = nullptr;     // list form: [S][Tpad] trial counts that differ from the count
     uint32_t *d_leave[2] = {nullptr, nullptr};  // EXP leave law: [S][Tpad] tables of the full and the last window
     double *d_G = nullptr;          // [Tpad] the tets' total face rates, and
     uint32_t *d_leave_list = nullptr;  // the entries the host decides: their number, (species, tet) each, values
@@ -346,7 +346,6 @@ struct steps_sim {
         drop(d_window_base);
         drop(d_stage);
         drop(d_rec);
-        drop(d_trial);
         free_list();
         drop(d_leave[0]);
         drop(d_leave[1]);
@@ -375,12 +374,12 @@ struct steps_sim {
         if (!sp && !(generic && B == 256)) return STEPS_OK;
         // a warp-tile kernel publishes per 32 tets and finds the tiles it waits
         // for from its tets' neighbours: it needs no lists
-        const bool warp = warp_tiles(model);
+        const bool warp = sp || model.dev.S <= kWarpGenericSpecies;
         const int64_t nt = (T + B - 1) / B, nwords = warp ? nt * (B / 32) : nt;
         std::vector<int32_t> off, nb;
         if (!warp) {
             try {
-                flow_neighbours(tab.nbr_dev, T, B, 0, off, nb);
+                flow_neighbours(tab.nbr_dev, T, B, off, nb);
                 off.push_back((int32_t)nb.size());
             } catch (const std::bad_alloc &) {
                 set_error("flow tables: out of host memory");
@@ -482,18 +481,9 @@ struct steps_sim {
         }
     }
 
-    // the global trial buffer the model-specialised kernels of this model need (if any)
-    int ensure_trial() {
-        if (d_trial || !(spec_global_trial(model) || spec_list)) return STEPS_OK;
-        if (!cuda_ok(cudaMalloc((void **)&d_trial, (size_t)S * (size_t)Tpad * 4), "trial buffer"))
-            return STEPS_ERR_OOM;
-        drop_graphs();  // the captured launches hold the old arguments
-        return STEPS_OK;
-    }
-
     void free_list() {
         for (void **p : {(void **)&d_tm[0], (void **)&d_tm[1], (void **)&d_list[0], (void **)&d_list[1],
-                         (void **)&d_lcnt, (void **)&d_tetrec, (void **)&d_src, (void **)&d_srcbits}) {
+                         (void **)&d_lcnt, (void **)&d_tetrec, (void **)&d_trial, (void **)&d_src, (void **)&d_srcbits}) {
             drop(*p);
             *p = nullptr;
         }
@@ -503,7 +493,8 @@ struct steps_sim {
     std::vector<Request> list_requests() {
         const size_t n = (size_t)Tpad * 4;
         std::vector<Request> r = {{(void **)&d_tm[0], n},       {(void **)&d_tm[1], n}, {(void **)&d_list[0], 2 * n},
-                                  {(void **)&d_list[1], 2 * n}, {(void **)&d_lcnt, 16}, {(void **)&d_tetrec, 4 * n}};
+                                  {(void **)&d_list[1], 2 * n}, {(void **)&d_lcnt, 16}, {(void **)&d_tetrec, 4 * n},
+                                  {(void **)&d_trial, (size_t)S * n}};
         if (model.dev.order0) {
             r.emplace_back((void **)&d_src, n);
             r.emplace_back((void **)&d_srcbits, n / 32);
@@ -524,16 +515,16 @@ struct steps_sim {
     // records and sources the masks, and the list is window k_total's. Windows
     // append tets in the order their warps meet them; building the list afresh
     // now and then keeps neighbours together.
-    int prepare_list() {
+    int prepare_list(cudaStream_t st) {
         if (!listing || (tm_valid && src_valid && list_valid && k_total - list_built < kListWindows)) return STEPS_OK;
         const unsigned grid = (unsigned)((T + 255) / 256);
         if (!tm_valid)
-            build_species_words<<<grid, 256, 0, stream>>>(d_cnt[cur], T, (size_t)Tpad, S, d_tm[cur], d_tm[1 - cur]);
-        if (!cuda_ok(cudaMemsetAsync(d_lcnt, 0, src_valid ? 12 : 16, stream), "tet lists")) return STEPS_ERR_CUDA;
+            build_species_words<<<grid, 256, 0, st>>>(d_cnt[cur], T, (size_t)Tpad, S, d_tm[cur], d_tm[1 - cur]);
+        if (!cuda_ok(cudaMemsetAsync(d_lcnt, 0, src_valid ? 12 : 16, st), "tet lists")) return STEPS_ERR_CUDA;
         if (!src_valid)
-            build_sources<<<grid, 256, 0, stream>>>(d_rmask, model.dev.order0, T, d_thr, d_orig, d_inv_nav, d_tetrec,
+            build_sources<<<grid, 256, 0, st>>>(d_rmask, model.dev.order0, T, d_thr, d_orig, d_inv_nav, d_tetrec,
                                                     d_srcbits, d_src, d_lcnt + 3);
-        build_list<<<grid, 256, 0, stream>>>(d_tm[cur], T, d_srcbits, d_list[k_total & 1], d_lcnt + k_total % 3);
+        build_list<<<grid, 256, 0, st>>>(d_tm[cur], T, d_srcbits, d_list[k_total & 1], d_lcnt + k_total % 3);
         if (!cuda_ok(cudaGetLastError(), "tet lists")) return STEPS_ERR_CUDA;
         tm_valid = src_valid = list_valid = true;
         list_built = k_total;
@@ -624,7 +615,7 @@ struct steps_sim {
         uint32_t scale[kMaxSpecies] = {};
         for (int s = 0; s < S; ++s) scale[s] = species_scale(model, tab, s, tau_k);
         StepArgs a = args(cur, k_total, nullptr, tau_k, scale);
-        int rc = prepare_list();
+        int rc = prepare_list(stream);
         if (!rc) rc = launch(a, stream);
         if (rc) return rc;
         ++launches;
@@ -759,7 +750,7 @@ struct steps_sim {
             if (!cuda_ok(cudaGetLastError(), "set window base")) return STEPS_ERR_CUDA;
             ++launches;
             while (n - done >= kGraphWindows) {
-                int rc = prepare_list();
+                int rc = prepare_list(stream);
                 if (rc) return rc;
                 if (!cuda_ok(cudaGraphLaunch(graph[cur], stream), "cudaGraphLaunch")) return STEPS_ERR_CUDA;
                 launches += kGraphWindows + 1;
@@ -769,7 +760,7 @@ struct steps_sim {
         }
         for (; done < n; ++done) {
             StepArgs a = args(cur, k_total, nullptr, tab.tau, scale_full);
-            int rc = prepare_list();
+            int rc = prepare_list(stream);
             if (!rc) rc = launch(a, stream);
             if (rc) return rc;
             ++launches;
@@ -1015,8 +1006,6 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
                 cudaGetLastError();
                 return STEPS_ERR_OOM;
             }
-            int rc = s->ensure_trial();
-            if (rc) return rc;
         }
     } else {
         s->spec_why = "not requested";
@@ -1065,7 +1054,6 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
         alloc((void **)&s->d_inv_perm, T * 4);
     }
     if (src->d_rmask) alloc((void **)&s->d_rmask, Tpad * 4);
-    if (src->d_trial) alloc((void **)&s->d_trial, S * Tpad * 4);
     if (src->d_tm[0])
         for (const steps_sim::Request &r : s->list_requests()) want.push_back(r);
     if (src->d_leave[0]) {
@@ -1656,9 +1644,16 @@ struct steps_batch {
     struct Work {
         BlockWork *d = nullptr;
         int64_t n = 0;
+        bool built = false;
         cudaGraphExec_t graph = nullptr;
     };
     Work work[4];  // block sizes 64, 128, 256, 512
+    // members whose windows go through the list form in this run (their blocks
+    // are not in `work`), its kernel and their blocks
+    std::vector<char> listed;
+    void *spec_list = nullptr;
+    Work lwork;
+    uint32_t *h_lcnt = nullptr;  // pinned: their list lengths after the run
     uint64_t launches = 0;
     bool use_spec = false;      // run the model-specialised batched kernel
     bool spec_forced = false;
@@ -1666,14 +1661,11 @@ struct steps_batch {
     std::string spec_why;
     std::vector<float> tune_ms;  // autotune timings per candidate block (ms per window)
     bool flow = false;           // full windows of member groups as flow launches (specialised kernel)
-    // flow launches, per block size: the neighbour tiles of every work entry
-    // (CSR over work indices), the entries' finished-window words followed by
-    // the item counter, and the groups: consecutive members whose tables fit
-    // in about half of L2 (at least one member each), so that a group's
-    // windows run from L2
+    // flow launches, per block size: the finished-window words of every work
+    // entry's warp tiles followed by the item counter, and the groups:
+    // consecutive members whose tables fit in about half of L2 (at least one
+    // member each), so that a group's windows run from L2
     struct Flow {
-        int32_t *d_tnb_off = nullptr;
-        int32_t *d_tnb = nullptr;
         uint32_t *d_flow = nullptr;
         std::vector<std::pair<int64_t, int64_t>> groups;  // (first work entry, entries)
         int64_t nwords = 0;
@@ -1687,33 +1679,75 @@ struct steps_batch {
             if (w.graph) cudaGraphExecDestroy(w.graph);
             cudaFree(w.d);
         }
-        for (auto &f : fl) {
-            cudaFree(f.d_tnb_off);
-            cudaFree(f.d_tnb);
-            cudaFree(f.d_flow);
-        }
+        for (auto &f : fl) cudaFree(f.d_flow);
         cudaFree(d_reps);
         cudaFree(d_err);
+        cudaFree(lwork.d);
+        cudaFreeHost(h_lcnt);
         cudaFreeHost(h_err);
         cudaFreeHost(h_last);
         cudaFreeHost(h_reps);
     }
 
-    int build_work(int b) {
-        Work &w = work[slot(b)];
-        if (w.d) return STEPS_OK;
-        std::vector<BlockWork> v;
-        for (size_t j = 0; j < members.size(); ++j) {
-            const int64_t tiles = (members[j]->T + b - 1) / b;
-            for (int64_t t = 0; t < tiles; ++t) v.push_back(BlockWork{(int32_t)j, (int32_t)t});
-        }
+    // `v` as a work list on the device
+    static int upload_work(Work &w, const std::vector<BlockWork> &v) {
         w.n = (int64_t)v.size();
         if (w.n == 0) return STEPS_OK;
         if (!cuda_ok(cudaMalloc((void **)&w.d, v.size() * sizeof(BlockWork)), "steps_batch: alloc work"))
             return STEPS_ERR_OOM;
-        if (!cuda_ok(cudaMemcpy(w.d, v.data(), v.size() * sizeof(BlockWork), cudaMemcpyHostToDevice),
-                     "steps_batch: upload work"))
-            return STEPS_ERR_CUDA;
+        return cuda_ok(cudaMemcpy(w.d, v.data(), v.size() * sizeof(BlockWork), cudaMemcpyHostToDevice),
+                       "steps_batch: upload work")
+                   ? STEPS_OK
+                   : STEPS_ERR_CUDA;
+    }
+
+    int build_work(int b) {
+        Work &w = work[slot(b)];
+        if (w.built) return STEPS_OK;
+        std::vector<BlockWork> v;
+        for (size_t j = 0; j < members.size(); ++j) {
+            const int64_t tiles = listed[j] ? 0 : (members[j]->T + b - 1) / b;
+            for (int64_t t = 0; t < tiles; ++t) v.push_back(BlockWork{(int32_t)j, (int32_t)t});
+        }
+        w.built = true;
+        return upload_work(w, v);
+    }
+
+    // The members of this run's list form, by what is known of their states; the
+    // work lists and graphs follow when they change.
+    int choose_forms() {
+        std::vector<char> want(members.size(), 0);
+        for (size_t j = 0; j < members.size(); ++j) {
+            const steps_sim *m = members[j];
+            want[j] = use_spec && !flow && m->spec_list && m->fill <= kListFill;
+            if (want[j]) spec_list = m->spec_list;
+        }
+        if (want != listed) {
+            for (Work *w : {&work[0], &work[1], &work[2], &work[3], &lwork}) {
+                if (w->graph) cudaGraphExecDestroy(w->graph);
+                cudaFree(w->d);
+                *w = Work{};
+            }
+            listed = std::move(want);
+        }
+        if (!lwork.built) {
+            std::vector<BlockWork> v;
+            for (size_t j = 0; j < members.size(); ++j) {
+                const int64_t n = listed[j] ? list_blocks(members[j]->T, 256) : 0;
+                for (int64_t t = 0; t < n; ++t) v.push_back(BlockWork{(int32_t)j, (int32_t)t});
+            }
+            lwork.built = true;
+            int rc = upload_work(lwork, v);
+            if (rc) return rc;
+        }
+        for (size_t j = 0; j < members.size(); ++j) {
+            steps_sim *m = members[j];
+            if (m->listing != (bool)listed[j]) m->drop_graphs();
+            m->listing = listed[j];
+            if (!m->listing) m->tm_valid = m->list_valid = false;  // the other kernels leave them behind
+            int rc = m->prepare_list(stream);
+            if (rc) return rc;
+        }
         return STEPS_OK;
     }
 
@@ -1735,6 +1769,7 @@ struct steps_batch {
         Work &w = work[slot(b)];
         int rc = use_spec && spec[slot(b)] ? launch_spec_batch(spec[slot(b)], w.d, w.n, d_reps, max_S, b, st)
                                            : launch_step_batch(w.d, w.n, d_reps, max_S, max_R, any_order0, b, st);
+        if (!rc && lwork.n) rc = launch_spec_batch(spec_list, lwork.d, lwork.n, d_reps, max_S, 256, st);
         if (!rc) rc = launch_advance(d_reps, (int32_t)members.size(), st);
         launches += 2;
         return rc;
@@ -1762,7 +1797,7 @@ struct steps_batch {
         return rc;
     }
 
-    // the flow tables of block size b (once; build_work(b) first)
+    // the flow words and groups of block size b (once; build_work(b) first)
     int build_flow(int b) {
         Flow &f = fl[slot(b)];
         if (f.d_flow) return STEPS_OK;
@@ -1770,14 +1805,12 @@ struct steps_batch {
         if (!cuda_ok(cudaGetDevice(&dev), "steps_batch: device") ||
             !cuda_ok(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev), "steps_batch: L2 size"))
             return STEPS_ERR_CUDA;
-        std::vector<int32_t> off, nb;
         std::vector<std::pair<int64_t, int64_t>> groups;
         int64_t nwork = 0;
-        const bool warp = warp_tiles(members[0]->model);  // (flow runs on specialised kernels only)
         try {
             int64_t gfirst = 0, gbytes = 0;
             for (steps_sim *m : members) {
-                const int64_t B = b, T = m->T, tiles = (T + B - 1) / B, base = nwork;
+                const int64_t T = m->T, tiles = (T + b - 1) / b;
                 // counts (both buffers) and tables the member's windows touch
                 const int64_t bytes = T * (8 * (int64_t)m->S + 40) + (m->d_rmask ? 4 * T : 0);
                 if (nwork > gfirst && gbytes + bytes > (int64_t)l2 / 2) {
@@ -1786,10 +1819,8 @@ struct steps_batch {
                     gbytes = 0;
                 }
                 gbytes += bytes;
-                if (!warp) flow_neighbours(m->tab.nbr_dev, T, B, base, off, nb);
                 nwork += tiles;
             }
-            off.push_back((int32_t)nb.size());
             if (nwork > gfirst) groups.emplace_back(gfirst, nwork - gfirst);
         } catch (const std::bad_alloc &) {
             set_error("steps_batch: flow tables: out of host memory");
@@ -1799,23 +1830,11 @@ struct steps_batch {
             set_error("steps_batch: flow tables do not match the work list");
             return STEPS_ERR_STATE;
         }
-        // (a warp-tile kernel publishes per 32 tets and needs no lists)
-        const int64_t nwords = warp ? nwork * (b / 32) : nwork;
-        if ((!warp && (!cuda_ok(cudaMalloc((void **)&f.d_tnb_off, off.size() * 4), "steps_batch: flow tables") ||
-                       !cuda_ok(cudaMalloc((void **)&f.d_tnb, nb.size() * 4), "steps_batch: flow tables"))) ||
-            !cuda_ok(cudaMalloc((void **)&f.d_flow, ((size_t)nwords + 1) * 4), "steps_batch: flow tables")) {
-            cudaFree(f.d_tnb_off);
-            cudaFree(f.d_tnb);
-            cudaFree(f.d_flow);
-            f.d_tnb_off = f.d_tnb = nullptr;
-            f.d_flow = nullptr;
+        // flow runs on the specialised kernels only: warp tiles, which publish per 32 tets and need no lists
+        const int64_t nwords = nwork * (b / 32);
+        if (!cuda_ok(cudaMalloc((void **)&f.d_flow, ((size_t)nwords + 1) * 4), "steps_batch: flow words"))
             return STEPS_ERR_OOM;
-        }
-        if ((!warp &&
-             (!cuda_ok(cudaMemcpy(f.d_tnb_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice), "steps_batch") ||
-              !cuda_ok(cudaMemcpy(f.d_tnb, nb.data(), nb.size() * 4, cudaMemcpyHostToDevice), "steps_batch"))) ||
-            !cuda_ok(cudaMemset(f.d_flow, 0, ((size_t)nwords + 1) * 4), "steps_batch"))
-            return STEPS_ERR_CUDA;
+        if (!cuda_ok(cudaMemset(f.d_flow, 0, ((size_t)nwords + 1) * 4), "steps_batch")) return STEPS_ERR_CUDA;
         f.nwords = nwords;
         f.groups = std::move(groups);
         return STEPS_OK;
@@ -1835,8 +1854,7 @@ struct steps_batch {
                 if (!cuda_ok(cudaMemsetAsync(f.d_flow + f.nwords, 0, 4, stream), "steps_batch: flow counter"))
                     return STEPS_ERR_CUDA;
                 FlowArgs a;
-                a.tnb_off = f.d_tnb_off;
-                a.tnb = f.d_tnb;
+                a.tnb_off = a.tnb = nullptr;
                 a.tile_done = f.d_flow;
                 a.fetch = f.d_flow + f.nwords;
                 a.nwin = (uint32_t)nw;
@@ -1928,6 +1946,8 @@ int steps_batch_create(steps_sim *const *members, int32_t n, const steps_batch_o
     if (!cuda_ok(cudaMallocHost((void **)&b->h_reps, sizeof(RepEntry) * n), "steps_batch_create: host alloc") ||
         !cuda_ok(cudaMallocHost((void **)&b->h_last, sizeof(RepEntry) * n), "steps_batch_create: host alloc") ||
         !cuda_ok(cudaMallocHost((void **)&b->h_err, 4), "steps_batch_create: host alloc") ||
+        (std::any_of(b->members.begin(), b->members.end(), [](const steps_sim *m) { return m->spec_list != nullptr; }) &&
+         !cuda_ok(cudaMallocHost((void **)&b->h_lcnt, (size_t)n * 16), "steps_batch_create: host alloc")) ||
         !cuda_ok(cudaMalloc((void **)&b->d_reps, sizeof(RepEntry) * n), "steps_batch_create: alloc") ||
         !cuda_ok(cudaMalloc((void **)&b->d_err, 4), "steps_batch_create: alloc") ||
         !cuda_ok(cudaMemset(b->d_err, 0, 4), "steps_batch_create: memset"))
@@ -1953,12 +1973,8 @@ int steps_batch_create(steps_sim *const *members, int32_t n, const steps_batch_o
         return STEPS_ERR_ARG;
     }
     b->spec_forced = o.specialize > 0 || any_exp;
+    b->listed.assign((size_t)n, 0);
     b->use_spec = uniform && (o.specialize > 0 || any_exp || (o.specialize == 0 && tets >= kSpecializeMinTets));
-    if (b->use_spec)
-        for (steps_sim *m : b->members) {
-            int rc = m->ensure_trial();
-            if (rc) return rc;
-        }
     int rc = b->build_work(b->block);
     if (rc) return rc;
     *out = b.release();
@@ -2005,7 +2021,7 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
             if (int rl = m->upload_leave(partial[j], b->stream)) return rl;
         nmax = std::max(nmax, nfull[j]);
     }
-    for (steps_sim *m : b->members) m->tm_valid = m->list_valid = false;  // the batched kernels leave them behind
+    if (int rf = b->choose_forms()) return rf;
     // table for the full windows
     for (size_t j = 0; j < n; ++j) {
         steps_sim *m = b->members[j];
@@ -2016,6 +2032,8 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
         e.args.err = b->d_err;
         e.cnt[0] = m->d_cnt[0];
         e.cnt[1] = m->d_cnt[1];
+        e.tm[0] = m->d_tm[0];
+        e.tm[1] = m->d_tm[1];
         e.parity = (uint32_t)m->cur;
         e.window_end = m->k_total + (uint64_t)nfull[j];
     }
@@ -2119,6 +2137,11 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
             m->k_grid += nfull[j];
         }
     }
+    for (size_t j = 0; j < n; ++j)
+        if (b->listed[j] && !cuda_ok(cudaMemcpyAsync(b->h_lcnt + 4 * j, b->members[j]->d_lcnt, 16,
+                                                     cudaMemcpyDeviceToHost, b->stream),
+                                     "steps_batch_run: list length"))
+            return STEPS_ERR_CUDA;
     if (!cuda_ok(cudaMemcpyAsync(b->h_err, b->d_err, 4, cudaMemcpyDeviceToHost, b->stream),
                  "steps_batch_run: error word"))
         return STEPS_ERR_CUDA;
@@ -2127,6 +2150,8 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
 
 int batch_finish(steps_batch *b) {
     if (!cuda_ok(cudaStreamSynchronize(b->stream), "steps_batch_run")) return STEPS_ERR_CUDA;
+    for (size_t j = 0; j < b->members.size(); ++j)
+        if (b->listed[j]) b->members[j]->fill_from(b->h_lcnt + 4 * j);
     const uint32_t err = *b->h_err;
     if (err) {
         cudaMemset(b->d_err, 0, 4);

@@ -98,7 +98,9 @@ struct StepArgs {
 // Shared memory of one warp of the warp-tile step (steps_warp.cuh): 32
 // consecutive tets, one per lane, of a model with up to kWarpMaxSpecies
 // species.
-constexpr int kWarpMaxSpecies = 12;
+constexpr int kWarpMaxSpecies = 32;
+constexpr int kWarpGenericSpecies = 12;  // of a model given at run time
+constexpr int kManySpecies = 12;         // above: a warp first looks whether any reaction is possible
 constexpr int kWarpMapCap = 160;    // Philox blocks listed at a time
 constexpr int kWarpQueueCap = 160;  // waiting movers: 31 left over + four words of 32 lanes
 
@@ -115,7 +117,10 @@ struct WarpTile {
     int32_t trial[SM][32];          // trial counts that differ from the count, and those drawn by bit planes
     uint4 thr[32];
     int4 nbr[32];
-    uint4 pre[32];                  // words of the species up to and including each, a byte each (x, y, z); w: all words
+    // words of the species up to and including each, a byte each, four to a
+    // word; the last word: all words of the tet
+    static constexpr int kPre = ((SM + 3) / 4 + 1 + 3) / 4;
+    uint4 pre[32][kPre];
     uint32_t tet[32];
     union {
         struct {
@@ -183,6 +188,7 @@ struct RepEntry {
     ModelDev model;
     StepArgs args;
     int32_t *cnt[2];
+    uint32_t *tm[2];              // list form: the species words of cnt
     uint32_t parity;
     uint32_t pad_;
     uint64_t window_end;

@@ -18,9 +18,11 @@ void set_error(const std::string &msg);
 
 // sizeof(WarpTile<S>) for a species count known at run time
 constexpr size_t warp_tile_bytes(int S) {
-    return sizeof(WarpTile<1>) + (size_t)(S - 1) * (sizeof(WarpTile<2>) - sizeof(WarpTile<1>));
+    return sizeof(WarpTile<1>) + (size_t)(S - 1) * 256 + (size_t)(((S + 3) / 4 + 4) / 4 - 1) * 512;
 }
-static_assert(warp_tile_bytes(kWarpMaxSpecies) == sizeof(WarpTile<kWarpMaxSpecies>), "warp tile rows");
+static_assert(warp_tile_bytes(12) == sizeof(WarpTile<12>) && warp_tile_bytes(20) == sizeof(WarpTile<20>) &&
+                  warp_tile_bytes(kWarpMaxSpecies) == sizeof(WarpTile<kWarpMaxSpecies>),
+              "warp tile rows");
 // and sizeof(ListTile<S>)
 constexpr size_t list_tile_bytes(int S) {
     return sizeof(ListTile<1>) + (size_t)(S - 1) * (sizeof(ListTile<2>) - sizeof(ListTile<1>));
@@ -105,11 +107,6 @@ int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, co
 int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEntry *reps, int S, int block,
                       void *stream);
 std::string spec_program_source(const HostModel &hm, int block);
-// whether the specialised block-tile kernels keep the trial counts in StepArgs::trial
-bool spec_global_trial(const HostModel &hm);
-// whether a model's kernels, specialised or not, run on warp tiles: flow launches then wait and publish per 32 tets, whatever
-// the block size
-bool warp_tiles(const HostModel &hm);
 // the list form's step kernel for launch_spec (models of more species than warp tiles take), or nullptr
 void *spec_list_kernel(const HostModel &hm);
 

@@ -189,7 +189,7 @@ int prefetch_distance(const void *kernel, int block, size_t smem) {
 
 int launch_step(const ModelDev &m, const StepArgs &a, int block, void *stream) {
     if (a.T <= 0) return STEPS_OK;
-    if (m.S <= kWarpMaxSpecies) return launch_warp(m, a, block, stream);
+    if (m.S <= kWarpGenericSpecies) return launch_warp(m, a, block, stream);
     switch (block) {
     case 64: return launch_step_b<64>(m, a, stream);
     case 128: return launch_step_b<128>(m, a, stream);
@@ -211,7 +211,7 @@ int launch_flow(const ModelDev &m, const StepArgs &a, const FlowArgs &f, int blo
         set_error("flow launches of the generic step kernel need 256-thread blocks");
         return STEPS_ERR_ARG;
     }
-    if (m.S <= kWarpMaxSpecies) return launch_warp_flow(m, a, f, block, stream);
+    if (m.S <= kWarpGenericSpecies) return launch_warp_flow(m, a, f, block, stream);
     return m.order0 ? launch_flow_z<true>(m, a, f, stream) : launch_flow_z<false>(m, a, f, stream);
 }
 

@@ -78,35 +78,22 @@ Nvrtc &nvrtc() {
     return n;
 }
 
-}  // namespace
-
-// Models with many species keep the trial counts in a global buffer: their
-// tile's shared memory then fits more resident blocks per SM.
-bool spec_global_trial(const HostModel &hm) { return hm.dev.S >= 16; }
-
-// Models with few species run on warp tiles (steps_warp.cuh): their loops
-// over species are unrolled.
-bool warp_tiles(const HostModel &hm) { return hm.dev.S <= kWarpMaxSpecies; }
-
-namespace {
-
 std::string hex_u32(uint32_t v) {
     std::ostringstream o;
     o << "0x" << std::hex << v << "u";
     return o.str();
 }
 
-// The generated policy: the same functions as RtModel with the model's
+// The generated policy of the list form: the functions of RtModel with the model's
 // structure as constants. Propensity forms (all in float, as RtModel):
 //   order 0: k / inv_nav            order 1: k x
 //   order 2: ((k inv_nav) x) y      dimer:   ((k inv_nav) x) (x - 1)
-// (RtModel's extra factors of 1 are exact and left out.) block: entries of a
-// count row; list: for the list form.
-std::string policy_source(const HostModel &hm, int block, bool list) {
+// (RtModel's extra factors of 1 are exact and left out.)
+std::string list_policy_source(const HostModel &hm) {
+    constexpr int block = 32;  // entries of a count row
     const ModelDev &m = hm.dev;
     std::ostringstream o;
     o << "namespace steps {\nnamespace {\nstruct SpecModel {\n";
-    o << "    static constexpr bool kGlobalTrial = " << (spec_global_trial(hm) ? "true" : "false") << ";\n";
     o << "    static constexpr bool kExpLeave = " << (hm.leave_exp ? "true" : "false") << ";\n";
     o << "    __device__ static int S(const ModelDev &) { return " << m.S << "; }\n";
     o << "    __device__ static int R(const ModelDev &) { return " << m.R << "; }\n";
@@ -140,8 +127,7 @@ std::string policy_source(const HostModel &hm, int block, bool list) {
     // SSA loop would inline every reaction's occupancy update there
     o << "    template <class F>\n    __device__ static void for_changes(const RxnTab &tb, int r, F f) {\n";
     o << "        RtModel<false>::for_changes(tb, r, f);\n    }\n";
-    if (list)  // as ssa_lane calls them
-        o << "    template <int RM>\n    __device__ __forceinline__ static float sums(const RxnTab &tb, const ModelDev &m, "
+    o << "    template <int RM>\n    __device__ __forceinline__ static float sums(const RxnTab &tb, const ModelDev &m, "
              "const int32_t *cnt, float inv_nav, uint32_t active, bool, float *psum) {\n"
              "        return propensity_sums<SpecModel, RM>(tb, m, cnt, inv_nav, active, psum);\n    }\n"
              "    template <int RM>\n    __device__ __forceinline__ static int pick(const RxnTab &tb, const ModelDev &m, "
@@ -220,71 +206,48 @@ std::string warp_policy_source(const HostModel &hm) {
     return o.str();
 }
 
-int reaction_bucket(int R) { return R <= 8 ? 8 : R <= 16 ? 16 : R <= 24 ? 24 : 32; }
-
 std::string program_source(const HostModel &hm, int block) {
     std::ostringstream o;
     const std::string b = std::to_string(block);
-    if (warp_tiles(hm)) {
-        const std::string args = "<" + b + ", " + std::to_string(std::max(1, hm.dev.R)) + ", " +
-                                 std::to_string(hm.dev.S) + ", steps::SpecModel";
-        const std::string head = "extern \"C\" __global__ void __launch_bounds__(" + b + ", " +
-                                 std::to_string(1024 / block) + ")\n";
-        const std::string member = "const steps::BlockWork *__restrict__ work, const steps::RepEntry *__restrict__ reps, ";
-        o << "#include \"steps_warp.cuh\"\n" << warp_policy_source(hm);
-        o << head << "steps_spec_step(const __grid_constant__ steps::ModelDev m, const __grid_constant__ "
-          << "steps::StepArgs a) {\n    steps::warp_step" << args << ">(m, a, (int64_t)blockIdx.x);\n}\n";
-        o << head << "steps_spec_flow(const __grid_constant__ steps::ModelDev m, const __grid_constant__ "
-          << "steps::StepArgs a, const __grid_constant__ steps::FlowArgs f) {\n    steps::warp_step" << args
-          << ", 1>(m, a, 0, &f);\n}\n";
-        o << head << "steps_spec_batch(" << member << "int32_t prefetch) {\n"
-          << "    steps::batch_member<" << b << ">(work, reps, prefetch, [](const steps::ModelDev &m, const "
-          << "steps::StepArgs &a, int64_t tile) { steps::warp_step" << args << ">(m, a, tile); });\n}\n";
-        o << head << "steps_spec_batch_flow(" << member << "const __grid_constant__ steps::FlowArgs f, uint32_t work0, "
-          << "int32_t prefetch) {\n"
-          << "    steps::batch_flow_member<" << b << ">(work, reps, f, work0, prefetch, [&f](const steps::ModelDev &m, "
-          << "const steps::StepArgs &a, int64_t tile, uint32_t q, uint32_t dep) { steps::warp_step" << args
-          << ", 2>(m, a, tile, &f, q, dep); });\n}\n";
-        return o.str();
-    }
-    // models with many species keep trial counts in global memory; at 256
-    // threads their tiles then fit five resident blocks per SM with a 32-entry
-    // block map and 48 registers per thread
-    const bool five = spec_global_trial(hm) && block == 256;
-    if (five) o << "#define STEPS_MAP_CAP 32\n";
-    o << "#include \"steps_step.cuh\"\n" << policy_source(hm, block, false);
-    o << "extern \"C\" __global__ void __launch_bounds__(" << block << ", " << (five ? 5 : 2048 / block / 2) << ")\n"
-      << "steps_spec_step(const __grid_constant__ steps::ModelDev m, const __grid_constant__ steps::StepArgs a) {\n"
-      << "    steps::step_tile<" << block << ", " << reaction_bucket(hm.dev.R) << ", steps::SpecModel>(m, a, "
-      << "(int64_t)blockIdx.x);\n}\n";
-    o << "extern \"C\" __global__ void __launch_bounds__(" << block << ", " << (five ? 5 : 2048 / block / 2) << ")\n"
-      << "steps_spec_flow(const __grid_constant__ steps::ModelDev m, const __grid_constant__ steps::StepArgs a, "
-      << "const __grid_constant__ steps::FlowArgs f) {\n"
-      << "    steps::flow_tiles<" << block << ", " << reaction_bucket(hm.dev.R) << ", steps::SpecModel>(m, a, f);\n}\n";
-    o << "extern \"C\" __global__ void __launch_bounds__(" << block << ", " << 2048 / block / 2 << ")\n"
-      << "steps_spec_batch(const steps::BlockWork *__restrict__ work, const steps::RepEntry *__restrict__ reps, "
+    const std::string args = "<" + b + ", " + std::to_string(std::max(1, hm.dev.R)) + ", " +
+                             std::to_string(hm.dev.S) + ", steps::SpecModel";
+    const std::string head = "extern \"C\" __global__ void __launch_bounds__(" + b + ", " +
+                             std::to_string(1024 / block) + ")\n";
+    const std::string member = "const steps::BlockWork *__restrict__ work, const steps::RepEntry *__restrict__ reps, ";
+    o << "#include \"steps_warp.cuh\"\n" << warp_policy_source(hm);
+    o << head << "steps_spec_step(const __grid_constant__ steps::ModelDev m, const __grid_constant__ "
+      << "steps::StepArgs a) {\n    steps::warp_step" << args << ">(m, a, (int64_t)blockIdx.x);\n}\n";
+    o << head << "steps_spec_flow(const __grid_constant__ steps::ModelDev m, const __grid_constant__ "
+      << "steps::StepArgs a, const __grid_constant__ steps::FlowArgs f) {\n    steps::warp_step" << args
+      << ", 1>(m, a, 0, &f);\n}\n";
+    o << head << "steps_spec_batch(" << member << "int32_t prefetch) {\n"
+      << "    steps::batch_member<" << b << ">(work, reps, prefetch, [](const steps::ModelDev &m, const "
+      << "steps::StepArgs &a, int64_t tile) { steps::warp_step" << args << ">(m, a, tile); });\n}\n";
+    o << head << "steps_spec_batch_flow(" << member << "const __grid_constant__ steps::FlowArgs f, uint32_t work0, "
       << "int32_t prefetch) {\n"
-      << "    steps::batch_tile<" << block << ", " << reaction_bucket(hm.dev.R) << ", steps::SpecModel>(work, reps, "
-      << "prefetch);\n}\n";
-    o << "extern \"C\" __global__ void __launch_bounds__(" << block << ", " << 2048 / block / 2 << ")\n"
-      << "steps_spec_batch_flow(const steps::BlockWork *__restrict__ work, const steps::RepEntry *__restrict__ reps, "
-      << "const __grid_constant__ steps::FlowArgs f, uint32_t work0, int32_t prefetch) {\n"
-      << "    steps::batch_flow_tile<" << block << ", " << reaction_bucket(hm.dev.R) << ", steps::SpecModel>(work, reps, "
-      << "f, work0, prefetch);\n}\n";
+      << "    steps::batch_flow_member<" << b << ">(work, reps, f, work0, prefetch, [&f](const steps::ModelDev &m, "
+      << "const steps::StepArgs &a, int64_t tile, uint32_t q, uint32_t dep) { steps::warp_step" << args
+      << ", 2>(m, a, tile, &f, q, dep); });\n}\n";
     return o.str();
 }
 
-// The list form's program: one step kernel (256-thread blocks).
+// The list form's program: a plain and a batched step kernel (256-thread blocks).
 constexpr int kListBlock = 256;
+constexpr int kListMinSpecies = 13;
 
 std::string list_program_source(const HostModel &hm) {
     std::ostringstream o;
     const std::string b = std::to_string(kListBlock);
-    o << "#include \"steps_list.cuh\"\n" << policy_source(hm, 32, true);
+    o << "#include \"steps_list.cuh\"\n" << list_policy_source(hm);
     o << "extern \"C\" __global__ void __launch_bounds__(" << b << ", " << 1024 / kListBlock << ")\n"
       << "steps_spec_list(const __grid_constant__ steps::ModelDev m, const __grid_constant__ steps::StepArgs a) {\n"
       << "    steps::list_step<" << b << ", " << std::max(1, hm.dev.R) << ", " << hm.dev.S
       << ", steps::SpecModel>(m, a, blockIdx.x, gridDim.x);\n}\n";
+    o << "extern \"C\" __global__ void __launch_bounds__(" << b << ", " << 1024 / kListBlock << ")\n"
+      << "steps_spec_list_batch(const steps::BlockWork *__restrict__ work, const steps::RepEntry *__restrict__ reps) {\n"
+      << "    steps::batch_member<" << b << ">(work, reps, 0, [](const steps::ModelDev &m, const steps::StepArgs &a, "
+      << "int64_t tile) {\n        steps::list_step<" << b << ", " << std::max(1, hm.dev.R) << ", " << hm.dev.S
+      << ", steps::SpecModel>(m, a, (uint32_t)tile, (uint32_t)steps::list_blocks(a.T, " << b << "));\n    });\n}\n";
     return o.str();
 }
 
@@ -298,8 +261,7 @@ struct Compiled {
     size_t smem_set_flow = 0;           // the flow kernel
     size_t smem_set_batch_flow = 0;     // the batched flow kernel
     size_t smem_set_batch = 0;          // and the batched one
-    bool warp = false;                  // warp-tile kernels
-    cudaKernel_t kern_list = nullptr;   // or the list form's step kernel alone
+    cudaKernel_t kern_list = nullptr;   // or the list form's plain step kernel (kern_batch: its batched one)
     size_t smem = 0;                    // dynamic shared memory per block
 };
 
@@ -357,14 +319,11 @@ Compiled *compiled(const HostModel &hm, int block, bool list, std::string *why) 
         return nullptr;
     }
     auto c = std::make_shared<Compiled>();
-    const size_t S = (size_t)hm.dev.S;
-    c->warp = !list && warp_tiles(hm);
-    c->smem = list                 ? (size_t)(kListBlock / 32) * list_tile_bytes(hm.dev.S)
-              : warp_tiles(hm) ? (size_t)(block / 32) * warp_tile_bytes(hm.dev.S)
-                                   : (S + 1 + (spec_global_trial(hm) ? 0 : S)) * (size_t)block * sizeof(int32_t);
+    c->smem = list ? (size_t)(kListBlock / 32) * list_tile_bytes(hm.dev.S) : (size_t)(block / 32) * warp_tile_bytes(hm.dev.S);
     bool ok = cudaLibraryLoadData(&c->lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0) == cudaSuccess;
     if (list) {
-        ok = ok && cudaLibraryGetKernel(&c->kern_list, c->lib, "steps_spec_list") == cudaSuccess;
+        ok = ok && cudaLibraryGetKernel(&c->kern_list, c->lib, "steps_spec_list") == cudaSuccess &&
+             cudaLibraryGetKernel(&c->kern_batch, c->lib, "steps_spec_list_batch") == cudaSuccess;
     } else {
         ok = ok && cudaLibraryGetKernel(&c->kern, c->lib, "steps_spec_step") == cudaSuccess &&
              cudaLibraryGetKernel(&c->kern_batch, c->lib, "steps_spec_batch") == cudaSuccess &&
@@ -400,7 +359,7 @@ void *spec_kernel(const HostModel &hm, int block, std::string *why) {
 }
 
 void *spec_list_kernel(const HostModel &hm) {
-    return hm.dev.S > kWarpMaxSpecies ? (void *)compiled(hm, kListBlock, true, nullptr) : nullptr;
+    return hm.dev.S >= kListMinSpecies ? (void *)compiled(hm, kListBlock, true, nullptr) : nullptr;
 }
 
 int launch_spec(void *spec, const ModelDev &m, const StepArgs &a, int block, void *stream) {
@@ -410,10 +369,7 @@ int launch_spec(void *spec, const ModelDev &m, const StepArgs &a, int block, voi
     if (c->kern_list) block = kListBlock;
     const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set)) return STEPS_ERR_CUDA;
-    StepArgs b = a;
-    if (b.prefetch) b.prefetch = prefetch_distance(fn, block, smem);
-    ModelDev mm = m;
-    void *args[2] = {(void *)&mm, (void *)&b};
+    void *args[2] = {(void *)&m, (void *)&a};
     const unsigned grid = (unsigned)(c->kern_list ? list_blocks(a.T, block) : (a.T + block - 1) / block);
     // programmatic dependent launch, as the generic step kernel
     cudaLaunchConfig_t cfg = {};
@@ -449,14 +405,10 @@ int launch_spec_flow(void *spec, const ModelDev &m, const StepArgs &a, const Flo
     }
     StepArgs b = a;
     b.window_base = nullptr;
-    // the item taken about half a resident wave later: its tables into L2
-    if (b.prefetch) b.prefetch = std::max(1, per_sm * sms / 2);
-    ModelDev mm = m;
-    FlowArgs ff = f;
-    void *args[3] = {(void *)&mm, (void *)&b, (void *)&ff};
+    void *args[3] = {(void *)&m, (void *)&b, (void *)&f};
     // one item per block, or the blocks resident at once
     const unsigned items = f.nwin * f.ntiles;
-    const unsigned grid = c->warp && warp_flow_persists(block) ? std::min(items, (unsigned)(per_sm * sms)) : items;
+    const unsigned grid = warp_flow_persists(block) ? std::min(items, (unsigned)(per_sm * sms)) : items;
     cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3((unsigned)block), args, smem, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         set_error(std::string("flow step kernel launch: ") + cudaGetErrorString(e));
@@ -472,9 +424,8 @@ int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, co
     const void *fn = (const void *)c->kern_batch_flow;
     const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set_batch_flow)) return STEPS_ERR_CUDA;
-    int32_t prefetch = prefetch_distance(fn, block, smem);
-    FlowArgs ff = f;
-    void *args[5] = {(void *)&work, (void *)&reps, (void *)&ff, (void *)&work0, (void *)&prefetch};
+    int32_t prefetch = 0;
+    void *args[5] = {(void *)&work, (void *)&reps, (void *)&f, (void *)&work0, (void *)&prefetch};
     const unsigned grid = f.nwin * f.ntiles;  // one item per block
     cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3((unsigned)block), args, smem, (cudaStream_t)stream);
     if (e != cudaSuccess) {
@@ -491,8 +442,9 @@ int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEnt
     const void *fn = (const void *)c->kern_batch;
     const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set_batch)) return STEPS_ERR_CUDA;
-    int32_t prefetch = prefetch_distance(fn, block, smem);
-    void *args[3] = {(void *)&work, (void *)&reps, (void *)&prefetch};
+    int32_t prefetch = 0;
+    void *args[3] = {(void *)&work, (void *)&reps, (void *)&prefetch};  // (the list form's takes the first two)
+    if (c->kern_list) block = kListBlock;
     cudaError_t e = cudaLaunchKernel(fn, dim3((unsigned)nblocks), dim3((unsigned)block), args, smem, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         set_error(std::string("specialised batched step kernel launch: ") + cudaGetErrorString(e));

@@ -179,8 +179,6 @@ __device__ __forceinline__ float propensity(const float4 q, const int32_t *cnt, 
 // constants from the kernel parameters. Z: the model has order-0 reactions.
 template <bool Z>
 struct RtModel {
-    static constexpr bool kGlobalTrial = false;  // trial counts in shared memory
-    static constexpr bool kExpLeave = false;     // the EULER leave law (species scale in shared memory)
     __device__ static int S(const ModelDev &m) { return m.S; }
     __device__ static int R(const ModelDev &m) { return m.R; }
     __device__ static uint32_t diffusive(const ModelDev &m) { return m.diffusive; }
@@ -352,15 +350,6 @@ __device__ __forceinline__ int32_t trial_count(const StepArgs &a, int s, int32_t
     return mm > N ? N : (int32_t)mm;
 }
 
-// The species factor of tet i's thresholds: the window's species scale R_s
-// (EULER), or the tet's own leave value L_{s,i} from the EXP table (the
-// tet's factor A is then its cumulative face shares).
-template <class P>
-__device__ __forceinline__ uint32_t species_R(const StepArgs &a, const uint32_t *s_scale, int s, int64_t i) {
-    if constexpr (P::kExpLeave) return __ldg(a.leave + (size_t)s * (size_t)a.Tpad + (size_t)i);
-    else return s_scale[s];
-}
-
 // Leave thresholds of one species: T_f = (A_f R_s) >> 31 (2^31 fixed point).
 __device__ __forceinline__ void species_thresholds(const uint4 &A, uint32_t R, uint32_t &T0, uint32_t &T1,
                                                    uint32_t &T2, uint32_t &T3) {
@@ -440,13 +429,9 @@ __device__ __forceinline__ int32_t bulk_species(const StepArgs &a, int32_t *nxt,
 // order), cut into Philox blocks of 4 words. Block b of the chunk belongs to
 // lane `owner` with first[lane] <= b < first[lane + 1]; the map caches the
 // owner, the species of the block's first word and the tet's trial
-// molecules before that species for the first kMapCap blocks (a program may
-// set a smaller map to fit more resident blocks; blocks past it are found by
-// search).
-#ifndef STEPS_MAP_CAP
-#define STEPS_MAP_CAP 160
-#endif
-constexpr int kMapCap = STEPS_MAP_CAP;
+// molecules before that species for the first kMapCap blocks (those past it are
+// found by search).
+constexpr int kMapCap = 160;
 
 struct WarpWork {
     int16_t tet[32];          // tile index of each lane's tet (-1: none)
@@ -510,7 +495,7 @@ __device__ __forceinline__ void diffuse_block(const StepArgs &a, int32_t *nxt, c
     const size_t Tpad = (size_t)a.Tpad;
     const uint4 rw = philox4x32_10(a.key0, a.key1, c0, s_tet[t], k, (kPurposeDiff << 28) | c3);
     uint32_t T0, T1, T2, T3;
-    species_thresholds(A, species_R<P>(a, s_scale, s, i0 + t), T0, T1, T2, T3);
+    species_thresholds(A, s_scale[s], T0, T1, T2, T3);
     uint32_t w = 4u * k;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -519,7 +504,7 @@ __device__ __forceinline__ void diffuse_block(const StepArgs &a, int32_t *nxt, c
                 s = __ffs(hm) - 1;
                 hm &= hm - 1;
                 end += (uint32_t)trial_all[s * tstride + t];
-                species_thresholds(A, species_R<P>(a, s_scale, s, i0 + t), T0, T1, T2, T3);
+                species_thresholds(A, s_scale[s], T0, T1, T2, T3);
             }
             const uint32_t x = word_of(rw, q) >> 1;
             if (x < T3) {
@@ -676,12 +661,8 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
     const int nlive = (int)min((int64_t)BLOCK, (int64_t)a.T - i0);
     const bool live = tid < nlive;
     int32_t *cnt_all = smem;                              // rows 0..S-1 counts, row S ones
-    // trial counts [S][tstride]: after the count rows in shared memory, or (for
-    // models with many species, to leave room for more resident blocks) the
-    // tile's columns of a global buffer
-    constexpr bool GT = P::kGlobalTrial;
-    int32_t *trial_all = GT ? a.trial + i0 : smem + (size_t)(S + 1) * BLOCK;
-    const size_t tstride = GT ? (size_t)a.Tpad : (size_t)BLOCK;
+    int32_t *trial_all = smem + (size_t)(S + 1) * BLOCK;  // trial counts [S][BLOCK]
+    constexpr size_t tstride = BLOCK;
     uint32_t c0, c3;  // RNG counter words of the window, set once the previous window is done
     const size_t Tpad = (size_t)a.Tpad;
     uint32_t bad = 0;
@@ -878,7 +859,7 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
             while (walk) {
                 const int s = __ffs(walk) - 1;
                 walk &= walk - 1;
-                if ((uint32_t)(((uint64_t)Aw * species_R<P>(a, s_scale, s, i0 + t)) >> 31) == 0u)
+                if ((uint32_t)(((uint64_t)Aw * s_scale[s]) >> 31) == 0u)
                     continue;  // draws nothing
                 const int32_t N = cnt_all[s * BLOCK + t];
                 const int32_t M = plain ? N
@@ -905,7 +886,7 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
             bw &= bw - 1;
             if ((bm >> s) & 1u)
                 cnt_all[s * BLOCK + t] -= bulk_species(a, nxt, s, trial_all[s * tstride + t], s_thr[t],
-                                                       species_R<P>(a, s_scale, s, i0 + t), s_nbr[t], s_tet[t], c0, c3);
+                                                       s_scale[s], s_nbr[t], s_tet[t], c0, c3);
         }
         // the chunk's Philox blocks: exclusive prefix of the lanes' block counts
         const uint32_t nb = (W + 3u) >> 2;
@@ -1012,6 +993,8 @@ __device__ __forceinline__ void batch_member(const BlockWork *__restrict__ work,
     if (threadIdx.x == 0) {
         t_args.cur = e->cnt[e->parity];
         t_args.nxt = e->cnt[e->parity ^ 1u];
+        t_args.tm_cur = e->tm[e->parity];
+        t_args.tm_nxt = e->tm[e->parity ^ 1u];
         t_args.prefetch = prefetch;  // tiles ahead within the member
         t_tile = bw.tile;
     }
@@ -1073,15 +1056,6 @@ __device__ __forceinline__ void batch_flow_member(const BlockWork *__restrict__ 
     }
     __syncthreads();
     step(t_model, t_args, (int64_t)s_tile, s_q, s_dep);
-}
-
-template <int BLOCK, int RM, class P>
-__device__ __forceinline__ void batch_flow_tile(const BlockWork *__restrict__ work, const RepEntry *__restrict__ reps,
-                                                const FlowArgs &f, uint32_t work0, int32_t prefetch) {
-    batch_flow_member<BLOCK>(work, reps, f, work0, prefetch,
-                             [&f](const ModelDev &m, const StepArgs &a, int64_t tile, uint32_t q, uint32_t dep) {
-                                 step_tile<BLOCK, RM, P, 2>(m, a, tile, &f, q, dep);
-                             });
 }
 
 }  // namespace

@@ -1,6 +1,6 @@
 // The warp-tile step for models given at run time (meshes below the
 // specialisation size, or without the run-time compiler) of up to
-// kWarpMaxSpecies species: plain, flow and batched kernels. The loops over
+// kWarpGenericSpecies species: plain, flow and batched kernels. The loops over
 // species are unrolled to 4 or 12, the reaction table is walked in loops.
 #include <algorithm>
 #include <string>
@@ -90,16 +90,16 @@ int launch_batch_sm(const BlockWork *work, int64_t nblocks, const RepEntry *reps
 }  // namespace
 
 int launch_warp(const ModelDev &m, const StepArgs &a, int block, void *stream) {
-    return m.S <= 4 ? launch_plain<4>(m, a, block, stream) : launch_plain<kWarpMaxSpecies>(m, a, block, stream);
+    return m.S <= 4 ? launch_plain<4>(m, a, block, stream) : launch_plain<kWarpGenericSpecies>(m, a, block, stream);
 }
 
 int launch_warp_flow(const ModelDev &m, const StepArgs &a, const FlowArgs &f, int block, void *stream) {
-    return m.S <= 4 ? launch_flow_sm<4>(m, a, f, block, stream) : launch_flow_sm<kWarpMaxSpecies>(m, a, f, block, stream);
+    return m.S <= 4 ? launch_flow_sm<4>(m, a, f, block, stream) : launch_flow_sm<kWarpGenericSpecies>(m, a, f, block, stream);
 }
 
 int launch_warp_batch(const BlockWork *work, int64_t nblocks, const RepEntry *reps, int max_S, int block, void *stream) {
     return max_S <= 4 ? launch_batch_sm<4>(work, nblocks, reps, block, stream)
-                      : launch_batch_sm<kWarpMaxSpecies>(work, nblocks, reps, block, stream);
+                      : launch_batch_sm<kWarpGenericSpecies>(work, nblocks, reps, block, stream);
 }
 
 }  // namespace steps

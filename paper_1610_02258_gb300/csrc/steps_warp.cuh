@@ -324,19 +324,24 @@ __device__ __forceinline__ void plane_groups(const StepArgs &a, WarpTile<SM> &w,
 // which no word reaches. (The byte dot product __dp4a in place of the shifts
 // and the population count took three times the instructions on this GPU.)
 template <int NP>
-__device__ __forceinline__ uint32_t species_of(const uint4 pre, uint32_t v4) {
-    uint32_t u = (v4 - pre.x) & 0x80808080u;
-    if constexpr (NP > 1) u |= ((v4 - pre.y) >> 1) & 0x40404040u;
-    if constexpr (NP > 2) u |= ((v4 - pre.z) >> 2) & 0x20202020u;
+__device__ __forceinline__ uint32_t species_of(const uint32_t *pre, uint32_t v4) {
+    uint32_t u = (v4 - pre[0]) & 0x80808080u;
+#pragma unroll
+    for (int j = 1; j < NP; ++j) u |= ((v4 - pre[j]) >> j) & (0x80808080u >> j);
     return (uint32_t)__popc(u);
 }
 
-// The same for a tet of 128 words or more, species by species.
-__device__ __forceinline__ uint32_t species_of_wide(const uint4 *pre, int S, uint32_t v) {
-    const uint8_t *pb = reinterpret_cast<const uint8_t *>(pre);
-    uint32_t c = 0;
-    while ((int)c < S - 1 && pb[c] <= v) ++c;
-    return c;
+// The same for a tet of 128 words or more, species by species, from its trial
+// counts (trial: its column).
+__device__ __forceinline__ uint32_t species_of_wide(const int32_t *trial, int S, uint32_t v) {
+    uint32_t end = 0;
+    int c = 0;
+    for (; c < S - 1; ++c) {
+        const int32_t M = trial[c * 32];
+        end += M < kBulkMin ? (uint32_t)M : 0u;
+        if (v < end) break;
+    }
+    return (uint32_t)c;
 }
 
 // The listed Philox blocks, n of them, 32 at a time, one per lane: word v
@@ -356,14 +361,20 @@ __device__ __forceinline__ void draw_words(const ModelDev &m, const StepArgs &a,
         const uint32_t o = w.d.map[min(b + lane, n - 1u)];
         const int t = (int)(o & 31u);
         const uint32_t k = o >> 5, v4 = k * 0x04040404u + 0x80808080u;
-        const uint4 pre = w.pre[t];
-        const int left = b + lane < n ? (int)(pre.w - 4u * k) : 0;  // words that decide a molecule
+        constexpr int NQ = WarpTile<SM>::kPre;
+        uint32_t pre[4 * NQ];
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) {
+            const uint4 x = w.pre[t][j];
+            pre[4 * j] = x.x, pre[4 * j + 1] = x.y, pre[4 * j + 2] = x.z, pre[4 * j + 3] = x.w;
+        }
+        const int left = b + lane < n ? (int)(pre[4 * NQ - 1] - 4u * k) : 0;  // words that decide a molecule
         const uint32_t Aw = w.thr[t].w;
         const uint4 rw = philox_rk(a.rk, c0, w.tet[t], k, (kPurposeDiff << 28) | c3);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             uint32_t c;
-            if constexpr (WIDE) c = species_of_wide(&w.pre[t], P::S(m), 4u * k + r);
+            if constexpr (WIDE) c = species_of_wide(&w.trial[0][t], P::S(m), 4u * k + r);
             else c = species_of<NP>(pre, v4 + r * 0x01010101u);
             if constexpr (P::kExpLeave) c = min(c, (uint32_t)P::S(m) - 1u);  // (a word past the last molecule)
             const uint32_t x = word_of(rw, (uint32_t)r) >> 1;
@@ -392,6 +403,21 @@ template <int SM, class P>
 __device__ __noinline__ void draw_words_wide(const ModelDev &m, const StepArgs &a, WarpTile<SM> &w, int32_t *nxt,
                                              const uint32_t *s_scale, int64_t i0, uint32_t n, uint32_t c0, uint32_t c3) {
     draw_words<SM, P, true>(m, a, w, nxt, s_scale, i0, n, c0, c3);
+}
+
+// Every species' trial count into w.trial, as draw_words_wide reads them: those
+// in the word stream, 0 for the others, bit-plane species (bm) as they are.
+// round: species whose trial count is there already.
+template <int SM, class P>
+__device__ __noinline__ void wide_trials(const ModelDev &m, const StepArgs &a, WarpTile<SM> &w, const uint32_t *s_scale,
+                                         int64_t i, uint32_t Aw, uint32_t bm, uint32_t round) {
+    const int lane = threadIdx.x & 31;
+    for (int s = 0; s < P::S(m); ++s) {
+        if ((bm >> s) & 1u) continue;
+        int32_t M = (round >> s) & 1u ? w.trial[s][lane] : w.cnt[s][lane];
+        if (!((P::diffusive(m) >> s) & 1u) || thr31(Aw, warp_R<P>(a, s_scale, s, i)) == 0u) M = 0;
+        w.trial[s][lane] = max(M, 0);
+    }
 }
 
 // Waits until the warp tiles holding the lanes' face neighbours, and the
@@ -479,6 +505,7 @@ __device__ __forceinline__ bool warp_window(const ModelDev &m, const StepArgs &a
     const uint64_t window = a.window + q + (a.window_base ? *a.window_base : 0ull);
     const uint32_t c0 = (uint32_t)window, c3 = (uint32_t)(window >> 32) & 0x0FFFFFFFu;
     int32_t any = 0;
+    uint32_t nz = 0;  // the tet's species (models of many: a warp of which may lack every reaction's reactants)
     {
         int32_t n[SM];
         const int32_t *src = cur + i;
@@ -493,6 +520,7 @@ __device__ __forceinline__ bool warp_window(const ModelDev &m, const StepArgs &a
         for (int s = 0; s < SM; ++s) {
             w.cnt[s][lane] = s < P::S(m) ? n[s] : 1;  // (row S holds ones: a missing reactant)
             any |= n[s];
+            if (SM > kManySpecies) nz |= n[s] != 0 ? 1u << s : 0u;
             if (n[s] != 0) *row = 0;
             row += Tpad;
         }
@@ -507,7 +535,13 @@ __device__ __forceinline__ bool warp_window(const ModelDev &m, const StepArgs &a
     // straight-line code for the whole warp, with both Philox blocks side by
     // side; only tets whose second attempt may fire run the event loop.
     uint32_t touched = 0;
-    if (P::R(m) > 0) {
+    bool possible = P::R(m) > 0;
+    if (SM > kManySpecies && possible) {  // lane r: can reaction r fire in any tet of the warp?
+        const uint32_t wnz = __reduce_or_sync(0xFFFFFFFFu, nz), wact = __reduce_or_sync(0xFFFFFFFFu, active);
+        const uint32_t need = lane < P::R(m) ? tb.need[lane] : 0u;
+        possible = __any_sync(0xFFFFFFFFu, lane < P::R(m) && ((wact >> lane) & 1u) && (wnz & need) == need);
+    }
+    if (possible) {
         double O[SM], tS[SM];
         int32_t *const cnt = &w.cnt[0][lane];
         const bool masked = a.rmask != nullptr;
@@ -570,11 +604,14 @@ __device__ __forceinline__ bool warp_window(const ModelDev &m, const StepArgs &a
     // threshold; those below kBulkMin join the tet's word stream
     uint32_t W = 0, bm = 0;
     const uint32_t round = a.occ ? touched : 0u;
+    // species somewhere in the warp (models of many species skip the others)
+    const uint32_t here = SM > kManySpecies ? __reduce_or_sync(0xFFFFFFFFu, nz | touched) : 0xFFFFFFFFu;
     {
-        uint32_t pre[3] = {0u, 0u, 0u};
+        constexpr int NQ = WarpTile<SM>::kPre;
+        uint32_t pre[4 * NQ] = {};
 #pragma unroll
         for (int s = 0; s < SM; ++s) {
-            if (s < P::S(m) && ((P::diffusive(m) >> s) & 1u)) {
+            if (s < P::S(m) && ((P::diffusive(m) >> s) & 1u) && ((here >> s) & 1u)) {
                 int32_t M = w.cnt[s][lane];
                 if ((round >> s) & 1u) M = w.trial[s][lane];
                 M = thr31(A.w, warp_R<P>(a, s_scale, s, i)) == 0u ? 0 : M;  // draws nothing
@@ -587,8 +624,14 @@ __device__ __forceinline__ bool warp_window(const ModelDev &m, const StepArgs &a
         }
 #pragma unroll
         for (int s = SM; s < 4 * NP; ++s) pre[s >> 2] |= 0x80u << (8 * (s & 3));
-        w.pre[lane] = make_uint4(pre[0], pre[1], pre[2], W);
+        pre[4 * NQ - 1] = W;
+#pragma unroll
+        for (int j = 0; j < NQ; ++j)
+            w.pre[lane][j] = make_uint4(pre[4 * j], pre[4 * j + 1], pre[4 * j + 2], pre[4 * j + 3]);
     }
+
+    const bool wide = __any_sync(0xFFFFFFFFu, W > 127u);
+    if (wide) wide_trials<SM, P>(m, a, w, s_scale, i, A.w, bm, round);
 
     // ---- bit-plane groups of the species with many trial molecules
     if (__any_sync(0xFFFFFFFFu, bm != 0u)) {
@@ -634,7 +677,6 @@ __device__ __forceinline__ bool warp_window(const ModelDev &m, const StepArgs &a
         }
         const uint32_t first = xs - nb;
         const uint32_t total = __shfl_sync(0xFFFFFFFFu, xs, 31);
-        const bool wide = __any_sync(0xFFFFFFFFu, W > 127u);
         uint32_t k = 0;
         for (uint32_t base = 0; base < total; base += kWarpMapCap) {
             const uint32_t lim = min(total, base + (uint32_t)kWarpMapCap);
@@ -650,14 +692,14 @@ __device__ __forceinline__ bool warp_window(const ModelDev &m, const StepArgs &a
         int32_t *out = nxt + i;
 #pragma unroll
         for (int s = 0; s < SM; ++s) {
-            if (s < P::S(m)) {
+            if (s < P::S(m) && ((here >> s) & 1u)) {
                 const int32_t N = w.cnt[s][lane];
                 if (N) {
                     if ((P::diffusive(m) >> s) & 1u) atomicAdd(out, N);
                     else *out = N;
                 }
-                out += Tpad;
             }
+            out += Tpad;
         }
     }
     if (bad) atomicOr(a.err, bad);

@@ -144,3 +144,24 @@ def test_recordings(capi):
     for k in range(10):
         o.run((k + 1) * dt)
         assert np.array_equal(rec[k], o.get_counts()[[0, 5]][:, tets])
+
+
+def test_batch_of_listed_and_other_members(capi):
+    """A batch whose members are in sparse and in dense states (list form and warp
+    tiles in one window), over two runs and then alone."""
+    pairs = [_pair(capi, 14, (9, 6, 5), 0.1, [1, 2], seed=3), _pair(capi, 14, (6, 6, 5), 0.05, [1, 40], seed=4)]
+    g, o, _ = _pair(capi, 14, (8, 5, 5), 0.1, [1], seed=6)
+    c = np.random.default_rng(3).integers(0, 6, (14, g.nt)).astype(np.int32)
+    for obj in (g, o):
+        obj.set_counts(c)
+    pairs.append((g, o, c))
+    b = capi.Batch([p[0] for p in pairs], block=256, specialize=1)
+    for k in (20.4, 21.7):
+        ends = [p[1].time + k * p[1].tau for p in pairs]
+        b.run(ends)
+        for (g, o, _), t in zip(pairs, ends):
+            o.run(t)
+            assert g.windows == o.windows and np.array_equal(g.get_counts(), o.get_counts())
+    b.close()
+    for g, o, _ in pairs:
+        _run(g, o, 5.5)
