@@ -1701,7 +1701,7 @@ struct steps_batch {
                    : STEPS_ERR_CUDA;
     }
 
-    int build_work(int b) {
+    int build_work(int b) try {
         Work &w = work[slot(b)];
         if (w.built) return STEPS_OK;
         std::vector<BlockWork> v;
@@ -1711,11 +1711,14 @@ struct steps_batch {
         }
         w.built = true;
         return upload_work(w, v);
+    } catch (const std::bad_alloc &) {
+        set_error("steps_batch: work list: out of host memory");
+        return STEPS_ERR_OOM;
     }
 
     // The members of this run's list form, by what is known of their states; the
     // work lists and graphs follow when they change.
-    int choose_forms() {
+    int choose_forms() try {
         std::vector<char> want(members.size(), 0);
         for (size_t j = 0; j < members.size(); ++j) {
             const steps_sim *m = members[j];
@@ -1749,6 +1752,9 @@ struct steps_batch {
             if (rc) return rc;
         }
         return STEPS_OK;
+    } catch (const std::bad_alloc &) {
+        set_error("steps_batch: work list: out of host memory");
+        return STEPS_ERR_OOM;
     }
 
     // the specialised batched kernel for block size b (compiled once); on
