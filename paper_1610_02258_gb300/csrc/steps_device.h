@@ -84,6 +84,7 @@ struct StepArgs {
     float tau_dn;                 // largest float <= tau_k
     int32_t occ;                  // STEPS_OCC_*
     int32_t prefetch;             // tiles ahead whose tables a block prefetches into L2 (0 = none)
+    int32_t lanes;                // tets per warp in window launches of run-time models: 32 or fewer
     int32_t *trial;               // [S][Tpad] trial counts, for kernels that keep them in global memory
     uint32_t *tm_cur, *tm_nxt;    // list form: [T] species bits of cur and nxt, a clear bit means count 0
     const uint4 *rec;             // [T] last face threshold, RNG key, 1 / (N_A V_L), active reactions

@@ -49,15 +49,24 @@ int checked(cudaError_t e, const char *what) {
 
 template <int SM>
 int launch_plain(const ModelDev &m, const StepArgs &a, int block, void *stream) {
-    // a small mesh's tiles go into smaller blocks until the blocks cover the
-    // SMs twice: its windows are bound by the latency of a tile, and warps of
-    // one block share an SM
-    while (block > 32 && ((int64_t)a.T + block - 1) / block < 2 * 152) block /= 2;
+    // A small mesh's windows are bound by the latency of a tile. Below a warp per
+    // scheduler (4 on each of 152 SMs), warps take fewer tets, whose queues are
+    // shorter: us per window, 32 tets -> this rule: 1,920 tets 7.4 -> 6.7, 8,670
+    // tets 20.4 -> 19.8; but two warps per scheduler instead of one for 30,720
+    // tets of 151 molecules 66 -> 73, and 2 tets a warp are no faster than 4.
+    StepArgs b = a;
+    while (b.lanes > 4 && ((int64_t)a.T + b.lanes - 1) / b.lanes < 4 * 152) b.lanes /= 2;
+    const int64_t warps = ((int64_t)a.T + b.lanes - 1) / b.lanes;
+    // warps of one block share an SM, so the blocks shrink until they cover the
+    // SMs twice: 256 threads -> this rule, 30,720 tets 67.4 -> 65.8, 17,340 to
+    // 52,020 tets of 14 molecules 22.2 -> 21.7, 24.4 -> 23.2, 24.7 -> 23.5 (up to
+    // four times: 21.7, 23.7, 25.0)
+    while (block > 32 && (warps * 32 + block - 1) / block < 2 * 152) block /= 2;
     const size_t smem = (size_t)(block / 32) * sizeof(WarpTile<SM>);
     if (!opt_in((const void *)warp_kernel<SM>, smem)) return STEPS_ERR_CUDA;
     // programmatic dependent launch, as the block-tile kernel
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(((int64_t)a.T + block - 1) / block));
+    cfg.gridDim = dim3((unsigned)((warps * 32 + block - 1) / block));
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = (cudaStream_t)stream;
@@ -66,7 +75,7 @@ int launch_plain(const ModelDev &m, const StepArgs &a, int block, void *stream) 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return checked(cudaLaunchKernelEx(&cfg, warp_kernel<SM>, m, a), "warp-tile kernel launch");
+    return checked(cudaLaunchKernelEx(&cfg, warp_kernel<SM>, m, b), "warp-tile kernel launch");
 }
 
 template <int SM>

@@ -16,8 +16,8 @@
 // molecules per tet, 0.07 events per tet and window) a window is about 24M
 // warp instructions, issued at two thirds of the slots; loading and applying
 // alone take 7 us. us per window, block tiles -> warp tiles, flow launches:
-// box 42.7 -> 28.5, at a tenth of the densities 24.0 -> 16.4, at ten times
-// 139 -> 105; 1.05M tets in window launches 94 -> 65. Registers: 64 at 32
+// box 42.7 -> 28.6, at a tenth of the densities 24.0 -> 15.3, at ten times
+// 139 -> 102; 1.05M tets in window launches 94 -> 65. Registers: 64 at 32
 // warps per SM; 48 at 40 warps spilled and was 10 % slower. Items per warp
 // instead of per block (warps out of step) missed the instruction cache: 35
 // us on the box.
@@ -459,18 +459,18 @@ __device__ __forceinline__ bool flow_nbr_wait(const uint32_t *done, uint32_t own
     return true;
 }
 
-// One diffusion window for the 32 tets from i0 on, one warp. FLOW as in
+// One diffusion window for the `lanes` tets from i0 on, one warp. FLOW as in
 // step_tile, with the finished-window words by warp tile
 // (dep): window a.window + q, buffers swapped when q is odd. False when the
 // tiles it waits for did not finish within the wait limit.
 template <int RM, int SM, class P, int FLOW>
 __device__ __forceinline__ bool warp_window(const ModelDev &m, const StepArgs &a, WarpTile<SM> &w, const RxnTab &tb,
                                             const uint32_t *s_scale, int64_t i0, const FlowArgs *f, uint32_t q,
-                                            uint32_t dep) {
+                                            uint32_t dep, int lanes = 32) {
     constexpr int NP = (SM + 3) / 4;
     const int lane = threadIdx.x & 31;
     const int64_t i = i0 + lane;
-    const bool live = i < a.T;
+    const bool live = i < a.T && lane < lanes;
     const uint32_t below = (1u << lane) - 1u;
     int32_t *const cur = (q & 1u) ? a.nxt : a.cur;
     int32_t *const nxt = (q & 1u) ? a.cur : a.nxt;
@@ -753,8 +753,9 @@ __device__ __forceinline__ void warp_step(const ModelDev &m, const StepArgs &a, 
             if (!PERSIST || __syncthreads_or(!done)) return;  // (a wait that ran out ends the block)
         }
     } else {
-        const int64_t i0 = tile * threads + warp * 32;
-        if (i0 < a.T) warp_window<RM, SM, P, FLOW>(m, a, w, tb, s_scale, i0, f, q, dep * (uint32_t)warps + (uint32_t)warp);
+        const int lanes = FLOW == 0 && BLOCK == 0 ? a.lanes : 32;
+        const int64_t i0 = (tile * warps + warp) * lanes;
+        if (i0 < a.T) warp_window<RM, SM, P, FLOW>(m, a, w, tb, s_scale, i0, f, q, dep * (uint32_t)warps + (uint32_t)warp, lanes);
     }
 }
 }  // namespace

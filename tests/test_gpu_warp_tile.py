@@ -97,3 +97,12 @@ def test_long_word_streams(capi, leave):
     Philox blocks in 32 tets than are listed at a time."""
     _check(capi, 12, (5, 5, 3), [13, 14, 15], leave=leave, windows=(1.0, 2.3))
     _check(capi, 12, (5, 5, 3), [9, 10, 11], leave=leave, windows=(1.0, 2.3))
+
+
+@pytest.mark.parametrize("cells,lanes", [(809, 4), (810, 8), (1618, 8), (1619, 16), (3237, 16), (3238, 32)])
+@pytest.mark.parametrize("S", [3, 6])
+def test_tets_per_warp(capi, cells, lanes, S):
+    """Models given at run time on either side of the sizes (4,856, 9,712 and
+    19,424 tets) below which a warp takes fewer tets, all with a ragged end."""
+    assert (6 * cells + lanes - 1) // lanes >= 608 or lanes == 4
+    _check_kernel(capi, S, (cells, 1, 1), SPARSE + EDGES, OCC, 0, False, 256, True, (2.0, 3.3), -1)
