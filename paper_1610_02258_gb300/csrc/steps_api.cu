@@ -274,6 +274,8 @@ struct steps_sim {
     uint64_t list_built = 0;        // the window the list was last built for
     double density = 0.0;           // molecules per tet when counts were last set
     double fill = 0.0;              // listed tets or non-zero counts per tet, last known
+    // each species' share of both when its counts were last set (of all species at once: equal shares)
+    double set_density[kMaxSpecies] = {}, set_fill[kMaxSpecies] = {};
     // time
     double t_base = 0.0;
     int64_t k_grid = 0;
@@ -1131,10 +1133,19 @@ static int put_counts(steps_sim *sim, int32_t s0, int32_t ns, const int32_t *cou
         return STEPS_ERR_ARG;
     }
     sim->tm_valid = sim->list_valid = false;
-    // counts of every species replace the state; of one, they add to what is known of it
+    // counts of every species replace the state; of one, they change what is known
+    // of it by as much as they differ from those set before
     const double sum = (double)((uint64_t)seen[3] << 32 | seen[2]);
-    sim->fill = (ns == sim->S ? 0.0 : sim->fill) + seen[1] / (double)T;
-    sim->density = (ns == sim->S ? 0.0 : sim->density) + sum / (double)T;
+    if (ns == sim->S) sim->fill = sim->density = 0.0;
+    for (int32_t s = s0; s < s0 + ns; ++s) {
+        const double f = seen[1] / (double)T / ns, d = sum / (double)T / ns;
+        sim->fill += ns == sim->S ? f : f - sim->set_fill[s];
+        sim->density += ns == sim->S ? d : d - sim->set_density[s];
+        sim->set_fill[s] = f;
+        sim->set_density[s] = d;
+    }
+    sim->fill = std::max(0.0, sim->fill);
+    sim->density = std::max(0.0, sim->density);
     scatter_to_device_order<<<(unsigned)((T + 255) / 256), 256, 0, sim->stream>>>(
         sim->d_stage, (int64_t)T, ns, sim->d_inv_perm, sim->d_cnt[sim->cur] + (size_t)s0 * Tpad, Tpad);
     if (!cuda_ok(cudaGetLastError(), "steps_set_counts: scatter")) return STEPS_ERR_CUDA;
