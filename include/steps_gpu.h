@@ -69,7 +69,8 @@ typedef struct steps_sim steps_sim;
 typedef struct steps_options {
     int32_t occupancy;   /* STEPS_OCC_MEAN or STEPS_OCC_END */
     int32_t reorder;     /* STEPS_REORDER_* */
-    int32_t block;       /* threads per block of the step kernel; 0 = default (256) */
+    int32_t block;       /* threads per block of the step kernel; 0 = default (256; small meshes on the generic
+                            kernel take smaller blocks, so that more of the chip works) */
     int32_t use_graph;   /* 1 = replay full windows from a captured CUDA graph (default), 0 = plain launches */
     int32_t specialize;  /* step kernel compiled for this model at run time (NVRTC): 0 = when the mesh has at
                             least 65,536 tets and NVRTC is available (default), 1 = always (sim creation fails
@@ -83,7 +84,9 @@ typedef struct steps_options {
                             72 full windows times, on its own windows, window launches, flow launches of
                             `block`-tet tiles and (specialised, block < 512) of 512-tet tiles, and keeps the
                             fastest (steps_sim_flow reports it); 1: flow at `block` where a flow kernel exists;
-                            -1: window launches. The results are the same bits in every form. */
+                            -1: window launches. The results are the same bits in every form. With 0 and -1, a
+                            specialised model of 13 or more species whose state holds few molecules per tet
+                            runs its windows, in window launches, over a list of the tets that hold something. */
     int32_t reserved[1]; /* set to 0 */
 } steps_options;
 

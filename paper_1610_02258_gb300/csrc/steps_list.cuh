@@ -1,16 +1,24 @@
-// The operator-split step in the list form: models with more than
-// kWarpMaxSpecies species, in states of few molecules per tet (the block-tile
-// step reads and zeroes every count of every tet). Included after
-// steps_warp.cuh, whose building blocks it shares; the same draws, formulas
-// and decisions, so the same bits.
+// The operator-split step in the list form: models with many species, in
+// states of few molecules per tet (a step over tiles reads every count of
+// every tet). Included after steps_warp.cuh, whose building blocks it shares;
+// the same draws, formulas and decisions, so the same bits.
 //
 // Every tet has a word of species bits beside its counts (StepArgs::tm_cur,
 // tm_nxt, in step with the count buffers): a set bit says that the count may
 // be non-zero. Warps work on 32 tets that hold something at a time, one per
 // lane, reading only their non-zero counts and their tables; an empty tet
 // costs nothing. Those tets are listed by the window before: whoever sets bits
-// of a tet's word in tm_nxt appends the tet to the next window's list. Tets with an active order-0 reaction (sources) have a list of their
-// own and are tested every window.
+// of a tet's word in tm_nxt appends the tet to the next window's list. Tets
+// with an active order-0 reaction (sources) have a list of their own and are
+// tested every window.
+//
+// What bounds it: scattered accesses to L2 and a chunk's chain of them (list
+// entry, record, counts, atomics, append). On the 1.03M-tet dendrite (0.12
+// molecules per tet) an empty launch takes 1.4 us, the chunks without
+// reactions and draws 8.7, all of it 14.6 us per window; block tiles, which
+// copied every count, took 39.8. Tried: one append per block, 14.5; places
+// reserved at the start of a chunk, 16.9; a scan of tiles for listed tets
+// instead of a list, 30.8.
 #pragma once
 
 #include "steps_warp.cuh"
