@@ -1811,13 +1811,16 @@ struct steps_batch {
         return STEPS_OK;
     }
 
+    // launches of a batched window: tiles, the list form, advance
+    uint64_t per_window(int b) const { return (work[slot(b)].n ? 1 : 0) + (lwork.n ? 1 : 0) + 1; }
+
     int window(int b, cudaStream_t st) {  // one batched window + advance
         Work &w = work[slot(b)];
         int rc = use_spec && spec[slot(b)] ? launch_spec_batch(spec[slot(b)], w.d, w.n, d_reps, max_S, b, st)
                                            : launch_step_batch(w.d, w.n, d_reps, max_S, max_R, any_order0, b, st);
         if (!rc && lwork.n) rc = launch_spec_batch(spec_list, lwork.d, lwork.n, d_reps, max_S, 256, st);
         if (!rc) rc = launch_advance(d_reps, (int32_t)members.size(), st);
-        launches += 2;
+        launches += per_window(b);
         return rc;
     }
 
@@ -1927,7 +1930,7 @@ struct steps_batch {
             if (rc) return rc;
             for (; n - done >= kGraphWindows; done += kGraphWindows) {
                 if (!cuda_ok(cudaGraphLaunch(work[slot(b)].graph, stream), "cudaGraphLaunch")) return STEPS_ERR_CUDA;
-                launches += 2 * kGraphWindows;
+                launches += per_window(b) * kGraphWindows;
             }
         }
         for (; done < n; ++done) {
