@@ -417,21 +417,29 @@ struct steps_sim {
                 return STEPS_ERR_OOM;
             }
         }
+        int rc = STEPS_OK;
         if ((!warp && (!cuda_ok(cudaMalloc((void **)&fl.d_tnb_off, off.size() * 4), "flow tables") ||
                        !cuda_ok(cudaMalloc((void **)&fl.d_tnb, nb.size() * 4), "flow tables"))) ||
-            !cuda_ok(cudaMalloc((void **)&fl.d_flow, ((size_t)nwords + 1) * 4), "flow tables")) {
+            !cuda_ok(cudaMalloc((void **)&fl.d_flow, ((size_t)nwords + 1) * 4), "flow tables"))
+            rc = STEPS_ERR_OOM;
+        // on the stream of the launches: a launch there waits for nothing the
+        // default stream still has to do, and a word of an earlier simulation
+        // in this memory would open a tile's wait at once
+        if (!rc &&
+            ((!warp && (!cuda_ok(cudaMemcpyAsync(fl.d_tnb_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice, stream),
+                                 "flow tables") ||
+                        !cuda_ok(cudaMemcpyAsync(fl.d_tnb, nb.data(), nb.size() * 4, cudaMemcpyHostToDevice, stream),
+                                 "flow tables"))) ||
+             !cuda_ok(cudaMemsetAsync(fl.d_flow, 0, ((size_t)nwords + 1) * 4, stream), "flow tables")))
+            rc = STEPS_ERR_CUDA;
+        if (rc) {
             cudaFree(fl.d_tnb_off);
             cudaFree(fl.d_tnb);
             cudaFree(fl.d_flow);
             fl.d_tnb_off = fl.d_tnb = nullptr;
             fl.d_flow = nullptr;
-            return STEPS_ERR_OOM;
+            return rc;
         }
-        if ((!warp &&
-             (!cuda_ok(cudaMemcpy(fl.d_tnb_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice), "flow tables") ||
-              !cuda_ok(cudaMemcpy(fl.d_tnb, nb.data(), nb.size() * 4, cudaMemcpyHostToDevice), "flow tables"))) ||
-            !cuda_ok(cudaMemset(fl.d_flow, 0, ((size_t)nwords + 1) * 4), "flow tables"))
-            return STEPS_ERR_CUDA;
         fl.spec = sp;
         fl.generic = generic;
         fl.block = (int)B;
@@ -1883,7 +1891,11 @@ struct steps_batch {
         const int64_t nwords = nwork * (b / 32);
         if (!cuda_ok(cudaMalloc((void **)&f.d_flow, ((size_t)nwords + 1) * 4), "steps_batch: flow words"))
             return STEPS_ERR_OOM;
-        if (!cuda_ok(cudaMemset(f.d_flow, 0, ((size_t)nwords + 1) * 4), "steps_batch")) return STEPS_ERR_CUDA;
+        if (!cuda_ok(cudaMemsetAsync(f.d_flow, 0, ((size_t)nwords + 1) * 4, stream), "steps_batch: flow words")) {
+            cudaFree(f.d_flow);
+            f.d_flow = nullptr;
+            return STEPS_ERR_CUDA;
+        }
         f.nwords = nwords;
         f.groups = std::move(groups);
         return STEPS_OK;
