@@ -1006,29 +1006,27 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
         cudaGetLastError();
         return STEPS_ERR_OOM;
     }
-    bool ok = cuda_ok(cudaMemset(s->d_nbr, 0xFF, Tpad * 16), "memset") &&
-              cuda_ok(cudaMemset(s->d_thr, 0, Tpad * 16), "memset") &&
-              cuda_ok(cudaMemset(s->d_inv_nav, 0, Tpad * 4), "memset") &&
-              cuda_ok(cudaMemcpy(s->d_nbr, s->tab.nbr_dev.data(), T * 16, cudaMemcpyHostToDevice), "upload nbr") &&
-              cuda_ok(cudaMemcpy(s->d_thr, s->tab.thr_dev.data(), T * 16, cudaMemcpyHostToDevice), "upload thr") &&
-              cuda_ok(cudaMemcpy(s->d_inv_nav, s->tab.inv_nav_dev.data(), T * 4, cudaMemcpyHostToDevice),
-                      "upload inv_nav") &&
-              cuda_ok(cudaMemset(s->d_cnt[0], 0, S * Tpad * 4), "memset") &&
-              cuda_ok(cudaMemset(s->d_cnt[1], 0, S * Tpad * 4), "memset") &&
-              cuda_ok(cudaMemset(s->d_err, 0, 24), "memset") && cuda_ok(cudaMemset(s->d_window_base, 0, 8), "memset");
+    // every upload on the simulation's stream, so that its launches come after
+    // them whatever the default stream is busy with
+    const cudaStream_t st = s->stream;
+    auto fill = [&](void *p, int byte, size_t n) { return cuda_ok(cudaMemsetAsync(p, byte, n, st), "memset"); };
+    auto put = [&](void *p, const void *src, size_t n, const char *what) {
+        return cuda_ok(cudaMemcpyAsync(p, src, n, cudaMemcpyHostToDevice, st), what);
+    };
+    bool ok = fill(s->d_nbr, 0xFF, Tpad * 16) && fill(s->d_thr, 0, Tpad * 16) && fill(s->d_inv_nav, 0, Tpad * 4) &&
+              put(s->d_nbr, s->tab.nbr_dev.data(), T * 16, "upload nbr") &&
+              put(s->d_thr, s->tab.thr_dev.data(), T * 16, "upload thr") &&
+              put(s->d_inv_nav, s->tab.inv_nav_dev.data(), T * 4, "upload inv_nav") &&
+              fill(s->d_cnt[0], 0, S * Tpad * 4) && fill(s->d_cnt[1], 0, S * Tpad * 4) && fill(s->d_err, 0, 24) &&
+              fill(s->d_window_base, 0, 8);
     if (ok && reordered)
-        ok = cuda_ok(cudaMemset(s->d_orig, 0, Tpad * 4), "memset") &&
-             cuda_ok(cudaMemcpy(s->d_orig, s->tab.perm.data(), T * 4, cudaMemcpyHostToDevice), "upload perm") &&
-             cuda_ok(cudaMemcpy(s->d_inv_perm, s->tab.inv_perm.data(), T * 4, cudaMemcpyHostToDevice),
-                     "upload inv_perm");
-    if (ok && s->model.leave_exp) {
-        ok = cuda_ok(cudaMemset(s->d_leave[0], 0, S * Tpad * 4), "memset") &&
-             cuda_ok(cudaMemset(s->d_leave[1], 0, S * Tpad * 4), "memset") &&
-             cuda_ok(cudaMemcpy(s->d_G, s->tab.G_dev.data(), T * 8, cudaMemcpyHostToDevice), "upload G") &&
-             s->upload_leave(s->tab.tau, s->stream) == STEPS_OK &&
-             cuda_ok(cudaStreamSynchronize(s->stream), "leave table upload");
-    }
-    if (!ok) return STEPS_ERR_CUDA;
+        ok = fill(s->d_orig, 0, Tpad * 4) && put(s->d_orig, s->tab.perm.data(), T * 4, "upload perm") &&
+             put(s->d_inv_perm, s->tab.inv_perm.data(), T * 4, "upload inv_perm");
+    if (ok && s->model.leave_exp)
+        ok = fill(s->d_leave[0], 0, S * Tpad * 4) && fill(s->d_leave[1], 0, S * Tpad * 4) &&
+             put(s->d_G, s->tab.G_dev.data(), T * 8, "upload G") && s->upload_leave(s->tab.tau, st) == STEPS_OK;
+    // (a clone on another stream reads the tables as soon as this call returns)
+    if (!ok || !cuda_ok(cudaStreamSynchronize(st), "steps_sim_create")) return STEPS_ERR_CUDA;
     // the model-specialised step kernel (compiled once per model and block size)
     constexpr int64_t kSpecializeMinTets = 65536;
     if (s->opt.specialize > 0 || (s->opt.specialize == 0 && s->T >= kSpecializeMinTets)) {
@@ -1253,15 +1251,16 @@ int steps_set_reac_mask(steps_sim *sim, int32_t reac, const uint8_t *active) {
         sim->h_rmask[d] = on ? (sim->h_rmask[d] | bit) : (sim->h_rmask[d] & ~bit);
     }
     if (!sim->d_rmask) {
-        if (!cuda_ok(cudaMalloc((void **)&sim->d_rmask, (size_t)sim->Tpad * 4), "steps_set_reac_mask: alloc") ||
-            !cuda_ok(cudaMemset(sim->d_rmask, 0, (size_t)sim->Tpad * 4), "steps_set_reac_mask: memset"))
+        if (!cuda_ok(cudaMalloc((void **)&sim->d_rmask, (size_t)sim->Tpad * 4), "steps_set_reac_mask: alloc"))
             return STEPS_ERR_OOM;
         sim->drop_graphs();  // kernel arguments change
+        if (!cuda_ok(cudaMemsetAsync(sim->d_rmask, 0, (size_t)sim->Tpad * 4, sim->stream), "steps_set_reac_mask: memset"))
+            return STEPS_ERR_CUDA;
     }
     sim->src_valid = sim->list_valid = false;
-    if (!cuda_ok(cudaStreamSynchronize(sim->stream), "steps_set_reac_mask") ||
-        !cuda_ok(cudaMemcpy(sim->d_rmask, sim->h_rmask.data(), T * 4, cudaMemcpyHostToDevice),
-                 "steps_set_reac_mask: copy"))
+    if (!cuda_ok(cudaMemcpyAsync(sim->d_rmask, sim->h_rmask.data(), T * 4, cudaMemcpyHostToDevice, sim->stream),
+                 "steps_set_reac_mask: copy") ||
+        !cuda_ok(cudaStreamSynchronize(sim->stream), "steps_set_reac_mask"))
         return STEPS_ERR_CUDA;
     return STEPS_OK;
 }
@@ -1738,12 +1737,12 @@ struct steps_batch {
     }
 
     // `v` as a work list on the device
-    static int upload_work(Work &w, const std::vector<BlockWork> &v) {
+    int upload_work(Work &w, const std::vector<BlockWork> &v) {
         w.n = (int64_t)v.size();
         if (w.n == 0) return STEPS_OK;
         if (!cuda_ok(cudaMalloc((void **)&w.d, v.size() * sizeof(BlockWork)), "steps_batch: alloc work"))
             return STEPS_ERR_OOM;
-        return cuda_ok(cudaMemcpy(w.d, v.data(), v.size() * sizeof(BlockWork), cudaMemcpyHostToDevice),
+        return cuda_ok(cudaMemcpyAsync(w.d, v.data(), v.size() * sizeof(BlockWork), cudaMemcpyHostToDevice, stream),
                        "steps_batch: upload work")
                    ? STEPS_OK
                    : STEPS_ERR_CUDA;
@@ -2011,7 +2010,7 @@ int steps_batch_create(steps_sim *const *members, int32_t n, const steps_batch_o
          !cuda_ok(cudaMallocHost((void **)&b->h_lcnt, (size_t)n * 16), "steps_batch_create: host alloc")) ||
         !cuda_ok(cudaMalloc((void **)&b->d_reps, sizeof(RepEntry) * n), "steps_batch_create: alloc") ||
         !cuda_ok(cudaMalloc((void **)&b->d_err, 4), "steps_batch_create: alloc") ||
-        !cuda_ok(cudaMemset(b->d_err, 0, 4), "steps_batch_create: memset"))
+        !cuda_ok(cudaMemsetAsync(b->d_err, 0, 4, b->stream), "steps_batch_create: memset"))
         return STEPS_ERR_OOM;
     // the model-specialised batched kernel: all members must share one model structure
     bool uniform = true;
@@ -2215,7 +2214,7 @@ int batch_finish(steps_batch *b) {
         if (b->listed[j]) b->members[j]->fill_from(b->h_lcnt + 4 * j);
     const uint32_t err = *b->h_err;
     if (err) {
-        cudaMemset(b->d_err, 0, 4);
+        cudaMemsetAsync(b->d_err, 0, 4, b->stream);
         if (err & 4u) {
             for (steps_sim *m : b->members) m->failed = true;
             set_error("steps_batch_run: a bulk copy into shared memory did not complete within its wait limit; "

@@ -72,3 +72,42 @@ def test_first_batch_flow_run(capi):
         for w, m in zip(ws, members):
             assert np.array_equal(m.get_counts(), _oracle(w, [t], w.seed))
         b.close()
+
+
+@pytest.mark.parametrize("leave", [0, 1])
+def test_setup_while_the_default_stream_is_busy(capi, leave):
+    """A simulation created, masked, filled, run and cloned on a side stream. The
+    tets keep their order, so that no upload follows the zeroed counts."""
+    import torch
+    w = I.config2(nx=2, t_end=1.5e-3)
+    on = (np.arange(w.tets.shape[0]) % 3 != 0).astype(np.uint8)
+    side, other = torch.cuda.Stream(), torch.cuda.Stream()
+    ends = [0.7e-3, 1.5e-3]
+    want = _oracle(w, ends, 9, leave, {0: on})
+    _busy()
+    g = capi.Simulation(w.verts, w.tets, w.model, 9, reorder=capi.STEPS_REORDER_NONE, leave_law=leave,
+                        cuda_stream=side.cuda_stream)
+    _busy()
+    g.set_reac_mask(0, on)
+    g.set_counts(w.counts)
+    c = g.clone(9, cuda_stream=other.cuda_stream)
+    c.set_counts(w.counts)
+    for t in ends:
+        g.run(t)
+        c.run(t)
+    torch.cuda.synchronize()
+    assert np.array_equal(g.get_counts(), want)
+    assert np.array_equal(c.get_counts(), want)
+
+
+def test_batch_while_the_default_stream_is_busy(capi):
+    import torch
+    ws = [I.config1(seed=50 + j) for j in range(3)]
+    side = torch.cuda.Stream()
+    members = [capi.from_workload(w, cuda_stream=side.cuda_stream) for w in ws]
+    _busy()
+    b = capi.Batch(members, block=64, cuda_stream=side.cuda_stream)
+    b.run([w.t_end for w in ws])
+    torch.cuda.synchronize()
+    for w, m in zip(ws, members):
+        assert np.array_equal(m.get_counts(), _oracle(w, [w.t_end], w.seed))
