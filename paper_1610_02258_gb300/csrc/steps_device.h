@@ -105,6 +105,10 @@ constexpr int kManySpecies = 12;         // above: a warp first looks whether an
 constexpr int kWarpMapCap = 160;    // Philox blocks listed at a time
 constexpr int kWarpQueueCap = 160;  // waiting movers: 31 left over + four words of 32 lanes
 
+// Entries of a warp-tile block's species scales: a word that decides no molecule
+// may be given the species after the last (species_of), whose scale is 0.
+constexpr int kScaleEntries = kMaxSpecies + 1;
+
 // Whether a flow launch's blocks (of a compile-time size) stay resident and take
 // item after item, else one item each.
 #if defined(__CUDACC__) || defined(__CUDACC_RTC__)

@@ -321,7 +321,8 @@ __device__ __forceinline__ void plane_groups(const StepArgs &a, WarpTile<SM> &w,
 // holds the words up to and including each species, a byte each, below 128;
 // v's byte with the top bit set, minus that, keeps the top bit where v has
 // reached it (no borrow between bytes). Rows past the last species hold 0x80,
-// which no word reaches. (The byte dot product __dp4a in place of the shifts
+// which no word reaches; with 32 species there is no such row, and a word past
+// the tet's last molecule gives 32 (kScaleEntries). (The byte dot product __dp4a in place of the shifts
 // and the population count took three times the instructions on this GPU.)
 template <int NP>
 __device__ __forceinline__ uint32_t species_of(const uint32_t *pre, uint32_t v4) {
@@ -722,7 +723,7 @@ __device__ __forceinline__ void warp_step(const ModelDev &m, const StepArgs &a, 
                                           const FlowArgs *f = nullptr, uint32_t q = 0, uint32_t dep = 0) {
     extern __shared__ __align__(16) unsigned char warp_smem[];
     __shared__ RxnTab tb;
-    __shared__ uint32_t s_scale[kMaxSpecies];
+    __shared__ uint32_t s_scale[kScaleEntries];
     static_assert(SM <= kWarpMaxSpecies, "species bound");
     const int threads = BLOCK ? BLOCK : (int)blockDim.x, warps = threads / 32;
     constexpr bool PERSIST = warp_flow_persists(BLOCK);
@@ -731,6 +732,7 @@ __device__ __forceinline__ void warp_step(const ModelDev &m, const StepArgs &a, 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     P::template build<32>(m, tb);  // (of up to 32 reactions, by the first warp)
     if (tid < kMaxSpecies) s_scale[tid] = a.scale[tid];
+    if (tid == 0) s_scale[kMaxSpecies] = 0u;
     __syncthreads();
     WarpTile<SM> &w = reinterpret_cast<WarpTile<SM> *>(warp_smem)[warp];
     if constexpr (FLOW == 1) {
