@@ -433,6 +433,12 @@ int steps_debug_flow_wait(int32_t deliver, int64_t limit_cycles);
  * too near an integer and were computed by the host instead. Errors:
  * STEPS_ERR_ARG (not an EXP simulation, bad tau_k). */
 int steps_debug_leave_table(steps_sim *sim, double tau_k, uint32_t *out, uint32_t *decided);
+/* The nth device allocation that simulations and batches make from now on, on
+ * the calling thread, fails as if the device were full (0: none does; a test
+ * of what follows a failure, without filling the device). *made (may be NULL)
+ * receives how many such allocations the thread has made so far. Errors:
+ * STEPS_ERR_ARG (nth < 0). */
+int steps_debug_fail_alloc(int32_t nth, int64_t *made);
 /* The host-side set-up of steps_sim_create alone, with no device work (for
  * tests of the host logic without a GPU): *tau (§2.1), the cumulative face
  * thresholds of every tet at the full window ([nt*4] uint32, 2^31 fixed

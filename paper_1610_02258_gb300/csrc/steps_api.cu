@@ -251,6 +251,20 @@ bool cuda_ok(cudaError_t e, const char *what) {
     return false;
 }
 
+// Device allocations of simulations and batches. A test makes one of its
+// thread's fail (steps_debug_fail_alloc): the paths that follow cannot be
+// reached by filling the device.
+thread_local int32_t t_fail_alloc = 0;
+thread_local int64_t t_allocs = 0;
+
+cudaError_t device_alloc(void **p, size_t bytes) {
+    if (t_fail_alloc > 0 && --t_fail_alloc == 0) return cudaErrorMemoryAllocation;
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaSuccess) ++t_allocs;
+    else cudaGetLastError();
+    return e;
+}
+
 }  // namespace
 
 struct steps_sim {
@@ -346,7 +360,7 @@ struct steps_sim {
         size_t n = 0;
         for (const Request &r : want) n += (r.second + 255) / 256 * 256;
         void *p = nullptr;
-        const cudaError_t e = cudaMalloc(&p, n);
+        const cudaError_t e = device_alloc(&p, n);
         if (e != cudaSuccess) return e;
         arena = static_cast<char *>(p);
         arena_bytes = n;
@@ -418,9 +432,9 @@ struct steps_sim {
             }
         }
         int rc = STEPS_OK;
-        if ((!warp && (!cuda_ok(cudaMalloc((void **)&fl.d_tnb_off, off.size() * 4), "flow tables") ||
-                       !cuda_ok(cudaMalloc((void **)&fl.d_tnb, nb.size() * 4), "flow tables"))) ||
-            !cuda_ok(cudaMalloc((void **)&fl.d_flow, ((size_t)nwords + 1) * 4), "flow tables"))
+        if ((!warp && (!cuda_ok(device_alloc((void **)&fl.d_tnb_off, off.size() * 4), "flow tables") ||
+                       !cuda_ok(device_alloc((void **)&fl.d_tnb, nb.size() * 4), "flow tables"))) ||
+            !cuda_ok(device_alloc((void **)&fl.d_flow, ((size_t)nwords + 1) * 4), "flow tables"))
             rc = STEPS_ERR_OOM;
         // on the stream of the launches: a launch there waits for nothing the
         // default stream still has to do, and a word of an earlier simulation
@@ -979,7 +993,7 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
     for (size_t d = 0; d < T && !reordered; ++d) reordered = s->tab.perm[d] != (int32_t)d;
     cudaError_t e = cudaSuccess;
     auto alloc = [&](void **p, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMalloc(p, bytes);
+        if (e == cudaSuccess) e = device_alloc(p, bytes);
     };
     alloc((void **)&s->d_cnt[0], S * Tpad * 4);
     alloc((void **)&s->d_cnt[1], S * Tpad * 4);
@@ -1251,7 +1265,7 @@ int steps_set_reac_mask(steps_sim *sim, int32_t reac, const uint8_t *active) {
         sim->h_rmask[d] = on ? (sim->h_rmask[d] | bit) : (sim->h_rmask[d] & ~bit);
     }
     if (!sim->d_rmask) {
-        if (!cuda_ok(cudaMalloc((void **)&sim->d_rmask, (size_t)sim->Tpad * 4), "steps_set_reac_mask: alloc"))
+        if (!cuda_ok(device_alloc((void **)&sim->d_rmask, (size_t)sim->Tpad * 4), "steps_set_reac_mask: alloc"))
             return STEPS_ERR_OOM;
         sim->drop_graphs();  // kernel arguments change
         if (!cuda_ok(cudaMemsetAsync(sim->d_rmask, 0, (size_t)sim->Tpad * 4, sim->stream), "steps_set_reac_mask: memset"))
@@ -1434,7 +1448,7 @@ int steps_run_record(steps_sim *sim, double t_end, double dt_rec, int32_t n_spec
         cudaFree(sim->d_rec);
         sim->d_rec = nullptr;
         sim->rec_bytes = 0;
-        if (!cuda_ok(cudaMalloc((void **)&sim->d_rec, need), "steps_run_record: alloc")) return STEPS_ERR_OOM;
+        if (!cuda_ok(device_alloc((void **)&sim->d_rec, need), "steps_run_record: alloc")) return STEPS_ERR_OOM;
         sim->rec_bytes = need;
     }
     int32_t *d_species = sim->d_rec, *d_tets = sim->d_rec + n_species;
@@ -1569,6 +1583,16 @@ int steps_debug_leave_table(steps_sim *sim, double tau_k, uint32_t *out, uint32_
                  "steps_debug_leave_table") ||
         !cuda_ok(cudaStreamSynchronize(sim->stream), "steps_debug_leave_table"))
         return STEPS_ERR_CUDA;
+    return STEPS_OK;
+}
+
+int steps_debug_fail_alloc(int32_t nth, int64_t *made) {
+    if (nth < 0) {
+        set_error("steps_debug_fail_alloc: nth must be >= 0");
+        return STEPS_ERR_ARG;
+    }
+    t_fail_alloc = nth;
+    if (made) *made = t_allocs;
     return STEPS_OK;
 }
 
@@ -1736,16 +1760,22 @@ struct steps_batch {
         cudaFreeHost(h_reps);
     }
 
-    // `v` as a work list on the device
+    // `v` as a work list on the device; after a failure the list counts as not
+    // built, so that a later run builds it or fails again
     int upload_work(Work &w, const std::vector<BlockWork> &v) {
+        if (!v.empty()) {
+            const size_t bytes = v.size() * sizeof(BlockWork);
+            BlockWork *d = nullptr;
+            if (!cuda_ok(device_alloc((void **)&d, bytes), "steps_batch: alloc work")) return STEPS_ERR_OOM;
+            if (!cuda_ok(cudaMemcpyAsync(d, v.data(), bytes, cudaMemcpyHostToDevice, stream), "steps_batch: upload work")) {
+                cudaFree(d);
+                return STEPS_ERR_CUDA;
+            }
+            w.d = d;
+        }
         w.n = (int64_t)v.size();
-        if (w.n == 0) return STEPS_OK;
-        if (!cuda_ok(cudaMalloc((void **)&w.d, v.size() * sizeof(BlockWork)), "steps_batch: alloc work"))
-            return STEPS_ERR_OOM;
-        return cuda_ok(cudaMemcpyAsync(w.d, v.data(), v.size() * sizeof(BlockWork), cudaMemcpyHostToDevice, stream),
-                       "steps_batch: upload work")
-                   ? STEPS_OK
-                   : STEPS_ERR_CUDA;
+        w.built = true;
+        return STEPS_OK;
     }
 
     int build_work(int b) try {
@@ -1756,7 +1786,6 @@ struct steps_batch {
             const int64_t tiles = listed[j] ? 0 : (members[j]->T + b - 1) / b;
             for (int64_t t = 0; t < tiles; ++t) v.push_back(BlockWork{(int32_t)j, (int32_t)t});
         }
-        w.built = true;
         return upload_work(w, v);
     } catch (const std::bad_alloc &) {
         set_error("steps_batch: work list: out of host memory");
@@ -1786,7 +1815,6 @@ struct steps_batch {
                 const int64_t n = listed[j] ? list_blocks(members[j]->T, 256) : 0;
                 for (int64_t t = 0; t < n; ++t) v.push_back(BlockWork{(int32_t)j, (int32_t)t});
             }
-            lwork.built = true;
             int rc = upload_work(lwork, v);
             if (rc) return rc;
         }
@@ -1888,7 +1916,7 @@ struct steps_batch {
         }
         // flow runs on the specialised kernels only: warp tiles, which publish per 32 tets and need no lists
         const int64_t nwords = nwork * (b / 32);
-        if (!cuda_ok(cudaMalloc((void **)&f.d_flow, ((size_t)nwords + 1) * 4), "steps_batch: flow words"))
+        if (!cuda_ok(device_alloc((void **)&f.d_flow, ((size_t)nwords + 1) * 4), "steps_batch: flow words"))
             return STEPS_ERR_OOM;
         if (!cuda_ok(cudaMemsetAsync(f.d_flow, 0, ((size_t)nwords + 1) * 4, stream), "steps_batch: flow words")) {
             cudaFree(f.d_flow);
@@ -1930,9 +1958,17 @@ struct steps_batch {
         return STEPS_OK;
     }
 
-    int run_windows(int b, int64_t n) {  // n windows at block size b
+    // What windows at block size b need, allocated. Called for every size a run
+    // may use before its first window: a run that fails in between would leave
+    // the members' counts ahead of their clocks.
+    int prepare(int b) {
         int rc = build_work(b);
         if (!rc) rc = prepare_spec(b);
+        return !rc && flow && use_spec && spec[slot(b)] ? build_flow(b) : rc;
+    }
+
+    int run_windows(int b, int64_t n) {  // n windows at block size b
+        int rc = prepare(b);
         if (rc) return rc;
         if (flow && use_spec && spec[slot(b)] && n >= 2) return flow_windows(b, n);
         int64_t done = 0;
@@ -2008,8 +2044,8 @@ int steps_batch_create(steps_sim *const *members, int32_t n, const steps_batch_o
         !cuda_ok(cudaMallocHost((void **)&b->h_err, 4), "steps_batch_create: host alloc") ||
         (std::any_of(b->members.begin(), b->members.end(), [](const steps_sim *m) { return m->spec_list != nullptr; }) &&
          !cuda_ok(cudaMallocHost((void **)&b->h_lcnt, (size_t)n * 16), "steps_batch_create: host alloc")) ||
-        !cuda_ok(cudaMalloc((void **)&b->d_reps, sizeof(RepEntry) * n), "steps_batch_create: alloc") ||
-        !cuda_ok(cudaMalloc((void **)&b->d_err, 4), "steps_batch_create: alloc") ||
+        !cuda_ok(device_alloc((void **)&b->d_reps, sizeof(RepEntry) * n), "steps_batch_create: alloc") ||
+        !cuda_ok(device_alloc((void **)&b->d_err, 4), "steps_batch_create: alloc") ||
         !cuda_ok(cudaMemsetAsync(b->d_err, 0, 4, b->stream), "steps_batch_create: memset"))
         return STEPS_ERR_OOM;
     // the model-specialised batched kernel: all members must share one model structure
@@ -2102,12 +2138,16 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
         return STEPS_ERR_CUDA;
     int64_t done = 0;
     int rc = STEPS_OK;
-    if (b->autotune && nmax >= 12) {
+    const int cand[3] = {128, 256, 512};
+    const bool tune = b->autotune && nmax >= 12;
+    for (int c = 0; c < 3 && tune && rc == STEPS_OK; ++c) rc = b->prepare(cand[c]);
+    if (rc == STEPS_OK) rc = b->prepare(b->block);
+    if (rc) return rc;
+    if (tune) {
         // time the candidate block sizes on alternating windows (one warm window
         // each, then two rounds of one timed window each), so that the state's
         // slow drift over the run cancels; keep 256 unless another is more than
         // 2 % faster
-        const int cand[3] = {128, 256, 512};
         b->tune_ms.assign(3, 0.f);
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (!cuda_ok(cudaEventCreate(&e0), "steps_batch_run: autotuner event") ||
@@ -2118,8 +2158,6 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
         float total[3] = {0.f, 0.f, 0.f};
         for (int round = 0; round < 2 && rc == STEPS_OK; ++round) {
             for (int c = 0; c < 3 && rc == STEPS_OK; ++c) {
-                rc = b->build_work(cand[c]);
-                if (rc) break;
                 if (round == 0) {
                     rc = b->run_windows(cand[c], 1);  // warm
                     if (rc) break;

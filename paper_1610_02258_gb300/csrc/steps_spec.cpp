@@ -420,6 +420,10 @@ int launch_spec_flow(void *spec, const ModelDev &m, const StepArgs &a, const Flo
 int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, const FlowArgs &f, uint32_t work0, int S,
                            int block, void *stream) {
     if (f.nwin == 0 || f.ntiles == 0) return STEPS_OK;
+    if (!work) {
+        set_error("specialised batched flow kernel launch: no work list");
+        return STEPS_ERR_STATE;
+    }
     Compiled *c = static_cast<Compiled *>(spec);
     const void *fn = (const void *)c->kern_batch_flow;
     const size_t smem = c->smem;
@@ -438,6 +442,10 @@ int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, co
 int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEntry *reps, int S, int block,
                       void *stream) {
     if (nblocks <= 0) return STEPS_OK;
+    if (!work) {
+        set_error("specialised batched step kernel launch: no work list");
+        return STEPS_ERR_STATE;
+    }
     Compiled *c = static_cast<Compiled *>(spec);
     const void *fn = (const void *)c->kern_batch;
     const size_t smem = c->smem;
