@@ -73,16 +73,20 @@ __device__ __forceinline__ int32_t round_trials32(double nbar, uint32_t w, int32
     return fl > (uint64_t)most ? most : (int32_t)fl;
 }
 
+// A propensity that is 0 where a reactant is absent, whatever the rate.
+__device__ __forceinline__ float careful_propensity(const float4 p, const int32_t *cnt, float inv_nav) {
+    const bool have = *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(cnt) + __float_as_uint(p.y)) &&
+                      *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(cnt) + __float_as_uint(p.z));
+    return have ? propensity(p, cnt, inv_nav, true) : 0.0f;
+}
+
 // First propensity sums of a tet whose plain sums are not finite (rates near
 // the float range): a reaction without all its reactants counts 0.
 __device__ __noinline__ float careful_sums(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
                                            uint32_t active, float *psum) {
     float a0 = 0.0f;
     for (int r = 0; r < m.R; ++r) {
-        const float4 p = tb.p[r];
-        const bool have = *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(cnt) + __float_as_uint(p.y)) &&
-                          *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(cnt) + __float_as_uint(p.z));
-        a0 = __fadd_rn(a0, ((active >> r) & 1u) && have ? propensity(p, cnt, inv_nav, true) : 0.0f);
+        a0 = __fadd_rn(a0, ((active >> r) & 1u) ? careful_propensity(tb.p[r], cnt, inv_nav) : 0.0f);
         if (psum) psum[r] = a0;
     }
     return a0;
@@ -96,6 +100,17 @@ __device__ __noinline__ int last_positive_tab(const RxnTab &tb, const ModelDev &
     for (int r = 0; r < m.R; ++r)
         if (((active >> r) & 1u) && propensity(tb.p[r], cnt, inv_nav, true) > 0.0f) last = r;
     return last;
+}
+
+// The pick from careful_sums, for a model without kept sums.
+__device__ __noinline__ int careful_pick(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
+                                         uint32_t active, float target) {
+    float sum = 0.0f;
+    for (int r = 0; r < m.R; ++r) {
+        sum = __fadd_rn(sum, ((active >> r) & 1u) ? careful_propensity(tb.p[r], cnt, inv_nav) : 0.0f);
+        if (!(sum <= target)) return r;
+    }
+    return last_positive_tab(tb, m, cnt, inv_nav, active);
 }
 
 // Model access for models given at run time: the reaction table, walked in a
@@ -140,7 +155,10 @@ struct RtWarp {
         float sum = 0.0f;
         for (int r = 0; r < m.R; ++r) {
             sum = __fadd_rn(sum, ((active >> r) & 1u) ? propensity(tb.p[r], cnt, inv_nav, z) : 0.0f);
-            if (!(sum <= target)) return r;
+            if (!(sum <= target)) {
+                // not a number: an infinite rate times an absent reactant, which first_sums counted 0
+                return sum == sum ? r : careful_pick(tb, m, cnt, inv_nav, active, target);
+            }
         }
         return last_positive_tab(tb, m, cnt, inv_nav, active);
     }
