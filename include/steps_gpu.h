@@ -439,6 +439,12 @@ int steps_debug_leave_table(steps_sim *sim, double tau_k, uint32_t *out, uint32_
  * receives how many such allocations the thread has made so far. Errors:
  * STEPS_ERR_ARG (nth < 0). */
 int steps_debug_fail_alloc(int32_t nth, int64_t *made);
+/* What a run (plain, recorded, batched or without allocation) makes of the
+ * device's error word: its return code and message (host only). *closed (may
+ * be NULL): whether the simulations are closed to further runs. Bits: 1 a
+ * negative count, 2 too many reactions in a tet, 4 a bulk copy and 8 a tile of
+ * a flow launch that did not come within the wait limit. */
+int steps_debug_error_word(uint32_t word, int32_t *closed);
 /* The host-side set-up of steps_sim_create alone, with no device work (for
  * tests of the host logic without a GPU): *tau (§2.1), the cumulative face
  * thresholds of every tet at the full window ([nt*4] uint32, 2^31 fixed

@@ -36,7 +36,7 @@ EXPORTS = [
     "steps_server_options_default", "steps_server_create", "steps_server_destroy", "steps_server_submit",
     "steps_server_step", "steps_server_job_state", "steps_server_take_result", "steps_server_stats",
     "steps_debug_host_tables", "steps_debug_wait", "steps_debug_flow_wait",
-    "steps_debug_leave_table", "steps_debug_fail_alloc",
+    "steps_debug_leave_table", "steps_debug_fail_alloc", "steps_debug_error_word",
 ]
 
 
@@ -108,6 +108,7 @@ def _load():
         "steps_debug_host_tables": (ctypes.c_int, [P, P, i32, ctypes.POINTER(ctypes.c_double), P, P]),
         "steps_debug_leave_table": (ctypes.c_int, [P, ctypes.c_double, P, ctypes.POINTER(ctypes.c_uint32)]),
         "steps_debug_fail_alloc": (ctypes.c_int, [i32, ctypes.POINTER(ctypes.c_int64)]),
+        "steps_debug_error_word": (ctypes.c_int, [ctypes.c_uint32, ctypes.POINTER(i32)]),
         "steps_server_options_default": (None, [ctypes.POINTER(steps_server_options)]),
         "steps_server_create": (ctypes.c_int, [ctypes.POINTER(steps_server_options), P, PP]),
         "steps_server_destroy": (None, [P]),
@@ -327,6 +328,13 @@ def steps_debug_fail_alloc(nth):
     made = ctypes.c_int64(0)
     _check(lib.steps_debug_fail_alloc(int(nth), ctypes.byref(made)))
     return made.value
+
+
+def steps_debug_error_word(word):
+    """(return code, whether the simulations are closed) of a device error word."""
+    closed = ctypes.c_int32(0)
+    rc = lib.steps_debug_error_word(int(word), ctypes.byref(closed))
+    return rc, bool(closed.value)
 
 
 def steps_debug_logf(x):

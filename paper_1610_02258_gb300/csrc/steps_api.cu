@@ -1332,6 +1332,22 @@ int enqueue_run(steps_sim *sim, double t_end) {
     return STEPS_OK;
 }
 
+// The return code of a device error word, with its message. *closed: a wait
+// ran out, the counts are not valid and the simulations of the launch are
+// closed to further runs.
+int error_word(uint32_t err, const char *who, bool *closed) {
+    *closed = (err & 12u) != 0u;
+    if (err == 0) return STEPS_OK;
+    set_error(std::string(who) +
+              (err & 4u ? ": a bulk copy into shared memory did not complete within its wait limit; a copy may still "
+                          "be in flight, so what the launch ran is closed to further runs"
+               : err & 8u ? ": a tile of a flow launch waited beyond its limit for the tiles it depends on; the counts "
+                            "are not valid, so what the launch ran is closed to further runs"
+               : err & 2u ? ": a tet fired more than 2^24 reactions in one window (rates too large)"
+                          : ": a negative count was seen on the device"));
+    return *closed ? STEPS_ERR_TIMEOUT : STEPS_ERR_STATE;
+}
+
 // Waits for the simulation's stream and turns the device error word into a
 // return code (and clears it).
 int finish_run(steps_sim *sim, const char *who) {
@@ -1341,25 +1357,11 @@ int finish_run(steps_sim *sim, const char *who) {
         !cuda_ok(cudaStreamSynchronize(sim->stream), who))
         return STEPS_ERR_CUDA;
     if (sim->listing) sim->fill_from(c);
-    if (err) {
-        cudaMemsetAsync(sim->d_err, 0, 4, sim->stream);
-        if (err & 4u) {
-            sim->failed = true;
-            set_error(std::string(who) + ": a bulk copy into shared memory did not complete within its wait limit; "
-                                         "a copy may still be in flight, so this simulation is closed to further runs");
-            return STEPS_ERR_TIMEOUT;
-        }
-        if (err & 8u) {
-            sim->failed = true;
-            set_error(std::string(who) + ": a tile of a flow launch waited beyond its limit for the tiles it depends "
-                                         "on; the counts are not valid, so this simulation is closed to further runs");
-            return STEPS_ERR_TIMEOUT;
-        }
-        set_error(std::string(who) + (err & 2u ? ": a tet fired more than 2^24 reactions in one window (rates too large)"
-                                               : ": a negative count was seen on the device"));
-        return STEPS_ERR_STATE;
-    }
-    return STEPS_OK;
+    if (err) cudaMemsetAsync(sim->d_err, 0, 4, sim->stream);
+    bool closed = false;
+    const int rc = error_word(err, who, &closed);
+    if (closed) sim->failed = true;
+    return rc;
 }
 
 // One recording: counts of the chosen species (rows of cur) at the chosen
@@ -1594,6 +1596,13 @@ int steps_debug_fail_alloc(int32_t nth, int64_t *made) {
     t_fail_alloc = nth;
     if (made) *made = t_allocs;
     return STEPS_OK;
+}
+
+int steps_debug_error_word(uint32_t word, int32_t *closed) {
+    bool c = false;
+    const int rc = error_word(word, "steps_debug_error_word", &c);
+    if (closed) *closed = c ? 1 : 0;
+    return rc;
 }
 
 int steps_debug_wait(int32_t deliver, int64_t limit_cycles) {
@@ -2251,19 +2260,11 @@ int batch_finish(steps_batch *b) {
     for (size_t j = 0; j < b->members.size(); ++j)
         if (b->listed[j]) b->members[j]->fill_from(b->h_lcnt + 4 * j);
     const uint32_t err = *b->h_err;
-    if (err) {
-        cudaMemsetAsync(b->d_err, 0, 4, b->stream);
-        if (err & 4u) {
-            for (steps_sim *m : b->members) m->failed = true;
-            set_error("steps_batch_run: a bulk copy into shared memory did not complete within its wait limit; "
-                      "a copy may still be in flight, so every member is closed to further runs");
-            return STEPS_ERR_TIMEOUT;
-        }
-        set_error(err & 2u ? "steps_batch_run: a tet fired more than 2^24 reactions in one window"
-                           : "steps_batch_run: a negative count was seen on the device");
-        return STEPS_ERR_STATE;
-    }
-    return STEPS_OK;
+    if (err) cudaMemsetAsync(b->d_err, 0, 4, b->stream);
+    bool closed = false;
+    const int rc = error_word(err, "steps_batch_run", &closed);
+    for (steps_sim *m : b->members) m->failed = m->failed || closed;
+    return rc;
 }
 
 std::string sim_structure_key(const steps_sim *sim) { return spec_program_source(sim->model, 256); }
@@ -2444,16 +2445,8 @@ extern "C" int steps_run_noalloc(steps_sim *sim, int32_t *d_counts, double t_end
     if (!cuda_ok(cudaMemcpyAsync(&err, sc.err, 4, cudaMemcpyDeviceToHost, st), "steps_run_noalloc: error word") ||
         !cuda_ok(cudaStreamSynchronize(st), "steps_run_noalloc"))
         return STEPS_ERR_CUDA;
-    if (err & 4u) {
-        sim->failed = true;
-        set_error("steps_run_noalloc: a bulk copy into shared memory did not complete within its wait limit; "
-                  "a copy may still be in flight, so this simulation is closed to further runs");
-        return STEPS_ERR_TIMEOUT;
-    }
-    if (err) {
-        set_error(err & 2u ? "steps_run_noalloc: a tet fired more than 2^24 reactions in one window"
-                           : "steps_run_noalloc: a negative count was seen on the device");
-        return STEPS_ERR_STATE;
-    }
-    return STEPS_OK;
+    bool closed = false;
+    rc = error_word(err, "steps_run_noalloc", &closed);
+    if (closed) sim->failed = true;
+    return rc;
 }
