@@ -1049,14 +1049,13 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
             set_error("steps_sim_create: the specialised step kernel could not be built: " + s->spec_why);
             return STEPS_ERR_CUDA;
         }
-        if (s->spec) {
+        if (s->spec && s->opt.flow != 1) {
             s->spec_list = spec_list_kernel(s->model);
             if (s->spec_list)
                 for (const steps_sim::Request &r : s->list_requests()) alloc(r.first, r.second);
-            if (e != cudaSuccess) {
-                set_error(std::string("steps_sim_create: device allocation failed: ") + cudaGetErrorString(e));
-                cudaGetLastError();
-                return STEPS_ERR_OOM;
+            if (e != cudaSuccess) {  // no room for the list form: the simulation runs its tiles
+                s->free_list();
+                s->spec_list = nullptr;
             }
         }
     } else {
@@ -1106,15 +1105,21 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
         alloc((void **)&s->d_inv_perm, T * 4);
     }
     if (src->d_rmask) alloc((void **)&s->d_rmask, Tpad * 4);
-    if (src->d_tm[0])
-        for (const steps_sim::Request &r : s->list_requests()) want.push_back(r);
     if (src->d_leave[0]) {
         alloc((void **)&s->d_leave[0], S * Tpad * 4);
         alloc((void **)&s->d_leave[1], S * Tpad * 4);
         alloc((void **)&s->d_G, Tpad * 8);
         alloc((void **)&s->d_leave_list, kLeaveListBytes);
     }
-    const cudaError_t e = s->alloc_arena(want);
+    const size_t base = want.size();
+    if (src->d_tm[0])
+        for (const steps_sim::Request &r : s->list_requests()) want.push_back(r);
+    cudaError_t e = s->alloc_arena(want);
+    if (e != cudaSuccess && want.size() > base) {  // no room for the list form: the clone runs its tiles
+        want.resize(base);
+        s->spec_list = nullptr;
+        e = s->alloc_arena(want);
+    }
     if (e != cudaSuccess) {
         set_error(std::string("steps_sim_clone: device allocation failed: ") + cudaGetErrorString(e));
         cudaGetLastError();

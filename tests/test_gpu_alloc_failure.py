@@ -83,3 +83,63 @@ def test_batch_runs_after_a_failed_allocation(capi, kind, block, flow):
             break
     else:
         raise AssertionError("a run makes more allocations than expected")
+
+
+def _sparse(capi, **kw):
+    verts, tets = I.kuhn_box_mesh(6, 6, 5, 0.5 * I.UM)
+    m = _many_species()
+    c = np.zeros((14, tets.shape[0]), np.int32)
+    c[:4, ::20] = 5
+    g = capi.Simulation(verts, tets, m, 70, specialize=1, **kw)
+    o = oracle.OracleSim(verts, tets, m, seed=70, occ=oracle.OCC, prec=32)
+    for obj in (g, o):
+        obj.set_counts(c)
+    return g, o, c
+
+
+def _equal_run(g, o):
+    g.run(20.4 * o.tau)
+    o.run(20.4 * o.tau)
+    assert g.windows == o.windows and np.array_equal(g.get_counts(), o.get_counts())
+
+
+def _list_bytes(g):
+    return (10 + g.S) * ((g.nt + 31) // 32 * 32) * 4 + 16
+
+
+def test_a_simulation_needs_no_room_for_the_list_form(capi):
+    """Each allocation of a creation in turn: those of the simulation proper end it,
+    those of the list form (sparse states of 13 or more species) do not."""
+    full = _sparse(capi)[0].device_bytes
+    without = refused = 0
+    for nth in range(1, 40):
+        capi.steps_debug_fail_alloc(nth)
+        try:
+            g, o, _ = _sparse(capi)
+        except capi.StepsError as e:
+            assert e.code == -4 and without == 0, e
+            refused += 1
+            continue
+        finally:
+            capi.steps_debug_fail_alloc(0)
+        if g.device_bytes == full:
+            break
+        assert g.device_bytes == full - _list_bytes(g)
+        without += 1
+        _equal_run(g, o)
+    assert without >= 5 and refused >= 5
+
+
+def test_a_clone_needs_no_room_for_the_list_form(capi):
+    g, o, c = _sparse(capi)
+    capi.steps_debug_fail_alloc(1)
+    k = g.clone(70)
+    assert k.device_bytes == g.device_bytes - _list_bytes(g)
+    k.set_counts(c)
+    _equal_run(k, o)
+
+
+def test_flow_simulations_hold_no_list_buffers(capi):
+    g, o, _ = _sparse(capi, flow=True)
+    assert g.device_bytes == _sparse(capi)[0].device_bytes - _list_bytes(g)
+    _equal_run(g, o)
