@@ -315,10 +315,11 @@ struct steps_sim {
     bool src_valid = false;         // the records and the sources match the reaction masks
     bool listing = false;           // the present run's windows go through the list form
     uint64_t list_built = 0;        // the window the list was last built for
-    double density = 0.0;           // molecules per tet when counts were last set
-    double fill = 0.0;              // listed tets or non-zero counts per tet, last known
-    // each species' share of both when its counts were last set (of all species at once: equal shares)
-    double set_density[kMaxSpecies] = {}, set_fill[kMaxSpecies] = {};
+    // Molecules per tet when all counts were last set; listed tets or non-zero
+    // counts per tet, last known. Counts of single species leave both unknown
+    // (negative): a run that needs one of them looks at the state (measure).
+    double density = 0.0;
+    double fill = 0.0;
     // time
     double t_base = 0.0;
     int64_t k_grid = 0;
@@ -555,8 +556,30 @@ struct steps_sim {
         return r;
     }
 
+    // density and fill of the present state; waits for the stream
+    int measure(cudaStream_t st) {
+        uint32_t seen[4] = {0, 0, 0, 0};
+        const int64_t n = (int64_t)S * Tpad;  // (the padding is zero)
+        if (!cuda_ok(cudaMemsetAsync(d_err + 2, 0, 16, st), "state measure")) return STEPS_ERR_CUDA;
+        any_negative<true><<<input_blocks(n), kInputThreads, 0, st>>>(d_cnt[cur], n, d_err + 2);
+        if (!cuda_ok(cudaGetLastError(), "state measure") ||
+            !cuda_ok(cudaMemcpyAsync(seen, d_err + 2, 16, cudaMemcpyDeviceToHost, st), "state measure") ||
+            !cuda_ok(cudaStreamSynchronize(st), "state measure"))
+            return STEPS_ERR_CUDA;
+        found(seen);
+        return STEPS_OK;
+    }
+
+    // density and fill from any_negative's words over all counts
+    void found(const uint32_t seen[4]) {
+        fill = seen[1] / (double)T;
+        density = (double)((uint64_t)seen[3] << 32 | seen[2]) / (double)T;
+    }
+
     // Before a run: the form of its windows, by what is known of the state.
     int choose_form() {
+        if (spec_list && opt.flow != 1 && fill < 0.0)
+            if (int rc = measure(stream)) return rc;
         const bool want = spec_list && opt.flow != 1 && fill <= kListFill;
         if (want != listing) drop_graphs();
         listing = want;
@@ -735,6 +758,8 @@ struct steps_sim {
     // fastest flow form is kept when it is more than 2 % faster than window
     // launches. The windows taken are ordinary windows of the run.
     int tune_flow(int64_t *used) {
+        if (density < 0.0)
+            if (int rc = measure(stream)) return rc;
         // the best form depends on the state: by powers of two of the molecules per tet
         const auto key = std::make_tuple((const void *)spec, T, opt.block, (int)std::lrint(std::log2(density + 0.01)));
         {
@@ -1186,19 +1211,8 @@ static int put_counts(steps_sim *sim, int32_t s0, int32_t ns, const int32_t *cou
         return STEPS_ERR_ARG;
     }
     sim->tm_valid = sim->list_valid = false;
-    // counts of every species replace the state; of one, they change what is known
-    // of it by as much as they differ from those set before
-    const double sum = (double)((uint64_t)seen[3] << 32 | seen[2]);
-    if (ns == sim->S) sim->fill = sim->density = 0.0;
-    for (int32_t s = s0; s < s0 + ns; ++s) {
-        const double f = seen[1] / (double)T / ns, d = sum / (double)T / ns;
-        sim->fill += ns == sim->S ? f : f - sim->set_fill[s];
-        sim->density += ns == sim->S ? d : d - sim->set_density[s];
-        sim->set_fill[s] = f;
-        sim->set_density[s] = d;
-    }
-    sim->fill = std::max(0.0, sim->fill);
-    sim->density = std::max(0.0, sim->density);
+    if (ns == sim->S) sim->found(seen);
+    else sim->fill = sim->density = -1.0;
     scatter_to_device_order<<<(unsigned)((T + 255) / 256), 256, 0, sim->stream>>>(
         sim->d_stage, (int64_t)T, ns, sim->d_inv_perm, sim->d_cnt[sim->cur] + (size_t)s0 * Tpad, Tpad);
     if (!cuda_ok(cudaGetLastError(), "steps_set_counts: scatter")) return STEPS_ERR_CUDA;
@@ -1811,8 +1825,11 @@ struct steps_batch {
     int choose_forms() try {
         std::vector<char> want(members.size(), 0);
         for (size_t j = 0; j < members.size(); ++j) {
-            const steps_sim *m = members[j];
-            want[j] = use_spec && !flow && m->spec_list && m->fill <= kListFill;
+            steps_sim *m = members[j];
+            want[j] = use_spec && !flow && m->spec_list;
+            if (want[j] && m->fill < 0.0)
+                if (int rc = m->measure(stream)) return rc;
+            want[j] = want[j] && m->fill <= kListFill;
             if (want[j]) spec_list = m->spec_list;
         }
         if (want != listed) {

@@ -1,0 +1,83 @@
+"""GPU tests of when a run takes the list form (models of 13 or more species in
+sparse states) and when the tiles, seen from whether a run's tuning of the
+launch form took place (tiles) or not (list form), with counts equal to the
+oracle's either way."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1610_02258_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+S = 14
+
+
+@pytest.fixture(scope="module")
+def capi():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1610_02258_gb300.build import build
+    build()
+    from paper_1610_02258_gb300 import capi as c
+    return c
+
+
+def _pair(capi, seed, grid=(8, 6, 5), source=0.0):
+    names = [f"S{i}" for i in range(S)]
+    reac = [([names[0]], [names[1]], 30.0), ([names[1]], [names[0]], 20.0)]
+    if source:
+        reac.append(([], [names[2]], source))
+    m = I.model_from_lists(names, [1e-11 / (1 + i) for i in range(S)], reac)
+    verts, tets = I.kuhn_box_mesh(*grid, 0.5 * I.UM)
+    g = capi.Simulation(verts, tets, m, seed, specialize=1)
+    o = oracle.OracleSim(verts, tets, m, seed=seed, occ=oracle.OCC, prec=32)
+    return g, o
+
+
+def _run(g, o, windows=80.4):
+    t = o.time + windows * o.tau
+    g.run(t)
+    o.run(t)
+    assert g.windows == o.windows and np.array_equal(g.get_counts(), o.get_counts())
+
+
+def _tiles(g):
+    return g.flow[1][0] > 0.0
+
+
+def _set(capi, g, o, c, species=None):
+    o.set_counts(c)
+    if species is None:
+        g.set_counts(c)
+    for s in species or []:
+        capi.steps_set_counts(g._sim, s, c[s])
+
+
+def test_empty_species_set_one_by_one_leave_a_dense_state_dense(capi):
+    g, o = _pair(capi, 1)
+    c = np.zeros((S, g.nt), np.int32)
+    c[0] = 9
+    _set(capi, g, o, c)
+    _set(capi, g, o, c, range(1, S))
+    _run(g, o)
+    assert _tiles(g)
+
+
+def test_a_sparse_state_set_species_by_species_is_listed(capi):
+    g, o = _pair(capi, 2)
+    c = np.zeros((S, g.nt), np.int32)
+    c[0] = 9
+    _set(capi, g, o, c)
+    c[0] = 0
+    c[:, ::60] = 2
+    _set(capi, g, o, c, range(S))
+    _run(g, o)
+    assert not _tiles(g)
+    c = o.get_counts()
+    c[3] = 5
+    _set(capi, g, o, c, [3])
+    _run(g, o)
+    assert _tiles(g)
+
