@@ -44,7 +44,7 @@ constexpr int kGraphWindows = 16;  // full windows per captured graph (even: buf
 // crowd at one end, 0.37: 15.8 -> 19.1.
 constexpr double kListFill = 0.33;
 constexpr uint64_t kListWindows = 128;       // windows after which a list is built afresh
-constexpr int64_t kListCheckWindows = 1024;  // windows after which a run looks at the list's length
+constexpr uint64_t kListCheckWindows = 1024;  // windows after which a run looks at the list's length
 constexpr int64_t kFlowTuneWindows = 72;  // windows the launch-form tuning takes (3 rounds of up to 3 groups)
 
 __global__ void scatter_to_device_order(const int32_t *src, int64_t nt, int32_t S, const int32_t *inv_perm,
@@ -315,6 +315,7 @@ struct steps_sim {
     bool src_valid = false;         // the records and the sources match the reaction masks
     bool listing = false;           // the present run's windows go through the list form
     uint64_t list_built = 0;        // the window the list was last built for
+    uint64_t looked = 0;            // the window its length was last looked at
     // Molecules per tet when all counts were last set; listed tets or non-zero
     // counts per tet, last known. Counts of single species leave both unknown
     // (negative): a run that needs one of them looks at the state (measure).
@@ -576,12 +577,24 @@ struct steps_sim {
         density = (double)((uint64_t)seen[3] << 32 | seen[2]) / (double)T;
     }
 
-    // Before a run: the form of its windows, by what is known of the state.
+    // Before a run, and within long ones: the form of its windows, by what is
+    // known of the state. A list's length is looked at (the stream waited for)
+    // every kListCheckWindows, also over the intervals of a recording.
     int choose_form() {
+        if (listing && k_total - looked >= kListCheckWindows) {
+            uint32_t c[4];
+            if (!cuda_ok(cudaMemcpyAsync(c, d_lcnt, 16, cudaMemcpyDeviceToHost, stream), "list length") ||
+                !cuda_ok(cudaStreamSynchronize(stream), "list length"))
+                return STEPS_ERR_CUDA;
+            fill_from(c);
+        }
         if (spec_list && opt.flow != 1 && fill < 0.0)
             if (int rc = measure(stream)) return rc;
         const bool want = spec_list && opt.flow != 1 && fill <= kListFill;
-        if (want != listing) drop_graphs();
+        if (want != listing) {
+            drop_graphs();
+            looked = k_total;
+        }
         listing = want;
         if (!listing) tm_valid = list_valid = false;  // the other kernels leave them behind
         return STEPS_OK;
@@ -608,22 +621,16 @@ struct steps_sim {
     }
 
     // n full windows in the list form, as long as the state stays sparse: their
-    // number into *done. The list's length is looked at every kListCheckWindows.
+    // number into *done
     int list_windows(int64_t n, int64_t *done) {
         while (listing && *done < n) {
-            const int64_t m = std::min(n - *done, kListCheckWindows);
-            int rc = window_launches(m);
+            int rc = choose_form();
+            if (rc) return rc;
+            if (!listing) break;
+            const int64_t m = std::min(n - *done, (int64_t)(kListCheckWindows - (k_total - looked)));
+            rc = window_launches(m);
             if (rc) return rc;
             *done += m;
-            if (*done < n) {
-                uint32_t c[4];
-                if (!cuda_ok(cudaMemcpyAsync(c, d_lcnt, 16, cudaMemcpyDeviceToHost, stream), "list length") ||
-                    !cuda_ok(cudaStreamSynchronize(stream), "list length"))
-                    return STEPS_ERR_CUDA;
-                fill_from(c);
-                rc = choose_form();
-                if (rc) return rc;
-            }
         }
         return STEPS_OK;
     }
@@ -631,6 +638,7 @@ struct steps_sim {
     // the fill from the list's lengths after the last window enqueued
     void fill_from(const uint32_t c[4]) {
         if (list_valid) fill = ((double)c[k_total % 3] + (d_src ? 0.5 * (double)c[3] : 0.0)) / (double)T;
+        looked = k_total;
     }
 
     void drop_graphs() {
@@ -1851,7 +1859,10 @@ struct steps_batch {
         }
         for (size_t j = 0; j < members.size(); ++j) {
             steps_sim *m = members[j];
-            if (m->listing != (bool)listed[j]) m->drop_graphs();
+            if (m->listing != (bool)listed[j]) {
+                m->drop_graphs();
+                m->looked = m->k_total;
+            }
             m->listing = listed[j];
             if (!m->listing) m->tm_valid = m->list_valid = false;  // the other kernels leave them behind
             int rc = m->prepare_list(stream);
@@ -2121,8 +2132,11 @@ namespace steps {
 
 // steps_batch_run without its final wait: every window is enqueued on the
 // batch's stream, the members' clocks advanced and the error word's copy to
-// the host enqueued. batch_finish waits and turns the word into a code.
-int batch_enqueue(steps_batch *b, const double *t_end) {
+// the host enqueued. batch_finish waits and turns the word into a code. While
+// members go through the list form, no member takes more than `most` full
+// windows (0: no limit) and *more says that there are others to run: the next
+// call looks at the lists' lengths and builds them afresh.
+int batch_enqueue(steps_batch *b, const double *t_end, int64_t most, bool *more) {
     CHECK_NULL(b, "steps_batch_run");
     CHECK_NULL(t_end, "steps_batch_run");
     const size_t n = b->members.size();
@@ -2136,6 +2150,8 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
     // members' own streams may still hold work
     for (steps_sim *m : b->members)
         if (!cuda_ok(cudaStreamSynchronize(m->stream), "steps_batch_run: member stream")) return STEPS_ERR_CUDA;
+    if (int rf = b->choose_forms()) return rf;
+    const bool sliced = most > 0 && std::count(b->listed.begin(), b->listed.end(), 1) > 0;
     // the window schedule of every member (the loop of steps_run)
     std::vector<int64_t> nfull(n, 0);
     std::vector<double> partial(n, 0.0);  // > 0: a shortened last window of this length
@@ -2143,12 +2159,16 @@ int batch_enqueue(steps_batch *b, const double *t_end) {
     for (size_t j = 0; j < n; ++j) {
         steps_sim *m = b->members[j];
         m->schedule(t_end[j], &nfull[j], &partial[j]);
+        if (sliced && nfull[j] > most) {
+            nfull[j] = most;
+            partial[j] = 0.0;
+            *more = true;
+        }
         // the shortened window's leave table first: it waits for the stream
         if (partial[j] > 0.0 && partial[j] != m->tab.tau)
             if (int rl = m->upload_leave(partial[j], b->stream)) return rl;
         nmax = std::max(nmax, nfull[j]);
     }
-    if (int rf = b->choose_forms()) return rf;
     // table for the full windows
     for (size_t j = 0; j < n; ++j) {
         steps_sim *m = b->members[j];
@@ -2296,8 +2316,13 @@ std::string sim_structure_key(const steps_sim *sim) { return spec_program_source
 extern "C" {
 
 int steps_batch_run(steps_batch *b, const double *t_end) {
-    int rc = steps::batch_enqueue(b, t_end);
-    return rc ? rc : steps::batch_finish(b);
+    for (bool more = true; more;) {
+        more = false;
+        int rc = steps::batch_enqueue(b, t_end, (int64_t)kListCheckWindows, &more);
+        if (!rc) rc = steps::batch_finish(b);
+        if (rc) return rc;
+    }
+    return STEPS_OK;
 }
 
 int steps_batch_specialized(const steps_batch *b, int32_t *specialized) {

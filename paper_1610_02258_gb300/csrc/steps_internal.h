@@ -115,7 +115,7 @@ void *spec_list_kernel(const HostModel &hm);
 // batches on different streams can run at the same time; and a key that is
 // equal for simulations whose models share one structure (one specialised
 // kernel serves them all).
-int batch_enqueue(steps_batch *b, const double *t_end);
+int batch_enqueue(steps_batch *b, const double *t_end, int64_t most = 0, bool *more = nullptr);
 int batch_finish(steps_batch *b);
 std::string sim_structure_key(const steps_sim *sim);
 

@@ -81,3 +81,44 @@ def test_a_sparse_state_set_species_by_species_is_listed(capi):
     _run(g, o)
     assert _tiles(g)
 
+
+
+def _filling(capi, seed):
+    """A few molecules, and a source in every tet that fills the mesh."""
+    g, o = _pair(capi, seed, source=3e-5)
+    c = np.zeros((S, g.nt), np.int32)
+    c[0, ::60] = 2
+    _set(capi, g, o, c)
+    return g, o
+
+
+def test_a_recording_leaves_the_list_form(capi):
+    """Intervals too short for a look of their own (100 windows) add up to one."""
+    import torch
+    g, o = _filling(capi, 3)
+    tets = np.arange(0, g.nt, 9, dtype=np.int32)
+    buf = torch.zeros((15, 1, tets.size), dtype=torch.int32, device="cuda")
+    dt = 100 * o.tau
+    assert g.run_record(15 * dt, dt, np.array([2], np.int32), tets, buf.data_ptr(), 15) == 15
+    assert _tiles(g)
+    for k in range(15):
+        o.run((k + 1) * dt)
+        assert np.array_equal(buf[k].cpu().numpy(), o.get_counts()[[2]][:, tets])
+    assert np.array_equal(g.get_counts(), o.get_counts())
+
+
+def test_a_batch_run_leaves_the_list_form(capi):
+    """One long run of a member that fills up and one that is dense from the start:
+    three launches a window (tiles, list, advance) become two on the way."""
+    pairs = [_filling(capi, 4), _pair(capi, 5, (6, 6, 5), 3e-5)]
+    g, o = pairs[1]
+    _set(capi, g, o, np.full((S, g.nt), 2, np.int32))
+    b = capi.Batch([p[0] for p in pairs], block=256, specialize=1)
+    windows = 1500.4
+    b.run([windows * o.tau for _, o in pairs])
+    for g, o in pairs:
+        o.run(windows * o.tau, threads=8)
+        assert g.windows == o.windows == 1501
+        assert np.array_equal(g.get_counts(), o.get_counts())
+    assert 1024 * 3 <= b.info[1] <= 1024 * 3 + 480 * 2
+    b.close()
