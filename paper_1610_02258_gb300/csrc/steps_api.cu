@@ -1828,18 +1828,39 @@ struct steps_batch {
         return STEPS_ERR_OOM;
     }
 
-    // The members of this run's list form, by what is known of their states; the
-    // work lists and graphs follow when they change.
-    int choose_forms() try {
+    // the members whose windows go through the list form, by what is known of their states
+    std::vector<char> wanted() const {
         std::vector<char> want(members.size(), 0);
         for (size_t j = 0; j < members.size(); ++j) {
-            steps_sim *m = members[j];
-            want[j] = use_spec && !flow && m->spec_list;
-            if (want[j] && m->fill < 0.0)
-                if (int rc = m->measure(stream)) return rc;
-            want[j] = want[j] && m->fill <= kListFill;
-            if (want[j]) spec_list = m->spec_list;
+            const steps_sim *m = members[j];
+            want[j] = use_spec && !flow && m->spec_list && m->fill >= 0.0 && m->fill <= kListFill;
         }
+        return want;
+    }
+
+    // the blocks of the listed members
+    int build_list_work() try {
+        if (lwork.built) return STEPS_OK;
+        std::vector<BlockWork> v;
+        for (size_t j = 0; j < members.size(); ++j) {
+            const int64_t n = listed[j] ? list_blocks(members[j]->T, 256) : 0;
+            for (int64_t t = 0; t < n; ++t) v.push_back(BlockWork{(int32_t)j, (int32_t)t});
+            if (listed[j]) spec_list = members[j]->spec_list;
+        }
+        return upload_work(lwork, v);
+    } catch (const std::bad_alloc &) {
+        set_error("steps_batch: work list: out of host memory");
+        return STEPS_ERR_OOM;
+    }
+
+    // Before a run: its members of the list form; the work lists and graphs
+    // follow when they change (a batch is created with those of its members'
+    // states, since freeing a list waits for the device).
+    int choose_forms() try {
+        for (steps_sim *m : members)
+            if (use_spec && !flow && m->spec_list && m->fill < 0.0)
+                if (int rc = m->measure(stream)) return rc;
+        std::vector<char> want = wanted();
         if (want != listed) {
             for (Work *w : {&work[0], &work[1], &work[2], &work[3], &lwork}) {
                 if (w->graph) cudaGraphExecDestroy(w->graph);
@@ -1848,15 +1869,7 @@ struct steps_batch {
             }
             listed = std::move(want);
         }
-        if (!lwork.built) {
-            std::vector<BlockWork> v;
-            for (size_t j = 0; j < members.size(); ++j) {
-                const int64_t n = listed[j] ? list_blocks(members[j]->T, 256) : 0;
-                for (int64_t t = 0; t < n; ++t) v.push_back(BlockWork{(int32_t)j, (int32_t)t});
-            }
-            int rc = upload_work(lwork, v);
-            if (rc) return rc;
-        }
+        if (int rc = build_list_work()) return rc;
         for (size_t j = 0; j < members.size(); ++j) {
             steps_sim *m = members[j];
             if (m->listing != (bool)listed[j]) {
@@ -2111,9 +2124,10 @@ int steps_batch_create(steps_sim *const *members, int32_t n, const steps_batch_o
         return STEPS_ERR_ARG;
     }
     b->spec_forced = o.specialize > 0 || any_exp;
-    b->listed.assign((size_t)n, 0);
     b->use_spec = uniform && (o.specialize > 0 || any_exp || (o.specialize == 0 && tets >= kSpecializeMinTets));
+    b->listed = b->wanted();
     int rc = b->build_work(b->block);
+    if (!rc) rc = b->build_list_work();
     if (rc) return rc;
     *out = b.release();
     return STEPS_OK;

@@ -122,3 +122,22 @@ def test_a_batch_run_leaves_the_list_form(capi):
         assert np.array_equal(g.get_counts(), o.get_counts())
     assert 1024 * 3 <= b.info[1] <= 1024 * 3 + 480 * 2
     b.close()
+
+
+def test_a_new_batch_has_its_members_work_lists(capi):
+    """The lists of a batch fit its members' states from its creation on: the first
+    run of a sparse and a dense member allocates (and frees) nothing."""
+    pairs = [_pair(capi, 6), _pair(capi, 7, (6, 6, 5))]
+    for (g, o), every in zip(pairs, (60, 1)):
+        c = np.zeros((S, g.nt), np.int32)
+        c[:, ::every] = 2
+        _set(capi, g, o, c)
+    b = capi.Batch([p[0] for p in pairs], block=256, specialize=1)
+    made = capi.steps_debug_fail_alloc(0)
+    b.run([20.4 * o.tau for _, o in pairs])
+    assert capi.steps_debug_fail_alloc(0) == made
+    assert b.info[1] == 3 * 21
+    for g, o in pairs:
+        o.run(20.4 * o.tau)
+        assert np.array_equal(g.get_counts(), o.get_counts())
+    b.close()
