@@ -421,12 +421,17 @@ int steps_debug_logf(const float *x, int64_t n, float *out);
  * ends, so the device stays usable. limit_cycles: 1 .. 2^31 (about a second
  * at most); else STEPS_ERR_ARG. */
 int steps_debug_wait(int32_t deliver, int64_t limit_cycles);
-/* The flow launch's bounded wait for the tiles a tile depends on, on its own
- * (a test of the failure path). One warp waits for 40 listed tiles to have
- * finished window 4: with deliver != 0 they all have (STEPS_OK); with
- * deliver = 0 one has not, and the wait gives up after limit_cycles clock
- * cycles (STEPS_ERR_TIMEOUT). limit_cycles: 1 .. 2^31; else STEPS_ERR_ARG. */
+/* The bounded waits of flow launches, on their own (tests of the failure path).
+ * Block tiles (models given at run time of more than 12 species): one warp
+ * waits for 40 listed tiles to have finished window 4: with deliver != 0 they
+ * all have (STEPS_OK); with deliver = 0 one has not, and the wait gives up after
+ * limit_cycles clock cycles (STEPS_ERR_TIMEOUT). Warp tiles (every other
+ * model): one warp, tile 1, waits for the tiles of its tets' face neighbours,
+ * 40 in all and its own among them, to have finished window 4: late = -1, they
+ * all have; else tile `late` (0 .. 39) has not. limit_cycles: 1 .. 2^31; else
+ * STEPS_ERR_ARG. */
 int steps_debug_flow_wait(int32_t deliver, int64_t limit_cycles);
+int steps_debug_flow_nbr_wait(int32_t late, int64_t limit_cycles);
 /* The EXP leave law's table for a window of length tau_k (> 0): out[s * nt +
  * tet] = floor(2^31 (1 - exp(-(tau_k D_s) G_tet))), host, original tet order.
  * The device computes it; *decided (may be NULL) receives how many entries lay

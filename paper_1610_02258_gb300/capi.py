@@ -37,6 +37,7 @@ EXPORTS = [
     "steps_server_step", "steps_server_job_state", "steps_server_take_result", "steps_server_stats",
     "steps_debug_host_tables", "steps_debug_wait", "steps_debug_flow_wait",
     "steps_debug_leave_table", "steps_debug_fail_alloc", "steps_debug_error_word",
+    "steps_debug_flow_nbr_wait",
 ]
 
 
@@ -108,6 +109,7 @@ def _load():
         "steps_debug_host_tables": (ctypes.c_int, [P, P, i32, ctypes.POINTER(ctypes.c_double), P, P]),
         "steps_debug_leave_table": (ctypes.c_int, [P, ctypes.c_double, P, ctypes.POINTER(ctypes.c_uint32)]),
         "steps_debug_fail_alloc": (ctypes.c_int, [i32, ctypes.POINTER(ctypes.c_int64)]),
+        "steps_debug_flow_nbr_wait": (ctypes.c_int, [i32, i64]),
         "steps_debug_error_word": (ctypes.c_int, [ctypes.c_uint32, ctypes.POINTER(i32)]),
         "steps_server_options_default": (None, [ctypes.POINTER(steps_server_options)]),
         "steps_server_create": (ctypes.c_int, [ctypes.POINTER(steps_server_options), P, PP]),
@@ -351,9 +353,14 @@ def steps_debug_wait(deliver, limit_cycles):
 
 
 def steps_debug_flow_wait(deliver, limit_cycles):
-    """The flow launch's bounded wait for the tiles a tile depends on, on its
-    own: raises StepsError (code -6, STEPS_ERR_TIMEOUT) when the wait ran out."""
+    """The bounded wait of block tiles in a flow launch, on its own: raises
+    StepsError (code -6, STEPS_ERR_TIMEOUT) when the wait ran out."""
     _check(lib.steps_debug_flow_wait(1 if deliver else 0, int(limit_cycles)))
+
+
+def steps_debug_flow_nbr_wait(late, limit_cycles):
+    """The same of warp tiles: one waits for 40 tiles, of which `late` (-1: none) never finishes."""
+    _check(lib.steps_debug_flow_nbr_wait(int(late), int(limit_cycles)))
 
 
 def steps_batch_options_default():

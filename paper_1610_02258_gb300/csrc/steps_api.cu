@@ -1711,6 +1711,42 @@ int steps_debug_flow_wait(int32_t deliver, int64_t limit_cycles) {
     return STEPS_OK;
 }
 
+int steps_debug_flow_nbr_wait(int32_t late, int64_t limit_cycles) {
+    constexpr int n = 40;  // warp tiles of 32 tets
+    if (limit_cycles < 1 || limit_cycles > (int64_t)1 << 31 || late < -1 || late >= n) {
+        set_error("steps_debug_flow_nbr_wait: limit_cycles must be in [1, 2^31], late in [-1, 39]");
+        return STEPS_ERR_ARG;
+    }
+    // of the 128 faces of tile 1's tets, three reach each tile and eight are boundary faces
+    int32_t h_nbr[128];
+    for (int k = 0; k < 128; ++k) h_nbr[k] = k < 3 * n ? 32 * (k % n) + k / 4 : -1;
+    uint32_t h_done[n];
+    for (int j = 0; j < n; ++j) h_done[j] = j == late ? 4u : 5u + (uint32_t)(j % 3);
+    void *d_nbr = nullptr;
+    uint32_t *d_done = nullptr, *status = nullptr;
+    int rc = STEPS_OK;
+    if (!cuda_ok(cudaMalloc(&d_nbr, sizeof(h_nbr)), "steps_debug_flow_nbr_wait: alloc") ||
+        !cuda_ok(cudaMalloc((void **)&d_done, sizeof(h_done)), "steps_debug_flow_nbr_wait: alloc") ||
+        !cuda_ok(cudaMalloc((void **)&status, 4), "steps_debug_flow_nbr_wait: alloc"))
+        rc = STEPS_ERR_OOM;
+    uint32_t st = 0;
+    if (!rc && (!cuda_ok(cudaMemcpy(d_nbr, h_nbr, sizeof(h_nbr), cudaMemcpyHostToDevice), "steps_debug_flow_nbr_wait") ||
+                !cuda_ok(cudaMemcpy(d_done, h_done, sizeof(h_done), cudaMemcpyHostToDevice), "steps_debug_flow_nbr_wait") ||
+                !cuda_ok(cudaMemset(status, 0xFF, 4), "steps_debug_flow_nbr_wait")))
+        rc = STEPS_ERR_CUDA;
+    if (!rc) rc = launch_nbr_wait_test(d_done, d_nbr, (long long)limit_cycles, status);
+    if (!rc && !cuda_ok(cudaMemcpy(&st, status, 4, cudaMemcpyDeviceToHost), "steps_debug_flow_nbr_wait"))
+        rc = STEPS_ERR_CUDA;
+    cudaFree(d_nbr);
+    cudaFree(d_done);
+    cudaFree(status);
+    if (rc) return rc;
+    if (st == 0u) return STEPS_OK;
+    set_error(st == 8u ? "steps_debug_flow_nbr_wait: the neighbour wait did not complete within its limit"
+                       : "steps_debug_flow_nbr_wait: unexpected status");
+    return st == 8u ? STEPS_ERR_TIMEOUT : STEPS_ERR_STATE;
+}
+
 int steps_debug_logf(const float *x, int64_t n, float *out) {
     CHECK_NULL(x, "steps_debug_logf");
     CHECK_NULL(out, "steps_debug_logf");

@@ -32,6 +32,13 @@ __global__ void __launch_bounds__(512, 2)
     });
 }
 
+// One warp, the tile of tets 32 to 63 (word 1), waits for window word 5 of the
+// tiles of its tets' face neighbours.
+__global__ void nbr_wait_test_kernel(const uint32_t *done, const int4 *nbr, long long limit, uint32_t *status) {
+    const bool ok = flow_nbr_wait(done, 1u, 32, nbr[threadIdx.x], 5u, limit);
+    if (threadIdx.x == 0) *status = ok ? 0u : 8u;
+}
+
 bool opt_in(const void *fn, size_t smem) {
     if (smem <= 44 * 1024) return true;  // with the static arrays below the 48 KB every launch may have
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -97,6 +104,11 @@ int launch_batch_sm(const BlockWork *work, int64_t nblocks, const RepEntry *reps
 }
 
 }  // namespace
+
+int launch_nbr_wait_test(const uint32_t *d_done, const void *d_nbr, long long limit, uint32_t *d_status) {
+    nbr_wait_test_kernel<<<1, 32>>>(d_done, (const int4 *)d_nbr, limit, d_status);
+    return checked(cudaSuccess, "flow wait test launch");
+}
 
 int launch_warp(const ModelDev &m, const StepArgs &a, int block, void *stream) {
     return m.S <= 4 ? launch_plain<4>(m, a, block, stream) : launch_plain<kWarpGenericSpecies>(m, a, block, stream);
