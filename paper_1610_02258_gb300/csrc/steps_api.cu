@@ -130,6 +130,13 @@ struct LeaveRates {
     double tauD[kMaxSpecies];  // tau_k D_s, 0 for immobile species
 };
 constexpr uint32_t kLeaveListCap = 4096;
+// Up to so many entries the host computes the whole table, behind the windows
+// already enqueued and without a wait (the copy, of 32 KB at most, is staged).
+// A recording of 40 intervals of 2.5 windows, us, device -> host: 144 entries
+// 1,770 -> 875, 1,440 entries 1,945 -> 996, 5,760 entries 1,980 -> 1,413. The
+// host takes 4 ns an entry: 19,200 entries took 3,650 from the host (on the
+// block tiles, which made 0.1 of that), 2,990 from the device.
+constexpr int64_t kLeaveHostEntries = 8192;
 constexpr size_t kLeaveListBytes = (2 + 3 * (size_t)kLeaveListCap) * 4;
 
 __global__ void leave_table(const double *G, int64_t T, size_t Tpad, int S, const __grid_constant__ LeaveRates r,
@@ -465,14 +472,34 @@ struct steps_sim {
         return STEPS_OK;
     }
 
-    // EXP leave law: the table of a window of length tau_k, into the full
-    // window's buffer (tau_k == tau) or the last window's, in stream order. The
-    // device computes it and the host decides the entries it lists
-    // (leave_table); *decided, if asked for, receives their number. Waits for
-    // the stream. 105,222 tets and 10 species: 2.6 ms when the host computed
-    // all of it, 0.05 ms now.
-    int upload_leave(double tau_k, cudaStream_t st, uint32_t *decided = nullptr) {
+    // EXP leave law: a table of more than kLeaveHostEntries waits for the stream,
+    // so it comes before a run's windows
+    bool leave_waits() const { return d_leave[0] && (int64_t)S * T > kLeaveHostEntries; }
+
+    // the table of a window of length tau_k, smaller ones from the host
+    int upload_leave(double tau_k, cudaStream_t st) {
         if (!d_leave[0]) return STEPS_OK;
+        if (leave_waits() || !std::isfinite(tab.tau)) return device_leave(tau_k, st);
+        try {
+            std::vector<uint32_t> t;
+            exp_leave_table(model, tab, tau_k, (size_t)Tpad, t);
+            return cuda_ok(cudaMemcpyAsync(tau_k == tab.tau ? d_leave[0] : d_leave[1], t.data(), t.size() * 4,
+                                           cudaMemcpyHostToDevice, st),
+                           "leave table")
+                       ? STEPS_OK
+                       : STEPS_ERR_CUDA;
+        } catch (const std::bad_alloc &) {
+            set_error("leave table: out of host memory");
+            return STEPS_ERR_OOM;
+        }
+    }
+
+    // The table of a window of length tau_k, into the full window's buffer
+    // (tau_k == tau) or the last window's, in stream order. The device computes
+    // it and the host decides the entries it lists (leave_table); *decided, if
+    // asked for, receives their number. Waits for the stream. 105,222 tets and
+    // 10 species: 2.6 ms when the host computed all of it, 0.05 ms now.
+    int device_leave(double tau_k, cudaStream_t st, uint32_t *decided = nullptr) {
         uint32_t *dst = tau_k == tab.tau ? d_leave[0] : d_leave[1];
         if (!std::isfinite(tab.tau))
             return cuda_ok(cudaMemsetAsync(dst, 0, (size_t)S * Tpad * 4, st), "leave table") ? STEPS_OK : STEPS_ERR_CUDA;
@@ -699,6 +726,8 @@ struct steps_sim {
     int window_launch(double tau_k) {  // one window of explicit length, plain launch
         uint32_t scale[kMaxSpecies] = {};
         for (int s = 0; s < S; ++s) scale[s] = species_scale(model, tab, s, tau_k);
+        if (d_leave[0] && !leave_waits() && tau_k != tab.tau)
+            if (int rl = upload_leave(tau_k, stream)) return rl;
         StepArgs a = args(cur, k_total, nullptr, tau_k, scale);
         int rc = prepare_list(stream);
         if (!rc) rc = launch(a, stream);
@@ -1323,7 +1352,7 @@ int refuse_failed(const steps_sim *sim, const char *who) {
 // (full windows of tau, then a shortened last window); no synchronisation.
 int enqueue_run(steps_sim *sim, double t_end) {
     if (int rf = sim->choose_form()) return rf;
-    if (sim->d_leave[0]) {  // the shortened window's leave table first: it waits for the stream
+    if (sim->leave_waits()) {  // the shortened window's leave table first
         int64_t full;
         double partial;
         sim->schedule(t_end, &full, &partial);
@@ -1602,7 +1631,7 @@ int steps_debug_leave_table(steps_sim *sim, double tau_k, uint32_t *out, uint32_
         set_error("steps_debug_leave_table: needs the EXP leave law and a finite window > 0");
         return STEPS_ERR_ARG;
     }
-    int rc = sim->upload_leave(tau_k, sim->stream, decided);
+    int rc = sim->device_leave(tau_k, sim->stream, decided);
     if (rc) return rc;
     const uint32_t *d = tau_k == sim->tab.tau ? sim->d_leave[0] : sim->d_leave[1];
     gather_to_original_order<<<(unsigned)((sim->T + 255) / 256), 256, 0, sim->stream>>>(
@@ -2214,8 +2243,8 @@ int batch_enqueue(steps_batch *b, const double *t_end, int64_t most, bool *more)
             partial[j] = 0.0;
             *more = true;
         }
-        // the shortened window's leave table first: it waits for the stream
-        if (partial[j] > 0.0 && partial[j] != m->tab.tau)
+        // the shortened window's leave table first where it waits for the stream
+        if (m->leave_waits() && partial[j] > 0.0 && partial[j] != m->tab.tau)
             if (int rl = m->upload_leave(partial[j], b->stream)) return rl;
         nmax = std::max(nmax, nfull[j]);
     }
@@ -2309,6 +2338,8 @@ int batch_enqueue(steps_batch *b, const double *t_end, int64_t most, bool *more)
             any_partial = true;
             uint32_t scale[kMaxSpecies] = {};
             for (int s = 0; s < m->S; ++s) scale[s] = species_scale(m->model, m->tab, s, partial[j]);
+            if (m->d_leave[0] && !m->leave_waits() && partial[j] != m->tab.tau)
+                if (int rl = m->upload_leave(partial[j], b->stream)) return rl;
             StepArgs a = m->args(0, w, nullptr, partial[j], scale);
             a.err = b->d_err;
             e.args = a;
