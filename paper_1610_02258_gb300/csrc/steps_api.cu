@@ -1971,9 +1971,9 @@ struct steps_batch {
 
     int window(int b, cudaStream_t st) {  // one batched window + advance
         Work &w = work[slot(b)];
-        int rc = use_spec && spec[slot(b)] ? launch_spec_batch(spec[slot(b)], w.d, w.n, d_reps, max_S, b, st)
+        int rc = use_spec && spec[slot(b)] ? launch_spec_batch(spec[slot(b)], w.d, w.n, d_reps, b, st)
                                            : launch_step_batch(w.d, w.n, d_reps, max_S, max_R, any_order0, b, st);
-        if (!rc && lwork.n) rc = launch_spec_batch(spec_list, lwork.d, lwork.n, d_reps, max_S, 256, st);
+        if (!rc && lwork.n) rc = launch_spec_batch(spec_list, lwork.d, lwork.n, d_reps, 256, st);
         if (!rc) rc = launch_advance(d_reps, (int32_t)members.size(), st);
         launches += per_window(b);
         return rc;
@@ -2067,7 +2067,7 @@ struct steps_batch {
                 a.fetch = f.d_flow + f.nwords;
                 a.nwin = (uint32_t)nw;
                 a.ntiles = (uint32_t)g.second;
-                rc = launch_spec_batch_flow(spec[slot(b)], work[slot(b)].d, d_reps, a, (uint32_t)g.first, max_S, b,
+                rc = launch_spec_batch_flow(spec[slot(b)], work[slot(b)].d, d_reps, a, (uint32_t)g.first, b,
                                             stream);
                 if (rc) return rc;
                 ++launches;

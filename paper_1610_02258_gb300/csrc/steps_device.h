@@ -173,7 +173,7 @@ inline int64_t list_blocks(int64_t T, int block) {
 }
 
 // Full windows of one simulation in one flow launch (flow_tiles; the batched
-// form: a group of members, batch_flow_tile): one block per item (window q,
+// form: a group of members, batch_flow_member): one block per item (window q,
 // tile t), q-major; the item (q, t) waits until every tile sharing a face
 // with t, t included, has finished window q - 1.
 struct FlowArgs {

@@ -213,19 +213,18 @@ std::string program_source(const HostModel &hm, int block) {
                              std::to_string(hm.dev.S) + ", steps::SpecModel";
     const std::string head = "extern \"C\" __global__ void __launch_bounds__(" + b + ", " +
                              std::to_string(1024 / block) + ")\n";
-    const std::string member = "const steps::BlockWork *__restrict__ work, const steps::RepEntry *__restrict__ reps, ";
+    const std::string member = "const steps::BlockWork *__restrict__ work, const steps::RepEntry *__restrict__ reps";
     o << "#include \"steps_warp.cuh\"\n" << warp_policy_source(hm);
     o << head << "steps_spec_step(const __grid_constant__ steps::ModelDev m, const __grid_constant__ "
       << "steps::StepArgs a) {\n    steps::warp_step" << args << ">(m, a, (int64_t)blockIdx.x);\n}\n";
     o << head << "steps_spec_flow(const __grid_constant__ steps::ModelDev m, const __grid_constant__ "
       << "steps::StepArgs a, const __grid_constant__ steps::FlowArgs f) {\n    steps::warp_step" << args
       << ", 1>(m, a, 0, &f);\n}\n";
-    o << head << "steps_spec_batch(" << member << "int32_t prefetch) {\n"
-      << "    steps::batch_member<" << b << ">(work, reps, prefetch, [](const steps::ModelDev &m, const "
+    o << head << "steps_spec_batch(" << member << ") {\n"
+      << "    steps::batch_member<" << b << ">(work, reps, 0, [](const steps::ModelDev &m, const "
       << "steps::StepArgs &a, int64_t tile) { steps::warp_step" << args << ">(m, a, tile); });\n}\n";
-    o << head << "steps_spec_batch_flow(" << member << "const __grid_constant__ steps::FlowArgs f, uint32_t work0, "
-      << "int32_t prefetch) {\n"
-      << "    steps::batch_flow_member<" << b << ">(work, reps, f, work0, prefetch, [&f](const steps::ModelDev &m, "
+    o << head << "steps_spec_batch_flow(" << member << ", const __grid_constant__ steps::FlowArgs f, uint32_t work0) {\n"
+      << "    steps::batch_flow_member<" << b << ">(work, reps, f, work0, [&f](const steps::ModelDev &m, "
       << "const steps::StepArgs &a, int64_t tile, uint32_t q, uint32_t dep) { steps::warp_step" << args
       << ", 2>(m, a, tile, &f, q, dep); });\n}\n";
     return o.str();
@@ -417,7 +416,7 @@ int launch_spec_flow(void *spec, const ModelDev &m, const StepArgs &a, const Flo
     return STEPS_OK;
 }
 
-int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, const FlowArgs &f, uint32_t work0, int S,
+int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, const FlowArgs &f, uint32_t work0,
                            int block, void *stream) {
     if (f.nwin == 0 || f.ntiles == 0) return STEPS_OK;
     if (!work) {
@@ -428,8 +427,7 @@ int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, co
     const void *fn = (const void *)c->kern_batch_flow;
     const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set_batch_flow)) return STEPS_ERR_CUDA;
-    int32_t prefetch = 0;
-    void *args[5] = {(void *)&work, (void *)&reps, (void *)&f, (void *)&work0, (void *)&prefetch};
+    void *args[4] = {(void *)&work, (void *)&reps, (void *)&f, (void *)&work0};
     const unsigned grid = f.nwin * f.ntiles;  // one item per block
     cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3((unsigned)block), args, smem, (cudaStream_t)stream);
     if (e != cudaSuccess) {
@@ -439,7 +437,7 @@ int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, co
     return STEPS_OK;
 }
 
-int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEntry *reps, int S, int block,
+int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEntry *reps, int block,
                       void *stream) {
     if (nblocks <= 0) return STEPS_OK;
     if (!work) {
@@ -450,8 +448,7 @@ int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEnt
     const void *fn = (const void *)c->kern_batch;
     const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set_batch)) return STEPS_ERR_CUDA;
-    int32_t prefetch = 0;
-    void *args[3] = {(void *)&work, (void *)&reps, (void *)&prefetch};  // (the list form's takes the first two)
+    void *args[2] = {(void *)&work, (void *)&reps};
     if (c->kern_list) block = kListBlock;
     cudaError_t e = cudaLaunchKernel(fn, dim3((unsigned)nblocks), dim3((unsigned)block), args, smem, (cudaStream_t)stream);
     if (e != cudaSuccess) {

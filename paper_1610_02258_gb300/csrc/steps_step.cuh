@@ -599,15 +599,14 @@ __device__ __forceinline__ bool flow_deps_wait(const FlowArgs &f, uint32_t t, ui
 //         over the whole block, after a barrier, for chunks with reacting
 //         tets; then each tet's remaining counts are added to its own entry
 //         of `nxt`. Z: the model has order-0 reactions.
-// FLOW (a launch of several windows): 1, the block takes its item (window
-// q, tile) from f's counter (flow_tiles); 2, the caller took it and passes q
-// and the tile's index among f's tiles, dep (batch_flow_tile). Tile `tile`
-// of window a.window + q then waits for the tiles listed for dep and
-// publishes dep when done. Returns false when the tile's copies or the tiles
-// it depends on did not arrive within the wait limits.
-template <int BLOCK, int RM, class P, int FLOW = 0>
+// FLOW (a launch of several windows, flow_tiles): the block takes its item
+// (window q, tile) from f's counter. The tile of window a.window + q then
+// waits for the tiles listed for it and publishes its word when done.
+// Returns false when the tile's copies or the tiles it depends on did not
+// arrive within the wait limits.
+template <int BLOCK, int RM, class P, bool FLOW = false>
 __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, int64_t tile,
-                                          const FlowArgs *f = nullptr, uint32_t q = 0, uint32_t dep = 0) {
+                                          const FlowArgs *f = nullptr) {
     extern __shared__ __align__(16) int32_t smem[];  // cnt [S + 1][BLOCK], trial [S][BLOCK]
     __shared__ __align__(16) uint4 s_thr[BLOCK];
     __shared__ __align__(16) int4 s_nbr[BLOCK];
@@ -641,18 +640,18 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
         ncalm = 0;
         next_chunk = 0;
         mbar_init(&bar, 1);
-        if constexpr (FLOW == 1) s_item = atomicAdd(f->fetch, 1u);
+        if constexpr (FLOW) s_item = atomicAdd(f->fetch, 1u);
     }
     P::template build<BLOCK>(m, tb);
     if (tid < S) s_scale[tid] = a.scale[tid];
     __syncthreads();
     // the window of this tile: q windows after a.window (buffers swapped when q is odd)
-    if constexpr (FLOW == 1) {
+    uint32_t q = 0;
+    if constexpr (FLOW) {
         const uint32_t item = s_item;
         if (item >= f->nwin * f->ntiles) return true;
         q = item / f->ntiles;
         tile = (int64_t)(item - q * f->ntiles);
-        dep = (uint32_t)tile;
     }
     int32_t *const cur = (q & 1u) ? a.nxt : a.cur;
     int32_t *const nxt = (q & 1u) ? a.cur : a.nxt;
@@ -688,8 +687,8 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
     // it to complete (and its memory to be visible); in a flow launch, for the
     // tiles this one depends on
     bool deps = true;
-    if constexpr (FLOW != 0) {
-        if (q > 0 && tid < 32) deps = flow_deps_wait(*f, dep, (uint32_t)(a.window + q));
+    if constexpr (FLOW) {
+        if (q > 0 && tid < 32) deps = flow_deps_wait(*f, (uint32_t)tile, (uint32_t)(a.window + q));
     } else {
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
@@ -943,10 +942,10 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
         }
     }
     if (bad) atomicOr(a.err, bad);
-    if constexpr (FLOW != 0) {
+    if constexpr (FLOW) {
         // publish: every thread's writes of this tile come before the release
         __syncthreads();
-        if (tid == 0) st_release_gpu(f->tile_done + dep, (uint32_t)(a.window + q + 1));
+        if (tid == 0) st_release_gpu(f->tile_done + tile, (uint32_t)(a.window + q + 1));
     }
     return true;
 }
@@ -965,7 +964,7 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
 // number of resident blocks.
 template <int BLOCK, int RM, class P>
 __device__ __forceinline__ void flow_tiles(const ModelDev &m, const StepArgs &a, const FlowArgs &f) {
-    step_tile<BLOCK, RM, P, 1>(m, a, 0, &f);
+    step_tile<BLOCK, RM, P, true>(m, a, 0, &f);
 }
 
 // One block of a batched launch: the member named by work[blockIdx.x] copies
@@ -1015,11 +1014,11 @@ __device__ __forceinline__ void batch_tile(const BlockWork *__restrict__ work, c
 // by member; item (q, i) is tile work0 + i of window q of its member (its own
 // window index and buffers). A member whose windows end earlier skips its
 // later items; nothing depends on them (the dependencies stay within a
-// member). f's tile lists and words are indexed by work entry.
+// member). f's words are indexed by work entry.
 template <int BLOCK, class F>
 __device__ __forceinline__ void batch_flow_member(const BlockWork *__restrict__ work,
                                                   const RepEntry *__restrict__ reps, const FlowArgs &f, uint32_t work0,
-                                                  int32_t prefetch, F step) {
+                                                  F step) {
     __shared__ __align__(16) ModelDev t_model;
     __shared__ __align__(16) StepArgs t_args;
     __shared__ uint32_t s_q, s_dep;
@@ -1052,7 +1051,6 @@ __device__ __forceinline__ void batch_flow_member(const BlockWork *__restrict__ 
     if (threadIdx.x == 0) {
         t_args.cur = e->cnt[e->parity];
         t_args.nxt = e->cnt[e->parity ^ 1u];
-        t_args.prefetch = prefetch;  // tiles ahead within the member
     }
     __syncthreads();
     step(t_model, t_args, (int64_t)s_tile, s_q, s_dep);

@@ -164,7 +164,8 @@ struct RtWarp {
     }
 };
 
-// The tile's species factor of species s for lane t's tet (species_R).
+// The species factor of tet i's thresholds: the window's species scale R_s
+// (EULER), or the tet's own leave value from the EXP table.
 template <class P>
 __device__ __forceinline__ uint32_t warp_R(const StepArgs &a, const uint32_t *s_scale, int s, int64_t i) {
     if constexpr (P::kExpLeave) return __ldg(a.leave + (size_t)((uint64_t)(uint32_t)s * (uint32_t)a.Tpad) + (size_t)i);
