@@ -102,13 +102,16 @@ __device__ __noinline__ int last_positive_tab(const RxnTab &tb, const ModelDev &
     return last;
 }
 
-// The pick from careful_sums, for a model without kept sums.
+// The pick of a model without kept sums when no plain running sum exceeded the
+// target: from careful_sums, whose sums are the plain ones unless those met an
+// infinite rate of an absent reactant and are not numbers from there on; else
+// the last reaction with a positive propensity.
 __device__ __noinline__ int careful_pick(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
                                          uint32_t active, float target) {
     float sum = 0.0f;
     for (int r = 0; r < m.R; ++r) {
         sum = __fadd_rn(sum, ((active >> r) & 1u) ? careful_propensity(tb.p[r], cnt, inv_nav) : 0.0f);
-        if (!(sum <= target)) return r;
+        if (sum > target) return r;
     }
     return last_positive_tab(tb, m, cnt, inv_nav, active);
 }
@@ -155,12 +158,9 @@ struct RtWarp {
         float sum = 0.0f;
         for (int r = 0; r < m.R; ++r) {
             sum = __fadd_rn(sum, ((active >> r) & 1u) ? propensity(tb.p[r], cnt, inv_nav, z) : 0.0f);
-            if (!(sum <= target)) {
-                // not a number: an infinite rate times an absent reactant, which first_sums counted 0
-                return sum == sum ? r : careful_pick(tb, m, cnt, inv_nav, active, target);
-            }
+            if (sum > target) return r;  // (never a sum that is not a number)
         }
-        return last_positive_tab(tb, m, cnt, inv_nav, active);
+        return careful_pick(tb, m, cnt, inv_nav, active, target);
     }
 };
 
