@@ -617,7 +617,7 @@ struct steps_sim {
         }
         if (spec_list && opt.flow != 1 && fill < 0.0)
             if (int rc = measure(stream)) return rc;
-        const bool want = spec_list && opt.flow != 1 && fill <= kListFill;
+        const bool want = spec_list && opt.flow != 1 && fill <= kListFill && plain_rates(model, tab);
         if (want != listing) {
             drop_graphs();
             looked = k_total;
@@ -1898,7 +1898,8 @@ struct steps_batch {
         std::vector<char> want(members.size(), 0);
         for (size_t j = 0; j < members.size(); ++j) {
             const steps_sim *m = members[j];
-            want[j] = use_spec && !flow && m->spec_list && m->fill >= 0.0 && m->fill <= kListFill;
+            want[j] = use_spec && !flow && m->spec_list && m->fill >= 0.0 && m->fill <= kListFill &&
+                      plain_rates(m->model, m->tab);
         }
         return want;
     }

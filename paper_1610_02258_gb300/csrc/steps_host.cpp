@@ -370,7 +370,18 @@ void build_tables(const HostMesh &mesh, const HostModel &model, int reorder, Tab
         }
         double nav = kAvogadro * (mesh.vol[(size_t)i] * 1000.0);
         t.inv_nav_dev[(size_t)d] = (float)(1.0 / nav);
+        t.inv_nav_max = std::max(t.inv_nav_max, t.inv_nav_dev[(size_t)d]);
     }
+}
+
+bool plain_rates(const HostModel &model, const Tables &t) {
+    for (int r = 0; r < model.dev.R; ++r) {
+        const ReacDesc &d = model.dev.reac[r];
+        // ((k / (N_A V)) x) y: infinite before the factor of an absent reactant
+        const double c = d.type == kOrder2 || d.type == kDimer ? (double)d.k * t.inv_nav_max * 2147483648.0 : (double)d.k;
+        if (d.type != kOrder0 && !(c <= 3.0e38)) return false;
+    }
+    return true;
 }
 
 uint32_t exp_leave_entry(double tauD, double G) {

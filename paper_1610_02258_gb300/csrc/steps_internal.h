@@ -61,10 +61,14 @@ struct Tables {
     std::vector<int32_t> nbr_dev;   // [T*4] device order, device indices
     std::vector<uint32_t> thr_dev;  // [T*4] device order
     std::vector<float> inv_nav_dev; // [T]
+    float inv_nav_max = 0.0f;
     std::vector<double> G_dev;      // [T] device order: sum of the face rates g over internal faces
 };
 void build_tables(const HostMesh &mesh, const HostModel &model, int reorder, Tables &t);
 uint32_t species_scale(const HostModel &model, const Tables &t, int s, double tau_k);
+// Whether no propensity of the model can be infinity times an absent reactant
+// (the list form's kernel takes such a tet's sums as they are).
+bool plain_rates(const HostModel &model, const Tables &t);
 // EXP leave law: out[s * Tpad + d] = floor(2^31 (1 - exp(-(tau_k D_s) G_d))) for every
 // species and device-order tet (0 for immobile species and the padding).
 void exp_leave_table(const HostModel &model, const Tables &t, double tau_k, size_t Tpad, std::vector<uint32_t> &out);

@@ -191,7 +191,7 @@ std::string warp_policy_source(const HostModel &hm) {
     o << "    template <int RM>\n    __device__ __forceinline__ static float first_sums(const RxnTab &tb, const "
          "ModelDev &m, const int32_t *cnt, float inv_nav, uint32_t active, bool masked, float *psum) {\n"
          "        const float a0 = sums<RM>(tb, m, cnt, inv_nav, active, masked, psum);\n"
-         "        if (a0 <= 3.0e38f) return a0;\n"
+         "        if (a0 <= kPlainSums) return a0;\n"
          "        float ps[RM];\n"
          "        const float a1 = careful_sums(tb, m, cnt, inv_nav, active, ps);\n"
          "        for (int r = 0; r < " << m.R << "; ++r) psum[r] = ps[r];\n"

@@ -172,6 +172,53 @@ __device__ __forceinline__ float propensity(const float4 q, const int32_t *cnt, 
     return __fmul_rn(__fmul_rn(c, __int2float_rn(x)), __int2float_rn(y));
 }
 
+// A propensity that is 0 where a reactant (a dimer's second molecule too) is
+// absent, whatever the rate.
+__device__ __forceinline__ float careful_propensity(const float4 q, const int32_t *cnt, float inv_nav) {
+    const int32_t x = *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(cnt) + __float_as_uint(q.y));
+    const int32_t y = *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(cnt) + __float_as_uint(q.z)) -
+                      (int32_t)(__float_as_uint(q.w) & 0xFFu);
+    return x != 0 && y != 0 ? propensity(q, cnt, inv_nav, true) : 0.0f;
+}
+
+// First propensity sums of a tet whose plain sums exceed this or are not
+// numbers (rates near the float range): a reaction without all its reactants
+// counts 0, in every form of the step, whatever tets share the warp. (Later
+// sums of the tet that are not numbers end its window.)
+constexpr float kPlainSums = 3.0e38f;
+
+__device__ __noinline__ float careful_sums(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
+                                           uint32_t active, float *psum) {
+    float a0 = 0.0f;
+    for (int r = 0; r < m.R; ++r) {
+        a0 = __fadd_rn(a0, ((active >> r) & 1u) ? careful_propensity(tb.p[r], cnt, inv_nav) : 0.0f);
+        if (psum) psum[r] = a0;
+    }
+    return a0;
+}
+
+// The pick when u2 a0 reaches every running sum: the last reaction with a
+// positive propensity, or -1.
+__device__ __noinline__ int last_positive_tab(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
+                                              uint32_t active) {
+    int last = -1;
+    for (int r = 0; r < m.R; ++r)
+        if (((active >> r) & 1u) && propensity(tb.p[r], cnt, inv_nav, true) > 0.0f) last = r;
+    return last;
+}
+
+// The pick from careful_sums; the last reaction with a positive propensity when
+// no running sum exceeds the target.
+__device__ __noinline__ int careful_pick(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
+                                         uint32_t active, float target) {
+    float sum = 0.0f;
+    for (int r = 0; r < m.R; ++r) {
+        sum = __fadd_rn(sum, ((active >> r) & 1u) ? careful_propensity(tb.p[r], cnt, inv_nav) : 0.0f);
+        if (sum > target) return r;
+    }
+    return last_positive_tab(tb, m, cnt, inv_nav, active);
+}
+
 // Model access of the step body. RtModel reads a model given at run time
 // (kernel parameters and the tile's reaction table). A model compiled into a
 // kernel at run time (steps_spec.cpp) provides the same functions with the
@@ -242,6 +289,25 @@ __device__ __forceinline__ int pick_reaction(const RxnTab &tb, const ModelDev &m
     for (int r = 0; r < RM; ++r)
         if (r < P::R(m)) n += psum[r] <= target ? 1 : 0;
     return n < P::R(m) ? n : last_positive<P, RM>(tb, m, cnt, inv_nav, active);
+}
+
+// The first event of a tet whose plain sums are no numbers, from careful_sums:
+// its reaction and time, and its changes made.
+template <int BLOCK, class P>
+__device__ __noinline__ bool careful_event(const RxnTab &tb, const ModelDev &m, const StepArgs &a, int32_t *cnt,
+                                           float inv_nav, uint32_t active, uint32_t tet, uint32_t c0, uint32_t c3,
+                                           int8_t *pick_out, float *dt_out) {
+    const float a0 = careful_sums(tb, m, cnt, inv_nav, active, nullptr);
+    if (!(a0 > 0.0f)) return false;
+    const uint4 w = philox4x32_10(a.key0, a.key1, c0, tet, 0u, (kPurposeReac << 28) | c3);
+    const float dt = __fdiv_rn(-steps_logf(unit24f(w.x)), a0);
+    if (dt > a.tau_dn) return false;
+    const int pick = careful_pick(tb, m, cnt, inv_nav, active, __fmul_rn(unit24f(w.y), a0));
+    if (pick < 0) return false;
+    P::for_changes(tb, pick, [&](int s, int d) { cnt[s * BLOCK] += d; });
+    *pick_out = (int8_t)pick;
+    *dt_out = dt;
+    return true;
 }
 
 // Stochastic rounding of a mean occupancy: floor(nbar) + [u < nbar - floor(nbar)]
@@ -798,6 +864,8 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
                     reacting = true;
                 }
             }
+        } else if (live && a0 != a0) {
+            reacting = careful_event<BLOCK, P>(tb, m, a, cnt, inv_nav, active, s_tet[tid], c0, c3, q_pick + tid, q_dt + tid);
         }
     }
     {

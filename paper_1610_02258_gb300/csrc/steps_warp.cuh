@@ -73,49 +73,6 @@ __device__ __forceinline__ int32_t round_trials32(double nbar, uint32_t w, int32
     return fl > (uint64_t)most ? most : (int32_t)fl;
 }
 
-// A propensity that is 0 where a reactant is absent, whatever the rate.
-__device__ __forceinline__ float careful_propensity(const float4 p, const int32_t *cnt, float inv_nav) {
-    const bool have = *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(cnt) + __float_as_uint(p.y)) &&
-                      *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(cnt) + __float_as_uint(p.z));
-    return have ? propensity(p, cnt, inv_nav, true) : 0.0f;
-}
-
-// First propensity sums of a tet whose plain sums are not finite (rates near
-// the float range): a reaction without all its reactants counts 0.
-__device__ __noinline__ float careful_sums(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
-                                           uint32_t active, float *psum) {
-    float a0 = 0.0f;
-    for (int r = 0; r < m.R; ++r) {
-        a0 = __fadd_rn(a0, ((active >> r) & 1u) ? careful_propensity(tb.p[r], cnt, inv_nav) : 0.0f);
-        if (psum) psum[r] = a0;
-    }
-    return a0;
-}
-
-// The pick when u2 a0 reaches every running sum: the last reaction with a
-// positive propensity, or -1.
-__device__ __noinline__ int last_positive_tab(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
-                                              uint32_t active) {
-    int last = -1;
-    for (int r = 0; r < m.R; ++r)
-        if (((active >> r) & 1u) && propensity(tb.p[r], cnt, inv_nav, true) > 0.0f) last = r;
-    return last;
-}
-
-// The pick of a model without kept sums when no plain running sum exceeded the
-// target: from careful_sums, whose sums are the plain ones unless those met an
-// infinite rate of an absent reactant and are not numbers from there on; else
-// the last reaction with a positive propensity.
-__device__ __noinline__ int careful_pick(const RxnTab &tb, const ModelDev &m, const int32_t *cnt, float inv_nav,
-                                         uint32_t active, float target) {
-    float sum = 0.0f;
-    for (int r = 0; r < m.R; ++r) {
-        sum = __fadd_rn(sum, ((active >> r) & 1u) ? careful_propensity(tb.p[r], cnt, inv_nav) : 0.0f);
-        if (sum > target) return r;
-    }
-    return last_positive_tab(tb, m, cnt, inv_nav, active);
-}
-
 // Model access for models given at run time: the reaction table, walked in a
 // loop; the running sums are summed again for a pick instead of kept
 // (unrolled by four, or with the sums kept, the loops were slower). 30,720
@@ -148,7 +105,7 @@ struct RtWarp {
     __device__ __forceinline__ static float first_sums(const RxnTab &tb, const ModelDev &m, const int32_t *cnt,
                                                        float inv_nav, uint32_t active, bool masked, float *psum) {
         const float a0 = sums<RM>(tb, m, cnt, inv_nav, active, masked, psum);
-        if (a0 <= 3.0e38f) return a0;
+        if (a0 <= kPlainSums) return a0;
         return careful_sums(tb, m, cnt, inv_nav, active, nullptr);
     }
     template <int RM>
@@ -158,8 +115,10 @@ struct RtWarp {
         float sum = 0.0f;
         for (int r = 0; r < m.R; ++r) {
             sum = __fadd_rn(sum, ((active >> r) & 1u) ? propensity(tb.p[r], cnt, inv_nav, z) : 0.0f);
-            if (sum > target) return r;  // (never a sum that is not a number)
+            if (sum > target) return r;
         }
+        // no sum exceeds the target, or the sums met an infinite rate of an
+        // absent reactant and are not numbers from there on
         return careful_pick(tb, m, cnt, inv_nav, active, target);
     }
 };
