@@ -86,7 +86,8 @@ typedef struct steps_options {
                             fastest (steps_sim_flow reports it); 1: flow at `block` where a flow kernel exists;
                             -1: window launches. The results are the same bits in every form. With 0 and -1, a
                             specialised model of 13 or more species whose state holds few molecules per tet
-                            runs its windows, in window launches, over a list of the tets that hold something. */
+                            runs its windows, in window launches, over a list of the tets that hold something
+                            (unless the device has no room for the lists). */
     int32_t reserved[1]; /* set to 0 */
 } steps_options;
 
@@ -205,8 +206,10 @@ int steps_set_reac_rate(steps_sim *sim, int32_t reac, double k);
  * d_out: caller-owned DEVICE memory of at least max_records * n_species *
  * n_tets int32, recording k - 1 at offset (k - 1) n_species n_tets, laid
  * out [species][tet] in the order given. The snapshots are taken on the
- * device with no host synchronisation between them; the call synchronises
- * once at the end. *n_records (may be NULL) receives the number written.
+ * device; the call synchronises at the end, and in between only where the host
+ * must see something first (under the EXP law, once per interval on meshes of
+ * more than 8,192 tets x species; every 1,024 windows of a sparse state's list;
+ * the tuning of the launch form). *n_records (may be NULL) receives the number written.
  * The selection is copied to a small device buffer the simulation keeps.
  * Errors: STEPS_ERR_ARG for bad species/tet indices, a non-positive dt_rec
  * or more recordings than max_records (checked before anything runs); the
@@ -281,7 +284,8 @@ void steps_batch_destroy(steps_batch *batch);
  * out the later launches. With block autotuning, the first run times three
  * windows at each candidate block size (real windows: results do not depend
  * on the block size) and keeps the fastest. Synchronises with the batch's
- * stream once. Errors as steps_run.
+ * stream at the end, and every 1,024 windows while members in sparse states run
+ * over lists of their tets. Errors as steps_run.
  */
 int steps_batch_run(steps_batch *batch, const double *t_end);
 
@@ -397,8 +401,8 @@ int steps_server_stats(const steps_server *srv, uint64_t *rounds, uint64_t *rebu
  * simulation's stream before returning.
  * Errors: d_counts holding a negative count gives STEPS_ERR_ARG before
  * anything changes (clock and d_counts as before the call); so does a
- * simulation under STEPS_LEAVE_EXP (a shortened window would need a table
- * built on the host); otherwise as steps_run.
+ * simulation under STEPS_LEAVE_EXP (a shortened window would need a table that
+ * the scratch has no room for); otherwise as steps_run.
  */
 int steps_run_noalloc(steps_sim *sim, int32_t *d_counts, double t_end);
 

@@ -38,10 +38,11 @@ namespace {
 constexpr int kGraphWindows = 16;  // full windows per captured graph (even: buffer parity is restored)
 // The list form runs a state of at most this many listed tets (or, from set
 // counts, non-zero counts) per tet. us per window, warp tiles -> list form:
-// 1.03M-tet dendrite, 0.12: 61.8 -> 14.6; 294,780-tet box with 14, 20 and 30
-// species at 0.2, 0.31, 0.48: 19.6 -> 15.3, 22.0 -> 16.2, 34.1 -> 16.7; but
-// with 14 at 1.0: 23.3 -> 28.3, and the 300k-tet dendrite, whose molecules
-// crowd at one end, 0.37: 15.8 -> 19.1.
+// 1.03M-tet dendrite, 0.12: 61.8 -> 14.6; 294,780-tet box with 14 and 20
+// species at 0.2 and 0.31: 19.6 -> 15.3, 22.0 -> 16.2; but with 14 at 1.0: 23.3
+// -> 28.3, and the 300k-tet dendrite, whose molecules crowd at one end, 0.37:
+// 15.8 -> 19.1. One line for every species count, set by the crowded states:
+// even ones gain beyond it (30 species at 0.48, 34.1 -> 16.7) and stay on tiles.
 constexpr double kListFill = 0.33;
 constexpr uint64_t kListWindows = 128;       // windows after which a list is built afresh
 constexpr uint64_t kListCheckWindows = 1024;  // windows after which a run looks at the list's length
@@ -135,7 +136,7 @@ constexpr uint32_t kLeaveListCap = 4096;
 // A recording of 40 intervals of 2.5 windows, us, device -> host: 144 entries
 // 1,770 -> 875, 1,440 entries 1,945 -> 996, 5,760 entries 1,980 -> 1,413. The
 // host takes 4 ns an entry: 19,200 entries took 3,650 from the host (on the
-// block tiles, which made 0.1 of that), 2,990 from the device.
+// block tiles, whose windows were slower too), 2,990 from the device.
 constexpr int64_t kLeaveHostEntries = 8192;
 constexpr size_t kLeaveListBytes = (2 + 3 * (size_t)kLeaveListCap) * 4;
 
@@ -243,8 +244,9 @@ void flow_neighbours(const std::vector<int32_t> &nbr_dev, int64_t T, int64_t B, 
 // Launch-form choices of tuned simulations, shared by every simulation of
 // the same compiled kernel, tet count, block size and molecules per tet (to a
 // power of two; clones of one prototype, the jobs of a stream): the first
-// one's tuning run decides. (A tenth of the benchmark box's molecules runs 14 %
-// faster in another form than the box.)
+// one's tuning run decides, and a simulation keeps the choice of its own first
+// run when its counts change. (A tenth of the benchmark box's molecules runs
+// 14 % faster in another form than the box.)
 struct FlowChoice {
     int pick;
     float ms[3];
@@ -1349,7 +1351,9 @@ int refuse_failed(const steps_sim *sim, const char *who) {
 }
 
 // Enqueues the windows of Algorithm 1 from the simulation's time to t_end
-// (full windows of tau, then a shortened last window); no synchronisation.
+// (full windows of tau, then a shortened last window). Waits for the stream
+// only where the host has to see something first: the tuning of the launch
+// form, a list's length (choose_form), a leave table of many entries.
 int enqueue_run(steps_sim *sim, double t_end) {
     if (int rf = sim->choose_form()) return rf;
     if (sim->leave_waits()) {  // the shortened window's leave table first
@@ -2489,8 +2493,8 @@ extern "C" int steps_run_noalloc(steps_sim *sim, int32_t *d_counts, double t_end
     }
     if (int rf = refuse_failed(sim, "steps_run_noalloc")) return rf;
     if (sim->d_leave[0]) {
-        set_error("steps_run_noalloc: the EXP leave law needs a host-built table for a shortened window; "
-                  "use steps_run");
+        set_error("steps_run_noalloc: the EXP leave law needs a leave table for a shortened window, which "
+                  "this call has no room for; use steps_run");
         return STEPS_ERR_ARG;
     }
     // the scratch address is per device, and the simulation's stream and

@@ -80,7 +80,7 @@ uint32_t exp_leave_entry(double tauD, double G);  // one entry, tauD = tau_k D_s
 // shared-memory size.
 int prefetch_distance(const void *kernel, int block, size_t smem);
 int launch_step(const ModelDev &m, const StepArgs &a, int block, void *stream);
-// the same for models of up to kWarpMaxSpecies species, on warp tiles (steps_warp.cu)
+// the same for run-time models of up to kWarpGenericSpecies species, on warp tiles (steps_warp.cu)
 int launch_warp(const ModelDev &m, const StepArgs &a, int block, void *stream);
 int launch_warp_flow(const ModelDev &m, const StepArgs &a, const FlowArgs &f, int block, void *stream);
 int launch_warp_batch(const BlockWork *work, int64_t nblocks, const RepEntry *reps, int max_S, int block, void *stream);
@@ -112,7 +112,7 @@ int launch_spec_batch_flow(void *spec, const BlockWork *work, RepEntry *reps, co
 int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEntry *reps, int block,
                       void *stream);
 std::string spec_program_source(const HostModel &hm, int block);
-// the list form's step kernel for launch_spec (models of more species than warp tiles take), or nullptr
+// the list form's step kernel for launch_spec (models of 13 or more species), or nullptr
 void *spec_list_kernel(const HostModel &hm);
 
 // steps_api.cu: steps_batch_run in two parts (enqueue every window and the

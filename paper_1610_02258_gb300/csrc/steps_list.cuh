@@ -146,9 +146,10 @@ __device__ __forceinline__ void list_planes(const StepArgs &a, const ListCtx<SM>
 }
 
 // The chunk's reactions (warp_window's; `possible`: those with all reactants
-// somewhere in the chunk, the others' propensities are 0). Out of line: few
-// chunks of a sparse state have any, and inlined its registers spilled in all
-// of them. Returns the species changed and, above them, error bits.
+// somewhere in the chunk, the others' propensities are 0), skipped by a chunk
+// without any. Models with rates near the float range keep to the tiles
+// (plain_rates): the sums are taken as they are. Returns the species changed
+// and, above them, error bits.
 template <int RM, int SM, class P>
 __device__ __forceinline__ uint64_t list_react(const ModelDev &m, const StepArgs &a, const ListCtx<SM> &x,
                                               const RxnTab &tb, uint32_t possible, bool live, float inv_nav,
