@@ -448,6 +448,12 @@ int steps_debug_leave_table(steps_sim *sim, double tau_k, uint32_t *out, uint32_
  * receives how many such allocations the thread has made so far. Errors:
  * STEPS_ERR_ARG (nth < 0). */
 int steps_debug_fail_alloc(int32_t nth, int64_t *made);
+/* The form of the step that simulations of 13 or more species created from now
+ * on, on the calling thread, and their clones take where the model is compiled
+ * (tests at small sizes): 0 by rule (default), 2 the list form for sparse
+ * states of any mesh size, 3 block tiles for every window. Errors:
+ * STEPS_ERR_ARG. */
+int steps_debug_form(int32_t form);
 /* What a run (plain, recorded, batched or without allocation) makes of the
  * device's error word: its return code and message (host only). *closed (may
  * be NULL): whether the simulations are closed to further runs. Bits: 1 a

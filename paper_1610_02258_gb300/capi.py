@@ -37,7 +37,7 @@ EXPORTS = [
     "steps_server_step", "steps_server_job_state", "steps_server_take_result", "steps_server_stats",
     "steps_debug_host_tables", "steps_debug_wait", "steps_debug_flow_wait",
     "steps_debug_leave_table", "steps_debug_fail_alloc", "steps_debug_error_word",
-    "steps_debug_flow_nbr_wait",
+    "steps_debug_flow_nbr_wait", "steps_debug_form",
 ]
 
 
@@ -110,6 +110,7 @@ def _load():
         "steps_debug_leave_table": (ctypes.c_int, [P, ctypes.c_double, P, ctypes.POINTER(ctypes.c_uint32)]),
         "steps_debug_fail_alloc": (ctypes.c_int, [i32, ctypes.POINTER(ctypes.c_int64)]),
         "steps_debug_flow_nbr_wait": (ctypes.c_int, [i32, i64]),
+        "steps_debug_form": (ctypes.c_int, [i32]),
         "steps_debug_error_word": (ctypes.c_int, [ctypes.c_uint32, ctypes.POINTER(i32)]),
         "steps_server_options_default": (None, [ctypes.POINTER(steps_server_options)]),
         "steps_server_create": (ctypes.c_int, [ctypes.POINTER(steps_server_options), P, PP]),
@@ -330,6 +331,12 @@ def steps_debug_fail_alloc(nth):
     made = ctypes.c_int64(0)
     _check(lib.steps_debug_fail_alloc(int(nth), ctypes.byref(made)))
     return made.value
+
+
+def steps_debug_form(form):
+    """The form that simulations of 13 or more species created from now on take
+    where compiled: 0 by rule, 2 the list form in sparse states, 3 block tiles."""
+    _check(lib.steps_debug_form(int(form)))
 
 
 def steps_debug_error_word(word):

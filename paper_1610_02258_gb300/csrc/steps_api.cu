@@ -44,9 +44,42 @@ constexpr int kGraphWindows = 16;  // full windows per captured graph (even: buf
 // 15.8 -> 19.1. One line for every species count, set by the crowded states:
 // even ones gain beyond it (30 species at 0.48, 34.1 -> 16.7) and stay on tiles.
 constexpr double kListFill = 0.33;
+// On smaller meshes than this, or with more tets listed, the tiles are faster: a
+// window in the list form takes some 11 us however little there is to do, and
+// the scattered accesses of many tets miss L2. us per window, the best tiles ->
+// list form, 14 and 30 species at 0.1 molecules per tet: 10,404 tets 5.5 -> 9.6
+// and 6.5 -> 9.2, 138,720 9.0 -> 12.3 and 10.4 -> 12.1, 294,780 15.2 -> 14.5 and
+// 18.3 -> 14.5, 599,964 30.7 -> 15.3 and 38.7 -> 15.5, 1,040,400 49.8 -> 20.6 and
+// 61.8 -> 21.6; there at 0.3 59.0 -> 73.7 and 79.1 -> 87.2.
+constexpr int64_t kListMinTets = 262144;
+constexpr double kListMost = 250000.0;
 constexpr uint64_t kListWindows = 128;       // windows after which a list is built afresh
 constexpr uint64_t kListCheckWindows = 1024;  // windows after which a run looks at the list's length
 constexpr int64_t kFlowTuneWindows = 72;  // windows the launch-form tuning takes (3 rounds of up to 3 groups)
+constexpr int64_t kFormTuneWindows = 90;  // with block tiles as two more candidates
+constexpr int kForms = 6;                 // window launches, flow, flow at 512; the same of block tiles (256)
+
+// Tets a resident wave of compiled warp tiles covers (their shared memory, at
+// most 32 warps per SM). Models of 13 or more species on larger meshes have
+// compiled block tiles too, whose copies run ahead (TMA, L2 prefetch) with 40
+// warps per SM. us per window in the best launch form, warp tiles -> block
+// tiles, 14, 20 and 30 species: 138,720 tets at 0.1 molecules per tet 10.9, 12.0
+// and 14.0 -> 9.0, 9.7 and 10.4, at 2 16.1, 17.9 and 18.8 -> 15.4, 18.4 and 19.4;
+// 1,040,400 tets at 0.5 67.6, 80.0 and 132 -> 65.6, 78.2 and 89.3, at 5 98, 116 and
+// 216 -> 124, 182 and 214. Within a wave warp tiles win throughout (69,360 tets,
+// 14 species at 0.1: 7.2 -> 8.7).
+int64_t warp_wave(int S) {
+    const size_t block = 8 * warp_tile_bytes(S) + 3072;  // 256 threads, and the static arrays
+    return (int64_t)152 * 32 * std::min<int64_t>(32, 8 * (int64_t)(227 * 1024 / block));
+}
+// The molecules per tet up to which window launches that were not timed go over
+// block tiles, by those figures,
+// up to which the tuning times them, and up to which a batch takes them (four
+// members of 69,360 tets and 30 species at 2 molecules per tet: 65 us on warp
+// tiles, 54 on block tiles)
+double tuned_block_density(int S) { return S >= 24 ? 5.0 : 2.0; }
+double batch_block_density(int S) { return S >= 24 ? 2.0 : 0.5; }
+double block_density(int S, int64_t T) { return S >= 24 ? 1.5 : T < kListMinTets ? 1.0 : 0.2; }
 
 __global__ void scatter_to_device_order(const int32_t *src, int64_t nt, int32_t S, const int32_t *inv_perm,
                                         int32_t *dst, size_t Tpad) {
@@ -244,12 +277,11 @@ void flow_neighbours(const std::vector<int32_t> &nbr_dev, int64_t T, int64_t B, 
 // Launch-form choices of tuned simulations, shared by every simulation of
 // the same compiled kernel, tet count, block size and molecules per tet (to a
 // power of two; clones of one prototype, the jobs of a stream): the first
-// one's tuning run decides, and a simulation keeps the choice of its own first
-// run when its counts change. (A tenth of the benchmark box's molecules runs
-// 14 % faster in another form than the box.)
+// one's tuning run decides. (A tenth of the benchmark box's molecules runs 14 %
+// faster in another form than the box.)
 struct FlowChoice {
     int pick;
-    float ms[3];
+    float ms[kForms];
 };
 std::mutex g_flow_mu;
 std::map<std::tuple<const void *, int64_t, int, int>, FlowChoice> g_flow_choice;
@@ -264,6 +296,7 @@ bool cuda_ok(cudaError_t e, const char *what) {
 // thread's fail (steps_debug_fail_alloc): the paths that follow cannot be
 // reached by filling the device.
 thread_local int32_t t_fail_alloc = 0;
+thread_local int32_t t_form = 0;  // steps_debug_form
 thread_local int64_t t_allocs = 0;
 
 cudaError_t device_alloc(void **p, size_t bytes) {
@@ -311,6 +344,12 @@ struct steps_sim {
     double *d_G = nullptr;          // [Tpad] the tets' total face rates, and
     uint32_t *d_leave_list = nullptr;  // the entries the host decides: their number, (species, tet) each, values
     std::string spec_why;           // why there is none
+    // block tiles (steps_step.cuh) compiled for a model of many species, for
+    // meshes of more than a resident wave of warp tiles, on first use
+    void *spec_block = nullptr;
+    bool block_tried = false;
+    bool blocky = false;            // the present run's window launches go over block tiles
+    int forced = 0;                 // a test's choice of form (steps_debug_form), or 0
     // list form (steps_list.cuh): its kernel, and per-simulation buffers
     void *spec_list = nullptr;
     uint32_t *d_tm[2] = {nullptr, nullptr};   // [Tpad] species words of both count buffers
@@ -339,7 +378,8 @@ struct steps_sim {
     // graphs of kGraphWindows full windows, one per starting buffer
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     // flow launches (a run's full windows in one launch), per block size: [0]
-    // the simulation's, [1] 512 (a tuning candidate when the block is smaller).
+    // the simulation's, [1] 512 (a tuning candidate when the block is smaller),
+    // [2] and [3] compiled block tiles of 256 and 512 tets.
     // Each holds its step kernel, the tiles' finished-window words and the item
     // counter (d_flow[nwords]) and, for a block-tile kernel, every tile's
     // neighbour tiles (tiles of `block` tets in device order, CSR).
@@ -354,9 +394,12 @@ struct steps_sim {
         int64_t ntiles = 0;  // items per window
         int64_t nwords = 0;
         size_t bytes = 0;
-    } flow[2];
-    int flow_pick = -1;  // flow = 0 (tuned): -1 not yet timed, 0 window launches, 1 + k flow launches of flow[k]
-    float flow_ms[3] = {0.f, 0.f, 0.f};  // tuning: ms per window of window launches, flow[0], flow[1]
+    } flow[4];
+    // flow = 0 (tuned): -1 not yet timed, 0 window launches, 1 + k flow launches
+    // of flow[k] (k < 2); on block tiles 3 window launches, 2 + k flow[k] (k >= 2)
+    int flow_pick = -1;
+    int pick_bucket = 0;         // the bucket of the density it was made for
+    float flow_ms[kForms] = {};  // tuning: ms per window of each
 
     // a clone's buffers: one allocation (a dozen, and as many frees, were most
     // of the time of admitting and retiring a served job)
@@ -424,13 +467,16 @@ struct steps_sim {
         Flow &fl = flow[k];
         if (fl.d_flow || fl.tried) return STEPS_OK;
         fl.tried = true;
-        const int64_t B = k == 0 ? opt.block : 512;
-        void *sp = k == 0 ? spec : (spec ? spec_kernel(model, 512, nullptr) : nullptr);
+        const int64_t B = k == 0 ? opt.block : k == 2 ? 256 : 512;
+        void *sp = k == 0   ? spec
+                   : k == 2 ? spec_block
+                   : !spec  ? nullptr
+                            : k == 1 ? spec_kernel(model, 512, nullptr) : spec_block_kernel(model, 512);
         const bool generic = k == 0 && !spec;
         if (!sp && !(generic && B == 256)) return STEPS_OK;
         // a warp-tile kernel publishes per 32 tets and finds the tiles it waits
         // for from its tets' neighbours: it needs no lists
-        const bool warp = sp || model.dev.S <= kWarpGenericSpecies;
+        const bool warp = k < 2 && (sp || model.dev.S <= kWarpGenericSpecies);
         const int64_t nt = (T + B - 1) / B, nwords = warp ? nt * (B / 32) : nt;
         std::vector<int32_t> off, nb;
         if (!warp) {
@@ -586,6 +632,33 @@ struct steps_sim {
         return r;
     }
 
+    bool wants_list() const {
+        return spec_list && opt.flow != 1 && fill >= 0.0 && fill <= kListFill &&
+               (forced || (T >= kListMinTets && fill * (double)T <= kListMost)) && plain_rates(model, tab);
+    }
+
+    // whether block tiles are a form of this simulation at all
+    bool block_possible() const {
+        return spec && S >= kListMinSpecies && (forced ? forced == 3 : opt.flow != 1 && T > warp_wave(S));
+    }
+
+    // their kernels, and the trial buffer they need
+    bool ensure_block() {
+        if (!spec_block && !block_tried && block_possible()) {
+            block_tried = true;
+            void *k = spec_block_kernel(model, 256);
+            if (k && ensure_trial()) spec_block = k;
+        }
+        return spec_block != nullptr;
+    }
+
+    // window launches over block tiles, at a density of d molecules per tet
+    bool wants_block(double d) {
+        if (!block_possible()) return false;
+        if (flow_pick >= 0 && !stale() ? flow_pick < 3 : !forced && !(d >= 0.0 && d <= block_density(S, T))) return false;
+        return ensure_block();
+    }
+
     // density and fill of the present state; waits for the stream
     int measure(cudaStream_t st) {
         uint32_t seen[4] = {0, 0, 0, 0};
@@ -606,6 +679,14 @@ struct steps_sim {
         density = (double)((uint64_t)seen[3] << 32 | seen[2]) / (double)T;
     }
 
+    // the trial buffer that block tiles of 16 or more species need
+    bool ensure_trial() {
+        if (d_trial || !spec_block_trial(model)) return true;
+        if (device_alloc((void **)&d_trial, (size_t)S * (size_t)Tpad * 4) != cudaSuccess) return false;
+        drop_graphs();  // (captured launches hold the arguments)
+        return true;
+    }
+
     // Before a run, and within long ones: the form of its windows, by what is
     // known of the state. A list's length is looked at (the stream waited for)
     // every kListCheckWindows, also over the intervals of a recording.
@@ -617,14 +698,13 @@ struct steps_sim {
                 return STEPS_ERR_CUDA;
             fill_from(c);
         }
-        if (spec_list && opt.flow != 1 && fill < 0.0)
+        if ((spec_list && opt.flow != 1 && fill < 0.0) || (block_possible() && density < 0.0))
             if (int rc = measure(stream)) return rc;
-        const bool want = spec_list && opt.flow != 1 && fill <= kListFill && plain_rates(model, tab);
-        if (want != listing) {
-            drop_graphs();
-            looked = k_total;
-        }
+        const bool want = wants_list(), block = !want && wants_block(density);
+        if (want != listing || block != blocky) drop_graphs();
+        if (want != listing) looked = k_total;
         listing = want;
+        blocky = block;
         if (!listing) tm_valid = list_valid = false;  // the other kernels leave them behind
         return STEPS_OK;
     }
@@ -721,7 +801,7 @@ struct steps_sim {
 
     // one window on the model-specialised kernel if there is one, else the generic one
     int launch(const StepArgs &a, cudaStream_t st) const {
-        if (listing) return launch_spec(spec_list, model.dev, a, opt.block, st);
+        if (listing || blocky) return launch_spec(listing ? spec_list : spec_block, model.dev, a, opt.block, st);
         return spec ? launch_spec(spec, model.dev, a, opt.block, st) : launch_step(model.dev, a, opt.block, st);
     }
 
@@ -768,43 +848,61 @@ struct steps_sim {
     // a flow kernel exists for the simulation's block size
     bool flow_possible() const { return spec || opt.block == 256; }
 
+    // the flow launches of a run's full windows: flow[k], or -1 for window launches
+    int flow_form() const {
+        if (!flow_possible()) return -1;
+        if (opt.flow == 1) return blocky ? 2 : 0;
+        return opt.flow != 0 ? -1 : flow_pick >= 4 ? (blocky ? flow_pick - 2 : -1) : flow_pick == 1 || flow_pick == 2 ? flow_pick - 1 : -1;
+    }
+
     // n full windows: flow launches or window launches (all give the same bits)
     int full_windows(int64_t n) {
         int64_t listed = 0;
         if (int rl = list_windows(n, &listed)) return rl;
         n -= listed;
         if (n == 0) return STEPS_OK;
-        if (opt.flow == 0 && flow_pick < 0 && flow_possible() && n >= kFlowTuneWindows) {
+        if (opt.flow == 0 && (flow_pick < 0 || stale()) && flow_possible() && forced != 3 && n >= tune_windows()) {
             int64_t used = 0;
             int rc = tune_flow(&used);
+            if (!rc) rc = choose_form();
             if (rc) return rc;
             n -= used;
         }
-        int k = -1;
-        if (n >= 2 && flow_possible()) {
-            if (opt.flow == 1) k = 0;
-            else if (opt.flow == 0 && flow_pick >= 1) k = flow_pick - 1;
-        }
+        const int k = n >= 2 ? flow_form() : -1;
         return k >= 0 ? flow_windows(n, k) : window_launches(n);
     }
 
 
+    // molecules per tet, to a power of two
+    int bucket() const { return (int)std::lrint(std::log2(std::max(density, 0.0) + 0.01)); }
+
+    // whether a tuned choice was made for another state: the next run that is
+    // long enough tunes again (or looks the choice up)
+    bool stale() const { return flow_pick >= 0 && density >= 0.0 && bucket() != pick_bucket; }
+
+    // full windows that the tuning takes
+    int64_t tune_windows() const {
+        return block_possible() && density <= tuned_block_density(S) ? kFormTuneWindows : kFlowTuneWindows;
+    }
+
     // The first run with enough full windows times the launch forms on
     // alternating groups of windows: window launches, flow launches at the
     // simulation's block size and, when that is below 512, flow launches of
-    // 512-tet tiles. One warm round, so that one-time costs do not decide,
-    // then two timed rounds, so that the state's slow drift cancels. The
-    // fastest flow form is kept when it is more than 2 % faster than window
-    // launches. The windows taken are ordinary windows of the run.
+    // 512-tet tiles; then both forms of block tiles where the model and mesh
+    // have them. One warm round, so that one-time costs do not decide, then two
+    // timed rounds, so that the state's slow drift cancels. The fastest other
+    // form is kept when it is more than 2 % faster than window launches. The
+    // windows taken are ordinary windows of the run.
     int tune_flow(int64_t *used) {
         if (density < 0.0)
             if (int rc = measure(stream)) return rc;
         // the best form depends on the state: by powers of two of the molecules per tet
-        const auto key = std::make_tuple((const void *)spec, T, opt.block, (int)std::lrint(std::log2(density + 0.01)));
+        const auto key = std::make_tuple((const void *)spec, T, opt.block, bucket());
+        pick_bucket = bucket();
         {
             std::lock_guard<std::mutex> lock(g_flow_mu);
             auto it = g_flow_choice.find(key);
-            if (it != g_flow_choice.end()) {
+            if (it != g_flow_choice.end() && (it->second.pick < 3 || ensure_block())) {
                 flow_pick = it->second.pick;
                 std::memcpy(flow_ms, it->second.ms, sizeof(flow_ms));
                 return STEPS_OK;
@@ -813,24 +911,31 @@ struct steps_sim {
         int rc = ensure_flow(0);
         if (!rc && opt.block < 512) rc = ensure_flow(1);
         if (rc) return rc;
-        const int nc = flow[0].d_flow ? (flow[1].d_flow ? 3 : 2) : 1;
-        if (nc == 1) {
-            flow_pick = 0;
-            return STEPS_OK;
+        int form[kForms] = {0}, nc = 1;
+        for (int k = 0; k < 2; ++k)
+            if (flow[k].d_flow) form[nc++] = 1 + k;
+        const int64_t windows = tune_windows();
+        if (windows == kFormTuneWindows && ensure_block()) {
+            form[nc++] = 3;
+            for (int k = 2; k < 4; ++k)
+                if (ensure_flow(k) == STEPS_OK && flow[k].d_flow) form[nc++] = 2 + k;
         }
-        cudaEvent_t e[4] = {};
+        flow_pick = 0;
+        if (nc == 1) return STEPS_OK;
+        cudaEvent_t e[kForms + 1] = {};
         for (auto &ev : e)
             if (!cuda_ok(cudaEventCreate(&ev), "flow tuning event")) {
                 for (auto &x : e)
                     if (x) cudaEventDestroy(x);
                 return STEPS_ERR_CUDA;
             }
-        float tot[3] = {0.f, 0.f, 0.f};
-        const int64_t g = kFlowTuneWindows / (3 * nc);  // windows per group
+        float tot[kForms] = {};
+        const int64_t g = windows / (3 * nc);  // windows per group (too few for a graph)
         for (int round = 0; round < 3 && rc == STEPS_OK; ++round) {
             for (int c = 0; c < nc && rc == STEPS_OK; ++c) {
                 if (!cuda_ok(cudaEventRecord(e[c], stream), "flow tuning")) rc = STEPS_ERR_CUDA;
-                if (!rc) rc = c == 0 ? window_launches(g) : flow_windows(g, c - 1);
+                blocky = form[c] == 3;
+                if (!rc) rc = form[c] % 3 == 0 ? window_launches(g) : flow_windows(g, form[c] >= 4 ? form[c] - 2 : form[c] - 1);
                 *used += g;
             }
             if (!rc && !cuda_ok(cudaEventRecord(e[nc], stream), "flow tuning")) rc = STEPS_ERR_CUDA;
@@ -841,13 +946,14 @@ struct steps_sim {
                 else if (round > 0) tot[c] += ms;
             }
         }
+        if (windows == kFormTuneWindows) drop_graphs();  // (captured before, perhaps of another form)
         for (auto &x : e) cudaEventDestroy(x);
         if (rc) return rc;
         int best = 1;
         for (int c = 2; c < nc; ++c)
             if (tot[c] < tot[best]) best = c;
-        for (int c = 0; c < nc; ++c) flow_ms[c] = tot[c] / (2.f * (float)g);
-        flow_pick = tot[best] < 0.98f * tot[0] ? best : 0;
+        for (int c = 0; c < nc; ++c) flow_ms[form[c]] = tot[c] / (2.f * (float)g);
+        flow_pick = tot[best] < 0.98f * tot[0] ? form[best] : 0;
         std::lock_guard<std::mutex> lock(g_flow_mu);
         FlowChoice ch;
         ch.pick = flow_pick;
@@ -989,7 +1095,7 @@ int steps_model_create(int32_t n_species, const double *diff, int32_t n_reac, co
 void steps_model_destroy(steps_model *model) { delete model; }
 
 int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t seed, const steps_options *opt,
-                     void *cuda_stream, steps_sim **out) {
+                     void *cuda_stream, steps_sim **out) try {
     CHECK_NULL(out, "steps_sim_create");
     *out = nullptr;
     CHECK_NULL(mesh, "steps_sim_create");
@@ -1036,6 +1142,7 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
     } else {
         steps_options_default(&s->opt);
     }
+    s->forced = t_form;
     s->model = model->m;
     s->model.leave_exp = s->opt.leave_law == STEPS_LEAVE_EXP;
     s->stream = (cudaStream_t)cuda_stream;
@@ -1113,7 +1220,7 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
             set_error("steps_sim_create: the specialised step kernel could not be built: " + s->spec_why);
             return STEPS_ERR_CUDA;
         }
-        if (s->spec && s->opt.flow != 1) {
+        if (s->spec && s->opt.flow != 1 && (s->forced ? s->forced == 2 : s->T >= kListMinTets)) {
             s->spec_list = spec_list_kernel(s->model);
             if (s->spec_list)
                 for (const steps_sim::Request &r : s->list_requests()) alloc(r.first, r.second);
@@ -1127,9 +1234,12 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
     }
     *out = s.release();
     return STEPS_OK;
+} catch (const std::bad_alloc &) {
+    set_error("steps_sim_create: out of host memory");
+    return STEPS_ERR_OOM;
 }
 
-int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, steps_sim **out) {
+int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, steps_sim **out) try {
     CHECK_NULL(out, "steps_sim_clone");
     *out = nullptr;
     CHECK_NULL(src, "steps_sim_clone");
@@ -1151,6 +1261,7 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
     s->seed = seed;
     s->spec = src->spec;
     s->spec_list = src->spec_list;
+    s->forced = src->forced;
     s->spec_why = src->spec_why;
     std::memcpy(s->scale_full, src->scale_full, sizeof(s->scale_full));
     const size_t Tpad = (size_t)s->Tpad, S = (size_t)s->S, T = (size_t)s->T;
@@ -1210,6 +1321,9 @@ int steps_sim_clone(const steps_sim *src, uint64_t seed, void *cuda_stream, step
     if (!ok || !cuda_ok(cudaStreamSynchronize(st), "steps_sim_clone")) return STEPS_ERR_CUDA;
     *out = s.release();
     return STEPS_OK;
+} catch (const std::bad_alloc &) {
+    set_error("steps_sim_clone: out of host memory");
+    return STEPS_ERR_OOM;
 }
 
 int steps_sim_device_bytes(const steps_sim *sim, int64_t *bytes) {
@@ -1219,7 +1333,8 @@ int steps_sim_device_bytes(const steps_sim *sim, int64_t *bytes) {
     *bytes = 2 * S * Tpad * 4 + Tpad * 16 * 2 + Tpad * 4 + 16 + S * T * 4 + (sim->d_orig ? Tpad * 4 + T * 4 : 0) +
              (sim->d_trial ? S * Tpad * 4 : 0) + (sim->d_tm[0] ? 10 * Tpad * 4 + 16 : 0) +
              (sim->d_src ? Tpad * 4 + Tpad / 8 : 0) + (sim->d_leave[0] ? 2 * S * Tpad * 4 + Tpad * 8 + (int64_t)kLeaveListBytes : 0) +
-             (sim->d_rmask ? Tpad * 4 : 0) + (int64_t)(sim->flow[0].bytes + sim->flow[1].bytes);
+             (sim->d_rmask ? Tpad * 4 : 0) + (int64_t)(sim->flow[0].bytes + sim->flow[1].bytes + sim->flow[2].bytes +
+                       sim->flow[3].bytes);
     return STEPS_OK;
 }
 
@@ -1539,12 +1654,8 @@ int steps_run_record(steps_sim *sim, double t_end, double dt_rec, int32_t n_spec
 int steps_sim_flow(const steps_sim *sim, int32_t *flow_block, float *tune_ms) {
     CHECK_NULL(sim, "steps_sim_flow");
     CHECK_NULL(flow_block, "steps_sim_flow");
-    int k = -1;
-    if (sim->flow_possible()) {
-        if (sim->opt.flow == 1) k = 0;
-        else if (sim->opt.flow == 0 && sim->flow_pick >= 1) k = sim->flow_pick - 1;
-    }
-    *flow_block = k < 0 ? 0 : k == 0 ? sim->opt.block : 512;
+    const int k = sim->flow_form();
+    *flow_block = k < 0 ? 0 : k == 0 ? sim->opt.block : k == 2 ? 256 : 512;
     if (tune_ms)
         for (int c = 0; c < 3; ++c) tune_ms[c] = sim->flow_ms[c];
     return STEPS_OK;
@@ -1655,6 +1766,15 @@ int steps_debug_fail_alloc(int32_t nth, int64_t *made) {
     }
     t_fail_alloc = nth;
     if (made) *made = t_allocs;
+    return STEPS_OK;
+}
+
+int steps_debug_form(int32_t form) {
+    if (form != 0 && form != 2 && form != 3) {
+        set_error("steps_debug_form: form must be 0, 2 or 3");
+        return STEPS_ERR_ARG;
+    }
+    t_form = form;
     return STEPS_OK;
 }
 
@@ -1830,6 +1950,8 @@ struct steps_batch {
     void *spec_list = nullptr;
     Work lwork;
     uint32_t *h_lcnt = nullptr;  // pinned: their list lengths after the run
+    void *spec_block = nullptr;  // block tiles for the others (256-thread blocks)
+    bool blocky = false;         // in this run
     uint64_t launches = 0;
     bool use_spec = false;      // run the model-specialised batched kernel
     bool spec_forced = false;
@@ -1902,8 +2024,7 @@ struct steps_batch {
         std::vector<char> want(members.size(), 0);
         for (size_t j = 0; j < members.size(); ++j) {
             const steps_sim *m = members[j];
-            want[j] = use_spec && !flow && m->spec_list && m->fill >= 0.0 && m->fill <= kListFill &&
-                      plain_rates(m->model, m->tab);
+            want[j] = use_spec && !flow && m->wants_list();
         }
         return want;
     }
@@ -1927,10 +2048,32 @@ struct steps_batch {
     // follow when they change (a batch is created with those of its members'
     // states, since freeing a list waits for the device).
     int choose_forms() try {
+        const bool many = use_spec && !flow && max_S >= kListMinSpecies;
         for (steps_sim *m : members)
-            if (use_spec && !flow && m->spec_list && m->fill < 0.0)
+            if (many && (m->fill < 0.0 || m->density < 0.0))
                 if (int rc = m->measure(stream)) return rc;
         std::vector<char> want = wanted();
+        // block tiles for the members that are not listed, by their tets and molecules together
+        int64_t tets = 0;
+        double molecules = 0.0;
+        bool forced = false;
+        for (size_t j = 0; j < members.size(); ++j)
+            if (!want[j]) {
+                tets += members[j]->T;
+                molecules += members[j]->density * (double)members[j]->T;
+                forced = forced || members[j]->forced == 3;
+            }
+        bool block = many && (forced || (tets > warp_wave(max_S) && molecules <= batch_block_density(max_S) * (double)tets));
+        if (block && !spec_block) spec_block = spec_block_kernel(members[0]->model, 256);
+        block = block && spec_block;
+        for (size_t j = 0; j < members.size() && block; ++j)
+            block = want[j] || members[j]->ensure_trial();
+        if (block != blocky)
+            for (Work &w : work) {
+                if (w.graph) cudaGraphExecDestroy(w.graph);
+                w.graph = nullptr;
+            }
+        blocky = block;
         if (want != listed) {
             for (Work *w : {&work[0], &work[1], &work[2], &work[3], &lwork}) {
                 if (w->graph) cudaGraphExecDestroy(w->graph);
@@ -1976,7 +2119,7 @@ struct steps_batch {
 
     int window(int b, cudaStream_t st) {  // one batched window + advance
         Work &w = work[slot(b)];
-        int rc = use_spec && spec[slot(b)] ? launch_spec_batch(spec[slot(b)], w.d, w.n, d_reps, b, st)
+        int rc = use_spec && spec[slot(b)] ? launch_spec_batch(blocky ? spec_block : spec[slot(b)], w.d, w.n, d_reps, b, st)
                                            : launch_step_batch(w.d, w.n, d_reps, max_S, max_R, any_order0, b, st);
         if (!rc && lwork.n) rc = launch_spec_batch(spec_list, lwork.d, lwork.n, d_reps, 256, st);
         if (!rc) rc = launch_advance(d_reps, (int32_t)members.size(), st);
@@ -2274,9 +2417,10 @@ int batch_enqueue(steps_batch *b, const double *t_end, int64_t most, bool *more)
     int64_t done = 0;
     int rc = STEPS_OK;
     const int cand[3] = {128, 256, 512};
-    const bool tune = b->autotune && nmax >= 12;
+    const bool tune = b->autotune && !b->blocky && nmax >= 12;
+    const int block = b->blocky ? 256 : b->block;
     for (int c = 0; c < 3 && tune && rc == STEPS_OK; ++c) rc = b->prepare(cand[c]);
-    if (rc == STEPS_OK) rc = b->prepare(b->block);
+    if (rc == STEPS_OK) rc = b->prepare(block);
     if (rc) return rc;
     if (tune) {
         // time the candidate block sizes on alternating windows (one warm window
@@ -2326,7 +2470,7 @@ int batch_enqueue(steps_batch *b, const double *t_end, int64_t most, bool *more)
         b->block = best_b;
         b->autotune = false;
     }
-    rc = b->run_windows(b->block, nmax - done);
+    rc = b->run_windows(tune ? b->block : block, nmax - done);
     if (rc) return rc;
     // shortened last windows: their table goes into the second pinned buffer
     // (h_reps may still be read by its queued upload)
@@ -2355,7 +2499,7 @@ int batch_enqueue(steps_batch *b, const double *t_end, int64_t most, bool *more)
         if (!cuda_ok(cudaMemcpyAsync(b->d_reps, b->h_last, sizeof(RepEntry) * n, cudaMemcpyHostToDevice, b->stream),
                      "steps_batch_run: upload"))
             return STEPS_ERR_CUDA;
-        rc = b->run_windows(b->block, 1);
+        rc = b->run_windows(tune ? b->block : block, 1);
         if (rc) return rc;
     }
     // members' clocks and buffers
@@ -2447,7 +2591,7 @@ namespace {
 struct NoAllocScratch {
     bool ready = false;
     int32_t *counts = nullptr;  // [2][kNoAllocMaxCounts]
-    uint32_t *err = nullptr;    // two words after the count buffers: window error word, input check flag
+    uint32_t *err = nullptr;    // after the count buffers: window error word, unused, any_negative's four
 };
 
 constexpr int kNoAllocMaxDevices = 64;
@@ -2516,29 +2660,34 @@ extern "C" int steps_run_noalloc(steps_sim *sim, int32_t *d_counts, double t_end
     // (padding and receiving rows must be zero) and both error words
     if (!cuda_ok(cudaMemsetAsync(buf[0], 0, S * Tpad * 4, st), "steps_run_noalloc: clear") ||
         !cuda_ok(cudaMemsetAsync(buf[1], 0, S * Tpad * 4, st), "steps_run_noalloc: clear") ||
-        !cuda_ok(cudaMemsetAsync(sc.err, 0, 8, st), "steps_run_noalloc: clear"))
+        !cuda_ok(cudaMemsetAsync(sc.err, 0, 24, st), "steps_run_noalloc: clear"))
         return STEPS_ERR_CUDA;
     // reject negative input counts before anything (clock, caller's buffer) changes
+    double density = 0.0;
     {
         const int64_t n = (int64_t)(S * T);
-        uint32_t neg = 0;
-        any_negative<false><<<input_blocks(n), kInputThreads, 0, st>>>(d_counts, n, sc.err + 1);
+        uint32_t seen[4] = {0, 0, 0, 0};  // (any_negative)
+        if (sim->block_possible()) any_negative<true><<<input_blocks(n), kInputThreads, 0, st>>>(d_counts, n, sc.err + 2);
+        else any_negative<false><<<input_blocks(n), kInputThreads, 0, st>>>(d_counts, n, sc.err + 2);
         if (!cuda_ok(cudaGetLastError(), "steps_run_noalloc: check") ||
-            !cuda_ok(cudaMemcpyAsync(&neg, sc.err + 1, 4, cudaMemcpyDeviceToHost, st), "steps_run_noalloc: check") ||
+            !cuda_ok(cudaMemcpyAsync(seen, sc.err + 2, 16, cudaMemcpyDeviceToHost, st), "steps_run_noalloc: check") ||
             !cuda_ok(cudaStreamSynchronize(st), "steps_run_noalloc: check"))
             return STEPS_ERR_CUDA;
-        if (neg) {
+        if (seen[0]) {
             set_error("steps_run_noalloc: negative count in d_counts");
             return STEPS_ERR_ARG;
         }
+        density = (double)((uint64_t)seen[3] << 32 | seen[2]) / (double)T;
     }
     const unsigned grid = (unsigned)((T + 255) / 256);
     scatter_to_device_order<<<grid, 256, 0, st>>>(d_counts, (int64_t)T, (int32_t)S, sim->d_inv_perm, buf[0], Tpad);
     if (!cuda_ok(cudaGetLastError(), "steps_run_noalloc: scatter")) return STEPS_ERR_CUDA;
 
     // the window loop of steps_run (Algorithm 1), with plain launches on the scratch buffers (never the list form)
-    if (sim->listing) sim->drop_graphs();
+    const bool block = sim->spec_block && sim->wants_block(density);  // (nothing is allocated or compiled here)
+    if (sim->listing || sim->blocky != block) sim->drop_graphs();
     sim->listing = sim->tm_valid = sim->list_valid = false;
+    sim->blocky = block;
     const double tau = sim->tab.tau;
     const bool finite = std::isfinite(tau);
     const double tol = finite ? 1e-9 * tau : 0.0;

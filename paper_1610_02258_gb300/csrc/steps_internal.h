@@ -114,6 +114,11 @@ int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEnt
 std::string spec_program_source(const HostModel &hm, int block);
 // the list form's step kernel for launch_spec (models of 13 or more species), or nullptr
 void *spec_list_kernel(const HostModel &hm);
+constexpr int kListMinSpecies = 13;
+// the block tiles' kernels for launch_spec, launch_spec_flow and launch_spec_batch (the same models), or nullptr;
+// and whether they keep the trial counts in StepArgs::trial
+void *spec_block_kernel(const HostModel &hm, int block);
+bool spec_block_trial(const HostModel &hm);
 
 // steps_api.cu: steps_batch_run in two parts (enqueue every window and the
 // error word's copy; then wait and map the word to a return code), so that

@@ -78,22 +78,29 @@ Nvrtc &nvrtc() {
     return n;
 }
 
+}  // namespace
+
+bool spec_block_trial(const HostModel &hm) { return hm.dev.S >= 16; }
+
+namespace {
+
 std::string hex_u32(uint32_t v) {
     std::ostringstream o;
     o << "0x" << std::hex << v << "u";
     return o.str();
 }
 
-// The generated policy of the list form: the functions of RtModel with the model's
-// structure as constants. Propensity forms (all in float, as RtModel):
+// The generated policy of the list form and of block tiles: the functions of
+// RtModel with the model's structure as constants (block: entries of a count
+// row). Propensity forms (all in float, as RtModel):
 //   order 0: k / inv_nav            order 1: k x
 //   order 2: ((k inv_nav) x) y      dimer:   ((k inv_nav) x) (x - 1)
 // (RtModel's extra factors of 1 are exact and left out.)
-std::string list_policy_source(const HostModel &hm) {
-    constexpr int block = 32;  // entries of a count row
+std::string table_policy_source(const HostModel &hm, int block) {
     const ModelDev &m = hm.dev;
     std::ostringstream o;
     o << "namespace steps {\nnamespace {\nstruct SpecModel {\n";
+    o << "    static constexpr bool kGlobalTrial = " << (spec_block_trial(hm) ? "true" : "false") << ";\n";
     o << "    static constexpr bool kExpLeave = " << (hm.leave_exp ? "true" : "false") << ";\n";
     o << "    __device__ static int S(const ModelDev &) { return " << m.S << "; }\n";
     o << "    __device__ static int R(const ModelDev &) { return " << m.R << "; }\n";
@@ -232,12 +239,11 @@ std::string program_source(const HostModel &hm, int block) {
 
 // The list form's program: a plain and a batched step kernel (256-thread blocks).
 constexpr int kListBlock = 256;
-constexpr int kListMinSpecies = 13;
 
 std::string list_program_source(const HostModel &hm) {
     std::ostringstream o;
     const std::string b = std::to_string(kListBlock);
-    o << "#include \"steps_list.cuh\"\n" << list_policy_source(hm);
+    o << "#include \"steps_list.cuh\"\n" << table_policy_source(hm, 32);
     o << "extern \"C\" __global__ void __launch_bounds__(" << b << ", " << 1024 / kListBlock << ")\n"
       << "steps_spec_list(const __grid_constant__ steps::ModelDev m, const __grid_constant__ steps::StepArgs a) {\n"
       << "    steps::list_step<" << b << ", " << std::max(1, hm.dev.R) << ", " << hm.dev.S
@@ -250,7 +256,34 @@ std::string list_program_source(const HostModel &hm) {
     return o.str();
 }
 
+// The block tiles' program: plain, flow and batched step kernels. With the
+// trial counts in global memory, five blocks of 256 threads fit an SM with a
+// 32-entry block map and 48 registers per thread.
+int reaction_bucket(int R) { return R <= 8 ? 8 : R <= 16 ? 16 : R <= 24 ? 24 : 32; }
+
+std::string block_program_source(const HostModel &hm, int block) {
+    std::ostringstream o;
+    const bool five = spec_block_trial(hm) && block == 256;
+    const std::string b = std::to_string(block), per_sm = std::to_string(1024 / block);
+    const std::string head = "extern \"C\" __global__ void __launch_bounds__(" + b + ", " + (five ? "5" : per_sm) + ")\n";
+    const std::string args = "<" + b + ", " + std::to_string(reaction_bucket(hm.dev.R)) + ", steps::SpecModel>";
+    if (five) o << "#define STEPS_MAP_CAP 32\n";
+    o << "#include \"steps_step.cuh\"\n" << table_policy_source(hm, block);
+    o << head << "steps_spec_step(const __grid_constant__ steps::ModelDev m, const __grid_constant__ steps::StepArgs a) "
+      << "{\n    steps::step_tile" << args << "(m, a, (int64_t)blockIdx.x);\n}\n";
+    o << head << "steps_spec_flow(const __grid_constant__ steps::ModelDev m, const __grid_constant__ steps::StepArgs a, "
+      << "const __grid_constant__ steps::FlowArgs f) {\n    steps::flow_tiles" << args << "(m, a, f);\n}\n";
+    o << "extern \"C\" __global__ void __launch_bounds__(" << b << ", " << per_sm << ")\n"
+      << "steps_spec_batch(const steps::BlockWork *__restrict__ work, const steps::RepEntry *__restrict__ reps, "
+      << "int32_t prefetch) {\n    steps::batch_tile" << args << "(work, reps, prefetch);\n}\n";
+    return o.str();
+}
+
+enum class Form { tiles, list, block };
+
 struct Compiled {
+    Form form = Form::tiles;
+    int block = 0;                      // threads per block
     cudaLibrary_t lib = nullptr;
     cudaKernel_t kern = nullptr;        // plain step kernel
     cudaKernel_t kern_batch = nullptr;  // batched step kernel
@@ -260,7 +293,6 @@ struct Compiled {
     size_t smem_set_flow = 0;           // the flow kernel
     size_t smem_set_batch_flow = 0;     // the batched flow kernel
     size_t smem_set_batch = 0;          // and the batched one
-    cudaKernel_t kern_list = nullptr;   // or the list form's plain step kernel (kern_batch: its batched one)
     size_t smem = 0;                    // dynamic shared memory per block
 };
 
@@ -273,14 +305,16 @@ std::string spec_program_source(const HostModel &hm, int block) { return program
 
 namespace {
 
-// Compiles (once per generated source) and loads the plain and batched kernels.
-Compiled *compiled(const HostModel &hm, int block, bool list, std::string *why) {
+// Compiles (once per generated source) and loads a form's kernels.
+Compiled *compiled(const HostModel &hm, int block, Form form, std::string *why) {
     Nvrtc &nv = nvrtc();
     if (!nv.handle) {
         if (why) *why = nv.why;
         return nullptr;
     }
-    const std::string src = list ? list_program_source(hm) : program_source(hm, block);
+    const std::string src = form == Form::list    ? list_program_source(hm)
+                            : form == Form::block ? block_program_source(hm, block)
+                                                  : program_source(hm, block);
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_cache.find(src);
     if (it != g_cache.end()) {
@@ -318,16 +352,20 @@ Compiled *compiled(const HostModel &hm, int block, bool list, std::string *why) 
         return nullptr;
     }
     auto c = std::make_shared<Compiled>();
-    c->smem = list ? (size_t)(kListBlock / 32) * list_tile_bytes(hm.dev.S) : (size_t)(block / 32) * warp_tile_bytes(hm.dev.S);
+    const auto get = [&](cudaKernel_t *k, const char *name) { return cudaLibraryGetKernel(k, c->lib, name) == cudaSuccess; };
     bool ok = cudaLibraryLoadData(&c->lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0) == cudaSuccess;
-    if (list) {
-        ok = ok && cudaLibraryGetKernel(&c->kern_list, c->lib, "steps_spec_list") == cudaSuccess &&
-             cudaLibraryGetKernel(&c->kern_batch, c->lib, "steps_spec_list_batch") == cudaSuccess;
+    const size_t S = (size_t)hm.dev.S;
+    c->form = form;
+    c->block = block;
+    if (form == Form::list) {
+        c->smem = (size_t)(kListBlock / 32) * list_tile_bytes(hm.dev.S);
+        ok = ok && get(&c->kern, "steps_spec_list") && get(&c->kern_batch, "steps_spec_list_batch");
     } else {
-        ok = ok && cudaLibraryGetKernel(&c->kern, c->lib, "steps_spec_step") == cudaSuccess &&
-             cudaLibraryGetKernel(&c->kern_batch, c->lib, "steps_spec_batch") == cudaSuccess &&
-             cudaLibraryGetKernel(&c->kern_flow, c->lib, "steps_spec_flow") == cudaSuccess &&
-             cudaLibraryGetKernel(&c->kern_batch_flow, c->lib, "steps_spec_batch_flow") == cudaSuccess;
+        c->smem = form == Form::block ? (S + 1 + (spec_block_trial(hm) ? 0 : S)) * (size_t)block * sizeof(int32_t)
+                                      : (size_t)(block / 32) * warp_tile_bytes(hm.dev.S);
+        ok = ok && get(&c->kern, "steps_spec_step") && get(&c->kern_batch, "steps_spec_batch") &&
+             get(&c->kern_flow, "steps_spec_flow") &&
+             (form == Form::block || get(&c->kern_batch_flow, "steps_spec_batch_flow"));
     }
     if (!ok) {
         cudaGetLastError();
@@ -354,22 +392,28 @@ bool opt_in(const void *fn, size_t smem, size_t *done) {
 }  // namespace
 
 void *spec_kernel(const HostModel &hm, int block, std::string *why) {
-    return (void *)compiled(hm, block, false, why);
+    return (void *)compiled(hm, block, Form::tiles, why);
 }
 
 void *spec_list_kernel(const HostModel &hm) {
-    return hm.dev.S >= kListMinSpecies ? (void *)compiled(hm, kListBlock, true, nullptr) : nullptr;
+    return hm.dev.S >= kListMinSpecies ? (void *)compiled(hm, kListBlock, Form::list, nullptr) : nullptr;
+}
+
+void *spec_block_kernel(const HostModel &hm, int block) {
+    return hm.dev.S >= kListMinSpecies ? (void *)compiled(hm, block, Form::block, nullptr) : nullptr;
 }
 
 int launch_spec(void *spec, const ModelDev &m, const StepArgs &a, int block, void *stream) {
     if (a.T <= 0) return STEPS_OK;
     Compiled *c = static_cast<Compiled *>(spec);
-    const void *fn = (const void *)(c->kern_list ? c->kern_list : c->kern);
-    if (c->kern_list) block = kListBlock;
+    const void *fn = (const void *)c->kern;
+    block = c->block;
     const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set)) return STEPS_ERR_CUDA;
-    void *args[2] = {(void *)&m, (void *)&a};
-    const unsigned grid = (unsigned)(c->kern_list ? list_blocks(a.T, block) : (a.T + block - 1) / block);
+    StepArgs b = a;
+    if (c->form == Form::block) b.prefetch = prefetch_distance(fn, block, smem);
+    void *args[2] = {(void *)&m, (void *)&b};
+    const unsigned grid = (unsigned)(c->form == Form::list ? list_blocks(a.T, block) : (a.T + block - 1) / block);
     // programmatic dependent launch, as the generic step kernel
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -404,10 +448,12 @@ int launch_spec_flow(void *spec, const ModelDev &m, const StepArgs &a, const Flo
     }
     StepArgs b = a;
     b.window_base = nullptr;
+    // block tiles: the item taken about half a resident wave later, its tables into L2
+    b.prefetch = std::max(1, per_sm * sms / 2);
     void *args[3] = {(void *)&m, (void *)&b, (void *)&f};
     // one item per block, or the blocks resident at once
     const unsigned items = f.nwin * f.ntiles;
-    const unsigned grid = warp_flow_persists(block) ? std::min(items, (unsigned)(per_sm * sms)) : items;
+    const unsigned grid = c->form == Form::tiles && warp_flow_persists(block) ? std::min(items, (unsigned)(per_sm * sms)) : items;
     cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3((unsigned)block), args, smem, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         set_error(std::string("flow step kernel launch: ") + cudaGetErrorString(e));
@@ -448,8 +494,9 @@ int launch_spec_batch(void *spec, const BlockWork *work, int64_t nblocks, RepEnt
     const void *fn = (const void *)c->kern_batch;
     const size_t smem = c->smem;
     if (!opt_in(fn, smem, &c->smem_set_batch)) return STEPS_ERR_CUDA;
-    void *args[2] = {(void *)&work, (void *)&reps};
-    if (c->kern_list) block = kListBlock;
+    block = c->block;
+    int32_t prefetch = c->form == Form::block ? prefetch_distance(fn, block, smem) : 0;
+    void *args[3] = {(void *)&work, (void *)&reps, (void *)&prefetch};  // (the last one: block tiles)
     cudaError_t e = cudaLaunchKernel(fn, dim3((unsigned)nblocks), dim3((unsigned)block), args, smem, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         set_error(std::string("specialised batched step kernel launch: ") + cudaGetErrorString(e));

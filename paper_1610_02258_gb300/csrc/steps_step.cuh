@@ -226,6 +226,8 @@ __device__ __noinline__ int careful_pick(const RxnTab &tb, const ModelDev &m, co
 // constants from the kernel parameters. Z: the model has order-0 reactions.
 template <bool Z>
 struct RtModel {
+    static constexpr bool kGlobalTrial = false;  // trial counts in shared memory
+    static constexpr bool kExpLeave = false;     // the EULER leave law (species scale in shared memory)
     __device__ static int S(const ModelDev &m) { return m.S; }
     __device__ static int R(const ModelDev &m) { return m.R; }
     __device__ static uint32_t diffusive(const ModelDev &m) { return m.diffusive; }
@@ -416,6 +418,15 @@ __device__ __forceinline__ int32_t trial_count(const StepArgs &a, int s, int32_t
     return mm > N ? N : (int32_t)mm;
 }
 
+// The species factor of tet i's thresholds: the window's species scale R_s
+// (EULER), or the tet's own leave value L_{s,i} from the EXP table (the
+// tet's factor A is then its cumulative face shares).
+template <class P>
+__device__ __forceinline__ uint32_t species_R(const StepArgs &a, const uint32_t *s_scale, int s, int64_t i) {
+    if constexpr (P::kExpLeave) return __ldg(a.leave + (size_t)s * (size_t)a.Tpad + (size_t)i);
+    else return s_scale[s];
+}
+
 // Leave thresholds of one species: T_f = (A_f R_s) >> 31 (2^31 fixed point).
 __device__ __forceinline__ void species_thresholds(const uint4 &A, uint32_t R, uint32_t &T0, uint32_t &T1,
                                                    uint32_t &T2, uint32_t &T3) {
@@ -496,8 +507,11 @@ __device__ __forceinline__ int32_t bulk_species(const StepArgs &a, int32_t *nxt,
 // lane `owner` with first[lane] <= b < first[lane + 1]; the map caches the
 // owner, the species of the block's first word and the tet's trial
 // molecules before that species for the first kMapCap blocks (those past it are
-// found by search).
-constexpr int kMapCap = 160;
+// found by search; a program may set a smaller map to fit more resident blocks).
+#ifndef STEPS_MAP_CAP
+#define STEPS_MAP_CAP 160
+#endif
+constexpr int kMapCap = STEPS_MAP_CAP;
 
 struct WarpWork {
     int16_t tet[32];          // tile index of each lane's tet (-1: none)
@@ -561,7 +575,7 @@ __device__ __forceinline__ void diffuse_block(const StepArgs &a, int32_t *nxt, c
     const size_t Tpad = (size_t)a.Tpad;
     const uint4 rw = philox4x32_10(a.key0, a.key1, c0, s_tet[t], k, (kPurposeDiff << 28) | c3);
     uint32_t T0, T1, T2, T3;
-    species_thresholds(A, s_scale[s], T0, T1, T2, T3);
+    species_thresholds(A, species_R<P>(a, s_scale, s, i0 + t), T0, T1, T2, T3);
     uint32_t w = 4u * k;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -570,7 +584,7 @@ __device__ __forceinline__ void diffuse_block(const StepArgs &a, int32_t *nxt, c
                 s = __ffs(hm) - 1;
                 hm &= hm - 1;
                 end += (uint32_t)trial_all[s * tstride + t];
-                species_thresholds(A, s_scale[s], T0, T1, T2, T3);
+                species_thresholds(A, species_R<P>(a, s_scale, s, i0 + t), T0, T1, T2, T3);
             }
             const uint32_t x = word_of(rw, q) >> 1;
             if (x < T3) {
@@ -726,8 +740,12 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
     const int nlive = (int)min((int64_t)BLOCK, (int64_t)a.T - i0);
     const bool live = tid < nlive;
     int32_t *cnt_all = smem;                              // rows 0..S-1 counts, row S ones
-    int32_t *trial_all = smem + (size_t)(S + 1) * BLOCK;  // trial counts [S][BLOCK]
-    constexpr size_t tstride = BLOCK;
+    // trial counts [S][tstride]: after the count rows in shared memory, or (for
+    // models with many species, to leave room for more resident blocks) the
+    // tile's columns of a global buffer
+    constexpr bool GT = P::kGlobalTrial;
+    int32_t *trial_all = GT ? a.trial + i0 : smem + (size_t)(S + 1) * BLOCK;
+    const size_t tstride = GT ? (size_t)a.Tpad : (size_t)BLOCK;
     uint32_t c0, c3;  // RNG counter words of the window, set once the previous window is done
     const size_t Tpad = (size_t)a.Tpad;
     uint32_t bad = 0;
@@ -926,7 +944,7 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
             while (walk) {
                 const int s = __ffs(walk) - 1;
                 walk &= walk - 1;
-                if ((uint32_t)(((uint64_t)Aw * s_scale[s]) >> 31) == 0u)
+                if ((uint32_t)(((uint64_t)Aw * species_R<P>(a, s_scale, s, i0 + t)) >> 31) == 0u)
                     continue;  // draws nothing
                 const int32_t N = cnt_all[s * BLOCK + t];
                 const int32_t M = plain ? N
@@ -953,7 +971,7 @@ __device__ __forceinline__ bool step_tile(const ModelDev &m, const StepArgs &a, 
             bw &= bw - 1;
             if ((bm >> s) & 1u)
                 cnt_all[s * BLOCK + t] -= bulk_species(a, nxt, s, trial_all[s * tstride + t], s_thr[t],
-                                                       s_scale[s], s_nbr[t], s_tet[t], c0, c3);
+                                                       species_R<P>(a, s_scale, s, i0 + t), s_nbr[t], s_tet[t], c0, c3);
         }
         // the chunk's Philox blocks: exclusive prefix of the lanes' block counts
         const uint32_t nb = (W + 3u) >> 2;

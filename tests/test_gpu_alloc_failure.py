@@ -23,8 +23,10 @@ def _capi():
 
 @pytest.fixture
 def capi(_capi):
+    _capi.steps_debug_form(2)  # the list form in sparse states of these small meshes
     yield _capi
     _capi.steps_debug_fail_alloc(0)
+    _capi.steps_debug_form(0)
 
 
 def _many_species():

@@ -1,5 +1,5 @@
 """GPU tests of when a run takes the list form (models of 13 or more species in
-sparse states) and when the tiles, seen from whether a run's tuning of the
+sparse states; here without the rule's mesh size) and when the tiles, seen from whether a run's tuning of the
 launch form took place (tiles) or not (list form), with counts equal to the
 oracle's either way."""
 import numpy as np
@@ -13,8 +13,15 @@ pytestmark = pytest.mark.gpu
 S = 14
 
 
+@pytest.fixture
+def capi(_capi):
+    _capi.steps_debug_form(2)
+    yield _capi
+    _capi.steps_debug_form(0)
+
+
 @pytest.fixture(scope="module")
-def capi():
+def _capi():
     import torch
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
