@@ -85,9 +85,12 @@ typedef struct steps_options {
                             `block`-tet tiles and (specialised, block < 512) of 512-tet tiles, and keeps the
                             fastest (steps_sim_flow reports it); 1: flow at `block` where a flow kernel exists;
                             -1: window launches. The results are the same bits in every form. With 0 and -1, a
-                            specialised model of 13 or more species whose state holds few molecules per tet
-                            runs its windows, in window launches, over a list of the tets that hold something
-                            (unless the device has no room for the lists). */
+                            specialised model of 13 or more species takes two more forms where they are faster:
+                            on meshes of 262,144 tets or more whose state holds few molecules per tet, window
+                            launches over a list of the tets that hold something (unless the device has no room
+                            for the lists); on meshes of about 80,000 tets or more at few molecules per tet, tiles
+                            of another layout, which the tuning times too (it then takes 90 windows). Counts of
+                            another density are timed again. */
     int32_t reserved[1]; /* set to 0 */
 } steps_options;
 
