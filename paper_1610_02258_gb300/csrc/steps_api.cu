@@ -72,14 +72,20 @@ int64_t warp_wave(int S) {
     const size_t block = 8 * warp_tile_bytes(S) + 3072;  // 256 threads, and the static arrays
     return (int64_t)152 * 32 * std::min<int64_t>(32, 8 * (int64_t)(227 * 1024 / block));
 }
-// The molecules per tet up to which window launches that were not timed go over
-// block tiles, by those figures,
-// up to which the tuning times them, and up to which a batch takes them (four
-// members of 69,360 tets and 30 species at 2 molecules per tet: 65 us on warp
-// tiles, 54 on block tiles)
-double tuned_block_density(int S) { return S >= 24 ? 5.0 : 2.0; }
-double batch_block_density(int S) { return S >= 24 ? 2.0 : 0.5; }
+// The molecules per tet up to which, by those figures, window launches that were
+// not timed go over block tiles, and the tuning times them.
 double block_density(int S, int64_t T) { return S >= 24 ? 1.5 : T < kListMinTets ? 1.0 : 0.2; }
+double tuned_block_density(int S) { return S >= 24 ? 5.0 : 2.0; }
+// The same for a batch, by its members together: four of 69,360 tets and 30
+// species at 2 molecules per tet, 65 us per window on warp tiles, 54 on block
+// tiles.
+double batch_block_density(int S) { return S >= 24 ? 2.0 : 0.5; }
+// Batches of run-time models of 5 to 12 species go over block tiles up to this
+// density. us per window of 16 members of 52,020 tets and 10 species, block ->
+// warp tiles: 0.05 molecules per tet 55 -> 67, 0.2 65 -> 73, 0.5 76 -> 79, 1.0
+// 88 -> 84, 3.0 113 -> 101; 3 species 40 -> 40, 44 -> 42, 51 -> 44, 59 -> 47, 72
+// -> 59.
+constexpr double kFewPerTet = 0.5;
 
 __global__ void scatter_to_device_order(const int32_t *src, int64_t nt, int32_t S, const int32_t *inv_perm,
                                         int32_t *dst, size_t Tpad) {
@@ -1952,6 +1958,7 @@ struct steps_batch {
     uint32_t *h_lcnt = nullptr;  // pinned: their list lengths after the run
     void *spec_block = nullptr;  // block tiles for the others (256-thread blocks)
     bool blocky = false;         // in this run
+    bool few = false;            // run-time models of 5 to 12 species in sparse states: block tiles, in this run
     uint64_t launches = 0;
     bool use_spec = false;      // run the model-specialised batched kernel
     bool spec_forced = false;
@@ -2049,8 +2056,9 @@ struct steps_batch {
     // states, since freeing a list waits for the device).
     int choose_forms() try {
         const bool many = use_spec && !flow && max_S >= kListMinSpecies;
+        const bool generic = !use_spec && max_S > 4 && max_S <= kWarpGenericSpecies;
         for (steps_sim *m : members)
-            if (many && (m->fill < 0.0 || m->density < 0.0))
+            if ((many || generic) && m->density < 0.0)  // (the fill is unknown with it)
                 if (int rc = m->measure(stream)) return rc;
         std::vector<char> want = wanted();
         // block tiles for the members that are not listed, by their tets and molecules together
@@ -2068,12 +2076,14 @@ struct steps_batch {
         block = block && spec_block;
         for (size_t j = 0; j < members.size() && block; ++j)
             block = want[j] || members[j]->ensure_trial();
-        if (block != blocky)
+        const bool sparse = generic && molecules <= kFewPerTet * (double)tets;
+        if (block != blocky || sparse != few)
             for (Work &w : work) {
                 if (w.graph) cudaGraphExecDestroy(w.graph);
                 w.graph = nullptr;
             }
         blocky = block;
+        few = sparse;
         if (want != listed) {
             for (Work *w : {&work[0], &work[1], &work[2], &work[3], &lwork}) {
                 if (w->graph) cudaGraphExecDestroy(w->graph);
@@ -2120,7 +2130,7 @@ struct steps_batch {
     int window(int b, cudaStream_t st) {  // one batched window + advance
         Work &w = work[slot(b)];
         int rc = use_spec && spec[slot(b)] ? launch_spec_batch(blocky ? spec_block : spec[slot(b)], w.d, w.n, d_reps, b, st)
-                                           : launch_step_batch(w.d, w.n, d_reps, max_S, max_R, any_order0, b, st);
+                                           : launch_step_batch(w.d, w.n, d_reps, max_S, max_R, any_order0, few, b, st);
         if (!rc && lwork.n) rc = launch_spec_batch(spec_list, lwork.d, lwork.n, d_reps, 256, st);
         if (!rc) rc = launch_advance(d_reps, (int32_t)members.size(), st);
         launches += per_window(b);

@@ -73,13 +73,13 @@ __global__ void advance_kernel(RepEntry *reps, int32_t n) {
 }  // namespace
 
 int launch_step_batch(const BlockWork *work, int64_t nblocks, RepEntry *reps, int max_S, int max_R,
-                      bool any_order0, int block, void *stream) {
+                      bool any_order0, bool few, int block, void *stream) {
     if (nblocks <= 0) return STEPS_OK;
     if (!work) {
         set_error("batched step kernel launch: no work list");
         return STEPS_ERR_STATE;
     }
-    if (max_S <= kWarpGenericSpecies) return launch_warp_batch(work, nblocks, reps, max_S, block, stream);
+    if (max_S <= kWarpGenericSpecies && !few) return launch_warp_batch(work, nblocks, reps, max_S, block, stream);
     switch (block) {
     case 64: return launch_batch_b<64>(work, nblocks, reps, max_S, max_R, any_order0, stream);
     case 128: return launch_batch_b<128>(work, nblocks, reps, max_S, max_R, any_order0, stream);

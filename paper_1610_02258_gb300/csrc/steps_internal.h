@@ -92,7 +92,7 @@ int launch_flow_wait_test(const int32_t *d_off, const int32_t *d_nb, uint32_t *d
 int launch_nbr_wait_test(const uint32_t *d_done, const void *d_nbr, long long limit, uint32_t *d_status);
 int launch_add_u64(uint64_t *p, uint64_t v, void *stream);
 int launch_step_batch(const BlockWork *work, int64_t nblocks, RepEntry *reps, int max_S, int max_R,
-                      bool any_order0, int block, void *stream);
+                      bool any_order0, bool few, int block, void *stream);
 int launch_advance(RepEntry *reps, int32_t n, void *stream);
 
 // steps_spec.cpp: the plain and batched step kernels specialised for one

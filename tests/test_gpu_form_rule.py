@@ -77,3 +77,29 @@ def test_batch_above_a_wave_together(capi):
             _equal(g, o)
     assert b.specialized
     b.close()
+
+
+@pytest.mark.parametrize("per_tet", [0.3, 3.0])
+def test_run_time_batches_on_either_side_of_the_density(capi, per_tet):
+    """Members of 10 and 3 species on the kernels for models given at run time: block
+    tiles below half a molecule per tet, warp tiles above; then the other way."""
+    ws = [I.config2(seed=80, nx=3), I.config1(seed=81), I.config2(seed=82, nx=2)]
+    sims, refs = [], []
+    for w in ws:
+        sims.append(capi.Simulation(w.verts, w.tets, w.model, w.seed, specialize=-1))
+        refs.append(oracle.OracleSim(w.verts, w.tets, w.model, seed=w.seed, occ=oracle.OCC, prec=32))
+    b = capi.Batch(sims, block=128, specialize=-1)
+    for k, d in enumerate((per_tet, 3.3 - per_tet)):
+        for g, o in zip(sims, refs):
+            rng = np.random.default_rng(k)
+            c = np.zeros((g.S, g.nt), np.int32)
+            n = int(d * g.nt)
+            np.add.at(c, (rng.integers(0, g.S, n), rng.integers(0, g.nt, n)), 1)
+            g.set_counts(c)
+            o.set_counts(c)
+        ends = [o.time + 18.4 * o.tau for o in refs]
+        b.run(ends)
+        for g, o, t in zip(sims, refs, ends):
+            o.run(t)
+            _equal(g, o)
+    b.close()
