@@ -6,6 +6,8 @@
 #include <cstring>
 #include <limits>
 #include <algorithm>
+#include <future>
+#include <system_error>
 #include <map>
 #include <tuple>
 #include <memory>
@@ -923,7 +925,9 @@ struct steps_sim {
         const int64_t windows = tune_windows();
         if (windows == kFormTuneWindows && ensure_block()) {
             form[nc++] = 3;
-            for (int k = 2; k < 4; ++k)
+            // (512-tet tiles, another program to compile, are only faster where a
+            // window is few waves: 138,720 tets and 20 species 10.8 -> 9.1 us)
+            for (int k = 2; k < (T < kListMinTets ? 4 : 3); ++k)
                 if (ensure_flow(k) == STEPS_OK && flow[k].d_flow) form[nc++] = 2 + k;
         }
         flow_pick = 0;
@@ -1221,12 +1225,28 @@ int steps_sim_create(const steps_mesh *mesh, const steps_model *model, uint64_t 
     // the model-specialised step kernel (compiled once per model and block size)
     constexpr int64_t kSpecializeMinTets = 65536;
     if (s->opt.specialize > 0 || (s->opt.specialize == 0 && s->T >= kSpecializeMinTets)) {
+        // the second program of a model of many species, compiled beside the
+        // first (2.1 s each): the list form's, or on smaller meshes block tiles,
+        // for this simulation or a batch of its clones (on meshes that have the
+        // list form's they come on first use)
+        const bool many = s->S >= kListMinSpecies && s->opt.flow != 1;
+        const bool list = many && (s->forced ? s->forced == 2 : s->T >= kListMinTets);
+        const bool block = many && !list && s->T < kListMinTets && (s->opt.specialize > 0 || s->T > warp_wave(s->S));
+        std::future<void *> second;
+        if (list || block) try {
+                second = std::async(std::launch::async, [&s, list]() -> void * {
+                    cudaSetDevice(s->device);
+                    return list ? spec_list_kernel(s->model) : spec_block_kernel(s->model, 256);
+                });
+            } catch (const std::system_error &) {  // no thread: compiled when it is asked for below
+            }
         s->spec = spec_kernel(s->model, s->opt.block, &s->spec_why);
+        if (second.valid()) second.get();
         if (!s->spec && s->opt.specialize > 0) {
             set_error("steps_sim_create: the specialised step kernel could not be built: " + s->spec_why);
             return STEPS_ERR_CUDA;
         }
-        if (s->spec && s->opt.flow != 1 && (s->forced ? s->forced == 2 : s->T >= kListMinTets)) {
+        if (s->spec && list) {
             s->spec_list = spec_list_kernel(s->model);
             if (s->spec_list)
                 for (const steps_sim::Request &r : s->list_requests()) alloc(r.first, r.second);

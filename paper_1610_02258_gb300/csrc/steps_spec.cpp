@@ -305,34 +305,19 @@ std::string spec_program_source(const HostModel &hm, int block) { return program
 
 namespace {
 
-// Compiles (once per generated source) and loads a form's kernels.
-Compiled *compiled(const HostModel &hm, int block, Form form, std::string *why) {
-    Nvrtc &nv = nvrtc();
-    if (!nv.handle) {
-        if (why) *why = nv.why;
-        return nullptr;
-    }
-    const std::string src = form == Form::list    ? list_program_source(hm)
-                            : form == Form::block ? block_program_source(hm, block)
-                                                  : program_source(hm, block);
-    std::lock_guard<std::mutex> lock(g_mu);
-    auto it = g_cache.find(src);
-    if (it != g_cache.end()) {
-        if (!it->second && why) *why = "an earlier build of this kernel failed";
-        return it->second.get();
-    }
+// A generated program's binary, or nothing and why.
+std::vector<char> build_program(Nvrtc &nv, const std::string &src, std::string *why) {
+    std::vector<char> cubin;
     nvrtc_program prog = nullptr;
     const char *hdr_src[4] = {kSrcDeviceH, kSrcStepCuh, kSrcWarpCuh, kSrcListCuh};
     const char *hdr_name[4] = {"steps_device.h", "steps_step.cuh", "steps_warp.cuh", "steps_list.cuh"};
     if (nv.create(&prog, src.c_str(), "steps_spec.cu", 4, hdr_src, hdr_name) != 0) {
         if (why) *why = "nvrtcCreateProgram failed";
-        g_cache[src] = nullptr;
-        return nullptr;
+        return cubin;
     }
     // the generic kernels' flags: no contraction, C++17, this GPU only
     const char *opts[] = {"--gpu-architecture=sm_103a", "-std=c++17", "-fmad=false", "-lineinfo", "--device-int128"};
     const int rc = nv.compile(prog, 5, opts);
-    std::vector<char> cubin;
     if (rc == 0) {
         size_t n = 0;
         if (nv.cubin_size(prog, &n) == 0 && n > 0) {
@@ -347,6 +332,35 @@ Compiled *compiled(const HostModel &hm, int block, Form form, std::string *why) 
         *why = "NVRTC compile failed: " + lg.substr(0, 2000);
     }
     nv.destroy(&prog);
+    return cubin;
+}
+
+// Compiles (once per generated source) and loads a form's kernels. Compiled
+// without the lock, so that two programs of a model are at the same time.
+Compiled *compiled(const HostModel &hm, int block, Form form, std::string *why) {
+    Nvrtc &nv = nvrtc();
+    if (!nv.handle) {
+        if (why) *why = nv.why;
+        return nullptr;
+    }
+    const std::string src = form == Form::list    ? list_program_source(hm)
+                            : form == Form::block ? block_program_source(hm, block)
+                                                  : program_source(hm, block);
+    const auto known = [&](Compiled **c) {
+        auto it = g_cache.find(src);
+        if (it == g_cache.end()) return false;
+        if (!it->second && why) *why = "an earlier build of this kernel failed";
+        *c = it->second.get();
+        return true;
+    };
+    Compiled *done = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        if (known(&done)) return done;
+    }
+    const std::vector<char> cubin = build_program(nv, src, why);
+    std::lock_guard<std::mutex> lock(g_mu);
+    if (known(&done)) return done;
     if (cubin.empty()) {
         g_cache[src] = nullptr;
         return nullptr;
